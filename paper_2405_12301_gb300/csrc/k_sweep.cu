@@ -47,7 +47,9 @@ template <int M, int D, int DIR, bool BULK> struct Layout {
     static constexpr size_t fp_off = 0;
     static constexpr size_t fm_off = fp_off + sizeof(T) * NF * W * NP;
     static constexpr size_t F_off = fm_off + sizeof(T) * NF * W * NP;
-    static constexpr size_t ref_off = align16(F_off + sizeof(T) * NF * W * NI);
+    static constexpr int NS = BULK ? 1 : 2;   // face-flux copies: FP64 keeps WENO(+) and WENO(-) apart
+    static constexpr int RF = 9;              // faces per FP64 sliding run
+    static constexpr size_t ref_off = align16(F_off + sizeof(T) * NS * NF * W * NI);
     static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * W : 0);
 };
 
@@ -157,24 +159,45 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
     }
     __syncthreads();
 
-    // ---- phase B: interface fluxes, one work item per (interface, component)
-    for (int u = threadIdx.x; u < NF * W * NI; u += NT) {
-        const int f = u / (W * NI);
-        const int r = u - f * (W * NI);
-        int w, j;
-        if (DIR == 0) { w = r / NI; j = r - w * NI; }
-        else { j = r / W; w = r - j * W; }
-        if (c0 + j - 1 >= n) continue;  // right of the last cell's right face
-        const T *P = sfp + f * W * NP;
-        const T *M = sfm + f * W * NP;
-        const int pw = DIR == 0 ? w * NP : w;
-        const int ps = DIR == 0 ? 1 : W;
-        // interface between local cells j-1 and j: f+ at points j..j+4, f- mirrored at j+5..j+1
-        const T Fh = weno5<T>(P[pw + j * ps], P[pw + (j + 1) * ps], P[pw + (j + 2) * ps], P[pw + (j + 3) * ps],
-                              P[pw + (j + 4) * ps], eps) +
-                     weno5<T>(M[pw + (j + 5) * ps], M[pw + (j + 4) * ps], M[pw + (j + 3) * ps],
-                              M[pw + (j + 2) * ps], M[pw + (j + 1) * ps], eps);
-        sF[f * W * NI + (DIR == 0 ? w * NI + j : j * W + w)] = Fh;
+    // ---- phase B: interface fluxes.  FP64: a sliding run of RF faces per work item
+    // (line, segment, component, sign), WENO(+) and WENO(-) kept apart; FP32-bulk:
+    // one work item per (interface, component)
+    const int nfaces = n - c0 + 1 < NI ? n - c0 + 1 : NI;  // none right of the last cell's right face
+    if constexpr (!BULK) {
+        const PairEps P = pair_eps(eps);
+        constexpr int NSEG = (NI + L::RF - 1) / L::RF;
+        const int pst = DIR == 0 ? 1 : W;
+        for (int u = threadIdx.x; u < 2 * NF * W * NSEG; u += NT) {
+            const int w = u % W, seg_ = (u / W) % NSEG, fs = u / (W * NSEG);
+            const int j0 = seg_ * L::RF, cnt = nfaces - j0 < L::RF ? nfaces - j0 : L::RF;
+            long long base;
+            if (cnt <= 0 || !line(w, base)) continue;
+            const bool minus = fs >= NF;
+            const double *src = (minus ? sfm + (fs - NF) * W * NP : sfp + fs * W * NP) + (DIR == 0 ? w * NP : w);
+            double *dst = sF + fs * W * NI + (DIR == 0 ? w * NI : w);
+            // face j: f+ at points j..j+4, f- mirrored at j+5..j+1
+            if (minus) weno5_slide_pair<L::RF>(src + (j0 + cnt + 4) * pst, -pst, P, dst + (j0 + cnt - 1) * pst, -pst, cnt);
+            else weno5_slide_pair<L::RF>(src + j0 * pst, pst, P, dst + j0 * pst, pst, cnt);
+        }
+    } else {
+        for (int u = threadIdx.x; u < NF * W * NI; u += NT) {
+            const int f = u / (W * NI);
+            const int r = u - f * (W * NI);
+            int w, j;
+            if (DIR == 0) { w = r / NI; j = r - w * NI; }
+            else { j = r / W; w = r - j * W; }
+            if (j >= nfaces) continue;
+            const T *P = sfp + f * W * NP;
+            const T *M = sfm + f * W * NP;
+            const int pw = DIR == 0 ? w * NP : w;
+            const int ps = DIR == 0 ? 1 : W;
+            // interface between local cells j-1 and j: f+ at points j..j+4, f- mirrored at j+5..j+1
+            const T Fh = weno5<T>(P[pw + j * ps], P[pw + (j + 1) * ps], P[pw + (j + 2) * ps], P[pw + (j + 3) * ps],
+                                  P[pw + (j + 4) * ps], eps) +
+                         weno5<T>(M[pw + (j + 5) * ps], M[pw + (j + 4) * ps], M[pw + (j + 3) * ps],
+                                  M[pw + (j + 2) * ps], M[pw + (j + 1) * ps], eps);
+            sF[f * W * NI + (DIR == 0 ? w * NI + j : j * W + w)] = Fh;
+        }
     }
     __syncthreads();
 
@@ -201,7 +224,14 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
         const int jr = DIR == 0 ? jl + 1 : jl + W;
         T rd[NF];
 #pragma unroll
-        for (int f = 0; f < NF; ++f) rd[f] = -(sF[f * W * NI + jr] - sF[f * W * NI + jl]) * ih;
+        for (int f = 0; f < NF; ++f) {
+            if constexpr (BULK) {
+                rd[f] = -(sF[f * W * NI + jr] - sF[f * W * NI + jl]) * ih;
+            } else {
+                const T *Fp = sF + f * W * NI, *Fm = Fp + NF * W * NI;
+                rd[f] = -((Fp[jr] + Fm[jr]) - (Fp[jl] + Fm[jl])) * ih;
+            }
+        }
         T *acc = reinterpret_cast<T *>(a.acc);
         if (EPI == EPI_STORE) {
 #pragma unroll

@@ -11,10 +11,10 @@
 //      the directions that need them: each thread its own point in x and y, and
 //      one halo point in the halo's direction;
 //   W. every x- and y-interface flux of the tile is reconstructed once, WENO(+)
-//      plus mirrored WENO(-): in 2D as sliding runs along tile columns and row
-//      segments; in 3D planes each thread its cell's left and bottom faces for
-//      every component (FP32-bulk: a face's two windows as one f32x2 pair), and
-//      the tile's last column/row faces spread over the threads;
+//      plus mirrored WENO(-): in FP64 as sliding runs along tile columns and row
+//      segments (weights in FP32 pairs); in FP32-bulk 3D planes each thread its
+//      cell's left and bottom faces for every component, a face's two windows as
+//      one f32x2 pair, and the tile's last column/row faces spread over the threads;
 //   C. each thread forms -(dF/dx) - (dG/dy) for its cell (Sec. 4.1) and either
 //      stores it (3D: the z sweep adds its part and runs the stage), writes L(U),
 //      or applies the SSP-RK3 stage combination (Eq. tt-ssprk3 without rounding)
@@ -43,15 +43,15 @@ constexpr int NYI = TX * (TY + 1);          // y interfaces: 32 x 9
 constexpr int NHY = 6 * TX;                 // y-halo points (rows -3..-1, TY..TY+2)
 constexpr int NHALO = NHY + 6 * TY;         // plus x-halo points: 240
 
-// 2D grids reconstruct faces with sliding runs (one thread per line segment,
-// component and sign; WENO(+) and WENO(-) kept apart); 3D planes (five
-// components) one thread per cell.
-template <int D> constexpr bool slide() { return D == 2; }
+// FP64 reconstructs faces with sliding runs (one thread per line segment,
+// component and sign; WENO(+) and WENO(-) kept apart); the FP32-bulk 3D planes
+// one thread per cell.
+template <bool BULK> constexpr bool slide() { return !BULK; }
 
 template <int D, bool BULK> struct Layout {
     using T = typename std::conditional<BULK, float, double>::type;
     static constexpr int NF = D + 2;
-    static constexpr int NS = slide<D>() ? 2 : 1;                             // face-flux copies
+    static constexpr int NS = slide<BULK>() ? 2 : 1;                             // face-flux copies
     static constexpr size_t F_off = 0;                                        // Fx, Fy
     static constexpr size_t fx_off = (sizeof(T) * NS * NF * (NXI + NYI) + 15) & ~size_t(15);
     static constexpr size_t fy_off = fx_off + sizeof(T) * 2 * NF * NXP;
@@ -258,57 +258,37 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
     }
     __syncthreads();
 
-    // ---- phase W: own left x face and bottom y face for every component, plus
-    // one of the remaining faces (top of the tile's top row, right of its last column)
-    // the shared arrays hold 2 f(+/-): reconstruct with 4 eps (twice the WENO5 value)
+    // ---- phase W: FP64 sliding runs; FP32-bulk the own left x face and bottom y face
+    // for every component, plus one of the remaining faces (top of the tile's top
+    // row, right of its last column).  The shared arrays hold 2 f(+/-): reconstruct with 4 eps (twice the WENO5 value)
     const T eps = T(4) * (BULK ? (T)a.eps_f : (T)a.eps);
-    // (FP32: WENO(+) and the mirrored WENO(-) of a face as one f32x2 pair)
-    auto face_x = [&](int f, int ly, int j) -> T {  // between local columns j-1 and j of row ly
-        const T *P = fx + f * NXP + ly * BXP;
-        const T *M = fx + (NF + f) * NXP + ly * BXP;
-        if constexpr (BULK)
-            return weno5_pm(make_float2(P[j], M[j + 5]), make_float2(P[j + 1], M[j + 4]),
-                            make_float2(P[j + 2], M[j + 3]), make_float2(P[j + 3], M[j + 2]),
-                            make_float2(P[j + 4], M[j + 1]), eps);
-        else
-            return weno5<T>(P[j], P[j + 1], P[j + 2], P[j + 3], P[j + 4], eps) +
-                   weno5<T>(M[j + 5], M[j + 4], M[j + 3], M[j + 2], M[j + 1], eps);
-    };
-    auto face_y = [&](int f, int lx, int j) -> T {  // between local rows j-1 and j of column lx
-        const T *P = fy + f * NYP + lx;
-        const T *M = fy + (NF + f) * NYP + lx;
-        if constexpr (BULK)
-            return weno5_pm(make_float2(P[j * TX], M[(j + 5) * TX]), make_float2(P[(j + 1) * TX], M[(j + 4) * TX]),
-                            make_float2(P[(j + 2) * TX], M[(j + 3) * TX]), make_float2(P[(j + 3) * TX], M[(j + 2) * TX]),
-                            make_float2(P[(j + 4) * TX], M[(j + 1) * TX]), eps);
-        else
-            return weno5<T>(P[j * TX], P[(j + 1) * TX], P[(j + 2) * TX], P[(j + 3) * TX], P[(j + 4) * TX], eps) +
-                   weno5<T>(M[(j + 5) * TX], M[(j + 4) * TX], M[(j + 3) * TX], M[(j + 2) * TX], M[(j + 1) * TX], eps);
-    };
     T fxl[NF], fyb[NF];
-    if constexpr (slide<D>()) {
-        // Two runs of TY + 1 = 9 windows per thread, one code path (a single
-        // unrolled copy keeps the kernel inside the instruction cache):
-        //   y: column `lane`, component w & 3, sign w >> 2, faces 0..8;
-        //   x: row lane & 7, component lane >> 3, sign w >> 2, faces 8 s .. 8 s + 8
-        //      for s = w & 3 -- neighbouring segments share one face and write it
-        //      with the same value (each window is formed from its own five points).
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sg = w >> 2;
+    if constexpr (slide<BULK>()) {
+        // Runs of TY + 1 = 9 windows, one code path, spread over the threads:
+        //   y: column, component, sign, faces 0..8 (a warp's lanes are 32 columns);
+        //   x: row, 8-cell segment, component, sign, faces 8 s .. 8 s + 8 (a warp's
+        //      lanes are 8 rows x 4 runs) -- neighbouring segments share one face and
+        //      write it with the same value (each window is formed from its own five
+        //      points).
+        const PairEps P = pair_eps(eps);
+        constexpr int NRY = 2 * NF * TX, NRX = 2 * NF * TY * (TX / 8);
 #pragma unroll 1
-        for (int item = 0; item < 2; ++item) {
+        for (int run = threadIdx.x; run < NRY + NRX; run += NT) {
             const T *p;
             T *out;
-            int st, os;
-            if (item == 0) {
-                const int f = w & 3;
-                p = fy + (sg * NF + f) * NYP + lane;
-                out = Fy + (sg * NF + f) * NYI + lane;
+            int st, os, sg;
+            if (run < NRY) {
+                const int fs = run >> 5, lx = run & 31;
+                sg = fs >= NF;
+                p = fy + fs * NYP + lx;
+                out = Fy + fs * NYI + lx;
                 st = TX;
                 os = TX;
             } else {
-                const int ly = lane & 7, f = lane >> 3, j0 = (w & 3) * 8;
-                p = fx + (sg * NF + f) * NXP + ly * BXP + j0;
-                out = Fx + (sg * NF + f) * NXI + ly * (TX + 1) + j0;
+                const int u = run - NRY, ly = u & 7, j0 = ((u >> 3) & 3) * 8, fs = u >> 5;
+                sg = fs >= NF;
+                p = fx + fs * NXP + ly * BXP + j0;
+                out = Fx + fs * NXI + ly * (TX + 1) + j0;
                 st = 1;
                 os = 1;
             }
@@ -318,9 +298,24 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
                 st = -st;
                 os = -os;
             }
-            weno5_slide<T, TY + 1>(p, st, eps, out, os);
+            weno5_slide_pair<TY + 1>(p, st, P, out, os);
         }
     } else {
+        // WENO(+) and the mirrored WENO(-) of a face as one f32x2 pair
+        auto face_x = [&](int f, int ly, int j) -> T {  // between local columns j-1 and j of row ly
+            const T *P = fx + f * NXP + ly * BXP;
+            const T *M = fx + (NF + f) * NXP + ly * BXP;
+            return weno5_pm(make_float2(P[j], M[j + 5]), make_float2(P[j + 1], M[j + 4]),
+                            make_float2(P[j + 2], M[j + 3]), make_float2(P[j + 3], M[j + 2]),
+                            make_float2(P[j + 4], M[j + 1]), eps);
+        };
+        auto face_y = [&](int f, int lx, int j) -> T {  // between local rows j-1 and j of column lx
+            const T *P = fy + f * NYP + lx;
+            const T *M = fy + (NF + f) * NYP + lx;
+            return weno5_pm(make_float2(P[j * TX], M[(j + 5) * TX]), make_float2(P[(j + 1) * TX], M[(j + 4) * TX]),
+                            make_float2(P[(j + 2) * TX], M[(j + 3) * TX]), make_float2(P[(j + 3) * TX], M[(j + 2) * TX]),
+                            make_float2(P[(j + 4) * TX], M[(j + 1) * TX]), eps);
+        };
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             fxl[f] = face_x(f, ty, tx);
@@ -350,7 +345,7 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
         T dx, dy;
-        if constexpr (slide<D>()) {  // F^ = WENO(+) + WENO(-) at the right/top and left/bottom faces
+        if constexpr (slide<BULK>()) {  // F^ = WENO(+) + WENO(-) at the right/top and left/bottom faces
             const int ox = f * NXI + ty * (TX + 1) + tx, oy = f * NYI + ty * TX + tx;
             const T *FxM = Fx + NF * NXI, *FyM = Fy + NF * NYI;
             dx = (Fx[ox + 1] + FxM[ox + 1]) - (Fx[ox] + FxM[ox]);

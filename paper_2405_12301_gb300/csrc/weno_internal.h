@@ -54,8 +54,8 @@ cudaError_t sweep_set_attributes();
 cudaError_t launch_xy(int dim, bool bulk, int epi, const SweepArgs &a, cudaStream_t s);
 // 2D FP32-bulk residual / stage in pair-difference form (EPI_RHS / EPI_STAGE).
 cudaError_t launch_xy2(int epi, const SweepArgs &a, cudaStream_t s);
-// z direction of a 3D grid, adding the accumulator and ending the residual (EPI_RHS / EPI_STAGE).
-cudaError_t launch_z(bool bulk, int epi, const SweepArgs &a, cudaStream_t s);
+// z direction of a 3D FP64 grid, adding the accumulator and ending the residual (EPI_RHS / EPI_STAGE).
+cudaError_t launch_z(int epi, const SweepArgs &a, cudaStream_t s);
 // z direction of a 3D FP32-bulk grid in pair-difference form (EPI_RHS / EPI_STAGE).
 cudaError_t launch_z2(int epi, const SweepArgs &a, cudaStream_t s);
 
