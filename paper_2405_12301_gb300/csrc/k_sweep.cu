@@ -50,7 +50,9 @@ template <int M, int D, int DIR, bool BULK> struct Layout {
     static constexpr int NS = BULK ? 1 : 2;   // face-flux copies: FP64 keeps WENO(+) and WENO(-) apart
     static constexpr int RF = 9;              // faces per FP64 sliding run
     static constexpr size_t ref_off = align16(F_off + sizeof(T) * NS * NF * W * NI);
-    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * W : 0);
+    // FP32-bulk: the lines' reference states; FP64: the rough windows' list
+    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * W : sizeof(unsigned) * ROUGH_CAP);
+    static_assert(2 * NF * W * NP <= 8192 && 2 * NF * W * NI <= 8192, "offsets of a RoughList entry");
 };
 
 // Split fluxes f(+/-) = (f(u) +/- alpha u) / 2 of a scalar law (Eq. lax-friedrichs).
@@ -74,6 +76,9 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
     T *sfm = reinterpret_cast<T *>(smem + L::fm_off);
     T *sF = reinterpret_cast<T *>(smem + L::F_off);
     RefState<D> *sref = reinterpret_cast<RefState<D> *>(smem + L::ref_off);
+    __shared__ int s_rough;
+    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(smem + L::ref_off)};
+    if (!BULK && threadIdx.x == 0) s_rough = 0;
 
     const long long dtbits = __double_as_longlong(a.ctl->dt);
     if (a.check_dt && dtbits == 0) return;  // the step is a no-op (time reached t_end)
@@ -173,12 +178,14 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
             long long base;
             if (cnt <= 0 || !line(w, base)) continue;
             const bool minus = fs >= NF;
-            const double *src = (minus ? sfm + (fs - NF) * W * NP : sfp + fs * W * NP) + (DIR == 0 ? w * NP : w);
-            double *dst = sF + fs * W * NI + (DIR == 0 ? w * NI : w);
-            // face j: f+ at points j..j+4, f- mirrored at j+5..j+1
-            if (minus) weno5_slide_pair<L::RF>(src + (j0 + cnt + 4) * pst, -pst, P, dst + (j0 + cnt - 1) * pst, -pst, cnt);
-            else weno5_slide_pair<L::RF>(src + j0 * pst, pst, P, dst + j0 * pst, pst, cnt);
+            // face j: f+ at points j..j+4, f- mirrored at j+5..j+1 (sfm follows sfp)
+            const int jp = minus ? j0 + cnt + 4 : j0, jo = minus ? j0 + cnt - 1 : j0, st_ = minus ? -pst : pst;
+            const int po = fs * W * NP + (DIR == 0 ? w * NP : w) + jp * pst;
+            const int oo = fs * W * NI + (DIR == 0 ? w * NI : w) + jo * pst;
+            weno5_slide_pair<W>(sfp, po, st_, P, sF, oo, st_, cnt, rough);
         }
+        __syncthreads();
+        rough_windows<W>(rough, sfp, sF, P);
     } else {
         for (int u = threadIdx.x; u < NF * W * NI; u += NT) {
             const int f = u / (W * NI);
@@ -213,6 +220,8 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
     const float anf = a.stage == 0 ? 0.0f : (a.stage == 1 ? 0.75f : (float)(1.0 / 3.0));
     const float anf_lo = a.stage == 2 ? (float)(1.0 / 3.0 - (double)(float)(1.0 / 3.0)) : 0.0f;
     const float2 bdtf = BULK ? f64_to_f32x2(bn * dt) : make_float2(0.0f, 0.0f);
+    double qout[NF];
+    bool has = false;
     for (int u = threadIdx.x; u < W * S; u += NT) {
         int w, i;
         if (DIR == 0) { w = u / S; i = u - w * S; }
@@ -280,14 +289,31 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
 #pragma unroll
                     for (int f = 0; f < NF; ++f) qf[f] = f64_to_f32(out[f]);
                     cmaxf = fmaxf(cmaxf, wavespeed_f32<D>(qf, a.gamma_f, b));
-                } else {
-                    cmax = fmax(cmax, wavespeed_f64<D>(out, a.gamma, b));
+                } else {  // (one cell per thread: its speed is formed below)
+                    static_assert(M != MODEL_EULER || W * S <= NT, "one cell per thread");
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) qout[f] = out[f];
+                    has = true;
+                    b = false;
                 }
                 bad |= b;
             }
         }
     }
-    if (EPI == EPI_STAGE) {
+    if constexpr (EPI == EPI_STAGE && M == MODEL_EULER && !BULK) {
+        // 1D: |u_x| + a is the x slot's
+        const int K = a.per_dir ? 2 : 1;
+        auto load = [&](long long, double *q) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) q[f] = qout[f];
+        };
+        if (K == 2)
+            speed_max_publish_f64<D, 2>(load, 0, has ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out],
+                                        a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
+        else
+            speed_max_publish_f64<D, 1>(load, 0, has ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out],
+                                        a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
+    } else if (EPI == EPI_STAGE) {
         if (BULK) cmax = (double)cmaxf;
         block_max_publish(cmax, bad, &a.ctl->alpha[a.slot_out], &a.ctl->status);
         // 1D: |u_x| + a equals |u| + a, so the x slot takes the same maximum

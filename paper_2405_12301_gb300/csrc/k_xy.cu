@@ -55,8 +55,10 @@ template <int D, bool BULK> struct Layout {
     static constexpr size_t F_off = 0;                                        // Fx, Fy
     static constexpr size_t fx_off = (sizeof(T) * NS * NF * (NXI + NYI) + 15) & ~size_t(15);
     static constexpr size_t fy_off = fx_off + sizeof(T) * 2 * NF * NXP;
+    // FP32-bulk: the tile's reference state; FP64: the rough windows' list
     static constexpr size_t ref_off = (fy_off + sizeof(T) * 2 * NF * NYP + 15) & ~size_t(15);
-    static constexpr size_t bytes = ref_off + sizeof(RefState<D>);
+    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) : sizeof(unsigned) * ROUGH_CAP);
+    static_assert(BULK || (2 * NF * (NXP + NYP) <= 8192 && 2 * NF * (NXI + NYI) <= 8192), "offsets of a RoughList entry");
 };
 }  // namespace xy
 
@@ -79,6 +81,9 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
     T *fx = reinterpret_cast<T *>(smem + L::fx_off);       // [2][NF][TY][BXP]
     T *fy = reinterpret_cast<T *>(smem + L::fy_off);       // [2][NF][BY][TX]
     RefState<D> &ref = *reinterpret_cast<RefState<D> *>(smem + L::ref_off);
+    __shared__ int s_rough;
+    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(smem + L::ref_off)};
+    if (!BULK && threadIdx.x == 0) s_rough = 0;
 
     // dt and alpha come from the control block; the FP32 path converts them on
     // the integer pipe (a cvt issues at FP64 rate on this GPU)
@@ -274,32 +279,29 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
         constexpr int NRY = 2 * NF * TX, NRX = 2 * NF * TY * (TX / 8);
 #pragma unroll 1
         for (int run = threadIdx.x; run < NRY + NRX; run += NT) {
-            const T *p;
-            T *out;
-            int st, os, sg;
+            int po, oo, st, sg;  // offsets from fx and Fx (fy and Fy follow them)
             if (run < NRY) {
                 const int fs = run >> 5, lx = run & 31;
                 sg = fs >= NF;
-                p = fy + fs * NYP + lx;
-                out = Fy + fs * NYI + lx;
+                po = 2 * NF * NXP + fs * NYP + lx;
+                oo = 2 * NF * NXI + fs * NYI + lx;
                 st = TX;
-                os = TX;
             } else {
                 const int u = run - NRY, ly = u & 7, j0 = ((u >> 3) & 3) * 8, fs = u >> 5;
                 sg = fs >= NF;
-                p = fx + fs * NXP + ly * BXP + j0;
-                out = Fx + fs * NXI + ly * (TX + 1) + j0;
+                po = fs * NXP + ly * BXP + j0;
+                oo = fs * NXI + ly * (TX + 1) + j0;
                 st = 1;
-                os = 1;
             }
             if (sg) {  // WENO(-): the same run read backwards from the far end
-                p += (TY + 5) * st;
-                out += TY * os;
+                po += (TY + 5) * st;
+                oo += TY * st;
                 st = -st;
-                os = -os;
             }
-            weno5_slide_pair<TY + 1>(p, st, P, out, os);
+            weno5_slide_pair<TX>(fx, po, st, P, Fx, oo, st, TY + 1, rough);
         }
+        __syncthreads();
+        rough_windows<TX>(rough, fx, Fx, P);
     } else {
         // WENO(+) and the mirrored WENO(-) of a face as one f32x2 pair
         auto face_x = [&](int f, int ly, int j) -> T {  // between local columns j-1 and j of row ly
@@ -376,28 +378,23 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
     }
     // EPI_STAGE (FP64): U' = a_n U^n + b_n (U^k + dt R)
     if constexpr (!BULK) {
-        double cmax = 0.0, sd[D];
-#pragma unroll
-        for (int e = 0; e < D; ++e) sd[e] = 0.0;
-        bool bad = false;
+        double out[NF];
         if (own) {
             const double an = a.stage == 0 ? 0.0 : (a.stage == 1 ? 0.75 : 1.0 / 3.0);
             const double bn = a.stage == 0 ? 1.0 : (a.stage == 1 ? 0.25 : 2.0 / 3.0);
-            double out[NF];
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
                 const double sf = uk[f] + dt * r[f];
                 out[f] = a.stage == 0 ? sf : an * un[f] + bn * sf;
                 a.Uout[f * N + cell] = out[f];
             }
-            cmax = wavespeed_f64<D>(out, a.gamma, bad);
-            if (PD && !bad) dirspeeds_f64<D>(out, a.gamma, sd);
         }
-        block_max_publish(cmax, bad, &a.ctl->alpha[a.slot_out], &a.ctl->status);
-        if constexpr (PD) {
+        speed_max_publish_f64<D, PD ? 1 + D : 1>(
+            [&](long long, double *q) {
 #pragma unroll
-            for (int e = 0; e < D; ++e) block_max_publish(sd[e], false, &a.ctl->alpha_dir[a.slot_out][e], &a.ctl->status);
-        }
+                for (int f = 0; f < NF; ++f) q[f] = out[f];
+            },
+            0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
     }
 }
 

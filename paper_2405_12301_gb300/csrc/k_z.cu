@@ -22,7 +22,8 @@ constexpr int NZI = TX * (TZ + 1);          // z interfaces: 32 x 9
 constexpr int NHALO = 6 * TX;               // 192 halo points
 constexpr int NF = 5;
 constexpr size_t fz_off = sizeof(double) * 2 * NF * NZI;
-constexpr size_t bytes = fz_off + sizeof(double) * 2 * NF * NZP;
+constexpr size_t rough_off = fz_off + sizeof(double) * 2 * NF * NZP;
+constexpr size_t bytes = rough_off + sizeof(unsigned) * ROUGH_CAP;
 }  // namespace zs
 
 template <int EPI, bool PD>
@@ -32,6 +33,9 @@ __global__ void __launch_bounds__(zs::NT) k_z(const SweepArgs a)
     extern __shared__ __align__(16) unsigned char smem[];
     double *Fz = reinterpret_cast<double *>(smem);           // [2][NF][TZ+1][TX]
     double *fz = reinterpret_cast<double *>(smem + fz_off);  // [2][NF][BZ][TX]
+    __shared__ int s_rough;
+    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(smem + rough_off)};
+    if (threadIdx.x == 0) s_rough = 0;
 
     const double dt = a.ctl->dt;
     if (a.check_dt && __double_as_longlong(dt) == 0) return;
@@ -102,16 +106,16 @@ __global__ void __launch_bounds__(zs::NT) k_z(const SweepArgs a)
 #pragma unroll 1
         for (int run = threadIdx.x; run < 2 * NF * TX; run += NT) {
             const int fs = run >> 5, lx = run & 31;
-            const double *p = fz + fs * NZP + lx;
-            double *out = Fz + fs * NZI + lx;
-            int st = TX;
+            int po = fs * NZP + lx, oo = fs * NZI + lx, st = TX;
             if (fs >= NF) {  // WENO(-): the same run read backwards from the far end
-                p += (TZ + 5) * TX;
-                out += TZ * TX;
+                po += (TZ + 5) * TX;
+                oo += TZ * TX;
                 st = -TX;
             }
-            weno5_slide_pair<TZ + 1>(p, st, P, out, st);
+            weno5_slide_pair<TX>(fz, po, st, P, Fz, oo, st, TZ + 1, rough);
         }
+        __syncthreads();
+        rough_windows<TX>(rough, fz, Fz, P);
     }
     __syncthreads();
 
@@ -132,26 +136,23 @@ __global__ void __launch_bounds__(zs::NT) k_z(const SweepArgs a)
         }
         return;
     }
-    double cmax = 0.0, sd[3] = {0.0, 0.0, 0.0};
-    bool bad = false;
+    double out[NF];
     if (own) {
         const double an = a.stage == 0 ? 0.0 : (a.stage == 1 ? 0.75 : 1.0 / 3.0);
         const double bn = a.stage == 0 ? 1.0 : (a.stage == 1 ? 0.25 : 2.0 / 3.0);
-        double out[NF];
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             const double sf = uk[f] + dt * r[f];
             out[f] = a.stage == 0 ? sf : an * un[f] + bn * sf;
             a.Uout[f * N + cell] = out[f];
         }
-        cmax = wavespeed_f64<3>(out, a.gamma, bad);
-        if (PD && !bad) dirspeeds_f64<3>(out, a.gamma, sd);
     }
-    block_max_publish(cmax, bad, &a.ctl->alpha[a.slot_out], &a.ctl->status);
-    if constexpr (PD) {
+    speed_max_publish_f64<3, PD ? 4 : 1>(
+        [&](long long, double *q) {
 #pragma unroll
-        for (int e = 0; e < 3; ++e) block_max_publish(sd[e], false, &a.ctl->alpha_dir[a.slot_out][e], &a.ctl->status);
-    }
+            for (int f = 0; f < NF; ++f) q[f] = out[f];
+        },
+        0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
 }
 
 template <int EPI, bool PD>

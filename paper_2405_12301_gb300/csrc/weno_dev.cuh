@@ -177,54 +177,6 @@ __device__ __forceinline__ T weno5(T a, T b, T c, T d, T e, T eps)
     return c + div_<T>(num, T(6) * sw);
 }
 
-// WENO5 of K consecutive windows along a line, sharing what neighbouring
-// windows have in common: window m is (p[m s], ..., p[(m + 4) s]) and its value
-// goes to out[m os].  Moving to the next window drops the first point, so its
-// first differences D1..D3, second differences t1, t2 and the 13/12 t^2 parts
-// of beta_1, beta_2 are the previous window's D2..D4, t0, t1 and beta_0, beta_1
-// parts; each window loads one new point and forms one new difference of each
-// kind.  Every window's value is formed from its five points by the same
-// operations wherever it sits in the run (the first window forms its shared
-// terms directly from the same differences), so a face computed by two runs
-// gets bitwise the same value.  A negative stride s walks a line backwards,
-// which turns the run into the mirrored WENO(-) of the faces in reverse order.
-template <typename T, int K>
-__device__ __forceinline__ void weno5_slide(const T *p, int s, T eps, T *out, int os)
-{
-    const T k13 = T(13.0 / 12.0), q = T(0.25);
-    const T v0 = *p, v1 = *(p += s);
-    T c = *(p += s), d = *(p += s);
-    T D1 = v1 - v0, D2 = c - v1, D3 = d - c;
-    T t1 = D3 - D2, t2 = D2 - D1;
-    T A1 = fma(k13 * t1, t1, eps), A2 = fma(k13 * t2, t2, eps);
-#pragma unroll
-    for (int m = 0; m < K; ++m) {
-        const T e = *(p += s);
-        const T D4 = e - d;
-        const T t0 = D4 - D3;
-        const T A0 = fma(k13 * t0, t0, eps);
-        const T s0 = fma(T(-3), D3, D4), s1 = D2 + D3, s2 = fma(T(3), D2, -D1);
-        T g0 = fma(q * s0, s0, A0), g1 = fma(q * s1, s1, A1), g2 = fma(q * s2, s2, A2);
-        g0 *= g0;
-        g1 *= g1;
-        g2 *= g2;
-        const T w0 = T(0.3) * (g1 * g2), w1 = T(0.6) * (g0 * g2), w2 = T(0.1) * (g0 * g1);
-        const T sw = w0 + w1 + w2;
-        const T num = fma(w0, t1 - t0, fma(T(-2) * w2, t1 - t2, fma(T(2), D3, D2) * sw));
-        *out = c + div_<T>(num, T(6) * sw);
-        out += os;
-        D1 = D2;
-        D2 = D3;
-        D3 = D4;
-        t2 = t1;
-        t1 = t0;
-        A2 = A1;
-        A1 = A0;
-        c = d;
-        d = e;
-    }
-}
-
 // ------------------------------------------------- packed FP32 pairs (f32x2)
 // Two independent FP32 streams in one float2: a .f32x2 instruction takes one
 // issue slot for both operations (the FMA pipe still does two), which is what
@@ -447,6 +399,20 @@ __device__ __forceinline__ double f32_to_f64_nz(float f)
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+// 1 / x of a normal x below 2^1021: an FP32 reciprocal of the mantissa, two
+// Newton-Raphson steps r (2 - x r) (4 FP64 instructions; a division takes ~9).
+// Within an ulp: the last step's error term is exact to 2^-44.
+__device__ __forceinline__ double rcp_f64(double x)
+{
+    const unsigned h = (unsigned)__double2hiint(x);
+    const float m = __uint_as_float(0x3F800000u | (__funnelshift_l((unsigned)__double2loint(x), h, 3) & 0x7FFFFFu));
+    const double y = f32_to_f64_nz(fast_rcp(m));
+    double r = __hiloint2double((int)((unsigned)__double2hiint(y) - ((h & 0x7FF00000u) - 0x3FF00000u) | (h & 0x80000000u)),
+                                __double2loint(y));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
 // The smoothness parameter as the pair formula takes it.
 struct PairEps {
     double eps;
@@ -489,11 +455,12 @@ __device__ __forceinline__ double weno5_diffs(double D1, double D2, double D3, d
     return c + num / (6.0 * sw);
 }
 
-// One window: D1..D4 and the centre value c in FP64; f2, f3 the pairs of D2 and
+// One window: D2, D3 and the centre value c in FP64; f2, f3 the pairs of D2 and
 // D3; u_r and A_r those of t_r and (13/3) t_r^2 + 4 eps; e0 = u1 - u0, ep = u2 - u1.
-__device__ __forceinline__ double weno5_pair_core(double D1, double D2, double D3, double D4, double c, float2 f2,
-                                                  float2 f3, float2 u0, float2 u2, float2 A0, float2 A1, float2 A2,
-                                                  float2 e0, float2 ep, const PairEps &P)
+// rough: the value is not good and the window has to take the FP64 formula.
+__device__ __forceinline__ double weno5_pair_core(double D2, double D3, double c, float2 f2, float2 f3,
+                                                  float2 u0, float2 u2, float2 A0, float2 A1, float2 A2,
+                                                  float2 e0, float2 ep, const PairEps &P, bool &rough)
 {
     const float2 s0 = pr_add(u0, make_float2(-2.0f * f3.x, -2.0f * f3.y)), s1 = pr_add(f2, f3),
                  s2 = pr_add(u2, make_float2(2.0f * f2.x, 2.0f * f2.y));
@@ -526,9 +493,8 @@ __device__ __forceinline__ double weno5_pair_core(double D1, double D2, double D
     const float em = fabsf(p0.x) + fabsf(p2.x);
     const int emh = (int)((__float_as_uint(em) >> 3) + 0x38000000u);  // as the high word of a double
     const int ch = __double2hiint(c) & 0x7FFFFFFF;
-    const bool rough = (emh > P.thr && emh > ch - (7 << 20)) || (unsigned)(ch - 1) < (953u << 20) ||  // 0 < |c| < 2^-70
-                       !(mn > 0x1p-80f) || !(sum < 0x1p100f) || !(sum * sc < 0x1p66f);
-    if (rough) return weno5_diffs(D1, D2, D3, D4, c, P.eps);
+    rough = (emh > P.thr && emh > ch - (7 << 20)) || (unsigned)(ch - 1) < (953u << 20) ||  // 0 < |c| < 2^-70
+            !(mn > 0x1p-80f) || !(sum < 0x1p100f) || !(sum * sc < 0x1p66f);
     const float2 x = pr_norm(pr_add(p0, p2));
     const double X = (fma(2.0, D3, D2) + f32_to_f64_nz(x.y)) + f32_to_f64_nz(x.x);
     return fma(X, 1.0 / 6.0, c);
@@ -539,22 +505,57 @@ __device__ __forceinline__ double weno5_pair(double a, double b, double c, doubl
 {
     const double D1 = b - a, D2 = c - b, D3 = d - c, D4 = e - d;
     const float2 u0 = split_sat(D4 - D3), u1 = split_sat(D3 - D2), u2 = split_sat(D2 - D1);
-    return weno5_pair_core(D1, D2, D3, D4, c, split_sat(D2), split_sat(D3), u0, u2, pair_t2(u0, P.g),
-                           pair_t2(u1, P.g), pair_t2(u2, P.g), pr_sub(u1, u0), pr_sub(u2, u1), P);
+    bool rough;
+    const double v = weno5_pair_core(D2, D3, c, split_sat(D2), split_sat(D3), u0, u2, pair_t2(u0, P.g),
+                                     pair_t2(u1, P.g), pair_t2(u2, P.g), pr_sub(u1, u0), pr_sub(u2, u1), P, rough);
+    return rough ? weno5_diffs(D1, D2, D3, D4, c, P.eps) : v;
 }
 
-// K consecutive windows along a line, as weno5_slide: each window forms one new
-// difference of each kind, and its value is bitwise weno5_pair of its points.
-// The loop stays rolled: a window is ~280 instructions plus the FP64 formula.
-template <int K>
-__device__ __forceinline__ void weno5_slide_pair(const double *p, int s, const PairEps &P, double *out, int os,
-                                                 int count = K)
+// The rough windows of a block, gathered in shared memory and evaluated densely
+// after the runs: taking the FP64 formula inside a run would hold the FP64 pipe
+// for the whole warp whenever one lane needs it.  An entry is the offset of the
+// window's first point, the offset of its value, and which of the strides
+// +-1, +-S its points have.  What does not fit is evaluated in place.
+struct RoughList {
+    int *count;      // shared, zeroed before a barrier that precedes the runs
+    unsigned *list;  // shared, CAP entries
+};
+constexpr int ROUGH_CAP = 1024;
+
+template <int S>
+__device__ __forceinline__ void rough_windows(const RoughList &L, const double *src, double *dst, const PairEps &P)
 {
+    const int n = *L.count < ROUGH_CAP ? *L.count : ROUGH_CAP;
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+        const unsigned w = L.list[e];
+        const int s = (w >> 26 & 1u ? S : 1) * (w >> 27 & 1u ? -1 : 1);
+        const double *p = src + (w & 0x1FFFu);
+        const double a = p[0], b = p[s], c = p[2 * s], d = p[3 * s], f = p[4 * s];
+        dst[w >> 13 & 0x1FFFu] = weno5_diffs(b - a, c - b, d - c, f - d, c, P.eps);
+    }
+}
+
+// `count` consecutive windows along a line: window m is the points at
+// src[po + m s], .., src[po + (m + 4) s] and its value goes to dst[oo + m os].
+// Neighbouring windows share all differences but one of each kind, so each window
+// forms one new; its value is bitwise weno5_pair of its points wherever it sits in
+// a run, so a face that two runs form gets the same value.  A negative stride walks
+// a line backwards, which turns the run into the mirrored WENO(-) of the faces in
+// reverse order.
+// Offsets are below 2^13 and |s| is 1 or S.  The loop stays rolled: a window is
+// ~280 instructions.
+template <int S>
+__device__ __forceinline__ void weno5_slide_pair(const double *src, int po, int s, const PairEps &P, double *dst, int oo,
+                                                 int os, int count, const RoughList &L)
+{
+    const double *p = src + po;
+    double *out = dst + oo;
+    const unsigned kind = (s == S || s == -S ? 1u << 26 : 0u) | (s < 0 ? 1u << 27 : 0u);
     const double v0 = *p, v1 = *(p += s);
     double c = *(p += s), d = *(p += s);
-    double D1 = v1 - v0, D2 = c - v1, D3 = d - c;
+    double D2 = c - v1, D3 = d - c;
     float2 f2 = split_sat(D2), f3 = split_sat(D3);
-    float2 u1 = split_sat(D3 - D2), u2 = split_sat(D2 - D1);
+    float2 u1 = split_sat(D3 - D2), u2 = split_sat(D2 - (v1 - v0));
     float2 A1 = pair_t2(u1, P.g), A2 = pair_t2(u2, P.g), ep = pr_sub(u2, u1);
 #pragma unroll 1
     for (int m = 0; m < count; ++m) {
@@ -562,9 +563,20 @@ __device__ __forceinline__ void weno5_slide_pair(const double *p, int s, const P
         const double D4 = e - d;
         const float2 f4 = split_sat(D4), u0 = split_sat(D4 - D3);
         const float2 A0 = pair_t2(u0, P.g), e0 = pr_sub(u1, u0);
-        *out = weno5_pair_core(D1, D2, D3, D4, c, f2, f3, u0, u2, A0, A1, A2, e0, ep, P);
+        bool rough;
+        const double v = weno5_pair_core(D2, D3, c, f2, f3, u0, u2, A0, A1, A2, e0, ep, P, rough);
+        if (!rough) {
+            *out = v;
+        } else {
+            const int k = atomicAdd(L.count, 1);
+            if (k < ROUGH_CAP) {
+                L.list[k] = (unsigned)(p - 4 * s - src) | (unsigned)(out - dst) << 13 | kind;
+            } else {
+                const double b = p[-3 * s];
+                *out = weno5_diffs(b - p[-4 * s], D2, D3, D4, c, P.eps);
+            }
+        }
         out += os;
-        D1 = D2;
         D2 = D3;
         D3 = D4;
         f2 = f3;
@@ -590,16 +602,15 @@ template <int D, int DIR, bool TWICE = false>
 __device__ __forceinline__ void split_flux_f64(const double *q, double alpha, double gm1, double *fp, double *fm)
 {
     constexpr int NF = D + 2;
-    const double rho = q[0];
-    const double ir = 1.0 / rho;
+    const double ir = rcp_f64(q[0]);
     double u[D];
-    double ke = 0.0;
+    double mu = 0.0;
 #pragma unroll
     for (int e = 0; e < D; ++e) {
         u[e] = q[1 + e] * ir;
-        ke += u[e] * u[e];
+        mu = e == 0 ? q[1] * u[0] : fma(q[1 + e], u[e], mu);
     }
-    const double p = gm1 * (q[D + 1] - 0.5 * rho * ke);
+    const double p = gm1 * fma(-0.5, mu, q[D + 1]);
     double F[NF];
     F[0] = q[1 + DIR];
 #pragma unroll
@@ -796,6 +807,125 @@ __device__ __forceinline__ float wavespeed_f32(const float *q, float gamma, bool
     const float p = (gamma - 1.0f) * (q[D + 1] - 0.5f * rho * u2);
     bad = !(rho > 0.0f) || !(p > 0.0f) || !isfinite(u2) || !isfinite(q[D + 1]);
     return bad ? 0.0f : sqrt_approx(u2) + sqrt_approx(gamma * p * ir);
+}
+
+// FP32 estimates of the speeds of an FP64 state: est[0] = |u| + a and, for K > 1,
+// est[1 + e] = |u_e| + a.  Returns whether the state is certainly physical and the
+// estimates are within 2^-16 of the FP64 values: the conserved fields of ordinary
+// size and the internal energy at least 2^-5 of the total and kinetic energies
+// (its FP32 rounding is 2^-21 of those).
+template <int D, int K>
+__device__ __forceinline__ bool speed_estimate(const double *q, float gamma, float *est)
+{
+    float f[D + 2];
+#pragma unroll
+    for (int k = 0; k < D + 2; ++k) f[k] = f64_to_f32(q[k]);
+    const float ir = fast_rcp(f[0]);
+    float u2 = 0.0f;
+#pragma unroll
+    for (int e = 0; e < D; ++e) {
+        const float ue = f[1 + e] * ir;
+        u2 = fmaf(ue, ue, u2);
+    }
+    const float ke = 0.5f * f[0] * u2, ie = f[D + 1] - ke;
+    const float a = sqrt_approx(gamma * (gamma - 1.0f) * ie * ir);
+    est[0] = sqrt_approx(u2) + a;
+    if (K > 1) {
+#pragma unroll
+        for (int e = 0; e < D; ++e) est[1 + e] = fabsf(f[1 + e] * ir) + a;
+    }
+    // f64_to_f32 is meaningful below 2^128 only: test the FP64 exponents
+    bool in = true;
+#pragma unroll
+    for (int k = 0; k < D + 2; ++k) in = in && (__double2hiint(q[k]) & 0x7FFFFFFF) < (1123 << 20);  // |q| < 2^100
+    return in && f[0] > 1e-30f && ie > 0.03125f * (fabsf(f[D + 1]) + ke) && est[0] < 1e30f;
+}
+
+// max over the block of the FP64 speeds of its threads' states (K = 1: |u| + a
+// into *slot0; K = 1 + D also |u_e| + a into slot_dir[e]), published with one
+// atomicMax per block and value, and the block's non-physical flag.  load(i, q)
+// gives the states i = begin, begin + step, .. < end of the calling thread.  Only
+// states whose FP32 estimate is within 2^-14 of the block's largest, or that have
+// no estimate, get the FP64 speeds (two divisions and two square roots, ~60
+// FP64 instructions): the maximum is theirs, bit for bit.  Every thread of the
+// block must call it.
+template <int D, int K, class Load>
+__device__ __forceinline__ void speed_max_publish_f64(Load load, long long begin, long long end, long long step,
+                                                      double gamma, unsigned long long *slot0,
+                                                      unsigned long long *slot_dir, int *status)
+{
+    __shared__ unsigned s_est[K];
+    __shared__ unsigned long long s_max[K];
+    __shared__ int s_bad;
+    if (threadIdx.x < K) {
+        s_est[threadIdx.x] = 0u;
+        s_max[threadIdx.x] = 0ull;
+    }
+    if (threadIdx.x == 0) s_bad = 0;
+    const float gf = (float)gamma;
+    float mine[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) mine[k] = 0.0f;
+    bool unsure = false;
+    for (long long i = begin; i < end; i += step) {
+        double q[D + 2];
+        float est[K];
+        load(i, q);
+        if (speed_estimate<D, K>(q, gf, est)) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) mine[k] = fmaxf(mine[k], est[k]);
+        } else {
+            unsure = true;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const unsigned m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mine[k]));
+        if ((threadIdx.x & 31) == 0 && m) atomicMax(s_est + k, m);
+    }
+    __syncthreads();
+    float thr[K];
+    bool need = unsure;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        thr[k] = __uint_as_float(s_est[k]) * (1.0f - 0x1p-14f);
+        need = need || (mine[k] > 0.0f && mine[k] >= thr[k]);
+    }
+    if (__any_sync(0xFFFFFFFFu, need)) {
+        unsigned long long best[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) best[k] = 0ull;
+        if (need) {
+            for (long long i = begin; i < end; i += step) {
+                double q[D + 2], v[K];
+                float est[K];
+                load(i, q);
+                bool go = !speed_estimate<D, K>(q, gf, est), bad;
+#pragma unroll
+                for (int k = 0; k < K; ++k) go = go || est[k] >= thr[k];
+                if (!go) continue;
+                v[0] = wavespeed_f64<D>(q, gamma, bad);
+                if (K > 1) dirspeeds_f64<D>(q, gamma, v + (K > 1));
+                if (bad) {
+                    s_bad = 1;
+                    continue;
+                }
+#pragma unroll
+                for (int k = 0; k < K; ++k) best[k] = max(best[k], (unsigned long long)__double_as_longlong(v[k]));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {  // the warp's maximum on the integer pipe: high words, then low words among them
+            const unsigned hi = (unsigned)(best[k] >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+            const unsigned ml = __reduce_max_sync(0xFFFFFFFFu, hi == mh ? (unsigned)best[k] : 0u);
+            if ((threadIdx.x & 31) == 0 && (mh | ml)) atomicMax(s_max + k, (unsigned long long)mh << 32 | ml);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < K && s_max[threadIdx.x])
+        atomicMax(threadIdx.x == 0 ? slot0 : slot_dir + (threadIdx.x - 1), s_max[threadIdx.x]);
+    if (threadIdx.x == 0 && s_bad) atomicOr(status, ST_NONPHYSICAL);
 }
 
 // FP32 variant for the FP32-bulk kernels: the max runs on the bit patterns of
