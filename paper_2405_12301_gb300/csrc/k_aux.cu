@@ -83,21 +83,10 @@ __global__ void k_copy_alpha(const Ctl *ctl, int slot, double *out)
 // the current call is spent.  Clears the stage alpha slots 1..3.
 __global__ void k_step_begin(Ctl *c)
 {
-    const double t = c->t, te = c->t_end;
-    const double alpha = __longlong_as_double((long long)c->alpha[0]);
-    double dt = c->dt_req > 0.0 ? c->dt_req : c->cfl_h / alpha;
-    double tn = t + dt;
-    if (!(dt > 0.0) || !isfinite(dt)) {
-        if (t < te && c->steps < c->max_steps) atomicOr(&c->status, ST_NONPHYSICAL);
-        dt = 0.0;
-        tn = t;
-    } else if (!(t < te) || c->steps >= c->max_steps) {
-        dt = 0.0;
-        tn = t;
-    } else if (tn >= te) {
-        dt = te - t;
-        tn = te;
-    }
+    double dt, tn;
+    if (next_dt(c->t, c->t_end, c->dt_req, c->cfl_h, __longlong_as_double((long long)c->alpha[0]), c->steps,
+                c->max_steps, dt, tn))
+        atomicOr(&c->status, ST_NONPHYSICAL);
     c->dt = dt;
     c->t_next = tn;
     c->bdt[0] = f64_to_f32x2(dt);

@@ -213,12 +213,10 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
     double cmax = 0.0;
     float cmaxf = 0.0f;
     bool bad = false;
-    // stage combination coefficients (Eq. tt-ssprk3): U' = a_n U^n + b_n (U^k + dt R)
-    const double an = a.stage == 0 ? 0.0 : (a.stage == 1 ? 0.75 : 1.0 / 3.0);
-    const double bn = a.stage == 0 ? 1.0 : (a.stage == 1 ? 0.25 : 2.0 / 3.0);
-    // FP32-bulk: a_n and b_n dt as hi + lo pairs (no systematic coefficient rounding)
+    // FP32-bulk: the stage combination U' = a_n U^n + b_n (U^k + dt R) (Eq. tt-ssprk3) with a_n and b_n dt as hi + lo pairs (no systematic coefficient rounding)
     const float anf = a.stage == 0 ? 0.0f : (a.stage == 1 ? 0.75f : (float)(1.0 / 3.0));
     const float anf_lo = a.stage == 2 ? (float)(1.0 / 3.0 - (double)(float)(1.0 / 3.0)) : 0.0f;
+    const double bn = a.stage == 0 ? 1.0 : (a.stage == 1 ? 0.25 : 2.0 / 3.0);
     const float2 bdtf = BULK ? f64_to_f32x2(bn * dt) : make_float2(0.0f, 0.0f);
     double qout[NF];
     bool has = false;
@@ -275,8 +273,7 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
                         }
                         out[f] = uk + f32_to_f64(dlt);
                     } else {
-                        const double s = uk + dt * r[f];
-                        out[f] = a.stage == 0 ? s : an * a.Un[f * N + cell] + bn * s;
+                        out[f] = stage_combine(a.stage, a.stage == 0 ? 0.0 : a.Un[f * N + cell], uk, r[f], dt);
                     }
                     a.Uout[f * N + cell] = out[f];
                 }

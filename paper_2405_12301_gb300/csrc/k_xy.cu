@@ -380,12 +380,9 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
     if constexpr (!BULK) {
         double out[NF];
         if (own) {
-            const double an = a.stage == 0 ? 0.0 : (a.stage == 1 ? 0.75 : 1.0 / 3.0);
-            const double bn = a.stage == 0 ? 1.0 : (a.stage == 1 ? 0.25 : 2.0 / 3.0);
-#pragma unroll
+        #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                const double sf = uk[f] + dt * r[f];
-                out[f] = a.stage == 0 ? sf : an * un[f] + bn * sf;
+                out[f] = stage_combine(a.stage, un[f], uk[f], r[f], dt);
                 a.Uout[f * N + cell] = out[f];
             }
         }

@@ -286,8 +286,19 @@ static int enqueue_sweeps(weno_ctx *h, SweepArgs a, int last, cudaStream_t s)
 
 // One SSP-RK3 step (Eq. tt-ssprk3 without rounding) on U in place; alpha(U^n)
 // must be in slot 0.  Capturable: no host synchronisation.
+// small 1D FP64 Euler grids run whole steps inside one kernel
+static bool runs_1d(const weno_ctx *h)
+{
+    return h->dim == 1 && !bulk(h) && h->p.model == WENO_MODEL_EULER && run1d_takes(h->n[0]);
+}
+
 static int enqueue_step(weno_ctx *h, double *U, cudaStream_t s)
 {
+    if (runs_1d(h)) {
+        const SweepArgs a = base_args(h);
+        CK(h, launch(h, 3, s, [&] { return launch_run1d(a, U, 1, s); }));
+        return WENO_OK;
+    }
     CK(h, launch(h, 7, s, [&] { return launch_step_begin(h->ctl, s); }));
     double *in[3] = {U, h->S1, h->S2};
     double *outs[3] = {h->S1, h->S2, U};
@@ -462,9 +473,13 @@ extern "C" int weno_run(weno_handle h, double *U, double t_end, double dt, int64
     if ((r = read_ctl(h))) return r;
     const long long s0 = h->ctl_host->steps;
     const int chunk = graph_steps > 0 ? graph_steps : 8;
-    if (graph_steps > 0 && (r = ensure_graph(h, U, graph_steps))) return r;
+    const bool one_kernel = graph_steps > 0 && runs_1d(h);  // a launch of graph_steps steps, no graph
+    if (graph_steps > 0 && !one_kernel && (r = ensure_graph(h, U, graph_steps))) return r;
     for (;;) {
-        if (graph_steps > 0) {
+        if (one_kernel) {
+            const SweepArgs a = base_args(h);
+            CK(h, launch(h, 3, h->stream, [&] { return launch_run1d(a, U, graph_steps, h->stream); }));
+        } else if (graph_steps > 0) {
             CK(h, cudaGraphLaunch(h->gexec, h->stream));
             h->launches += h->g_kernels;
         } else {

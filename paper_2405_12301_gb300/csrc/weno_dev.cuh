@@ -729,6 +729,39 @@ __device__ __forceinline__ void split_flux_diff(const float *dq, const RefState<
     }
 }
 
+// The SSP-RK3 stage combination in FP64, U' = a_n U^n + b_n (U^k + dt R) (stage 0:
+// U + dt R), with its roundings fixed so that every kernel gives the same bits.
+__device__ __forceinline__ double stage_combine(int stage, double un, double uk, double r, double dt)
+{
+    const double s = fma(dt, r, uk);
+    if (stage == 0) return s;
+    return fma(stage == 1 ? 0.25 : 2.0 / 3.0, s, __dmul_rn(stage == 1 ? 0.75 : 1.0 / 3.0, un));
+}
+
+// dt of the next step from alpha(U^n) (or the fixed dt), shortened so that the
+// time lands exactly on t_end; zero when the time is up or the step budget of the
+// current call is spent.  Returns whether the step is impossible (a dt that is not
+// a positive finite number while steps are wanted).
+__device__ __forceinline__ bool next_dt(double t, double t_end, double dt_req, double cfl_h, double alpha,
+                                        long long steps, long long max_steps, double &dt, double &t_next)
+{
+    dt = dt_req > 0.0 ? dt_req : cfl_h / alpha;
+    t_next = t + dt;
+    if (!(dt > 0.0) || !isfinite(dt)) {
+        dt = 0.0;
+        t_next = t;
+        return t < t_end && steps < max_steps;
+    }
+    if (!(t < t_end) || steps >= max_steps) {
+        dt = 0.0;
+        t_next = t;
+    } else if (t_next >= t_end) {
+        dt = t_end - t;
+        t_next = t_end;
+    }
+    return false;
+}
+
 // ------------------------------------------------------------- wavespeed
 
 // |u| + sqrt(gamma p / rho) in FP64 with the operation order of the plain
@@ -842,26 +875,23 @@ __device__ __forceinline__ bool speed_estimate(const double *q, float gamma, flo
 }
 
 // max over the block of the FP64 speeds of its threads' states (K = 1: |u| + a
-// into *slot0; K = 1 + D also |u_e| + a into slot_dir[e]), published with one
-// atomicMax per block and value, and the block's non-physical flag.  load(i, q)
-// gives the states i = begin, begin + step, .. < end of the calling thread.  Only
+// into s_max[0]; K = 1 + D also |u_e| + a into s_max[1 + e]) as bit patterns, and
+// its non-physical flag into *s_bad, in shared memory; the caller's next barrier
+// makes them visible.  load(i, q) gives the states i = begin, begin + step, .. < end of the calling thread.  Only
 // states whose FP32 estimate is within 2^-14 of the block's largest, or that have
 // no estimate, get the FP64 speeds (two divisions and two square roots, ~60
 // FP64 instructions): the maximum is theirs, bit for bit.  Every thread of the
 // block must call it.
 template <int D, int K, class Load>
-__device__ __forceinline__ void speed_max_publish_f64(Load load, long long begin, long long end, long long step,
-                                                      double gamma, unsigned long long *slot0,
-                                                      unsigned long long *slot_dir, int *status)
+__device__ __forceinline__ void speed_max_block_f64(Load load, long long begin, long long end, long long step,
+                                                    double gamma, unsigned long long *s_max, int *s_bad)
 {
     __shared__ unsigned s_est[K];
-    __shared__ unsigned long long s_max[K];
-    __shared__ int s_bad;
     if (threadIdx.x < K) {
         s_est[threadIdx.x] = 0u;
         s_max[threadIdx.x] = 0ull;
     }
-    if (threadIdx.x == 0) s_bad = 0;
+    if (threadIdx.x == 0) *s_bad = 0;
     const float gf = (float)gamma;
     float mine[K];
 #pragma unroll
@@ -908,7 +938,7 @@ __device__ __forceinline__ void speed_max_publish_f64(Load load, long long begin
                 v[0] = wavespeed_f64<D>(q, gamma, bad);
                 if (K > 1) dirspeeds_f64<D>(q, gamma, v + (K > 1));
                 if (bad) {
-                    s_bad = 1;
+                    *s_bad = 1;
                     continue;
                 }
 #pragma unroll
@@ -922,6 +952,18 @@ __device__ __forceinline__ void speed_max_publish_f64(Load load, long long begin
             if ((threadIdx.x & 31) == 0 && (mh | ml)) atomicMax(s_max + k, (unsigned long long)mh << 32 | ml);
         }
     }
+}
+
+// The same, published: one atomicMax per block and value, K = 1: *slot0, K > 1
+// also slot_dir[e].
+template <int D, int K, class Load>
+__device__ __forceinline__ void speed_max_publish_f64(Load load, long long begin, long long end, long long step,
+                                                      double gamma, unsigned long long *slot0,
+                                                      unsigned long long *slot_dir, int *status)
+{
+    __shared__ unsigned long long s_max[K];
+    __shared__ int s_bad;
+    speed_max_block_f64<D, K>(load, begin, end, step, gamma, s_max, &s_bad);
     __syncthreads();
     if (threadIdx.x < K && s_max[threadIdx.x])
         atomicMax(threadIdx.x == 0 ? slot0 : slot_dir + (threadIdx.x - 1), s_max[threadIdx.x]);

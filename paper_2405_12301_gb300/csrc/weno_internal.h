@@ -50,6 +50,10 @@ struct SweepArgs {
 // Launches the sweep of direction dir for a dim-dimensional grid.
 cudaError_t launch_sweep(int model, int dim, int dir, bool bulk, int epi, const SweepArgs &a, cudaStream_t s);
 cudaError_t sweep_set_attributes();
+// nsteps whole SSP-RK3 steps of a small 1D FP64 Euler grid on U in place; alpha(U)
+// must be in slot 0 (k_run1d.cu).
+bool run1d_takes(long long n);
+cudaError_t launch_run1d(const SweepArgs &a, double *U, int nsteps, cudaStream_t s);
 // Fused x+y residual of a 2D grid (EPI_RHS / EPI_STAGE) or of the z-planes of a 3D grid (EPI_STORE).
 cudaError_t launch_xy(int dim, bool bulk, int epi, const SweepArgs &a, cudaStream_t s);
 // 2D FP32-bulk residual / stage in pair-difference form (EPI_RHS / EPI_STAGE).
