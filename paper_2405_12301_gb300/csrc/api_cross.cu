@@ -11,7 +11,7 @@ namespace {
 struct CrossPrep {
     std::vector<CrossInst> ci;
     std::vector<CrossSet> cs;
-    long long work = 0, nvec = 0, samples = 0;
+    long long work = 0, fixed = 0, nvec = 0, samples = 0;
     int fp64 = 0, max_rank = 1;
     size_t off_inst = 0, off_sets = 0, off_vecs = 0, bytes = 0;
     std::string key;  // workload class of the autotuner
@@ -70,9 +70,7 @@ static int cross_prepare(weno_ctx *h, const weno_tt_instance *inst, int32_t n_in
         c.left = F.left;
         c.right = F.right;
         c.out = F.out;
-        c.work_begin = P.work;
-        // a work item fixes the index of the side the stencil does not move
-        P.work += F.flux_dir > F.mode ? F.n_left : F.n_right;
+        P.fixed += F.flux_dir > F.mode ? F.n_left : F.n_right;  // indices of the side the stencil does not move
         P.samples += F.n_left * F.n_right * c.n_mode;
         c.nsl = F.flux_dir < F.mode ? 7 : 1;
         c.nsr = F.flux_dir > F.mode ? 7 : 1;
@@ -81,7 +79,7 @@ static int cross_prepare(weno_ctx *h, const weno_tt_instance *inst, int32_t n_in
         c.rvec_off = P.nvec;
         P.nvec += F.n_right * c.nsr * 5 * cross_vec_len();
     }
-    if (P.work >= (1ll << 31)) return fail(h, WENO_ERR_ARG, "weno_cross_eval: more than 2^31 work items");
+    if (P.fixed >= (1ll << 31)) return fail(h, WENO_ERR_ARG, "weno_cross_eval: more than 2^31 fibers");
     P.fp64 = (flags & WENO_CROSS_FP64_CHECK) ? 1 : 0;
     const size_t esz = P.fp64 ? sizeof(double) : sizeof(float);
     P.off_inst = 64 + ((sizeof(int) * n_sets + 15) & ~size_t(15));
@@ -96,9 +94,11 @@ static int cross_prepare(weno_ctx *h, const weno_tt_instance *inst, int32_t n_in
     return WENO_OK;
 }
 
-// Descriptor upload and the launch arguments for scratch at `base`.
-static int cross_upload(weno_ctx *h, const CrossPrep &P, char *base, cudaStream_t s, CrossArgs &a)
+// The sets' work items for a kernel variant, descriptor upload and the launch
+// arguments for scratch at `base`.
+static int cross_upload(weno_ctx *h, CrossPrep &P, int variant, char *base, cudaStream_t s, CrossArgs &a)
 {
+    P.work = cross_plan(P.cs.data(), (int)P.cs.size(), P.fp64 != 0, variant);
     unsigned long long *counter = (unsigned long long *)base;
     int *dbad = (int *)(base + 64);
     CrossInst *dinst = (CrossInst *)(base + P.off_inst);
@@ -121,10 +121,10 @@ static int cross_upload(weno_ctx *h, const CrossPrep &P, char *base, cudaStream_
     return WENO_OK;
 }
 
-static void cross_config(const weno_ctx *h, const std::string &key, int &variant, int &cpsm)
+static void cross_config(const weno_ctx *h, const CrossPrep &P, int &variant, int &cpsm)
 {
-    cross_default(&variant, &cpsm);
-    auto it = h->tune.find(key);
+    cross_default(P.fp64 != 0, &variant, &cpsm);
+    auto it = h->tune.find(P.key);
     if (it != h->tune.end()) {
         variant = it->second.first;
         cpsm = it->second.second;
@@ -146,7 +146,7 @@ extern "C" int weno_cross_eval(weno_handle h, const weno_tt_instance *inst, int3
     int r = cross_prepare(h, inst, n_inst, sets, n_sets, flags, P);
     if (r) return r;
     int variant, cpsm;
-    cross_config(h, P.key, variant, cpsm);
+    cross_config(h, P, variant, cpsm);
     if (flags & WENO_CROSS_GRAPH) {
         // replay the graph captured for these exact descriptors (the device
         // arrays they point to may have new contents), or capture it now
@@ -169,7 +169,7 @@ extern "C" int weno_cross_eval(weno_handle h, const weno_tt_instance *inst, int3
         g.key = key;
         CK(h, cudaMalloc(&g.buf, P.bytes));
         CrossArgs a;
-        if ((r = cross_upload(h, P, (char *)g.buf, h->stream, a))) {
+        if ((r = cross_upload(h, P, variant, (char *)g.buf, h->stream, a))) {
             cudaFree(g.buf);
             return r;
         }
@@ -206,7 +206,7 @@ extern "C" int weno_cross_eval(weno_handle h, const weno_tt_instance *inst, int3
     }
     if ((r = grow(h, &h->xbuf, &h->xbuf_bytes, P.bytes))) return r;
     CrossArgs a;
-    if ((r = cross_upload(h, P, (char *)h->xbuf, h->stream, a))) return r;
+    if ((r = cross_upload(h, P, variant, (char *)h->xbuf, h->stream, a))) return r;
     CK(h, cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), h->stream));
     CK(h, launch(h, 7, h->stream, [&] { return launch_cross(a, variant, cpsm, h->stream); }, 2));
     return WENO_OK;
@@ -224,14 +224,14 @@ extern "C" int weno_cross_autotune(weno_handle h, const weno_tt_instance *inst, 
     int r = cross_prepare(h, inst, n_inst, sets, n_sets, flags, P);
     if (r) return r;
     if ((r = grow(h, &h->xbuf, &h->xbuf_bytes, P.bytes))) return r;
-    CrossArgs a;
-    if ((r = cross_upload(h, P, (char *)h->xbuf, h->stream, a))) return r;
     cudaEvent_t e0, e1;
     CK(h, cudaEventCreate(&e0));
     CK(h, cudaEventCreate(&e1));
     double best = 1e300;
     int bv = 0, bc = 4;
-    for (int v = 0; v < cross_num_variants(); ++v)
+    for (int v = 0; v < cross_num_variants(); ++v) {
+        CrossArgs a;
+        if ((r = cross_upload(h, P, v, (char *)h->xbuf, h->stream, a))) return r;
         for (int c = 1; c <= 4; ++c) {
             for (int k = 0; k <= reps; ++k) {  // the first run is a warm-up
                 if (k == 1) CK(h, cudaEventRecord(e0, h->stream));
@@ -248,6 +248,7 @@ extern "C" int weno_cross_autotune(weno_handle h, const weno_tt_instance *inst, 
                 bc = c;
             }
         }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     h->tune[P.key] = std::make_pair(bv, bc);

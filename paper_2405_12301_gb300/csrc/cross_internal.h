@@ -23,6 +23,7 @@ struct CrossSet {
     const int *right;
     void *out;
     long long work_begin;  // first work item of this set (prefix sum)
+    int jb, rows;          // fixed indices and rows of a work item (cross_plan)
     int nsl, nsr;          // shifted copies stored per left / right vector (7 or 1)
     long long lvec_off, rvec_off;  // element offsets of the set's vectors in CrossArgs::vecs
 };
@@ -47,7 +48,9 @@ int cross_max_rank();
 int cross_vec_len();
 int cross_num_variants();
 // The configuration used until the autotuner has timed a workload class.
-void cross_default(int *variant, int *ctas_per_sm);
+void cross_default(bool fp64, int *variant, int *ctas_per_sm);
+// Splits every set into work items for a variant (sets jb, rows, work_begin); returns their number.
+long long cross_plan(CrossSet *sets, int n_sets, bool fp64, int variant);
 void cross_variant(int v, int *threads, int *chunk);
 cudaError_t cross_set_attributes();
 

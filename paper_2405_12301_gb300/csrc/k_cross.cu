@@ -14,15 +14,21 @@
 //                 the 7 shifted ones where the stencil moves that side (FP32:
 //                 stored as differences from the centre vector, so rounding
 //                 scales with the variation along the stencil);
-//   k_cross       persistent; a work item fixes one index of the side the
-//                 stencil does not move (r for fd <= m, l for fd > m).  For each
-//                 chunk of samples (32 to 128, per variant) it contracts the
-//                 core rows G_m(i) with that fixed vector once into shared
-//                 memory; every sample (v, i) of the other side's index v
-//                 then needs only 7 dot products per field, followed by the
-//                 LF split fluxes at the 7 points and WENO5(+/-) at the two
-//                 interfaces of the sample.
+//   k_cross       persistent; a work item is a chunk of rows i of the core and a
+//                 block of one to four indices of the side the stencil does not
+//                 move (r for fd <= m, l for fd > m), small enough that the items
+//                 of the largest fiber set do not outlast the rest (cross_plan).
+//                 It contracts the core rows G_m(i) with the block's vectors once
+//                 into shared memory; every sample (v, i) of the other side's
+//                 index v then needs only 7 dot products per field, followed by
+//                 the LF split fluxes at the 7 points and WENO5(+/-) at the two
+//                 interfaces of the sample.  Where the stencil moves along the
+//                 fiber (fd = m) neighbouring samples share points and interfaces,
+//                 so those are formed once per chunk and varying index.
 // Ghost rows (Sec. 4.5) are mapped by the boundary rule of fd.
+#include <algorithm>
+#include <type_traits>
+
 #include "weno_dev.cuh"
 #include "weno_internal.h"
 #include "cross_internal.h"
@@ -32,20 +38,25 @@ namespace wg {
 constexpr int XT = 256;       // threads per CTA of k_cross_vecs
 constexpr int VP = 32;        // padded vector length (largest rank)
 constexpr int CS = VP + 4;    // shared-memory row stride: float4 reads of 8 consecutive rows hit distinct banks
-// FP32, stencil along the fiber: varying indices per block of the point-flux
-// path, so that each of its phases is one pass of the CTA's threads
-constexpr int fiber_vb(int threads, int chunk) { return threads / (chunk + 6) > 0 ? threads / (chunk + 6) : 1; }
-constexpr int FLS = 11;       // floats per point of the fiber path's split fluxes (10, padded odd:
+constexpr int JB = 4;         // fixed indices per work item at most
+constexpr int SP = 9;         // pitch of a warp's staged 32 x 8 piece of a core row's matrix
+constexpr int FLS = 11;       // values per point of the fiber path's split fluxes (10, padded odd:
                               // consecutive points of a warp fall on distinct banks)
 // k_cross is compiled for several (threads per CTA, samples per chunk) pairs;
 // the autotuner of api_cross.cu picks one, and the persistent grid size, per
-// workload class.  Until then variant 5 at 3 CTAs per SM runs: held to 80
+// workload class.  Until then variant 5 at 3 CTAs per SM runs (FP32): held to 80
 // registers it keeps 24 warps per SM, where the unbounded builds (225
-// registers) fit one CTA per SM whatever grid is asked for.
+// registers) fit one CTA per SM whatever grid is asked for; FP64, bound by its
+// pipe, takes the variant whose shared memory lets two CTAs share an SM.
 // minb > 1 asks the compiler for registers that fit minb CTAs per SM.
 struct CrossVariant { int threads, chunk, minb; };
 constexpr CrossVariant kCrossVariants[] = {{256, 64, 1}, {256, 32, 1}, {128, 64, 1}, {128, 32, 1},
                                            {256, 128, 1}, {256, 64, 3}, {128, 64, 6}};
+// rows of an FP64 chunk: at most 96 (shared memory)
+constexpr int variant_chunk(bool f64, int v)
+{
+    return f64 && kCrossVariants[v].chunk > 96 ? 96 : kCrossVariants[v].chunk;
+}
 constexpr int kNumCrossVariants = sizeof(kCrossVariants) / sizeof(kCrossVariants[0]);
 static_assert(kCrossVariants[5].threads == 256 && kCrossVariants[5].chunk == 64 && kCrossVariants[5].minb == 3,
               "cross_default names variant 5");
@@ -101,7 +112,10 @@ __device__ T right_entry(const CrossInst &in, int mode, const int *ridx, int f, 
 
 // ---------------------------------------------------------------- vectors
 // Lvec of a set: [n_left][nsl][5][VP], Rvec: [n_right][nsr][5][VP]; ns = 7
-// holds s = -3..3 (centre at 3), ns = 1 the centre only.  One CTA per set.
+// holds s = -3..3 (centre at 3), ns = 1 the centre only.  gridDim.y CTAs per set
+// share its vectors (one CTA per set took 0.96 ms on the 64-instance workload,
+// the largest set's ~10^5 entries in one CTA; a thread forms an entry's centre
+// once for all its shifted copies).
 template <bool F64>
 __global__ void __launch_bounds__(XT) k_cross_vecs(const CrossArgs A)
 {
@@ -119,7 +133,7 @@ __global__ void __launch_bounds__(XT) k_cross_vecs(const CrossArgs A)
     for (long long u = threadIdx.x; u < S.n_right * (2 - mode); u += XT)
         if ((unsigned)S.right[u] >= (unsigned)in.n[mode + 1 + u % (2 - mode)]) bad = 1;
     __syncthreads();
-    if (threadIdx.x == 0) A.bad[blockIdx.x] = bad;
+    if (threadIdx.x == 0 && blockIdx.y == 0) A.bad[blockIdx.x] = bad;
     if (bad) {
         if (threadIdx.x == 0) atomicOr(A.status, ST_BADINDEX);
         return;
@@ -130,53 +144,126 @@ __global__ void __launch_bounds__(XT) k_cross_vecs(const CrossArgs A)
         const long long nidx = side == 0 ? S.n_left : S.n_right;
         const int ns = side == 0 ? S.nsl : S.nsr;
         const int len = side == 0 ? rl : rr;
+        const bool empty = (side == 0 && mode == 0) || (side == 1 && mode == 2);
         T *out = vec + (side == 0 ? S.lvec_off : S.rvec_off);
-        const long long total = nidx * ns * 5 * VP;
-        for (long long u = threadIdx.x; u < total; u += XT) {
+        for (long long u = blockIdx.y * XT + threadIdx.x; u < nidx * 5 * VP; u += gridDim.y * XT) {
             const int a = (int)(u % VP);
             const int f = (int)((u / VP) % 5);
-            const int k = (int)((u / (5 * VP)) % ns);
-            const long long idx = u / (5 * VP * ns);
-            const int s = ns == 7 ? k - 3 : 0;
-            T v = T(0);
-            if (a < len) {
-                if ((side == 0 && mode == 0) || (side == 1 && mode == 2)) {
-                    v = T(1);  // empty side: the 1 x 1 identity
-                } else {
+            const long long idx = u / (5 * VP);
+            auto entry = [&](int s, bool &fl) {
+                return side == 0 ? left_entry<T>(in, mode, S.left + idx * mode, f, a, fd, s, fl)
+                                 : right_entry<T>(in, mode, S.right + idx * (2 - mode), f, a, fd, s, fl);
+            };
+            const bool live = a < len;
+            bool f0;
+            const T c = !live ? T(0) : empty ? T(1) : entry(0, f0);  // an empty side is the 1 x 1 identity
+            T *o = out + idx * ns * 5 * VP + f * VP + a;
+            for (int k = 0; k < ns; ++k) {
+                const int s = ns == 7 ? k - 3 : 0;
+                T v = c;
+                if (s != 0 && live) {
                     bool fl;
-                    v = side == 0 ? left_entry<T>(in, mode, S.left + idx * mode, f, a, fd, s, fl)
-                                  : right_entry<T>(in, mode, S.right + idx * (2 - mode), f, a, fd, s, fl);
+                    v = entry(s, fl);
                     if (fl && f == 1 + fd) v = -v;  // mirrored ghost row: normal momentum negated
-                    if (!F64 && s != 0) {
-                        bool f0;
-                        v -= side == 0 ? left_entry<T>(in, mode, S.left + idx * mode, f, a, fd, 0, f0)
-                                       : right_entry<T>(in, mode, S.right + idx * (2 - mode), f, a, fd, 0, f0);
-                    }
+                    if (!F64) v -= c;
                 }
+                o[(long long)k * 5 * VP] = v;
             }
-            out[u] = v;
         }
     }
 }
 
 // ------------------------------------------------------------------- main
+// Shared memory of k_cross in elements of T.
+template <int XT, int CH> struct CrossSmem {
+    static constexpr int CP = CH + 6;               // columns of a chunk, with the stencil halo of fd = m
+    static constexpr int c = 0;                     // [5][CP][CS] contracted core rows
+    static constexpr int cref = c + 5 * CP * CS;    // [5][CS]     the chunk's reference row (FP32, fd = m)
+    static constexpr int fixv = cref + 5 * CS;      // [5][VP][JB] the item's fixed vectors
+    static constexpr int fl = fixv + 5 * VP * JB;   // [XT][FLS]   fd = m: split fluxes of a block's points
+    static constexpr int stage = fl;                // [XT / 32][32][SP] (before fl is written) staged core pieces
+    static constexpr int ff = fl + (XT * FLS > XT * SP ? XT * FLS : XT * SP);  // [5][XT] face fluxes (doubled)
+    static constexpr int ct = ff + 5 * XT;          // [XT / 7 + 1][5] reference values (row i0)
+    static constexpr int total = ct + 5 * (XT / 7 + 1);
+};
+
+// RefState of a sample's centre (FP32), whose primitives multiply differences only.
+__device__ __forceinline__ void cross_ref(const float *ctr, float gm1, RefState<3> &rs)
+{
+#pragma unroll
+    for (int f = 0; f < 5; ++f) { rs.hi[f] = ctr[f]; rs.lo[f] = 0.0f; }
+    const float ir = 1.0f / ctr[0];
+    float ke = 0.0f;
+    rs.rho = ctr[0];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        rs.m[e] = ctr[1 + e];
+        rs.u[e] = ctr[1 + e] * ir;
+        ke += rs.m[e] * rs.u[e];
+    }
+    rs.H = ctr[4] + gm1 * (ctr[4] - 0.5f * ke);
+}
+
+// Twice the split fluxes of one stencil point: q the state (FP64) or its difference from rs (FP32).
+__device__ __forceinline__ void cross_flux(int fd, const float *q, const RefState<3> &rs, float alpha, double gm1, float *a5, float *b5)
+{
+    if (fd == 0) split_flux_diff<3, 0, true>(q, rs, alpha, (float)gm1, a5, b5);
+    else if (fd == 1) split_flux_diff<3, 1, true>(q, rs, alpha, (float)gm1, a5, b5);
+    else split_flux_diff<3, 2, true>(q, rs, alpha, (float)gm1, a5, b5);
+}
+__device__ __forceinline__ void cross_flux(int fd, const double *q, const RefState<3> &, double alpha, double gm1, double *a5, double *b5)
+{
+    if (fd == 0) split_flux_f64<3, 0, true>(q, alpha, gm1, a5, b5);
+    else if (fd == 1) split_flux_f64<3, 1, true>(q, alpha, gm1, a5, b5);
+    else split_flux_f64<3, 2, true>(q, alpha, gm1, a5, b5);
+}
+
+// Twice the flux of the face whose f(+) window is P[0], P[s], .., P[4 s] and whose
+// mirrored f(-) window is M[5 s], M[4 s], .., M[s] (FP32: one f32x2 pair).
+__device__ __forceinline__ float cross_face(const float *P, const float *M, int s, float eps, const PairEps &)
+{
+    return weno5_pm(make_float2(P[0], M[5 * s]), make_float2(P[s], M[4 * s]), make_float2(P[2 * s], M[3 * s]),
+                    make_float2(P[3 * s], M[2 * s]), make_float2(P[4 * s], M[s]), eps);
+}
+__device__ __forceinline__ double cross_face(const double *P, const double *M, int s, double, const PairEps &E)
+{
+    return weno5_pair(P[0], P[s], P[2 * s], P[3 * s], P[4 * s], E) + weno5_pair(M[5 * s], M[4 * s], M[3 * s], M[2 * s], M[s], E);
+}
+
+// Dot product of two zero-padded rows of l4 entries.  FP32: even and odd entries
+// accumulate in the two lanes of an f32x2 (one issue slot per two FMAs).
+__device__ __forceinline__ float row_dot(const float *x, const float *y, int, int l4)
+{
+    float2 s = bc2(0.0f);
+    for (int e = 0; e < l4; e += 4) {
+        const float4 p = *reinterpret_cast<const float4 *>(x + e), q = *reinterpret_cast<const float4 *>(y + e);
+        s = fma2(make_float2(p.z, p.w), make_float2(q.z, q.w), fma2(make_float2(p.x, p.y), make_float2(q.x, q.y), s));
+    }
+    return s.x + s.y;
+}
+__device__ __forceinline__ double row_dot(const double *x, const double *y, int l, int)
+{
+    double s = 0.0;
+    for (int e = 0; e < l; ++e) s = fma(x[e], y[e], s);
+    return s;
+}
+
 template <bool F64, int XT, int CH, int MINB>
 __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
 {
     using T = typename std::conditional<F64, double, float>::type;
-    constexpr int CP = CH + 6;  // chunk points including the stencil halo
+    using SM = CrossSmem<XT, CH>;
+    constexpr int CP = SM::CP, NWARP = XT / 32;
     extern __shared__ __align__(16) unsigned char dyn[];
-    T *C = reinterpret_cast<T *>(dyn);        // [5][CP][CS] contracted core rows of the chunk
-    T *Cref = C + 5 * CP * CS;                // [5][CS]     chunk reference row (FP32, fd == mode)
-    T *fixv = Cref + 5 * CS;                  // [5][CS]     the work item's fixed vector
-    // FP32, stencil along the fiber (role 1): per block of VB varying indices,
-    // the split fluxes of every chunk point, the face fluxes and the reference values
-    constexpr int VB = fiber_vb(XT, CH);
-    float *FL = reinterpret_cast<float *>(fixv + 5 * CS);  // [VB][CP][FLS] f(+) then f(-), 5 fields
-    float *FF = FL + VB * CP * FLS;                         // [VB][5][CH+1] face fluxes (doubled)
-    float *CT = FF + VB * 5 * (CH + 1);                     // [VB][5]       reference state (row i0)
+    T *base = reinterpret_cast<T *>(dyn);
+    T *C = base + SM::c, *Cref = base + SM::cref, *fixv = base + SM::fixv;
+    T *FL = base + SM::fl, *FF = base + SM::ff, *CT = base + SM::ct;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T *stage = base + SM::stage + warp * 32 * SP;
     __shared__ long long s_item;
     const T eps = T(4) * (T)A.eps;  // split fluxes are formed doubled: 4 eps gives twice the WENO5 value
+    PairEps E{};
+    if constexpr (F64) E = pair_eps(4.0 * A.eps);
     const double gm1 = A.gamma - 1.0;
     const T *vecs = reinterpret_cast<const T *>(A.vecs);
 
@@ -197,333 +284,273 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
         const CrossInst &in = A.inst[S.inst];
         const int mode = S.mode, fd = S.fd, n = S.n_mode;
         const int role = fd < mode ? 0 : (fd == mode ? 1 : 2);  // stencil moves: L / the core index / R
-        const long long j = item - S.work_begin;                 // fixed index: r (role 0, 1) or l (role 2)
         const int rl = mode == 0 ? 1 : in.r[mode - 1];
         const int rr = mode == 2 ? 1 : in.r[mode];
         const int clen = role == 2 ? rr : rl;                    // length of a contracted row
         const int cl4 = (clen + 3) & ~3;
         const long long nvar = role == 2 ? S.n_right : S.n_left;
+        const long long nfix = role == 2 ? S.n_left : S.n_right;
         const T *var = vecs + (role == 2 ? S.rvec_off : S.lvec_off);  // the varying side's vectors
         const int nsv = role == 2 ? S.nsr : S.nsl;
         const T alpha = (T)in.alpha;
         const T ih = (T)(0.5 / in.h[fd]);  // halves the doubled face fluxes
-        {   // fixed vector (centre) of this work item
-            const T *src = vecs + (role == 2 ? S.lvec_off + (j * S.nsl + (S.nsl == 7 ? 3 : 0)) * 5 * VP
-                                             : S.rvec_off + (j * S.nsr + (S.nsr == 7 ? 3 : 0)) * 5 * VP);
-            for (int u = threadIdx.x; u < 5 * VP; u += XT) fixv[(u / VP) * CS + u % VP] = src[u];
+        // the item: rows i0 .. i0 + cn, fixed indices j0 .. j0 + jn
+        const int jb = S.jb;
+        const long long njb = (nfix + jb - 1) / jb, w = item - S.work_begin;
+        const int i0 = (int)(w / njb) * S.rows;
+        const long long j0 = (w - (w / njb) * njb) * jb;
+        const int jn = nfix - j0 < jb ? (int)(nfix - j0) : jb;
+        const int cn = n - i0 < S.rows ? n - i0 : S.rows;
+        for (int u = threadIdx.x; u < 5 * VP * JB; u += XT) {  // the fixed side's centre vectors
+            const int jj = u / (5 * VP), x = u - jj * 5 * VP;
+            const T *src = vecs + (role == 2 ? S.lvec_off + ((j0 + jj) * S.nsl + (S.nsl == 7 ? 3 : 0)) * 5 * VP
+                                             : S.rvec_off + ((j0 + jj) * S.nsr + (S.nsr == 7 ? 3 : 0)) * 5 * VP);
+            fixv[x * JB + jj] = jj < jn ? src[x] : T(0);
         }
         const long long outstride_v = role == 2 ? 1 : (long long)n * S.n_right;   // along the varying index
-        const long long outbase_j = role == 2 ? j * (long long)n * S.n_right : j;  // fixed index offset
+        const long long outstride_j = role == 2 ? (long long)n * S.n_right : 1;   // along the fixed index
         T *out = reinterpret_cast<T *>(S.out);
         __syncthreads();
 
-        for (int i0 = 0; i0 < n; i0 += CH) {
-            const int cn = n - i0 < CH ? n - i0 : CH;             // samples in this chunk
-            const int p0 = role == 1 ? i0 - 3 : i0;               // first chunk point
-            const int np = role == 1 ? cn + 6 : cn;
-            // chunk reference row (FP32, stencil along the fiber): G(i0) . R
-            if (!F64 && role == 1) {
-                for (int u = threadIdx.x; u < 5 * cl4; u += XT) {
-                    const int f = u / cl4, x = u - f * cl4;
-                    T acc = T(0);
-                    if (x < clen) {
-                        const float *g = in.core[f][mode] + ((long long)i0 * rl + x) * rr;
-                        for (int y = 0; y < rr; ++y) acc += cvtf<T>(__ldg(g + y)) * fixv[f * CS + y];
-                    }
-                    Cref[f * CS + x] = acc;
-                }
-                __syncthreads();
-            }
-            // contracted rows: role 0/1: C[p][a] = G(p)[a][:] . R ; role 2: C[p][b] = L . G(p)[:][b]
-            // (rows zero-padded to a multiple of 4 entries for the float4 reads below)
-            for (int u = threadIdx.x; u < 5 * np * cl4; u += XT) {
-                const int f = u / (np * cl4);
-                const int rem = u - f * np * cl4;
-                const int pp = rem / cl4, x = rem - pp * cl4;
-                if (x >= clen) {
-                    C[(f * CP + pp) * CS + x] = T(0);
-                    continue;
-                }
-                bool flip = false;
-                int c = p0 + pp;
-                if (role == 1) c = xmap(in, fd, c, flip);
-                const float *g = in.core[f][mode] + (long long)c * rl * rr;
-                T acc = T(0);
-                if (role == 2) {
-                    for (int y = 0; y < rl; ++y) acc += fixv[f * CS + y] * cvtf<T>(__ldg(g + y * rr + x));
-                } else if (!F64 && role == 1) {
-                    const float *g0 = in.core[f][mode] + (long long)i0 * rl * rr;
-                    for (int y = 0; y < rr; ++y)
-                        acc += (__ldg(g + x * rr + y) - __ldg(g0 + x * rr + y)) * fixv[f * CS + y];
+        // One core row's matrix against the fixed vectors, by one warp, lane x the
+        // row entry.  Role 2: sum_y fixv[y] G[y][x], coalesced as it stands.
+        // Otherwise sum_y G[x][y] fixv[y] (minus the same of G0): pieces of 8
+        // columns go through the warp's stage, so that the loads take whole 32-byte
+        // sectors (a lane reading its own row touched 32 lines per load, and these
+        // loads were 85% of the kernel's L1 traffic).
+        auto contract = [&](int f, const float *g, const float *g0, T *acc) {
+#pragma unroll
+            for (int q = 0; q < JB; ++q) acc[q] = T(0);
+            const T *fv = fixv + f * VP * JB;
+            auto add = [&](T v, int y) {
+                if (jb == 1) {
+                    acc[0] += v * fv[y * JB];
                 } else {
-                    for (int y = 0; y < rr; ++y) acc += cvtf<T>(__ldg(g + x * rr + y)) * fixv[f * CS + y];
+#pragma unroll
+                    for (int q = 0; q < JB; ++q) acc[q] += v * fv[y * JB + q];
                 }
-                if (flip && f == 1 + fd) acc = F64 ? -acc : -acc - T(2) * Cref[f * CS + x];
-                C[(f * CP + pp) * CS + x] = acc;
+            };
+            if (role == 2) {
+                for (int y = 0; y < rl; ++y) add(lane < rr ? cvtf<T>(__ldg(g + y * rr + lane)) : T(0), y);
+            } else if (rr == 1) {
+                add(lane < rl ? cvtf<T>(__ldg(g + lane)) - (g0 ? cvtf<T>(__ldg(g0 + lane)) : T(0)) : T(0), 0);
+            } else {
+                for (int y0 = 0; y0 < rr; y0 += 8) {
+                    const int y = y0 + (lane & 7);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int x = 4 * k + (lane >> 3);
+                        T v = T(0);
+                        if (x < rl && y < rr) {
+                            v = cvtf<T>(__ldg(g + x * rr + y));
+                            if (g0) v -= cvtf<T>(__ldg(g0 + x * rr + y));
+                        }
+                        stage[x * SP + (lane & 7)] = v;
+                    }
+                    __syncwarp();
+                    const int ny = rr - y0 < 8 ? rr - y0 : 8;
+                    for (int k = 0; k < ny; ++k) add(stage[lane * SP + k], y0 + k);
+                    __syncwarp();
+                }
+            }
+        };
+        // chunk reference row (FP32, stencil along the fiber): G(i0) . R
+        if (!F64 && role == 1) {
+            for (int f = warp; f < 5; f += NWARP) {
+                T acc[JB];
+                contract(f, in.core[f][mode] + (long long)i0 * rl * rr, nullptr, acc);
+                if (lane < cl4) Cref[f * CS + lane] = acc[0];
             }
             __syncthreads();
+        }
+        // contracted rows, zero-padded to a multiple of 4 entries; column = point (fd = m)
+        // or (row, fixed index)
+        const int np = role == 1 ? cn + 6 : cn;
+        for (int u = warp; u < 5 * np; u += NWARP) {
+            const int f = u / np, pp = u - f * np;
+            bool flip = false;
+            int c = role == 1 ? i0 - 3 + pp : i0 + pp;
+            if (role == 1) c = xmap(in, fd, c, flip);
+            const float *g = in.core[f][mode];
+            T acc[JB];
+            contract(f, g + (long long)c * rl * rr, !F64 && role == 1 ? g + (long long)i0 * rl * rr : nullptr, acc);
+            if (flip && f == 1 + fd && lane < cl4) acc[0] = F64 ? -acc[0] : -acc[0] - T(2) * Cref[f * CS + lane];
+            if (lane < cl4) {
+                T *row = C + (f * CP + (role == 1 ? pp : pp * jb)) * CS + lane;
+                row[0] = acc[0];
+                if (jb > 1) {
+#pragma unroll
+                    for (int q = 1; q < JB; ++q)
+                        if (q < jb) row[q * CS] = acc[q];
+                }
+            }
+        }
+        __syncthreads();
 
-            if constexpr (!F64) if (role == 1) {
-                // The stencil moves along the fiber: neighbouring samples of one
-                // varying index share six of their seven points and one of their two
-                // faces, so each point's split flux and each face's WENO5(+/-) is
-                // formed once per block of VB varying indices (the values are the
-                // ones the per-sample path forms: the same dot products, split
-                // fluxes relative to row i0, and weno5_pm of the same windows).
-                for (long long vb0 = 0; vb0 < nvar; vb0 += VB) {
-                    // reference values (row i0) of the block's varying indices
-                    for (int u = threadIdx.x; u < VB * 5; u += XT) {
-                        const long long v = vb0 + u / 5;
+        if (role == 1) {
+            // The stencil moves along the fiber: neighbouring samples of one varying
+            // index share six of their seven points and one of their two faces, so
+            // each point's split flux and each face's WENO5(+/-) is formed once per
+            // block of vb varying indices (as many as make each phase one pass).
+            const int vb = XT / np;
+            for (long long v0 = 0; v0 < nvar; v0 += vb) {
+                const int nv = nvar - v0 < vb ? (int)(nvar - v0) : vb;
+                if constexpr (!F64) {  // reference values (row i0) of the block's varying indices
+                    for (int u = threadIdx.x; u < nv * 5; u += XT) {
                         const int f = u % 5;
-                        float racc = 0.0f;
-                        if (v < nvar) {
-                            const float *lv = reinterpret_cast<const float *>(var) + (v * nsv) * 5 * VP + f * VP;
-                            float2 ra2 = bc2(0.0f);
-                            for (int x = 0; x < cl4; x += 4) {
-                                const float4 l4 = *reinterpret_cast<const float4 *>(lv + x);
-                                const float4 r4 = *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(Cref) + f * CS + x);
-                                ra2 = fma2(make_float2(l4.z, l4.w), make_float2(r4.z, r4.w),
-                                           fma2(make_float2(l4.x, l4.y), make_float2(r4.x, r4.y), ra2));
-                            }
-                            racc = ra2.x + ra2.y;
-                        }
-                        CT[u] = racc;
+                        CT[u] = row_dot(var + (v0 + u / 5) * nsv * 5 * VP + f * VP, Cref + f * CS, clen, cl4);
                     }
                     __syncthreads();
-                    // split fluxes of every chunk point
-                    for (int u = threadIdx.x; u < VB * np; u += XT) {
-                        const int vl = u / np, pp = u - vl * np;
-                        const long long v = vb0 + vl;
-                        if (v >= nvar) continue;
-                        const float *lvb = reinterpret_cast<const float *>(var) + (v * nsv) * 5 * VP;
-                        float dq[5];
+                }
+                for (int u = threadIdx.x; u < nv * np; u += XT) {  // split fluxes of every chunk point
+                    const int vl = u / np, pp = u - vl * np;
+                    const T *lv = var + (v0 + vl) * nsv * 5 * VP;
+                    T q[5], a5[5], b5[5];
 #pragma unroll
-                        for (int f = 0; f < 5; ++f) {
-                            const float *lv = lvb + f * VP;
-                            const float *crow = reinterpret_cast<const float *>(C) + (f * CP + pp) * CS;
-                            float2 a2 = bc2(0.0f);
-                            for (int x = 0; x < cl4; x += 4) {
-                                const float4 l4 = *reinterpret_cast<const float4 *>(lv + x);
-                                const float4 c4 = *reinterpret_cast<const float4 *>(crow + x);
-                                a2 = fma2(make_float2(l4.z, l4.w), make_float2(c4.z, c4.w),
-                                          fma2(make_float2(l4.x, l4.y), make_float2(c4.x, c4.y), a2));
-                            }
-                            dq[f] = a2.x + a2.y;
-                        }
-                        RefState<3> rs;
-                        const float *ct = CT + vl * 5;
+                    for (int f = 0; f < 5; ++f) q[f] = row_dot(lv + f * VP, C + (f * CP + pp) * CS, clen, cl4);
+                    RefState<3> rs;
+                    if constexpr (!F64) cross_ref(CT + vl * 5, (float)gm1, rs);
+                    cross_flux(fd, q, rs, alpha, gm1, a5, b5);
+                    T *fl = FL + u * FLS;
 #pragma unroll
-                        for (int f = 0; f < 5; ++f) { rs.hi[f] = ct[f]; rs.lo[f] = 0.0f; }
-                        {
-                            const float ir = 1.0f / ct[0];
-                            float ke = 0.0f;
-                            rs.rho = ct[0];
-#pragma unroll
-                            for (int e = 0; e < 3; ++e) {
-                                rs.m[e] = ct[1 + e];
-                                rs.u[e] = ct[1 + e] * ir;
-                                ke += rs.m[e] * rs.u[e];
-                            }
-                            rs.H = ct[4] + (float)gm1 * (ct[4] - 0.5f * ke);
-                        }
-                        float a5[5], b5[5];
-                        if (fd == 0) split_flux_diff<3, 0, true>(dq, rs, (float)alpha, (float)gm1, a5, b5);
-                        else if (fd == 1) split_flux_diff<3, 1, true>(dq, rs, (float)alpha, (float)gm1, a5, b5);
-                        else split_flux_diff<3, 2, true>(dq, rs, (float)alpha, (float)gm1, a5, b5);
-                        float *fl = FL + (vl * CP + pp) * FLS;
-#pragma unroll
-                        for (int f = 0; f < 5; ++f) { fl[f] = a5[f]; fl[5 + f] = b5[f]; }
-                    }
-                    __syncthreads();
-                    // face fluxes j = 0..cn (face j lies before sample j)
-                    for (int u = threadIdx.x; u < VB * (cn + 1); u += XT) {
-                        const int vl = u / (cn + 1), j = u - vl * (cn + 1);
-                        if (vb0 + vl >= nvar) continue;
-                        const float *fl = FL + (vl * CP + j) * FLS;
-#pragma unroll
-                        for (int f = 0; f < 5; ++f) {
-                            const float *P = fl + f, *M = fl + 5 + f;  // point j + k at [k * FLS]
-                            FF[(vl * 5 + f) * (CH + 1) + j] = weno5_pm(
-                                make_float2(P[0], M[5 * FLS]), make_float2(P[FLS], M[4 * FLS]),
-                                make_float2(P[2 * FLS], M[3 * FLS]), make_float2(P[3 * FLS], M[2 * FLS]),
-                                make_float2(P[4 * FLS], M[FLS]), (float)eps);
-                        }
-                    }
-                    __syncthreads();
-                    for (int u = threadIdx.x; u < VB * cn; u += XT) {
-                        const int vl = u / cn, ii = u - vl * cn;
-                        const long long v = vb0 + vl;
-                        if (v >= nvar) continue;
-                        const int i = i0 + ii;
-#pragma unroll
-                        for (int f = 0; f < 5; ++f) {
-                            const float *F = FF + (vl * 5 + f) * (CH + 1);
-                            const long long o = (long long)f * S.n_left * n * S.n_right + outbase_j + v * outstride_v +
-                                                (long long)i * S.n_right;
-                            out[o] = -(F[ii + 1] - F[ii]) * ih;
-                        }
-                    }
-                    // (the next block's first writes go to CT and FL, which no thread
-                    // reads after the barrier above)
+                    for (int f = 0; f < 5; ++f) { fl[f] = a5[f]; fl[5 + f] = b5[f]; }
                 }
                 __syncthreads();
-                continue;
-            }
-            // samples (v, i): 7 stencil values per field, split fluxes, two interfaces
-            for (long long u = threadIdx.x; u < nvar * CH; u += XT) {
-                const long long v = u / CH;
-                const int ii = (int)(u - v * CH);
-                if (ii >= cn) continue;
-                T q7[5][7];  // FP64: values; FP32: differences from the reference state
-                T ctr[5];    // FP32: reference state
+                // face fluxes (face k lies before sample k), one work item per face and field
+                for (int u = threadIdx.x; u < 5 * nv * (cn + 1); u += XT) {
+                    const int f = u / (nv * (cn + 1)), r = u - f * (nv * (cn + 1));
+                    const int vl = r / (cn + 1), k = r - vl * (cn + 1);
+                    const T *fl = FL + (vl * np + k) * FLS + f;
+                    FF[f * XT + r] = cross_face(fl, fl + 5, FLS, eps, E);
+                }
+                __syncthreads();
+                for (int u = threadIdx.x; u < nv * cn; u += XT) {
+                    const int vl = u / cn, ii = u - vl * cn;
+                    const long long o = j0 * outstride_j + (v0 + vl) * outstride_v + (long long)(i0 + ii) * S.n_right;
 #pragma unroll
-                for (int f = 0; f < 5; ++f) {
-                    T acc[7];
-#pragma unroll
-                    for (int k = 0; k < 7; ++k) acc[k] = T(0);
-                    if (role == 1) {  // the same vector against the 7 rows i-3..i+3
-                        const T *lv = var + (v * nsv) * 5 * VP + f * VP;
-                        T racc = T(0);
-                        if constexpr (F64) {
-                            for (int x = 0; x < clen; ++x) {
-                                const T lx = lv[x];
-#pragma unroll
-                                for (int k = 0; k < 7; ++k) acc[k] += lx * C[(f * CP + ii + k) * CS + x];
-                            }
-                        } else {
-                            // f32x2: even and odd entries accumulate in the two lanes (one issue
-                            // slot per two FMAs), summed at the end
-                            float2 a2[7], ra2 = bc2(0.0f);
-#pragma unroll
-                            for (int k = 0; k < 7; ++k) a2[k] = bc2(0.0f);
-                            for (int x = 0; x < cl4; x += 4) {
-                                const float4 l4 = *reinterpret_cast<const float4 *>(lv + x);
-                                const float2 lxy = make_float2(l4.x, l4.y), lzw = make_float2(l4.z, l4.w);
-#pragma unroll
-                                for (int k = 0; k < 7; ++k) {
-                                    const float4 c4 = *reinterpret_cast<const float4 *>(C + (f * CP + ii + k) * CS + x);
-                                    a2[k] = fma2(lzw, make_float2(c4.z, c4.w), fma2(lxy, make_float2(c4.x, c4.y), a2[k]));
-                                }
-                                const float4 r4 = *reinterpret_cast<const float4 *>(Cref + f * CS + x);
-                                ra2 = fma2(lzw, make_float2(r4.z, r4.w), fma2(lxy, make_float2(r4.x, r4.y), ra2));
-                            }
-#pragma unroll
-                            for (int k = 0; k < 7; ++k) acc[k] = a2[k].x + a2[k].y;
-                            racc = ra2.x + ra2.y;
-                        }
-                        ctr[f] = racc;
-#pragma unroll
-                        for (int k = 0; k < 7; ++k) q7[f][k] = acc[k];
-                    } else {          // the 7 shifted vectors against the row of sample i
-                        const T *vv = var + (v * 7) * 5 * VP + f * VP;
-                        const T *crow = C + (f * CP + ii) * CS;
-                        if constexpr (F64) {
-                            for (int x = 0; x < clen; ++x) {
-                                const T cx = crow[x];
-#pragma unroll
-                                for (int k = 0; k < 7; ++k) acc[k] += vv[k * 5 * VP + x] * cx;
-                            }
-                        } else {  // f32x2 even / odd partial sums, as above
-                            float2 a2[7];
-#pragma unroll
-                            for (int k = 0; k < 7; ++k) a2[k] = bc2(0.0f);
-                            for (int x = 0; x < cl4; x += 4) {
-                                const float4 c4 = *reinterpret_cast<const float4 *>(crow + x);
-                                const float2 cxy = make_float2(c4.x, c4.y), czw = make_float2(c4.z, c4.w);
-#pragma unroll
-                                for (int k = 0; k < 7; ++k) {
-                                    const float4 w4 = *reinterpret_cast<const float4 *>(vv + k * 5 * VP + x);
-                                    a2[k] = fma2(make_float2(w4.z, w4.w), czw, fma2(make_float2(w4.x, w4.y), cxy, a2[k]));
-                                }
-                            }
-#pragma unroll
-                            for (int k = 0; k < 7; ++k) acc[k] = a2[k].x + a2[k].y;
-                        }
-                        ctr[f] = acc[3];
-#pragma unroll
-                        for (int k = 0; k < 7; ++k) q7[f][k] = (F64 || k != 3) ? acc[k] : T(0);
+                    for (int f = 0; f < 5; ++f) {
+                        const T *F = FF + f * XT + vl * (cn + 1) + ii;
+                        out[(long long)f * S.n_left * n * S.n_right + o] = -(F[1] - F[0]) * ih;
                     }
                 }
-                T fp7[5][7], fm7[5][7];
+                // (the next block's first writes go to CT and FL, which no thread reads
+                // after the barrier above)
+            }
+            continue;
+        }
+        // samples (v, column): 7 stencil values per field, split fluxes, two interfaces
+        const int ncol = cn * jb, jsh = jb == 4 ? 2 : jb == 2 ? 1 : 0;
+        for (long long u = threadIdx.x; u < nvar * ncol; u += XT) {
+            const long long v = (unsigned long long)u < (1ull << 32) ? (long long)((unsigned)u / (unsigned)ncol) : u / ncol;
+            const int col = (int)(u - v * ncol), ii = col >> jsh, jj = col & (jb - 1);
+            if (jj >= jn) continue;
+            T q7[5][7];  // FP64: values; FP32: differences from the reference state
+            T ctr[5];    // the centre (FP32: the reference state)
+#pragma unroll
+            for (int f = 0; f < 5; ++f) {  // the 7 shifted vectors against the column's row
+                T acc[7];
+                const T *vv = var + (v * 7) * 5 * VP + f * VP;
+                const T *crow = C + (f * CP + col) * CS;
                 if constexpr (F64) {
 #pragma unroll
-                    for (int k = 0; k < 7; ++k) {
-                        double qd[5], a5[5], b5[5];
+                    for (int k = 0; k < 7; ++k) acc[k] = T(0);
+                    for (int x = 0; x < clen; ++x) {
+                        const T cx = crow[x];
 #pragma unroll
-                        for (int f = 0; f < 5; ++f) qd[f] = q7[f][k];
-                        if (fd == 0) split_flux_f64<3, 0, true>(qd, (double)alpha, gm1, a5, b5);
-                        else if (fd == 1) split_flux_f64<3, 1, true>(qd, (double)alpha, gm1, a5, b5);
-                        else split_flux_f64<3, 2, true>(qd, (double)alpha, gm1, a5, b5);
-#pragma unroll
-                        for (int f = 0; f < 5; ++f) { fp7[f][k] = a5[f]; fm7[f][k] = b5[f]; }
+                        for (int k = 0; k < 7; ++k) acc[k] += vv[k * 5 * VP + x] * cx;
                     }
-                } else {
-                    RefState<3> rs;
+                } else {  // f32x2 even / odd partial sums, as row_dot
+                    float2 a2[7];
 #pragma unroll
-                    for (int f = 0; f < 5; ++f) { rs.hi[f] = ctr[f]; rs.lo[f] = 0.0f; }
-                    {
-                        const float ir = 1.0f / ctr[0];
-                        float ke = 0.0f;
-                        rs.rho = ctr[0];
+                    for (int k = 0; k < 7; ++k) a2[k] = bc2(0.0f);
+                    for (int x = 0; x < cl4; x += 4) {
+                        const float4 c4 = *reinterpret_cast<const float4 *>(crow + x);
+                        const float2 cxy = make_float2(c4.x, c4.y), czw = make_float2(c4.z, c4.w);
 #pragma unroll
-                        for (int e = 0; e < 3; ++e) {
-                            rs.m[e] = ctr[1 + e];
-                            rs.u[e] = ctr[1 + e] * ir;
-                            ke += rs.m[e] * rs.u[e];
+                        for (int k = 0; k < 7; ++k) {
+                            const float4 w4 = *reinterpret_cast<const float4 *>(vv + k * 5 * VP + x);
+                            a2[k] = fma2(make_float2(w4.z, w4.w), czw, fma2(make_float2(w4.x, w4.y), cxy, a2[k]));
                         }
-                        rs.H = ctr[4] + (float)gm1 * (ctr[4] - 0.5f * ke);
                     }
 #pragma unroll
-                    for (int k = 0; k < 7; ++k) {
-                        float dq[5], a5[5], b5[5];
-#pragma unroll
-                        for (int f = 0; f < 5; ++f) dq[f] = q7[f][k];
-                        if (fd == 0) split_flux_diff<3, 0, true>(dq, rs, alpha, (float)gm1, a5, b5);
-                        else if (fd == 1) split_flux_diff<3, 1, true>(dq, rs, alpha, (float)gm1, a5, b5);
-                        else split_flux_diff<3, 2, true>(dq, rs, alpha, (float)gm1, a5, b5);
-#pragma unroll
-                        for (int f = 0; f < 5; ++f) { fp7[f][k] = a5[f]; fm7[f][k] = b5[f]; }
-                    }
+                    for (int k = 0; k < 7; ++k) acc[k] = a2[k].x + a2[k].y;
                 }
-                const int i = i0 + ii;
+                ctr[f] = acc[3];
 #pragma unroll
-                for (int f = 0; f < 5; ++f) {
-                    const T *P = fp7[f], *M = fm7[f];
-                    T Flo, Fhi;
-                    if constexpr (F64) {
-                        Flo = weno5<T>(P[0], P[1], P[2], P[3], P[4], eps) + weno5<T>(M[5], M[4], M[3], M[2], M[1], eps);
-                        Fhi = weno5<T>(P[1], P[2], P[3], P[4], P[5], eps) + weno5<T>(M[6], M[5], M[4], M[3], M[2], eps);
-                    } else {  // WENO(+) and the mirrored WENO(-) of an interface as one f32x2 pair
-                        Flo = weno5_pm(make_float2(P[0], M[5]), make_float2(P[1], M[4]), make_float2(P[2], M[3]),
-                                       make_float2(P[3], M[2]), make_float2(P[4], M[1]), eps);
-                        Fhi = weno5_pm(make_float2(P[1], M[6]), make_float2(P[2], M[5]), make_float2(P[3], M[4]),
-                                       make_float2(P[4], M[3]), make_float2(P[5], M[2]), eps);
-                    }
-                    // out[f][l][i][r]: role 0/1 fix r (= j) and vary l (= v); role 2 fixes l, varies r
-                    const long long o = (long long)f * S.n_left * n * S.n_right + outbase_j + v * outstride_v +
-                                        (long long)i * S.n_right;
-                    out[o] = -(Fhi - Flo) * ih;
-                }
+                for (int k = 0; k < 7; ++k) q7[f][k] = (F64 || k != 3) ? acc[k] : T(0);
             }
-            __syncthreads();
+            T fp7[5][7], fm7[5][7];
+            RefState<3> rs;
+            if constexpr (!F64) cross_ref(ctr, (float)gm1, rs);
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                T q[5], a5[5], b5[5];
+#pragma unroll
+                for (int f = 0; f < 5; ++f) q[f] = q7[f][k];
+                cross_flux(fd, q, rs, alpha, gm1, a5, b5);
+#pragma unroll
+                for (int f = 0; f < 5; ++f) { fp7[f][k] = a5[f]; fm7[f][k] = b5[f]; }
+            }
+            // out[f][l][i][r]: role 0 varies l and fixes r, role 2 the other way round
+            const long long o = (j0 + jj) * outstride_j + v * outstride_v + (long long)(i0 + ii) * S.n_right;
+#pragma unroll
+            for (int f = 0; f < 5; ++f) {
+                const T Flo = cross_face(fp7[f], fm7[f], 1, eps, E), Fhi = cross_face(fp7[f] + 1, fm7[f] + 1, 1, eps, E);
+                out[(long long)f * S.n_left * n * S.n_right + o] = -(Fhi - Flo) * ih;
+            }
         }
     }
 }
 
-static size_t cross_dyn_bytes(bool f64, int threads, int chunk)
+template <bool F64, int XT, int CH> static constexpr size_t cross_dyn_bytes()
 {
-    const size_t e = f64 ? sizeof(double) : sizeof(float);
-    const int VB = fiber_vb(threads, chunk);
-    const size_t fiber = f64 ? 0 : sizeof(float) * (size_t)(VB * (chunk + 6) * FLS + VB * 5 * (chunk + 1) + VB * 5);
-    return e * (size_t)(5 * (chunk + 6) * CS + 2 * 5 * CS) + fiber;
+    return (F64 ? sizeof(double) : sizeof(float)) * (size_t)CrossSmem<XT, CH>::total;
 }
 
 int cross_vec_len() { return VP; }
 int cross_num_variants() { return kNumCrossVariants; }
-void cross_default(int *variant, int *ctas_per_sm)
+void cross_default(bool fp64, int *variant, int *ctas_per_sm)
 {
-    *variant = 5;  // {256, 64, 3}
-    *ctas_per_sm = 3;
+    *variant = fp64 ? 1 : 5;  // {256, 32, 1} and {256, 64, 3}
+    *ctas_per_sm = fp64 ? 2 : 3;
+}
+
+// Work items of a set for the chunk length of a variant: jb fixed indices and
+// `rows` rows each.  Several fixed indices share a core row's loads and the
+// varying vectors; where there are few fixed indices the columns are rows.  With
+// fewer than a few items per resident CTA the rows are halved (to 8 rows per
+// fixed index, 16 where the stencil needs 6 halo rows).
+long long cross_items(const CrossSet &S, int rows)
+{
+    const long long nfix = S.fd > S.mode ? S.n_left : S.n_right;
+    return (nfix + S.jb - 1) / S.jb * ((S.n_mode + rows - 1) / rows);
+}
+long long cross_plan(CrossSet *sets, int n_sets, bool fp64, int variant)
+{
+    const int chunk = variant_chunk(fp64, variant);
+    long long total = 0;
+    for (int k = 0; k < n_sets; ++k) {
+        CrossSet &S = sets[k];
+        const long long nfix = S.fd > S.mode ? S.n_left : S.n_right;
+        S.jb = S.fd == S.mode ? 1 : nfix >= 3 ? JB : (int)nfix;
+        S.rows = chunk / S.jb;
+        total += cross_items(S, S.rows);
+    }
+    for (int cut = 0; cut < 3 && total < 6ll * sm_count(); ++cut) {
+        total = 0;
+        for (int k = 0; k < n_sets; ++k) {
+            CrossSet &S = sets[k];
+            const int least = S.fd == S.mode ? 16 : 8;
+            if (S.rows / 2 >= least) S.rows /= 2;
+            total += cross_items(S, S.rows);
+        }
+    }
+    total = 0;
+    for (int k = 0; k < n_sets; ++k) {
+        sets[k].work_begin = total;
+        total += cross_items(sets[k], sets[k].rows);
+    }
+    return total;
 }
 void cross_variant(int v, int *threads, int *chunk)
 {
@@ -534,9 +561,9 @@ void cross_variant(int v, int *threads, int *chunk)
 template <bool F64, int V>
 static cudaError_t set_attr()
 {
-    constexpr int XT_ = kCrossVariants[V].threads, CH_ = kCrossVariants[V].chunk, MB_ = kCrossVariants[V].minb;
+    constexpr int XT_ = kCrossVariants[V].threads, CH_ = variant_chunk(F64, V), MB_ = kCrossVariants[V].minb;
     return cudaFuncSetAttribute(k_cross<F64, XT_, CH_, MB_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)cross_dyn_bytes(F64, XT_, CH_));
+                                (int)cross_dyn_bytes<F64, XT_, CH_>());
 }
 
 // Shared-memory limits of every variant, set once before any launch (and so
@@ -558,8 +585,8 @@ cudaError_t cross_set_attributes()
 template <bool F64, int V>
 static cudaError_t launch_main(const CrossArgs &a, long long blocks, cudaStream_t s)
 {
-    constexpr int XT_ = kCrossVariants[V].threads, CH_ = kCrossVariants[V].chunk, MB_ = kCrossVariants[V].minb;
-    k_cross<F64, XT_, CH_, MB_><<<(unsigned)blocks, XT_, cross_dyn_bytes(F64, XT_, CH_), s>>>(a);
+    constexpr int XT_ = kCrossVariants[V].threads, CH_ = variant_chunk(F64, V), MB_ = kCrossVariants[V].minb;
+    k_cross<F64, XT_, CH_, MB_><<<(unsigned)blocks, XT_, cross_dyn_bytes<F64, XT_, CH_>(), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -570,8 +597,10 @@ cudaError_t launch_cross(const CrossArgs &a, int variant, int ctas_per_sm, cudaS
     if (variant < 0 || variant >= kNumCrossVariants || ctas_per_sm < 1) return cudaErrorInvalidValue;
     cudaError_t ea = cross_set_attributes();
     if (ea != cudaSuccess) return ea;
-    if (a.fp64) k_cross_vecs<true><<<a.n_sets, XT, 0, s>>>(a);
-    else k_cross_vecs<false><<<a.n_sets, XT, 0, s>>>(a);
+    // enough CTAs per set that all of them together fill the GPU a few times over
+    const int per_set = (int)std::min(64ll, std::max(4ll, (8ll * sm_count() + a.n_sets - 1) / a.n_sets));
+    if (a.fp64) k_cross_vecs<true><<<dim3(a.n_sets, per_set), XT, 0, s>>>(a);
+    else k_cross_vecs<false><<<dim3(a.n_sets, per_set), XT, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     long long blocks = (long long)sm_count() * ctas_per_sm;
