@@ -18,6 +18,7 @@ struct CrossInst {
 struct CrossSet {
     int inst, mode, fd;
     int n_mode;
+    int r_mode;            // entries of a core row's matrix, r_{mode-1} r_mode
     long long n_left, n_right;
     const int *left;
     const int *right;

@@ -15,7 +15,7 @@
 //                 stored as differences from the centre vector, so rounding
 //                 scales with the variation along the stencil);
 //   k_cross       persistent; a work item is a chunk of rows i of the core and a
-//                 block of one to four indices of the side the stencil does not
+//                 block of up to eight indices of the side the stencil does not
 //                 move (r for fd <= m, l for fd > m), small enough that the items
 //                 of the largest fiber set do not outlast the rest (cross_plan).
 //                 It contracts the core rows G_m(i) with the block's vectors once
@@ -38,7 +38,10 @@ namespace wg {
 constexpr int XT = 256;       // threads per CTA of k_cross_vecs
 constexpr int VP = 32;        // padded vector length (largest rank)
 constexpr int CS = VP + 4;    // shared-memory row stride: float4 reads of 8 consecutive rows hit distinct banks
-constexpr int JB = 4;         // fixed indices per work item at most
+// fixed indices per work item at most; with fd = m, where a chunk's points carry a
+// 6-point halo, 4 (FP32) or 1
+constexpr int cross_jb(bool f64) { return f64 ? 4 : 8; }
+constexpr int JB1 = 4;
 constexpr int SP = 9;         // pitch of a warp's staged 32 x 8 piece of a core row's matrix
 constexpr int FLS = 11;       // values per point of the fiber path's split fluxes (10, padded odd:
                               // consecutive points of a warp fall on distinct banks)
@@ -51,7 +54,7 @@ constexpr int FLS = 11;       // values per point of the fiber path's split flux
 // minb > 1 asks the compiler for registers that fit minb CTAs per SM.
 struct CrossVariant { int threads, chunk, minb; };
 constexpr CrossVariant kCrossVariants[] = {{256, 64, 1}, {256, 32, 1}, {128, 64, 1}, {128, 32, 1},
-                                           {256, 128, 1}, {256, 64, 3}, {128, 64, 6}};
+                                           {256, 128, 1}, {256, 64, 3}, {128, 64, 6}, {256, 64, 2}};
 // rows of an FP64 chunk: at most 96 (shared memory)
 constexpr int variant_chunk(bool f64, int v)
 {
@@ -175,11 +178,12 @@ __global__ void __launch_bounds__(XT) k_cross_vecs(const CrossArgs A)
 
 // ------------------------------------------------------------------- main
 // Shared memory of k_cross in elements of T.
-template <int XT, int CH> struct CrossSmem {
+template <bool F64, int XT, int CH> struct CrossSmem {
+    static constexpr int JB = cross_jb(F64);
     static constexpr int CP = CH + 6;               // columns of a chunk, with the stencil halo of fd = m
     static constexpr int c = 0;                     // [5][CP][CS] contracted core rows
-    static constexpr int cref = c + 5 * CP * CS;    // [5][CS]     the chunk's reference row (FP32, fd = m)
-    static constexpr int fixv = cref + 5 * CS;      // [5][VP][JB] the item's fixed vectors
+    static constexpr int cref = c + 5 * CP * CS;    // [5][JB1][CS] the chunk's reference row (FP32, fd = m)
+    static constexpr int fixv = cref + 5 * JB1 * CS;  // [5][VP][JB] the item's fixed vectors
     static constexpr int fl = fixv + 5 * VP * JB;   // [XT][FLS]   fd = m: split fluxes of a block's points
     static constexpr int stage = fl;                // [XT / 32][32][SP] (before fl is written) staged core pieces
     static constexpr int ff = fl + (XT * FLS > XT * SP ? XT * FLS : XT * SP);  // [5][XT] face fluxes (doubled)
@@ -252,8 +256,8 @@ template <bool F64, int XT, int CH, int MINB>
 __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
 {
     using T = typename std::conditional<F64, double, float>::type;
-    using SM = CrossSmem<XT, CH>;
-    constexpr int CP = SM::CP, NWARP = XT / 32;
+    using SM = CrossSmem<F64, XT, CH>;
+    constexpr int CP = SM::CP, JB = SM::JB, NWARP = XT / 32;
     extern __shared__ __align__(16) unsigned char dyn[];
     T *base = reinterpret_cast<T *>(dyn);
     T *C = base + SM::c, *Cref = base + SM::cref, *fixv = base + SM::fixv;
@@ -314,20 +318,35 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
 
         // One core row's matrix against the fixed vectors, by one warp, lane x the
         // row entry.  Role 2: sum_y fixv[y] G[y][x], coalesced as it stands.
-        // Otherwise sum_y G[x][y] fixv[y] (minus the same of G0): pieces of 8
+        // Otherwise sum_y G[x][y] fixv[y] (of G - G0 if there is a G0): pieces of 8
         // columns go through the warp's stage, so that the loads take whole 32-byte
         // sectors (a lane reading its own row touched 32 lines per load, and these
-        // loads were 85% of the kernel's L1 traffic).
-        auto contract = [&](int f, const float *g, const float *g0, T *acc) {
+        // loads were 85% of the kernel's L1 traffic).  An entry's sums for all fixed
+        // indices are formed at once (FP32: in f32x2 pairs of indices).
+        T acc[JB];
+        auto contract_n = [&](auto nq, int f, const float *g, const float *g0) {
+            constexpr int NQ = decltype(nq)::value;  // fixed indices (1, or a multiple of 4)
 #pragma unroll
             for (int q = 0; q < JB; ++q) acc[q] = T(0);
             const T *fv = fixv + f * VP * JB;
             auto add = [&](T v, int y) {
-                if (jb == 1) {
-                    acc[0] += v * fv[y * JB];
+                const T *r = fv + y * JB;
+                if constexpr (NQ == 1) {
+                    acc[0] = fma(v, r[0], acc[0]);
+                } else if constexpr (F64) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) acc[q] = fma(v, r[q], acc[q]);
                 } else {
 #pragma unroll
-                    for (int q = 0; q < JB; ++q) acc[q] += v * fv[y * JB + q];
+                    for (int q = 0; q < NQ; q += 4) {
+                        const float4 r4 = *reinterpret_cast<const float4 *>(r + q);
+                        const float2 lo2 = fma2(bc2(v), make_float2(r4.x, r4.y), make_float2(acc[q], acc[q + 1]));
+                        const float2 hi2 = fma2(bc2(v), make_float2(r4.z, r4.w), make_float2(acc[q + 2], acc[q + 3]));
+                        acc[q] = lo2.x;
+                        acc[q + 1] = lo2.y;
+                        acc[q + 2] = hi2.x;
+                        acc[q + 3] = hi2.y;
+                    }
                 }
             };
             if (role == 2) {
@@ -337,34 +356,42 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
             } else {
                 for (int y0 = 0; y0 < rr; y0 += 8) {
                     const int y = y0 + (lane & 7);
+                    const int e = (lane >> 3) * rr + y;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
-                        const int x = 4 * k + (lane >> 3);
+                        if (4 * k >= rl) break;
                         T v = T(0);
-                        if (x < rl && y < rr) {
-                            v = cvtf<T>(__ldg(g + x * rr + y));
-                            if (g0) v -= cvtf<T>(__ldg(g0 + x * rr + y));
+                        if (4 * k + (lane >> 3) < rl && y < rr) {
+                            v = cvtf<T>(__ldg(g + e + 4 * k * rr));
+                            if (g0) v -= cvtf<T>(__ldg(g0 + e + 4 * k * rr));
                         }
-                        stage[x * SP + (lane & 7)] = v;
+                        stage[(4 * k + (lane >> 3)) * SP + (lane & 7)] = v;
                     }
                     __syncwarp();
                     const int ny = rr - y0 < 8 ? rr - y0 : 8;
-                    for (int k = 0; k < ny; ++k) add(stage[lane * SP + k], y0 + k);
+                    const T *sr = stage + (lane < rl ? lane : 0) * SP;
+                    for (int k = 0; k < ny; ++k) add(lane < rl ? sr[k] : T(0), y0 + k);
                     __syncwarp();
                 }
             }
         };
+        auto contract = [&](int f, const float *g, const float *g0) {
+            if (jb == 1) contract_n(std::integral_constant<int, 1>(), f, g, g0);
+            else if (JB == 4 || jb <= 4) contract_n(std::integral_constant<int, 4>(), f, g, g0);
+            else contract_n(std::integral_constant<int, JB>(), f, g, g0);
+        };
         // chunk reference row (FP32, stencil along the fiber): G(i0) . R
         if (!F64 && role == 1) {
             for (int f = warp; f < 5; f += NWARP) {
-                T acc[JB];
-                contract(f, in.core[f][mode] + (long long)i0 * rl * rr, nullptr, acc);
-                if (lane < cl4) Cref[f * CS + lane] = acc[0];
+                contract(f, in.core[f][mode] + (long long)i0 * rl * rr, nullptr);
+#pragma unroll
+                for (int q = 0; q < JB1; ++q)
+                    if (lane < cl4 && q < jb) Cref[(f * JB1 + q) * CS + lane] = acc[q];
             }
             __syncthreads();
         }
-        // contracted rows, zero-padded to a multiple of 4 entries; column = point (fd = m)
-        // or (row, fixed index)
+        // contracted rows, zero-padded to a multiple of 4 entries; column = (row or
+        // point, fixed index)
         const int np = role == 1 ? cn + 6 : cn;
         for (int u = warp; u < 5 * np; u += NWARP) {
             const int f = u / np, pp = u - f * np;
@@ -372,16 +399,16 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
             int c = role == 1 ? i0 - 3 + pp : i0 + pp;
             if (role == 1) c = xmap(in, fd, c, flip);
             const float *g = in.core[f][mode];
-            T acc[JB];
-            contract(f, g + (long long)c * rl * rr, !F64 && role == 1 ? g + (long long)i0 * rl * rr : nullptr, acc);
-            if (flip && f == 1 + fd && lane < cl4) acc[0] = F64 ? -acc[0] : -acc[0] - T(2) * Cref[f * CS + lane];
+            contract(f, g + (long long)c * rl * rr, !F64 && role == 1 ? g + (long long)i0 * rl * rr : nullptr);
+            flip = flip && f == 1 + fd;
             if (lane < cl4) {
-                T *row = C + (f * CP + (role == 1 ? pp : pp * jb)) * CS + lane;
-                row[0] = acc[0];
-                if (jb > 1) {
+                T *row = C + (f * CP + pp * jb) * CS + lane;
 #pragma unroll
-                    for (int q = 1; q < JB; ++q)
-                        if (q < jb) row[q * CS] = acc[q];
+                for (int q = 0; q < JB; ++q) {
+                    if (q < jb) {
+                        if (flip) acc[q] = F64 ? -acc[q] : -acc[q] - T(2) * Cref[(f * JB1 + (q & (JB1 - 1))) * CS + lane];
+                        row[q * CS] = acc[q];
+                    }
                 }
             }
         }
@@ -391,23 +418,28 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
             // The stencil moves along the fiber: neighbouring samples of one varying
             // index share six of their seven points and one of their two faces, so
             // each point's split flux and each face's WENO5(+/-) is formed once per
-            // block of vb varying indices (as many as make each phase one pass).
+            // block of vb lines (varying index, fixed index), as many as make each
+            // phase one pass.
             const int vb = XT / np;
-            for (long long v0 = 0; v0 < nvar; v0 += vb) {
-                const int nv = nvar - v0 < vb ? (int)(nvar - v0) : vb;
-                if constexpr (!F64) {  // reference values (row i0) of the block's varying indices
+            const long long nline = nvar * jn;
+            for (long long l0 = 0; l0 < nline; l0 += vb) {
+                const int nv = nline - l0 < vb ? (int)(nline - l0) : vb;
+                if constexpr (!F64) {  // reference values (row i0) of the block's lines
                     for (int u = threadIdx.x; u < nv * 5; u += XT) {
                         const int f = u % 5;
-                        CT[u] = row_dot(var + (v0 + u / 5) * nsv * 5 * VP + f * VP, Cref + f * CS, clen, cl4);
+                        const long long l = l0 + u / 5, v = l / jn;
+                        CT[u] = row_dot(var + v * nsv * 5 * VP + f * VP, Cref + (f * JB1 + (int)(l - v * jn)) * CS, clen, cl4);
                     }
                     __syncthreads();
                 }
                 for (int u = threadIdx.x; u < nv * np; u += XT) {  // split fluxes of every chunk point
                     const int vl = u / np, pp = u - vl * np;
-                    const T *lv = var + (v0 + vl) * nsv * 5 * VP;
+                    const long long l = l0 + vl, v = l / jn;
+                    const int col = pp * jb + (int)(l - v * jn);
+                    const T *lv = var + v * nsv * 5 * VP;
                     T q[5], a5[5], b5[5];
 #pragma unroll
-                    for (int f = 0; f < 5; ++f) q[f] = row_dot(lv + f * VP, C + (f * CP + pp) * CS, clen, cl4);
+                    for (int f = 0; f < 5; ++f) q[f] = row_dot(lv + f * VP, C + (f * CP + col) * CS, clen, cl4);
                     RefState<3> rs;
                     if constexpr (!F64) cross_ref(CT + vl * 5, (float)gm1, rs);
                     cross_flux(fd, q, rs, alpha, gm1, a5, b5);
@@ -426,7 +458,8 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
                 __syncthreads();
                 for (int u = threadIdx.x; u < nv * cn; u += XT) {
                     const int vl = u / cn, ii = u - vl * cn;
-                    const long long o = j0 * outstride_j + (v0 + vl) * outstride_v + (long long)(i0 + ii) * S.n_right;
+                    const long long l = l0 + vl, v = l / jn;
+                    const long long o = (j0 + (l - v * jn)) * outstride_j + v * outstride_v + (long long)(i0 + ii) * S.n_right;
 #pragma unroll
                     for (int f = 0; f < 5; ++f) {
                         const T *F = FF + f * XT + vl * (cn + 1) + ii;
@@ -439,11 +472,10 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
             continue;
         }
         // samples (v, column): 7 stencil values per field, split fluxes, two interfaces
-        const int ncol = cn * jb, jsh = jb == 4 ? 2 : jb == 2 ? 1 : 0;
+        const int ncol = cn * jn;
         for (long long u = threadIdx.x; u < nvar * ncol; u += XT) {
             const long long v = (unsigned long long)u < (1ull << 32) ? (long long)((unsigned)u / (unsigned)ncol) : u / ncol;
-            const int col = (int)(u - v * ncol), ii = col >> jsh, jj = col & (jb - 1);
-            if (jj >= jn) continue;
+            const int cu = (int)(u - v * ncol), ii = cu / jn, jj = cu - ii * jn, col = ii * jb + jj;
             T q7[5][7];  // FP64: values; FP32: differences from the reference state
             T ctr[5];    // the centre (FP32: the reference state)
 #pragma unroll
@@ -504,7 +536,7 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
 
 template <bool F64, int XT, int CH> static constexpr size_t cross_dyn_bytes()
 {
-    return (F64 ? sizeof(double) : sizeof(float)) * (size_t)CrossSmem<XT, CH>::total;
+    return (F64 ? sizeof(double) : sizeof(float)) * (size_t)CrossSmem<F64, XT, CH>::total;
 }
 
 int cross_vec_len() { return VP; }
@@ -518,8 +550,9 @@ void cross_default(bool fp64, int *variant, int *ctas_per_sm)
 // Work items of a set for the chunk length of a variant: jb fixed indices and
 // `rows` rows each.  Several fixed indices share a core row's loads and the
 // varying vectors; where there are few fixed indices the columns are rows.  With
-// fewer than a few items per resident CTA the rows are halved (to 8 rows per
-// fixed index, 16 where the stencil needs 6 halo rows).
+// fd = m several fixed indices pay for the larger share of halo rows only where a
+// row's matrix is large (64 entries).  With fewer than a few items per resident
+// CTA the rows are halved.
 long long cross_items(const CrossSet &S, int rows)
 {
     const long long nfix = S.fd > S.mode ? S.n_left : S.n_right;
@@ -532,15 +565,16 @@ long long cross_plan(CrossSet *sets, int n_sets, bool fp64, int variant)
     for (int k = 0; k < n_sets; ++k) {
         CrossSet &S = sets[k];
         const long long nfix = S.fd > S.mode ? S.n_left : S.n_right;
-        S.jb = S.fd == S.mode ? 1 : nfix >= 3 ? JB : (int)nfix;
-        S.rows = chunk / S.jb;
+        const int most = S.fd != S.mode ? cross_jb(fp64) : fp64 || S.r_mode < 64 ? 1 : JB1;
+        S.jb = (int)((nfix + (nfix + most - 1) / most - 1) / ((nfix + most - 1) / most));  // blocks of equal size
+        S.rows = S.fd != S.mode ? chunk / S.jb : S.jb == 1 ? chunk : (chunk + 6) / S.jb - 6;
         total += cross_items(S, S.rows);
     }
     for (int cut = 0; cut < 3 && total < 6ll * sm_count(); ++cut) {
         total = 0;
         for (int k = 0; k < n_sets; ++k) {
             CrossSet &S = sets[k];
-            const int least = S.fd == S.mode ? 16 : 8;
+            const int least = S.fd == S.mode ? (S.jb == 1 ? 16 : 8) : 4;
             if (S.rows / 2 >= least) S.rows /= 2;
             total += cross_items(S, S.rows);
         }
@@ -576,7 +610,7 @@ cudaError_t cross_set_attributes()
 #define X(V) \
     if ((r = set_attr<false, V>()) != cudaSuccess) e = r; \
     if ((r = set_attr<true, V>()) != cudaSuccess) e = r;
-    X(0) X(1) X(2) X(3) X(4) X(5) X(6)
+    X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
 #undef X
     if (e == cudaSuccess) done = true;
     return e;
@@ -608,7 +642,7 @@ cudaError_t launch_cross(const CrossArgs &a, int variant, int ctas_per_sm, cudaS
     if (blocks < 1) blocks = 1;
 #define X(V)                                                                             \
     if (variant == V) return a.fp64 ? launch_main<true, V>(a, blocks, s) : launch_main<false, V>(a, blocks, s);
-    X(0) X(1) X(2) X(3) X(4) X(5) X(6)
+    X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
 #undef X
     return cudaErrorInvalidValue;
 }
