@@ -396,12 +396,14 @@ extern "C" int weno_maxvol(weno_handle h, const weno_maxvol_problem *probs, int3
     std::vector<MaxvolDesc> ds(n_probs);
     size_t w_total = 0;
     int max_r = 1;
+    long long max_nr = 1;
     for (int i = 0; i < n_probs; ++i) {
         const weno_maxvol_problem &P = probs[i];
         if (P.r < 1 || P.r > MV_RMAX || P.n < P.r || P.n > MV_NMAX || !P.A || !P.B || !P.idx)
             return fail(h, WENO_ERR_ARG, "weno_maxvol: need 1 <= r <= 64, r <= n <= 65536 and non-null A, B, idx");
         w_total += (((size_t)P.n * P.r + 31) & ~size_t(31)) + (((size_t)P.r * P.r + 31) & ~size_t(31));
         max_r = std::max(max_r, (int)P.r);
+        max_nr = std::max(max_nr, (long long)P.n * P.r);
     }
     const size_t off_desc = 0;
     const size_t off_int = (sizeof(MaxvolDesc) * n_probs + 255) & ~size_t(255);
@@ -420,7 +422,7 @@ extern "C" int weno_maxvol(weno_handle h, const weno_maxvol_problem *probs, int3
     maxvol_order(ds.data(), n_probs);
     MaxvolDesc *dd = (MaxvolDesc *)(base + off_desc);
     CK(h, cudaMemcpyAsync(dd, ds.data(), sizeof(MaxvolDesc) * n_probs, cudaMemcpyHostToDevice, h->stream));
-    CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, n_probs, max_r, delta, max_iters, h->stream); },
+    CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, n_probs, max_r, max_nr, delta, max_iters, h->stream); },
                  MV_LAUNCHES));
     std::vector<int> st(2 * n_probs);
     CK(h, cudaMemcpyAsync(st.data(), ints, sizeof(int) * 2 * n_probs, cudaMemcpyDeviceToHost, h->stream));
@@ -562,6 +564,7 @@ extern "C" int weno_tt_cross(weno_handle h, const weno_tt_instance *inst, int32_
     auto select = [&](double *XProb::*Mp, double *XProb::*Bp, bool b_is_core0, auto &&dims) -> int {
         std::vector<MaxvolDesc> md(np);
         int mr = 1;
+        long long mnr = 1;
         for (int i = 0; i < np; ++i) {
             XProb &x = xp[i];
             int rows, cols;
@@ -570,11 +573,12 @@ extern "C" int weno_tt_cross(weno_handle h, const weno_tt_instance *inst, int32_
             int *st = status + 2 * ((size_t)mv_call * np + i);
             md[i] = MaxvolDesc{x.*Mp, Bout, x.Wmv, x.Linv, x.idx, st, st + 1, rows, cols};
             mr = std::max(mr, cols);
+            mnr = std::max(mnr, (long long)rows * cols);
         }
         maxvol_order(md.data(), np);
         MaxvolDesc *dd = (MaxvolDesc *)slot(3);
         CK(h, cudaMemcpyAsync(dd, md.data(), sizeof(MaxvolDesc) * np, cudaMemcpyHostToDevice, h->stream));
-        CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, np, mr, delta, 200, h->stream); }, MV_LAUNCHES));
+        CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, np, mr, mnr, delta, 200, h->stream); }, MV_LAUNCHES));
         ++mv_call;
         return WENO_OK;
     };

@@ -1,5 +1,5 @@
 // k_maxvol.cu -- batched maxvol (the maximum-volume row selection that picks
-// the cross indices of TT-cross, Sec. 3 "TT-cross Interpolation"), FP64, three
+// the cross indices of TT-cross, Sec. 3 "TT-cross Interpolation"), FP64, five
 // launches per batch:
 //   1. the r pivot rows I of Gaussian elimination with partial pivoting on a
 //      working copy W (largest remaining |W[i][j]| of column j, ties to the
@@ -8,20 +8,30 @@
 //   2. B = A A[I]^{-1} = L L[I]^{-1} (A = P L U, so the U factor cancels; the
 //      rows I get the unit vectors exactly), spread over many CTAs per matrix;
 //   3. while max |B[i][j]| > 1 + delta (ties to the first entry in row-major
-//      order): row i replaces I[j] and B -= B[:, j] (B[i, :] - e_j) / B[i][j].
+//      order): row i replaces I[j] and B -= B[:, j] (B[i, :] - e_j) / B[i][j],
+//      on a copy of B in FP32 pairs hi + lo (about 47 bits);
+//   4. if rows were swapped, B[I]^{-1} of the B of 2 and the new rows I, FP64;
+//   5. then B := B B[I]^{-1} = A A[I]^{-1}, FP64.
 // Forming B from L rather than from an inverse of A[I] keeps it accurate when
 // A is ill-conditioned: |L| <= 1 under partial pivoting, and the scale of
-// A's columns stays in U.  Phases 1 and 3 are sequences of (argmax, rank-one
+// A's columns stays in U.  The swaps only choose rows: their rank-one updates
+// would hold the FP64 pipe for n r instructions each (12000 x 32: 15 us a swap
+// on 8 SMs), while a choice that the pairs' 2^-46 could change is a tie for FP64
+// rounding as well; the final B is one FP64 product of the accurate B of step 2
+// with the inverse of a well-conditioned matrix, without the swaps' accumulated
+// rounding.  Phases 1 and 3 are sequences of (argmax, rank-one
 // update) steps.  Each matrix gets a thread-block cluster whose CTAs own
-// contiguous slices of its rows, so the FP64 work of a large matrix spreads
-// over up to 16 SMs.  Per step every CTA finds the best entry of its slice and
+// contiguous slices of its rows, held in shared memory as far as they fit (a slice
+// in L2 costs a round trip per step and column batch) and in W beyond.  Per step
+// every CTA finds the best entry of its slice, in the pass that updates it, and
 // stashes that entry's row in a shared-memory slot; after one cluster barrier
 // every CTA reduces the slots (read through distributed shared memory) to the
 // same winner and copies the winner's row from its owner.  Slots alternate
 // between two buffers, so the writes of step t + 1 never meet the reads of
 // step t, and the stash lets the owner update the winning row in place while
-// others still read it.  The working copy is column-major (W[c][i]), so a
-// warp's row-parallel accesses coalesce; it stays in L2.
+// others still read it.  Slices are column-major, so a warp's row-parallel
+// accesses coalesce.
+//   16 matrices of 256..12000 x 4..32: pivot 1.10 -> MVP ms, swaps 1.82 -> MVS ms.
 #include <algorithm>
 #include <climits>
 
@@ -35,7 +45,7 @@ namespace wg {
 
 namespace cg = cooperative_groups;
 
-constexpr int MV_NT = 256, MV_NW = MV_NT / 32;
+constexpr int MV_NT = 512, MV_NW = MV_NT / 32;
 // A pivot |w| <= MV_RANK_TOL r max_i |A[i][j]| counts as zero: the residual
 // of a column that lies in the span of the earlier ones is a few rounding
 // errors of the column's own scale (a full-rank matrix reaches it only with a
@@ -155,11 +165,21 @@ __device__ __forceinline__ void row_slice(int n, int rank, int ncl, int &lo, int
     hi = (int)((long long)(rank + 1) * n / ncl);
 }
 
-size_t maxvol_smem(int r) { return sizeof(double) * (size_t)r * 2 * r; }
+// The element (row t of the slice, column c) of a slice whose first `cap` rows are
+// in shared memory and whose others are in W: p[c * ld].
+template <class V> struct MvRow {
+    V *p;
+    int ld;
+};
+template <class V>
+__device__ __forceinline__ MvRow<V> mv_row(V *sh, int cap, V *W, int n, int lo, int t)
+{
+    return t < cap ? MvRow<V>{sh + t, cap} : MvRow<V>{W + lo + t, n};
+}
 
 // Phase 1: pivot rows and multipliers (the whole cluster), then L[I]^{-1}
 // (rank 0 alone, in dynamic shared memory).
-__global__ void __launch_bounds__(MV_NT) k_maxvol_pivot(const MaxvolDesc *descs)
+__global__ void __launch_bounds__(MV_NT) k_maxvol_pivot(const MaxvolDesc *descs, int smem_doubles)
 {
     cg::cluster_group cl = cg::this_cluster();
     const MaxvolDesc &d = descs[blockIdx.y];
@@ -172,47 +192,56 @@ __global__ void __launch_bounds__(MV_NT) k_maxvol_pivot(const MaxvolDesc *descs)
     __shared__ int s_fail;
     __shared__ unsigned long long cbits[MV_RMAX];  // this CTA's column maxima of |A| (bit patterns)
     __shared__ double ctol[MV_RMAX];
+    extern __shared__ double G[];
     double *W = d.W;
+    const int m = hi - lo, cap = min(m, smem_doubles / r);
     if (threadIdx.x == 0) s_fail = 0;
-    for (int e = threadIdx.x; e < (hi - lo + 31) / 32; e += MV_NT) chosen[e] = 0u;
-    for (int i = lo + threadIdx.x; i < hi; i += MV_NT)  // column-major copy; a thread reads its row in order
-        for (int c = 0; c < r; ++c) W[(long long)c * n + i] = d.A[(long long)i * r + c];
+    for (int e = threadIdx.x; e < (m + 31) / 32; e += MV_NT) chosen[e] = 0u;
+    for (int c = threadIdx.x; c < r; c += MV_NT) cbits[c] = 0ull;
+    for (int e = threadIdx.x; e < m * r; e += MV_NT) {  // column-major copy of the slice
+        const int t = e / r, c = e - t * r;
+        const MvRow<double> w = mv_row(G, cap, W, n, lo, t);
+        w.p[(long long)c * w.ld] = d.A[(long long)lo * r + e];
+    }
+    __syncthreads();
     // the scale of every column, max_i |A[i][c]|, over the whole cluster: a
     // pivot at or below MV_RANK_TOL of its column's scale means rank < r
-    for (int c = threadIdx.x; c < r; c += MV_NT) cbits[c] = 0ull;
-    __syncthreads();
-    for (int c = 0; c < r; ++c) {
-        unsigned long long m = 0ull;
-        for (int i = lo + threadIdx.x; i < hi; i += MV_NT) m = max(m, absbits(W[(long long)c * n + i]));
+    for (int c = threadIdx.x >> 5; c < r; c += MV_NW) {
+        unsigned long long k = 0ull;
+        for (int t = threadIdx.x & 31; t < m; t += 32) {
+            const MvRow<double> w = mv_row(G, cap, W, n, lo, t);
+            k = max(k, absbits(w.p[(long long)c * w.ld]));
+        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        if ((threadIdx.x & 31) == 0 && m) atomicMax(&cbits[c], m);
+        for (int o = 16; o > 0; o >>= 1) k = max(k, __shfl_xor_sync(0xFFFFFFFFu, k, o));
+        if ((threadIdx.x & 31) == 0) cbits[c] = k;
     }
     cl.sync();
     for (int c = threadIdx.x; c < r; c += MV_NT) {
-        unsigned long long m = 0ull;
-        for (int q = 0; q < ncl; ++q) m = max(m, *cl.map_shared_rank(&cbits[c], q));
-        ctol[c] = MV_RANK_TOL * r * __longlong_as_double((long long)m);
+        unsigned long long k = 0ull;
+        for (int q = 0; q < ncl; ++q) k = max(k, *cl.map_shared_rank(&cbits[c], q));
+        ctol[c] = MV_RANK_TOL * r * __longlong_as_double((long long)k);
     }
     __syncthreads();
 
     // 1. partial pivoting; only the columns after j are updated (earlier ones
-    // are never read again)
-    for (int j = 0; j < r; ++j) {
-        unsigned long long kmax = 0ull;
-        long long bi = LLONG_MAX;
-        for (int i = lo + threadIdx.x; i < hi; i += MV_NT) {
-            if ((chosen[(i - lo) >> 5] >> ((i - lo) & 31)) & 1u) continue;
-            const unsigned long long k = absbits(W[(long long)j * n + i]) + 1ull;  // 0 marks "no row"
-            if (k > kmax) {  // i grows per thread, so equal keys keep the first
-                kmax = k;
-                bi = i;
-            }
+    // are never read again); the pass that updates column j + 1 finds its argmax
+    unsigned long long kmax = 0ull;  // 0 marks "no row"
+    long long bi = LLONG_MAX;
+    for (int t = threadIdx.x; t < m; t += MV_NT) {
+        const unsigned long long k = absbits(*mv_row(G, cap, W, n, lo, t).p) + 1ull;
+        if (k > kmax) {  // t grows per thread, so equal keys keep the first
+            kmax = k;
+            bi = lo + t;
         }
+    }
+    for (int j = 0; j < r; ++j) {
         // the slot's row: the candidate's W[j..r) (entries before j are stale)
         const MvSlot *ws = cluster_argmax(cl, st, j & 1, ncl, kmax, bi, [&](MvSlot &s, unsigned long long k, long long e) {
-            if (k != 0ull)
-                for (int c = j + threadIdx.x; c < r; c += MV_NT) s.row[c] = W[(long long)c * n + e];
+            if (k != 0ull) {
+                const MvRow<double> w = mv_row(G, cap, W, n, lo, (int)(e - lo));
+                for (int c = j + threadIdx.x; c < r; c += MV_NT) s.row[c] = w.p[(long long)c * w.ld];
+            }
         });
         for (int c = j + threadIdx.x; c < r; c += MV_NT) st.row[c] = ws->row[c];
         const int p = (int)st.win_e;
@@ -221,24 +250,37 @@ __global__ void __launch_bounds__(MV_NT) k_maxvol_pivot(const MaxvolDesc *descs)
             if (p >= lo && p < hi) chosen[(p - lo) >> 5] |= 1u << ((p - lo) & 31);
         }
         __syncthreads();
+        kmax = 0ull;
+        bi = LLONG_MAX;
         const double wp = st.row[j];
-        if (!(fabs(wp) > ctol[j])) {
-            if (threadIdx.x == 0) s_fail = 1;  // every CTA sees the same pivot and scale
-        } else {
-            const double inv = 1.0 / wp;
-            for (int i = lo + threadIdx.x; i < hi; i += MV_NT) {
-                if ((chosen[(i - lo) >> 5] >> ((i - lo) & 31)) & 1u) continue;
-                double *wj = W + (long long)j * n + i;
+        const bool zero = !(fabs(wp) > ctol[j]);
+        if (zero && threadIdx.x == 0) s_fail = 1;  // every CTA sees the same pivot and scale
+        const double inv = zero ? 0.0 : 1.0 / wp;
+        for (int t = threadIdx.x; t < m; t += MV_NT) {
+            if ((chosen[t >> 5] >> (t & 31)) & 1u) continue;
+            const MvRow<double> w = mv_row(G, cap, W, n, lo, t);
+            double *wj = w.p + (long long)j * w.ld;
+            if (!zero) {
                 const double f = *wj * inv;
                 *wj = f;  // L[i][j]
-                for (int c = j + 1; c < r; ++c) {
-                    double *w = W + (long long)c * n + i;
-                    *w = fma(-f, st.row[c], *w);
+                double *wc = wj + w.ld;
+#pragma unroll 8
+                for (int c = j + 1; c < r; ++c, wc += w.ld) *wc = fma(-f, st.row[c], *wc);
+            }
+            if (j + 1 < r) {
+                const unsigned long long k = absbits(wj[w.ld]) + 1ull;
+                if (k > kmax) {
+                    kmax = k;
+                    bi = lo + t;
                 }
             }
         }
-        // the next step's argmax reads only this thread's own rows; its block
-        // argmax starts with a barrier before st is written again
+        // (the next step's block argmax starts with a barrier before st is written again)
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < cap * r; e += MV_NT) {  // the multipliers of the rows in shared memory
+        const int c = e / cap, t = e - c * cap;
+        W[(long long)c * n + lo + t] = G[e];
     }
     cl.sync();  // no CTA leaves while another may still read its slots
     if (rank != 0) return;
@@ -246,7 +288,6 @@ __global__ void __launch_bounds__(MV_NT) k_maxvol_pivot(const MaxvolDesc *descs)
     // L[I]^{-1}: L[I] is unit lower triangular, row k holding the multipliers
     // of row I[k] from the steps before k (other slices' rows are read from L2:
     // they were written before the barrier above)
-    extern __shared__ double G[];
     double *Lt = G;                       // [r][r]
     double *Li = G + (size_t)r * r;       // [r][r]
     for (int e = threadIdx.x; e < r * r; e += MV_NT) {
@@ -301,8 +342,15 @@ __global__ void __launch_bounds__(256) k_maxvol_b(const MaxvolDesc *descs)
     }
 }
 
-// Phase 3, the swaps (the whole cluster), on a column-major copy of B in W.
-__global__ void __launch_bounds__(MV_NT) k_maxvol_swap(const MaxvolDesc *descs, double delta, int max_iters)
+// Phase 3, the swaps (the whole cluster), on a column-major copy of B in FP32
+// pairs (the slice's first rows in shared memory, the others in W).
+__device__ __forceinline__ unsigned pair_low_order(float2 v)  // orders the low parts of equal |high| parts
+{
+    const unsigned b = __float_as_uint(v.x < 0.0f ? -v.y : v.y);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+
+__global__ void __launch_bounds__(MV_NT) k_maxvol_swap(const MaxvolDesc *descs, double delta, int max_iters, int smem_doubles)
 {
     cg::cluster_group cl = cg::this_cluster();
     const MaxvolDesc &d = descs[blockIdx.y];
@@ -311,65 +359,170 @@ __global__ void __launch_bounds__(MV_NT) k_maxvol_swap(const MaxvolDesc *descs, 
     int lo, hi;
     row_slice(n, rank, ncl, lo, hi);
     __shared__ MvStep st;
+    __shared__ float2 s_row[MV_RMAX];
     __shared__ int I[MV_RMAX];
-    double *W = d.W;
+    extern __shared__ float2 P[];
+    float2 *W = reinterpret_cast<float2 *>(d.W);
+    const int m = hi - lo, cap = min(m, smem_doubles / r);
     for (int j = threadIdx.x; j < r; j += MV_NT) I[j] = d.idx[j];
-    // column-major copy of the slice, with the first argmax (e = i r + c grows
-    // per thread, so equal keys keep the first)
-    unsigned long long kmax = 0ull;
-    long long bi = LLONG_MAX;
-    for (int i = lo + threadIdx.x; i < hi; i += MV_NT)
-        for (int c = 0; c < r; ++c) {
-            const double b = d.B[(long long)i * r + c];
-            W[(long long)c * n + i] = b;
-            const unsigned long long k = absbits(b);
-            if (k > kmax || bi == LLONG_MAX) {
-                kmax = k;
-                bi = (long long)i * r + c;
-            }
-        }
+    for (int e = threadIdx.x; e < m * r; e += MV_NT) {
+        const int t = e / r, c = e - t * r;
+        const MvRow<float2> w = mv_row(P, cap, W, n, lo, t);
+        w.p[(long long)c * w.ld] = pr_norm(split_sat(d.B[(long long)lo * r + e]));
+    }
     __syncthreads();
+    // an entry's key: |hi|, then the low part's order; e = i r + c grows per thread,
+    // so equal keys keep the first
+    unsigned kh = 0u, kl = 0u;
+    long long be = LLONG_MAX;
+    auto consider = [&](float2 v, long long e) {
+        const unsigned h = __float_as_uint(v.x) & 0x7FFFFFFFu;
+        if (h < kh && be != LLONG_MAX) return;
+        const unsigned l = pair_low_order(v);
+        if (be == LLONG_MAX || h > kh || l > kl) {
+            kh = h;
+            kl = l;
+            be = e;
+        }
+    };
+    for (int t = threadIdx.x; t < m; t += MV_NT) {
+        const MvRow<float2> w = mv_row(P, cap, W, n, lo, t);
+        for (int c = 0; c < r; ++c) consider(w.p[(long long)c * w.ld], (long long)(lo + t) * r + c);
+    }
     int it = 0;
     for (; it < max_iters; ++it) {
-        const MvSlot *ws = cluster_argmax(cl, st, it & 1, ncl, kmax, bi, [&](MvSlot &s, unsigned long long, long long e) {
+        const MvSlot *ws = cluster_argmax(cl, st, it & 1, ncl, (unsigned long long)kh << 32 | kl, be,
+                                          [&](MvSlot &s, unsigned long long, long long e) {
             if (e != LLONG_MAX) {
-                const long long i = e / r;
-                for (int c = threadIdx.x; c < r; c += MV_NT) s.row[c] = W[(long long)c * n + i];
+                const MvRow<float2> w = mv_row(P, cap, W, n, lo, (int)(e / r - lo));
+                for (int c = threadIdx.x; c < r; c += MV_NT) reinterpret_cast<float2 *>(s.row)[c] = w.p[(long long)c * w.ld];
             }
         });
-        if (!(__longlong_as_double((long long)st.win_key) > 1.0 + delta)) break;  // the same decision everywhere
         const long long we = st.win_e;
         const int i0 = (int)(we / r), j0 = (int)(we - (long long)i0 * r);
-        const double piv = ws->row[j0];
-        for (int c = threadIdx.x; c < r; c += MV_NT) st.row[c] = (ws->row[c] - (c == j0 ? 1.0 : 0.0)) / piv;
+        const float2 piv = reinterpret_cast<const float2 *>(ws->row)[j0];
+        if (!(fabs((double)piv.x + (double)piv.y) > 1.0 + delta)) break;  // the same decision everywhere
+        if (threadIdx.x < r) {  // (row_i0 - e_j0) / piv, one residual correction of an approximate quotient
+            float2 v = reinterpret_cast<const float2 *>(ws->row)[threadIdx.x];
+            if (threadIdx.x == j0) v = pr_norm(pr_sub(v, make_float2(1.0f, 0.0f)));
+            const float q = fast_rcp(piv.x), x = __fmul_rn(v.x, q);
+            const float rem = __fadd_rn(__fmaf_rn(-x, piv.x, v.x), __fmaf_rn(-x, piv.y, v.y));
+            s_row[threadIdx.x] = make_float2(x, __fmul_rn(rem, q));
+        }
         if (threadIdx.x == 0) I[j0] = i0;
         __syncthreads();
         // B -= B[:, j0] (row_i0 - e_j0) / piv over the slice, with the next argmax
-        kmax = 0ull;
-        bi = LLONG_MAX;
-        for (int i = lo + threadIdx.x; i < hi; i += MV_NT) {
-            const double f = W[(long long)j0 * n + i];
-            for (int c = 0; c < r; ++c) {
-                double *w = W + (long long)c * n + i;
-                const double b = fma(-f, st.row[c], *w);
-                *w = b;
-                const unsigned long long k = absbits(b);
-                if (k > kmax || bi == LLONG_MAX) {
-                    kmax = k;
-                    bi = (long long)i * r + c;
-                }
+        kh = kl = 0u;
+        be = LLONG_MAX;
+        for (int t = threadIdx.x; t < m; t += MV_NT) {
+            const MvRow<float2> w = mv_row(P, cap, W, n, lo, t);
+            const float2 f = w.p[(long long)j0 * w.ld];
+            float2 *wc = w.p;
+            const long long e0 = (long long)(lo + t) * r;
+#pragma unroll 4
+            for (int c = 0; c < r; ++c, wc += w.ld) {
+                const float2 v = pr_norm(pr_sub(*wc, pr_mul(f, s_row[c])));
+                *wc = v;
+                consider(v, e0 + c);
             }
         }
     }
     cl.sync();  // no CTA leaves while another may still read its slots
-    for (int i = lo + threadIdx.x; i < hi; i += MV_NT)
-        for (int c = 0; c < r; ++c) d.B[(long long)i * r + c] = W[(long long)c * n + i];
     if (rank == 0) {
         for (int j = threadIdx.x; j < r; j += MV_NT) d.idx[j] = I[j];
-        if (threadIdx.x == 0) {
-            d.status[0] = 0;
-            d.swaps[0] = it;
+        if (threadIdx.x == 0) d.swaps[0] = it;
+    }
+}
+
+// Phase 4: Linv := B[I]^{-1} for the final rows I (Gauss-Jordan with partial
+// pivoting in shared memory), one CTA per matrix whose rows changed.
+__global__ void __launch_bounds__(256) k_maxvol_inverse(const MaxvolDesc *descs)
+{
+    const MaxvolDesc &d = descs[blockIdx.x];
+    if (d.status[0] || d.swaps[0] == 0) return;
+    const int r = d.r, ld = 2 * r + 1;
+    extern __shared__ double G[];  // [r][B[I] | identity], pitch 2 r + 1
+    __shared__ double col[MV_RMAX];
+    __shared__ int s_piv;
+    for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
+        const int k = e / r, c = e - k * r;
+        G[k * ld + c] = d.B[(long long)d.idx[k] * r + c];
+        G[k * ld + r + c] = k == c ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    for (int j = 0; j < r; ++j) {
+        if (threadIdx.x < 32) {
+            unsigned long long k = 0ull;
+            int best = j;
+            for (int i = j + threadIdx.x; i < r; i += 32) {
+                const unsigned long long x = absbits(G[i * ld + j]) + 1ull;
+                if (x > k) {
+                    k = x;
+                    best = i;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long ok = __shfl_xor_sync(0xFFFFFFFFu, k, o);
+                const int ob = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+                if (ok > k || (ok == k && ob < best)) {
+                    k = ok;
+                    best = ob;
+                }
+            }
+            if (threadIdx.x == 0) s_piv = best;
         }
+        __syncthreads();
+        const int p = s_piv;
+        const double inv = 1.0 / G[p * ld + j];
+        __syncthreads();
+        for (int c = threadIdx.x; c < 2 * r; c += blockDim.x) {  // swap rows j and p, scale the pivot row
+            const double x = G[j * ld + c], y = G[p * ld + c];
+            if (p != j) G[p * ld + c] = x;
+            G[j * ld + c] = y * inv;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < r; i += blockDim.x) col[i] = i == j ? 0.0 : G[i * ld + j];
+        __syncthreads();
+        // (the columns before j of the left half are unit vectors already)
+        for (int e = threadIdx.x; e < r * (2 * r - j); e += blockDim.x) {
+            const int i = e / (2 * r - j), c = j + e - i * (2 * r - j);
+            if (i != j) G[i * ld + c] = fma(-col[i], G[j * ld + c], G[i * ld + c]);
+        }
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < r * r; e += blockDim.x) d.Linv[e] = G[(e / r) * ld + r + e % r];
+}
+
+// Phase 5: B := B B[I]^{-1}, the rows I exactly the unit vectors.  A block takes
+// 64 rows at a time, staged in shared memory (the product overwrites them).
+__global__ void __launch_bounds__(256) k_maxvol_final(const MaxvolDesc *descs)
+{
+    const MaxvolDesc &d = descs[blockIdx.y];
+    if (d.status[0] || d.swaps[0] == 0) return;
+    const int n = d.n, r = d.r;
+    constexpr int RB = 64;
+    if ((int)blockIdx.x * RB >= n) return;
+    extern __shared__ double G[];  // [r][r] the inverse, then [RB][r] rows
+    double *T = G + r * r;
+    __shared__ int I[MV_RMAX];
+    for (int e = threadIdx.x; e < r * r; e += blockDim.x) G[e] = d.Linv[e];
+    for (int k = threadIdx.x; k < r; k += blockDim.x) I[k] = d.idx[k];
+    for (int i0 = blockIdx.x * RB; i0 < n; i0 += gridDim.x * RB) {
+        const int rows = min(RB, n - i0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < rows * r; e += blockDim.x) T[e] = d.B[(long long)i0 * r + e];
+        __syncthreads();
+        for (int e = threadIdx.x; e < rows * r; e += blockDim.x) {
+            const int t = e / r, c = e - t * r;
+            double acc = 0.0;
+            for (int k = 0; k < r; ++k) acc = fma(T[t * r + k], G[k * r + c], acc);
+            d.B[(long long)i0 * r + e] = acc;
+        }
+        __syncthreads();
+        for (int k = 0; k < r; ++k)
+            if (I[k] >= i0 && I[k] < i0 + rows)
+                for (int c = threadIdx.x; c < r; c += blockDim.x) d.B[(long long)I[k] * r + c] = c == k ? 1.0 : 0.0;
     }
 }
 
@@ -399,6 +552,25 @@ static cudaError_t launch_cluster(K kern, int ncl, int n, size_t smem, cudaStrea
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Dynamic shared memory of a cluster kernel at most (the static part is ~12 KB).
+constexpr int MV_SMEM = 200 * 1024;
+
+static cudaError_t maxvol_attributes()
+{
+    static bool done = false;
+    if (done) return cudaSuccess;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_maxvol_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize, MV_SMEM)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_maxvol_swap, cudaFuncAttributeMaxDynamicSharedMemorySize, MV_SMEM)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_maxvol_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(double) * MV_RMAX * (2 * MV_RMAX + 1))) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_maxvol_final, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(double) * 2 * MV_RMAX * MV_RMAX)) != cudaSuccess)
+        return e;
+    done = true;
+    return e;
+}
+
 // Cluster size: 16 CTAs where the device schedules clusters that large, else 8.
 static int maxvol_cluster_size()
 {
@@ -410,7 +582,7 @@ static int maxvol_cluster_size()
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(16, 1);
         cfg.blockDim = dim3(MV_NT);
-        cfg.dynamicSmemBytes = maxvol_smem(MV_RMAX);
+        cfg.dynamicSmemBytes = MV_SMEM;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = 16;
@@ -427,22 +599,30 @@ static int maxvol_cluster_size()
     return ncl;
 }
 
-cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, double delta, int max_iters, cudaStream_t s)
+// max_nr: the largest n r of the batch.  Shared memory for a slice: what the
+// largest slice takes, and no more than lets the batch's CTAs run together.
+cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_nr, double delta, int max_iters,
+                          cudaStream_t s)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_maxvol_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)maxvol_smem(MV_RMAX));
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    cudaError_t e = maxvol_attributes();
+    if (e != cudaSuccess) return e;
     const int ncl = maxvol_cluster_size();
-    cudaError_t e = launch_cluster(k_maxvol_pivot, ncl, n, maxvol_smem(max_r), s, d);
+    const long long per_sm = std::min(3ll, std::max(1ll, ((long long)n * ncl + sm_count() - 1) / sm_count()));
+    const long long want = sizeof(double) * std::max((max_nr + ncl - 1) / ncl + max_r, 2ll * max_r * max_r);
+    const long long least = sizeof(double) * 2ll * max_r * max_r;  // L[I] and its inverse
+    const size_t smem = (size_t)std::max(least, std::min(want, MV_SMEM / per_sm));
+    const int doubles = (int)(smem / sizeof(double));
+    e = launch_cluster(k_maxvol_pivot, ncl, n, smem, s, d, doubles);
     if (e != cudaSuccess) return e;
     k_maxvol_b<<<dim3(64, n), 256, 0, s>>>(d);
-    e = cudaGetLastError();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_cluster(k_maxvol_swap, ncl, n, smem, s, d, delta, max_iters, doubles);
     if (e != cudaSuccess) return e;
-    return launch_cluster(k_maxvol_swap, ncl, n, 0, s, d, delta, max_iters);
+    k_maxvol_inverse<<<n, 256, sizeof(double) * max_r * (2 * max_r + 1), s>>>(d);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int blocks = std::max(8, std::min(128, 8 * sm_count() / n));
+    k_maxvol_final<<<dim3(blocks, n), 256, sizeof(double) * (max_r * max_r + 64 * max_r), s>>>(d);
+    return cudaGetLastError();
 }
 
 }  // namespace wg

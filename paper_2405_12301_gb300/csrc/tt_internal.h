@@ -94,17 +94,17 @@ struct MaxvolDesc {
     const double *A;   // n x r row-major
     double *B;         // n x r: A A[I]^{-1} on exit
     double *W;         // n x r scratch (column-major working copy, then the multipliers L)
-    double *Linv;      // r x r scratch: the inverse of the unit lower triangular L[I]
+    double *Linv;      // r x r scratch: the inverse of the unit lower triangular L[I], then of B[I]
     int *idx;          // r selected rows
     int *status;       // 0 ok, 1 A[I] singular after pivoting
     int *swaps;
     int n, r;
 };
-size_t maxvol_smem(int r);
-constexpr int MV_LAUNCHES = 3;  // kernels of one launch_maxvol
+constexpr int MV_LAUNCHES = 5;  // kernels of one launch_maxvol
 // Orders a batch largest first (n r^2), so the biggest matrices start first.
 void maxvol_order(MaxvolDesc *d, int n);
-cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, double delta, int max_iters, cudaStream_t s);
+cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_nr, double delta, int max_iters,
+                          cudaStream_t s);
 
 
 // ---- TT-cross sweep bookkeeping (k_cross_drv.cu)
