@@ -15,31 +15,53 @@ using namespace wg;
 
 namespace {
 
+// A TSQR tree: level 0 factors chunks of the matrix's rows, each further level
+// groups of the R factors of the one before, until one R is left.
 struct QRPlan {
-    long long m = 0;
-    int k = 0, b = 32, C = 1, sub = 1, top_sub = 0;
-    long long chunk_rows = 0;
-    double *A = nullptr, *tau = nullptr, *Rc = nullptr, *tau_top = nullptr, *T = nullptr;
+    struct Level {
+        long long m = 0, rows = 0;  // rows of the level's matrix, rows per chunk
+        int C = 1, sub = 1;         // chunks, sub-blocks per chunk
+        double *A = nullptr, *tau = nullptr, *R = nullptr, *X = nullptr;  // (X: the stack of the chunks' top rows)
+    };
+    int k = 0, b = 32;
+    std::vector<Level> L;
+    std::vector<Level> buf;  // the buffers taken for it
+    double *T = nullptr;
 };
+constexpr int QR_MAXL = 24;  // levels at most (a matrix of 2^27 rows takes 15)
 
-// Chunking of an m x k QR: sub-blocks of b >= k rows, at most 16 per chunk,
-// every chunk at least k rows long when there are several.
-void qr_plan(QRPlan &q, long long m, int k)
+// Sub-blocks of b >= k rows, at most spc per chunk, every chunk at least k rows
+// long when there are several; then g R factors per chunk: two where the batch is
+// small (the tree's depth is the time), four where it fills the GPU.
+// more: plan for that many chunks beyond what m needs (to size buffers).
+void qr_plan(QRPlan &q, long long m, int k, int spc, int g, int more = 0)
 {
-    q.m = m;
     q.k = k;
     q.b = k <= 32 ? 32 : (k + 31) / 32 * 32;
-    int C = (int)std::max(1LL, (m + 16LL * q.b - 1) / (16LL * q.b));
-    for (;; --C) {
+    q.L.clear();
+    QRPlan::Level l;
+    l.m = m;
+    const long long per = (long long)spc * q.b;
+    for (int C = (int)std::max(1LL, (m + per - 1) / per);; --C) {
         const long long cr = (m + C - 1) / C;
         if (C == 1 || (cr >= k && m - (long long)(C - 1) * cr >= k)) {
-            q.C = C;
-            q.chunk_rows = std::max(1LL, cr);
+            l.C = C;
+            l.rows = std::max(1LL, cr);
             break;
         }
     }
-    q.sub = (int)((q.chunk_rows + q.b - 1) / q.b);
-    q.top_sub = q.C > 1 ? (int)(((long long)q.C * k + q.b - 1) / q.b) : 0;
+    l.sub = (int)((l.rows + q.b - 1) / q.b);
+    q.L.push_back(l);
+    q.L[0].C += more;
+    while (q.L.back().C > 1) {
+        const int C = q.L.back().C;
+        l = QRPlan::Level();
+        l.m = (long long)C * k;
+        l.C = (C + g - 1) / g;
+        l.sub = g;
+        l.rows = (long long)g * k;
+        q.L.push_back(l);
+    }
 }
 
 struct Bump {  // counts (base == nullptr) or hands out 256-byte aligned pieces
@@ -54,55 +76,72 @@ struct Bump {  // counts (base == nullptr) or hands out 256-byte aligned pieces
     }
 };
 
-void qr_take(Bump &bp, QRPlan &q)
+// Buffers for the QR of an m x k matrix and for applying it to p columns, also for
+// any smaller m of the same k and spc (whose plan has at most one chunk more).
+void qr_take(Bump &bp, QRPlan &q, long long m, int k, int spc, int g, int p)
 {
-    q.tau = bp.take<double>((size_t)q.C * q.sub * q.k);
-    q.Rc = bp.take<double>((size_t)q.C * q.k * q.k);
-    if (q.C > 1) {
-        q.tau_top = bp.take<double>((size_t)q.top_sub * q.k);
-        q.T = bp.take<double>((size_t)q.k * q.k);
-    } else {
-        q.T = q.Rc;
+    QRPlan big;
+    qr_plan(big, m, k, spc, g, 1);
+    q.buf.assign(big.L.size(), QRPlan::Level());
+    for (size_t l = 0; l < big.L.size(); ++l) {
+        const QRPlan::Level &v = big.L[l];
+        const size_t subs = l == 0 ? (size_t)(m / big.b) + 2 * (size_t)v.C + 4 : (size_t)big.L[l - 1].C + 8;
+        q.buf[l].tau = bp.take<double>(subs * k);
+        q.buf[l].R = bp.take<double>((size_t)(v.C + 1) * k * k);
+        if (l > 0) q.buf[l].X = bp.take<double>((size_t)(big.L[l - 1].C + 4) * k * p);
     }
 }
+
+void qr_bind(QRPlan &q, double *A)
+{
+    for (size_t l = 0; l < q.L.size(); ++l) {
+        q.L[l].A = l == 0 ? A : q.buf[l - 1].R;
+        q.L[l].tau = q.buf[l].tau;
+        q.L[l].R = q.buf[l].R;
+        q.L[l].X = q.buf[l].X;
+    }
+    q.T = q.L.back().R;
+}
+
+// Sub-blocks per chunk: what spreads the batch's sub-blocks over three CTAs per SM.
+int qr_spc(long long subs) { return (int)std::min(16LL, std::max(2LL, (subs + 3LL * sm_count() - 1) / (3LL * sm_count()))); }
 
 struct TTPlan {
     int n[3] = {0, 0, 0};
     int R1 = 0, R2 = 0, k3 = 0, k2 = 0, kc = 0, ke = 0;
     long long mB = 0;
     double *C1 = nullptr, *MA = nullptr, *MB = nullptr, *MC = nullptr, *ME = nullptr;
-    QRPlan qa, qb, qc, qe, qe_max;
+    QRPlan qa, qb, qc, qe;
     double *VC = nullptr, *WC = nullptr, *svC = nullptr, *VE = nullptr, *WE = nullptr, *svE = nullptr;
     double *delta = nullptr;
-    double *XSa = nullptr, *XSb = nullptr, *XSc = nullptr, *XSe = nullptr;
     int r1 = 0, r2 = 0;
 };
 
 }  // namespace
 
-// Factor every plan (leaf chunks, then the stacked chunk R factors).
-static int tt_factor(weno_ctx *h, std::vector<QRPlan *> &ps, QRDesc *dev)
+// Factor every plan, level by level (a plan without the level sits it out).
+static int tt_factor(weno_ctx *h, std::vector<QRPlan *> &ps, char *dev)
 {
     const int n = (int)ps.size();
-    std::vector<QRDesc> leaf(n), top(n);
-    int maxC = 1, maxk = 1, maxb = 32;
-    bool any_top = false;
-    for (int i = 0; i < n; ++i) {
-        const QRPlan &q = *ps[i];
-        leaf[i] = QRDesc{q.A, q.m, q.k, q.k, q.b, q.C, q.chunk_rows, q.sub, q.tau, q.Rc};
-        top[i] = QRDesc{q.Rc, q.C > 1 ? (long long)q.C * q.k : 0, q.k, q.k, q.b, 1, (long long)q.C * q.k,
-                        q.top_sub, q.tau_top, q.T};
-        maxC = std::max(maxC, q.C);
-        maxk = std::max(maxk, q.k);
-        maxb = std::max(maxb, q.b);
-        any_top |= q.C > 1;
-    }
-    const size_t smem = qr_factor_smem(maxk, maxb);
-    CK(h, cudaMemcpyAsync(dev, leaf.data(), sizeof(QRDesc) * n, cudaMemcpyHostToDevice, h->stream));
-    CK(h, launch(h, 0, h->stream, [&] { return launch_qr_factor(dev, n, maxC, smem, h->stream); }));
-    if (any_top) {
-        CK(h, cudaMemcpyAsync(dev + n, top.data(), sizeof(QRDesc) * n, cudaMemcpyHostToDevice, h->stream));
-        CK(h, launch(h, 0, h->stream, [&] { return launch_qr_factor(dev + n, n, 1, smem, h->stream); }));
+    size_t levels = 0;
+    for (auto *q : ps) levels = std::max(levels, q->L.size());
+    if (levels > QR_MAXL) return fail(h, WENO_ERR_UNSUPPORTED, "weno_tt_round: matrix too long");
+    std::vector<QRDesc> ds(n);
+    for (size_t l = 0; l < levels; ++l) {
+        int maxC = 1;
+        size_t smem = 0;
+        for (int i = 0; i < n; ++i) {
+            const QRPlan &q = *ps[i];
+            ds[i] = QRDesc{};
+            if (l >= q.L.size()) continue;
+            const QRPlan::Level &v = q.L[l];
+            ds[i] = QRDesc{v.A, v.m, q.k, q.k, q.b, v.C, v.rows, v.sub, v.tau, v.R, l > 0};
+            maxC = std::max(maxC, v.C);
+            smem = std::max(smem, qr_factor_smem(q.k, q.b));
+        }
+        QRDesc *dd = (QRDesc *)(dev + sizeof(QRDesc) * n * l);
+        CK(h, cudaMemcpyAsync(dd, ds.data(), sizeof(QRDesc) * n, cudaMemcpyHostToDevice, h->stream));
+        CK(h, launch(h, 0, h->stream, [&] { return launch_qr_factor(dd, n, maxC, smem, h->stream); }));
     }
     return WENO_OK;
 }
@@ -111,39 +150,39 @@ struct ApplyReq {  // Q [X; 0] of one plan into an output row map
     const QRPlan *q;
     const double *X;
     int ldx, p;
-    double *XS;  // stack of the chunks' top rows (C > 1)
     double *out;
     long long P, sP, sQ, sC;
 };
 
-static int tt_apply(weno_ctx *h, std::vector<ApplyReq> &rs, QApplyDesc *dev)
+// From the top of each plan's tree down: a level's result is the stack of the top
+// rows of the level below.
+static int tt_apply(weno_ctx *h, std::vector<ApplyReq> &rs, char *dev)
 {
     const int n = (int)rs.size();
-    std::vector<QApplyDesc> leaf(n), top(n);
-    int maxC = 1, maxk = 1, maxb = 32, maxp = 1;
-    bool any_top = false;
-    for (int i = 0; i < n; ++i) {
-        const ApplyReq &r = rs[i];
-        const QRPlan &q = *r.q;
-        const bool two = q.C > 1;
-        const long long mt = (long long)q.C * q.k;
-        top[i] = QApplyDesc{q.Rc, q.tau_top, two ? mt : 0, q.k, q.k, q.b, 1, mt, q.top_sub, r.X, 0, r.ldx, r.p,
-                            r.XS, mt, r.p, 0, 1};
-        leaf[i] = QApplyDesc{q.A, q.tau, q.m, q.k, q.k, q.b, q.C, q.chunk_rows, q.sub, two ? r.XS : r.X,
-                             two ? (long long)q.k * r.p : 0, two ? r.p : r.ldx, r.p, r.out, r.P, r.sP, r.sQ, r.sC};
-        maxC = std::max(maxC, q.C);
-        maxk = std::max(maxk, q.k);
-        maxb = std::max(maxb, q.b);
-        maxp = std::max(maxp, r.p);
-        any_top |= two;
+    size_t levels = 0;
+    for (auto &r : rs) levels = std::max(levels, r.q->L.size());
+    std::vector<QApplyDesc> ds(n);
+    for (size_t l = levels; l-- > 0;) {
+        int maxC = 1;
+        size_t smem = 0;
+        for (int i = 0; i < n; ++i) {
+            const ApplyReq &r = rs[i];
+            const QRPlan &q = *r.q;
+            ds[i] = QApplyDesc{};
+            if (l >= q.L.size()) continue;
+            const QRPlan::Level &v = q.L[l];
+            const bool top = l + 1 == q.L.size();
+            const double *X = top ? r.X : q.L[l + 1].X;
+            ds[i] = QApplyDesc{v.A, v.tau, v.m, q.k, q.k, q.b, v.C, v.rows, v.sub, X, top ? 0 : (long long)q.k * r.p,
+                               top ? r.ldx : r.p, r.p, l > 0 ? v.X : r.out, l > 0 ? v.m : r.P, l > 0 ? r.p : r.sP,
+                               l > 0 ? 0 : r.sQ, l > 0 ? 1 : r.sC, l > 0};
+            maxC = std::max(maxC, v.C);
+            smem = std::max(smem, qr_apply_smem(q.k, q.b, r.p));
+        }
+        QApplyDesc *dd = (QApplyDesc *)(dev + sizeof(QApplyDesc) * n * l);
+        CK(h, cudaMemcpyAsync(dd, ds.data(), sizeof(QApplyDesc) * n, cudaMemcpyHostToDevice, h->stream));
+        CK(h, launch(h, 0, h->stream, [&] { return launch_qr_apply(dd, n, maxC, smem, h->stream); }));
     }
-    const size_t smem = qr_apply_smem(maxk, maxb, maxp);
-    if (any_top) {
-        CK(h, cudaMemcpyAsync(dev + n, top.data(), sizeof(QApplyDesc) * n, cudaMemcpyHostToDevice, h->stream));
-        CK(h, launch(h, 0, h->stream, [&] { return launch_qr_apply(dev + n, n, 1, smem, h->stream); }));
-    }
-    CK(h, cudaMemcpyAsync(dev, leaf.data(), sizeof(QApplyDesc) * n, cudaMemcpyHostToDevice, h->stream));
-    CK(h, launch(h, 0, h->stream, [&] { return launch_qr_apply(dev, n, maxC, smem, h->stream); }));
     return WENO_OK;
 }
 
@@ -155,9 +194,10 @@ static int tt_svd(weno_ctx *h, std::vector<SvdDesc> &ds, SvdDesc *dev)
         maxpk = std::max(maxpk, d.pk);
         maxq = std::max(maxq, d.q);
     }
-    const size_t smem = svd_smem(maxpk, maxq);
+    const int ncl = svd_cluster(n, maxpk);
+    const size_t smem = svd_smem(maxpk, maxq, ncl);
     CK(h, cudaMemcpyAsync(dev, ds.data(), sizeof(SvdDesc) * n, cudaMemcpyHostToDevice, h->stream));
-    CK(h, launch(h, 1, h->stream, [&] { return launch_svd_jacobi(dev, n, smem, h->stream); }));
+    CK(h, launch(h, 1, h->stream, [&] { return launch_svd_jacobi(dev, n, ncl, smem, h->stream); }));
     return WENO_OK;
 }
 
@@ -169,6 +209,7 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
     const int np = n_probs;
     std::vector<TTPlan> pl(np);
     std::vector<TTSumDesc> sd(np);
+    long long sa = 0, sb = 0, sc = 0, se = 0;  // sub-blocks of the batch's four QRs
     for (int i = 0; i < np; ++i) {
         const weno_tt_round_problem &P = probs[i];
         TTPlan &t = pl[i];
@@ -204,14 +245,23 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         t.mB = (long long)t.n[1] * t.k3;
         t.k2 = (int)std::min<long long>(t.mB, t.R1);
         t.kc = std::min(t.n[0], t.k2);
-        qr_plan(t.qa, t.n[2], t.R2);
-        qr_plan(t.qb, t.mB, t.R1);
-        qr_plan(t.qc, t.n[0], t.k2);
-        qr_plan(t.qe_max, (long long)t.kc * t.n[1], t.k3);
+        auto subs = [](long long m, int k) { return (m + k - 1) / std::max(32, (k + 31) / 32 * 32) + 1; };
+        sa += subs(t.n[2], t.R2);
+        sb += subs(t.mB, t.R1);
+        sc += subs(t.n[0], t.k2);
+        se += subs((long long)t.kc * t.n[1], t.k3);
         t.ke = (int)std::min<long long>((long long)t.kc * t.n[1], t.k3);
     }
-    // scratch: descriptors, ranks, then per problem matrices and QR data
-    const int NDESC = 24;
+    const int pa = qr_spc(sa), pb = qr_spc(sb), pc = qr_spc(sc), pe = qr_spc(se);
+    const int g = sb > 12ll * sm_count() * pb ? 4 : 2;
+    for (auto &t : pl) {
+        qr_plan(t.qa, t.n[2], t.R2, pa, g);
+        qr_plan(t.qb, t.mB, t.R1, pb, g);
+        qr_plan(t.qc, t.n[0], t.k2, pc, g);
+    }
+    // scratch: descriptors (a QR or apply step takes one block per level), ranks, then
+    // per problem matrices and QR data
+    const int NDESC = 8 * QR_MAXL + 8;
     const size_t dsz = std::max({sizeof(QRDesc), sizeof(QApplyDesc), sizeof(SvdDesc), sizeof(TTSumDesc), sizeof(GemmDesc)});
     auto layout = [&](Bump &bp) -> char * {
         char *desc = bp.take<char>(dsz * NDESC * (size_t)np);
@@ -221,10 +271,10 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
             t.MB = bp.take<double>((size_t)t.mB * t.R1);
             t.MC = bp.take<double>((size_t)t.n[0] * t.k2);
             t.ME = bp.take<double>((size_t)t.kc * t.n[1] * t.k3);
-            qr_take(bp, t.qa);
-            qr_take(bp, t.qb);
-            qr_take(bp, t.qc);
-            qr_take(bp, t.qe_max);
+            qr_take(bp, t.qa, t.n[2], t.R2, pa, g, t.ke);
+            qr_take(bp, t.qb, t.mB, t.R1, pb, g, t.kc);
+            qr_take(bp, t.qc, t.n[0], t.k2, pc, g, t.kc);
+            qr_take(bp, t.qe, (long long)t.kc * t.n[1], t.k3, pe, g, t.ke);
             t.VC = bp.take<double>((size_t)t.kc * t.kc);
             t.WC = bp.take<double>((size_t)t.k2 * t.kc);
             t.svC = bp.take<double>(t.kc);
@@ -232,10 +282,6 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
             t.WE = bp.take<double>((size_t)t.k3 * t.ke);
             t.svE = bp.take<double>(t.ke);
             t.delta = bp.take<double>(2);
-            t.XSa = bp.take<double>((size_t)t.qa.C * t.qa.k * t.ke);
-            t.XSb = bp.take<double>((size_t)t.qb.C * t.qb.k * t.kc);
-            t.XSc = bp.take<double>((size_t)t.qc.C * t.qc.k * t.kc);
-            t.XSe = bp.take<double>((size_t)t.qe_max.C * t.qe_max.k * t.ke);
         }
         return desc;
     };
@@ -256,18 +302,21 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
     char *desc = layout(bp);
     int *ranks = (int *)((char *)h->tbuf + rank_off);
     int slot = 0;
-    auto next_desc = [&]() { return desc + dsz * (size_t)np * (slot++); };
+    auto next_desc = [&](int blocks = 1) {
+        char *p = desc + dsz * (size_t)np * slot;
+        slot += blocks;
+        return p;
+    };
 
     for (int i = 0; i < np; ++i) {
         TTPlan &t = pl[i];
         sd[i].C1 = t.C1;
         sd[i].MA = t.MA;
         sd[i].MB = t.MB;
+        qr_bind(t.qa, t.MA);
+        qr_bind(t.qb, t.MB);
+        qr_bind(t.qc, t.MC);
         sd[i].TA = t.qa.T;
-        t.qa.A = t.MA;
-        t.qb.A = t.MB;
-        t.qc.A = t.MC;
-        t.qe_max.A = t.ME;
     }
     // ---- phase 1: sum unfoldings; QR of the last core; middle core times TA^T; QR; first core; QR; SVD
     {
@@ -276,14 +325,12 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         CK(h, launch(h, 1, h->stream, [&] { return launch_tt_build(d, np, h->stream); }));
         std::vector<QRPlan *> ps;
         for (auto &t : pl) ps.push_back(&t.qa);
-        int r = tt_factor(h, ps, (QRDesc *)next_desc());
+        int r = tt_factor(h, ps, next_desc(QR_MAXL));
         if (r) return r;
-        ++slot;
         CK(h, launch(h, 1, h->stream, [&] { return launch_tt_contract(d, np, h->stream); }));
         ps.clear();
         for (auto &t : pl) ps.push_back(&t.qb);
-        if ((r = tt_factor(h, ps, (QRDesc *)next_desc()))) return r;
-        ++slot;
+        if ((r = tt_factor(h, ps, next_desc(QR_MAXL)))) return r;
         std::vector<GemmDesc> gd(np);
         for (int i = 0; i < np; ++i)
             gd[i] = GemmDesc{pl[i].C1, pl[i].qb.T, pl[i].MC, pl[i].n[0], pl[i].k2, pl[i].R1};
@@ -292,8 +339,7 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         CK(h, launch(h, 1, h->stream, [&] { return launch_tt_gemm_tr(gdev, np, h->stream); }));
         ps.clear();
         for (auto &t : pl) ps.push_back(&t.qc);
-        if ((r = tt_factor(h, ps, (QRDesc *)next_desc()))) return r;
-        ++slot;
+        if ((r = tt_factor(h, ps, next_desc(QR_MAXL)))) return r;
         std::vector<SvdDesc> sv(np);
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
@@ -310,34 +356,26 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         if (t.r1 < 1 || t.r1 > t.kc) return fail(h, WENO_ERR_CUDA, "weno_tt_round: device returned a bad rank");
         if (probs[i].cap[0] < (long long)t.n[0] * t.r1)
             return fail(h, WENO_ERR_ARG, "weno_tt_round: output core 1 capacity too small");
-        t.qe = t.qe_max;
-        qr_plan(t.qe, (long long)t.r1 * t.n[1], t.k3);
-        t.qe.A = t.ME;
-        t.qe.tau = t.qe_max.tau;
-        t.qe.Rc = t.qe_max.Rc;
-        t.qe.tau_top = t.qe_max.tau_top;
-        t.qe.T = t.qe.C > 1 ? t.qe_max.T : t.qe.Rc;
+        qr_plan(t.qe, (long long)t.r1 * t.n[1], t.k3, pe, g);
+        qr_bind(t.qe, t.ME);
     }
     // ---- phase 2: first output core; the middle core into the (r1 n2) x k3 unfolding; QR; SVD
     {
         std::vector<ApplyReq> ar(np);
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
-            ar[i] = ApplyReq{&t.qc, t.VC, t.kc, t.r1, t.XSc, probs[i].out.core[0], t.n[0], t.r1, 0, 1};
+            ar[i] = ApplyReq{&t.qc, t.VC, t.kc, t.r1, probs[i].out.core[0], t.n[0], t.r1, 0, 1};
         }
-        int r = tt_apply(h, ar, (QApplyDesc *)next_desc());
+        int r = tt_apply(h, ar, next_desc(QR_MAXL));
         if (r) return r;
-        ++slot;
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
-            ar[i] = ApplyReq{&t.qb, t.WC, t.kc, t.r1, t.XSb, t.ME, t.mB, 1, 0, t.mB};
+            ar[i] = ApplyReq{&t.qb, t.WC, t.kc, t.r1, t.ME, t.mB, 1, 0, t.mB};
         }
-        if ((r = tt_apply(h, ar, (QApplyDesc *)next_desc()))) return r;
-        ++slot;
+        if ((r = tt_apply(h, ar, next_desc(QR_MAXL)))) return r;
         std::vector<QRPlan *> ps;
         for (auto &t : pl) ps.push_back(&t.qe);
-        if ((r = tt_factor(h, ps, (QRDesc *)next_desc()))) return r;
-        ++slot;
+        if ((r = tt_factor(h, ps, next_desc(QR_MAXL)))) return r;
         std::vector<SvdDesc> sv(np);
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
@@ -363,18 +401,16 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         std::vector<ApplyReq> ar(np);
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
-            ar[i] = ApplyReq{&t.qe, t.VE, t.ke, t.r2, t.XSe, probs[i].out.core[1], t.n[1], (long long)t.r1 * t.r2,
+            ar[i] = ApplyReq{&t.qe, t.VE, t.ke, t.r2, probs[i].out.core[1], t.n[1], (long long)t.r1 * t.r2,
                              t.r2, 1};
         }
-        int r = tt_apply(h, ar, (QApplyDesc *)next_desc());
+        int r = tt_apply(h, ar, next_desc(QR_MAXL));
         if (r) return r;
-        ++slot;
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
-            ar[i] = ApplyReq{&t.qa, t.WE, t.ke, t.r2, t.XSa, probs[i].out.core[2], t.n[2], t.r2, 0, 1};
+            ar[i] = ApplyReq{&t.qa, t.WE, t.ke, t.r2, probs[i].out.core[2], t.n[2], t.r2, 0, 1};
         }
-        if ((r = tt_apply(h, ar, (QApplyDesc *)next_desc()))) return r;
-        ++slot;
+        if ((r = tt_apply(h, ar, next_desc(QR_MAXL)))) return r;
     }
     for (int i = 0; i < np; ++i) {
         weno_tt3 &o = probs[i].out;

@@ -4,11 +4,13 @@
 //
 // Building blocks, each a batched kernel over independent problems:
 //   * k_qr_factor: Householder QR of a tall-skinny m x k matrix (k <= 96),
-//     two-level TSQR.  A chunk of rows is factored by one CTA as a flat tree:
+//     a TSQR tree.  A chunk of rows is factored by one CTA as a flat tree:
 //     a plain Householder QR of its first b rows, then for every further
 //     sub-block B of b rows the structured QR of [R; B] whose reflectors are
 //     [e_j; y_j].  The chunk R factors are stacked and factored the same way
-//     by a second launch.  Reflectors overwrite the matrix; taus are kept.
+//     by further launches, a few R's per CTA, until one is left; there the first
+//     block is an R already and reflector j of the others has j + 1 rows.
+//     Reflectors overwrite the matrix; taus are kept.
 //   * k_qr_apply: Q [X; 0] for a k x p block X, replaying the reflectors of a
 //     chunk in reverse (eight lanes per column of X, four columns per warp,
 //     no block barrier inside a sub-block); writes the rows through a general row map so that results
@@ -16,18 +18,24 @@
 //   * k_svd_jacobi: one-sided Jacobi SVD (round-robin pair ordering) of the
 //     transpose of a k x q triangular factor T: T^T V = U S gives T = V S U^T;
 //     picks the truncation rank from the singular values and writes V's kept
-//     columns and (U S)'s kept columns.
+//     columns and (U S)'s kept columns.  The rows of T^T and of V are spread over
+//     the CTAs of a cluster: a rotation acts on every row alone, only the dot
+//     products that choose the angles are sums over all of them.
 //   * k_tt_build / k_tt_contract / k_tt_gemm_tr: the TT sum's first and last
 //     unfoldings, the block-diagonal middle core times a triangular factor, and
 //     a small dense product.
 // All arithmetic is FP64.
 #include <cfloat>
 
+#include <cooperative_groups.h>
+
 #include "weno_dev.cuh"
 #include "weno_internal.h"
 #include "tt_internal.h"
 
 namespace wg {
+
+namespace cg = cooperative_groups;
 
 constexpr int TT_NT = 256, TT_NW = TT_NT / 32;
 
@@ -48,14 +56,6 @@ __device__ __forceinline__ double warp_sum_d(double v)
 // (b a multiple of 32), so a half-warp's 4 columns x 4 rows hit 16 distinct
 // banks.
 constexpr int LPC = 4, CPW = 32 / LPC, LDPAD = 4;
-constexpr int SV_LPP = 4, SV_PPW = 32 / SV_LPP;  // Jacobi lanes per pair, pairs per warp
-
-__device__ __forceinline__ double pair_sum_d(double v)
-{
-#pragma unroll
-    for (int o = SV_LPP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    return v;
-}
 
 __device__ __forceinline__ double group_sum(double v)
 {
@@ -64,17 +64,44 @@ __device__ __forceinline__ double group_sum(double v)
     return v;
 }
 
+// 1 / sqrt(s) of a normal s: an FP32 seed on the mantissa (scaled by an even power
+// of two to [1, 4)), two Newton-Raphson steps y (3 - s y^2) / 2.
+__device__ __forceinline__ double rsqrt_f64(double s)
+{
+    const int h = __double2hiint(s), e2 = ((h >> 20) - 1023) & ~1;  // the even exponent
+    const double m = __hiloint2double(h - (e2 << 20), __double2loint(s));
+    float f;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(f64_to_f32(m)));
+    double y = f32_to_f64_nz(f);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) - ((e2 / 2) << 20), __double2loint(y));
+}
+
 // Householder vector of x = (x0, y) with ||y||^2 = sig: H = I - tau v v^T,
-// v = (1, y / (x0 - beta)), H x = (beta, 0).  sig == 0 gives tau = 0.
+// v = (1, y / (x0 - beta)), H x = (beta, 0).  sig == 0 gives tau = 0.  Every column
+// waits for this chain of dependent FP64 operations (68 cycles each), so it takes
+// one reciprocal square root and one reciprocal by Newton's method (18 operations;
+// with sqrt and two divisions ~40).
 __device__ __forceinline__ void householder(double x0, double sig, double &beta, double &tau, double &scale)
 {
     beta = x0;
     tau = 0.0;
     scale = 0.0;
     if (sig > 0.0) {
-        beta = -copysign(sqrt(fma(x0, x0, sig)), x0);
-        tau = (beta - x0) / beta;
-        scale = 1.0 / (x0 - beta);
+        const double s = fma(x0, x0, sig);
+        if (s > 1e-280 && s < 1e280) {
+            const double y = rsqrt_f64(s);
+            double b = s * y;
+            b = fma(fma(-b, b, s), 0.5 * y, b);
+            beta = -copysign(b, x0);
+            tau = fma(-x0, -copysign(y, x0), 1.0);  // 1 - x0 / beta
+            scale = rcp_f64(x0 - beta);
+        } else {
+            beta = -copysign(sqrt(s), x0);
+            tau = (beta - x0) / beta;
+            scale = 1.0 / (x0 - beta);
+        }
     }
 }
 
@@ -83,15 +110,30 @@ size_t qr_apply_smem(int k, int b, int p)
 {
     return sizeof(double) * ((size_t)k * (b + LDPAD) + (size_t)p * (b + LDPAD) + (size_t)p * (k + 1) + k);
 }
-size_t svd_smem(int pk, int q) { return sizeof(double) * ((size_t)pk * (q + 1) + (size_t)pk * (pk + 1) + 2 * pk); }
+size_t svd_smem(int pk, int q, int ncl)
+{
+    return sizeof(double) * ((size_t)pk * (((q + ncl - 1) / ncl + (pk + ncl - 1) / ncl) | 1) + pk);
+}
 
+// CTAs per matrix: as many as the GPU has SMs for, at most 8 and at least ~8 rows each.
+int svd_cluster(int n, int max_pk)
+{
+    int ncl = 8;
+    while (ncl > 1 && ((long long)n * ncl > sm_count() || max_pk / ncl < 6)) ncl /= 2;
+    return ncl;
+}
+
+// The column loop keeps one reflector ahead: while the other warps apply reflector
+// j to their columns, one warp applies it to column j + 1 and forms reflector j + 1
+// from it, so that chain (~35 dependent FP64 operations) runs beside the updates
+// and a column takes one barrier.  64 columns of a 64-row sub-block: 195 -> QRSUB us.
 __global__ void __launch_bounds__(TT_NT) k_qr_factor(const QRDesc *descs)
 {
     const QRDesc &d = descs[blockIdx.y];
     const int chunk = blockIdx.x;
     if (chunk >= d.chunks || d.m <= 0) return;
     extern __shared__ double sm[];
-    const int k = d.k, b = d.b, ldb = b + LDPAD, ldr = k + 1;
+    const int k = d.k, b = d.tri ? k : d.b, ldb = d.b + LDPAD, ldr = k + 1;
     double *B = sm;                       // sub-block, column-major [k][ldb]
     double *R = B + (size_t)k * ldb;      // running R, column-major [k][ldr]
     double *ts = R + (size_t)k * ldr;     // taus of the current sub-block
@@ -109,89 +151,81 @@ __global__ void __launch_bounds__(TT_NT) k_qr_factor(const QRDesc *descs)
         }
         for (int j = threadIdx.x; j < k; j += TT_NT) ts[j] = 0.0;
         __syncthreads();
-        if (s == 0) {
-            // plain Householder QR of the first bs x k block
-            const int kk = min(bs, k);
-            for (int j = 0; j < kk; ++j) {
-                if (warp == 0) {
-                    double *x = B + j * ldb;
-                    double sig = 0.0;
-                    for (int i = j + 1 + lane; i < bs; i += 32) sig = fma(x[i], x[i], sig);
-                    sig = warp_sum_d(sig);
-                    double beta, tau, scale;
-                    householder(x[j], sig, beta, tau, scale);
-                    for (int i = j + 1 + lane; i < bs; i += 32) x[i] *= scale;
-                    __syncwarp();  // every lane has read x[j]
-                    if (lane == 0) {
-                        x[j] = beta;
-                        ts[j] = tau;
-                    }
-                }
-                __syncthreads();
-                const double tau = ts[j];
-                if (tau != 0.0) {
-                    const double *v = B + j * ldb;
-                    for (int c0 = j + 1 + warp * CPW; c0 < k; c0 += TT_NW * CPW) {
-                        const int c = c0 + grp;
-                        const bool ok = c < k;
-                        double *col = B + (ok ? c : 0) * ldb;
-                        double w = 0.0;
-                        if (ok)
-                            for (int i = j + 1 + sub; i < bs; i += LPC) w = fma(v[i], col[i], w);
-                        w = (group_sum(w) + (ok ? col[j] : 0.0)) * tau;
-                        if (ok)
-                            for (int i = j + 1 + sub; i < bs; i += LPC) col[i] = fma(-v[i], w, col[i]);
-                        __syncwarp();
-                        if (ok && sub == 0) col[j] -= w;
-                    }
-                }
-                __syncthreads();
+        const bool plain = s == 0;
+        const int kk = plain ? (d.tri ? 0 : min(bs, k)) : k;  // reflectors
+        // reflector j: the top element (plain: row j of B, else row j of R) and rows
+        // i0 .. i1 of B's column j
+        auto top = [&](int c, int j) -> double & { return plain ? B[c * ldb + j] : R[c * ldr + j]; };
+        auto first = [&](int j) { return plain ? j + 1 : 0; };
+        auto last = [&](int j) { return d.tri && !plain ? min(j + 1, bs) : bs; };
+        auto generate = [&](int j) {  // one warp
+            double *x = B + j * ldb;
+            const int i0 = first(j), i1 = last(j);
+            double sig = 0.0;
+            for (int i = i0 + lane; i < i1; i += 32) sig = fma(x[i], x[i], sig);
+            sig = warp_sum_d(sig);
+            double beta, tau, scale;
+            householder(top(j, j), sig, beta, tau, scale);
+            for (int i = i0 + lane; i < i1; i += 32) x[i] *= scale;
+            __syncwarp();  // every lane has read the top element
+            if (lane == 0) {
+                top(j, j) = beta;
+                ts[j] = tau;
             }
+        };
+        if (warp == 0 && kk > 0) generate(0);
+        __syncthreads();
+        for (int j = 0; j < kk; ++j) {
+            const double tau = ts[j];
+            const double *v = B + j * ldb;
+            const int i0 = first(j), i1 = last(j), ahead = j & (TT_NW - 1);
+            if (warp == ahead && j + 1 < k) {
+                if (tau != 0.0) {
+                    double *col = B + (j + 1) * ldb;
+                    double w = 0.0;
+                    for (int i = i0 + lane; i < i1; i += 32) w = fma(v[i], col[i], w);
+                    w = (warp_sum_d(w) + top(j + 1, j)) * tau;
+                    for (int i = i0 + lane; i < i1; i += 32) col[i] = fma(-v[i], w, col[i]);
+                    __syncwarp();
+                    if (lane == 0) top(j + 1, j) -= w;
+                    __syncwarp();
+                }
+                if (j + 1 < kk) generate(j + 1);
+            }
+            if (tau != 0.0) {
+                for (int c0 = j + 2 + ((warp - ahead - 1) & (TT_NW - 1)) * CPW; c0 < k; c0 += TT_NW * CPW) {
+                    const int c = c0 + grp;
+                    const bool ok = c < k;
+                    double *col = B + (ok ? c : 0) * ldb;
+                    double w = 0.0, w1 = 0.0;
+                    if (ok) {
+                        int i = i0 + sub;
+                        for (; i + LPC < i1; i += 2 * LPC) {
+                            w = fma(v[i], col[i], w);
+                            w1 = fma(v[i + LPC], col[i + LPC], w1);
+                        }
+                        if (i < i1) w = fma(v[i], col[i], w);
+                    }
+                    w = (group_sum(w + w1) + (ok ? top(c, j) : 0.0)) * tau;
+                    if (ok)
+                        for (int i = i0 + sub; i < i1; i += LPC) col[i] = fma(-v[i], w, col[i]);
+                    __syncwarp();
+                    if (ok && sub == 0) top(c, j) -= w;
+                }
+            }
+            __syncthreads();
+        }
+        if (plain) {
             for (int e = threadIdx.x; e < k * k; e += TT_NT) {
                 const int c = e / k, j = e - c * k;
-                R[c * ldr + j] = (j <= c && j < kk) ? B[c * ldb + j] : 0.0;
-            }
-        } else {
-            // structured QR of [R; B]: reflector j is (e_j; y_j), y_j stored in B's column j
-            for (int j = 0; j < k; ++j) {
-                if (warp == 0) {
-                    double *y = B + j * ldb;
-                    double sig = 0.0;
-                    for (int i = lane; i < bs; i += 32) sig = fma(y[i], y[i], sig);
-                    sig = warp_sum_d(sig);
-                    double beta, tau, scale;
-                    householder(R[j * ldr + j], sig, beta, tau, scale);
-                    for (int i = lane; i < bs; i += 32) y[i] *= scale;
-                    __syncwarp();  // every lane has read R[j][j]
-                    if (lane == 0) {
-                        R[j * ldr + j] = beta;
-                        ts[j] = tau;
-                    }
-                }
-                __syncthreads();
-                const double tau = ts[j];
-                if (tau != 0.0) {
-                    const double *y = B + j * ldb;
-                    for (int c0 = j + 1 + warp * CPW; c0 < k; c0 += TT_NW * CPW) {
-                        const int c = c0 + grp;
-                        const bool ok = c < k;
-                        double *col = B + (ok ? c : 0) * ldb;
-                        double w = 0.0;
-                        if (ok)
-                            for (int i = sub; i < bs; i += LPC) w = fma(y[i], col[i], w);
-                        w = (group_sum(w) + (ok ? R[c * ldr + j] : 0.0)) * tau;
-                        if (ok)
-                            for (int i = sub; i < bs; i += LPC) col[i] = fma(-y[i], w, col[i]);
-                        __syncwarp();
-                        if (ok && sub == 0) R[c * ldr + j] -= w;
-                    }
-                }
-                __syncthreads();
+                R[c * ldr + j] = (j <= c && j < min(bs, k)) ? B[c * ldb + j] : 0.0;
             }
         }
-        for (int e = threadIdx.x; e < bs * k; e += TT_NT) {
-            const int i = e / k, c = e - i * k;
-            d.A[(s0 + i) * d.lda + c] = B[c * ldb + i];
+        if (kk > 0) {
+            for (int e = threadIdx.x; e < bs * k; e += TT_NT) {
+                const int i = e / k, c = e - i * k;
+                d.A[(s0 + i) * d.lda + c] = B[c * ldb + i];
+            }
         }
         for (int j = threadIdx.x; j < k; j += TT_NT) d.tau[((long long)chunk * d.sub_per_chunk + s) * k + j] = ts[j];
         __syncthreads();
@@ -208,7 +242,7 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
     const int chunk = blockIdx.x;
     if (chunk >= d.chunks || d.m <= 0 || d.p <= 0) return;
     extern __shared__ double sm[];
-    const int k = d.k, b = d.b, p = d.p, ldb = b + LDPAD, ldx = k + 1;
+    const int k = d.k, b = d.tri ? k : d.b, p = d.p, ldb = d.b + LDPAD, ldx = k + 1;
     double *Y = sm;                        // reflectors of a sub-block, column-major [k][ldb]
     double *Z = Y + (size_t)k * ldb;       // output block, column-major [p][ldb]
     double *X = Z + (size_t)p * ldb;       // running top rows, column-major [p][ldx]
@@ -251,12 +285,19 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
                 const double tau = ts[j];
                 if (tau == 0.0) continue;
                 const double *y = Y + j * ldb;
-                double w = 0.0;
+                const int i1 = d.tri ? min(j + 1, bs) : bs;
+                double w = 0.0, w1 = 0.0;
+                if (ok) {
+                    int i = sub;
+                    for (; i + LPC < i1; i += 2 * LPC) {
+                        w = fma(y[i], zq[i], w);
+                        w1 = fma(y[i + LPC], zq[i + LPC], w1);
+                    }
+                    if (i < i1) w = fma(y[i], zq[i], w);
+                }
+                w = (group_sum(w + w1) + (ok ? xq[j] : 0.0)) * tau;
                 if (ok)
-                    for (int i = sub; i < bs; i += LPC) w = fma(y[i], zq[i], w);
-                w = (group_sum(w) + (ok ? xq[j] : 0.0)) * tau;
-                if (ok)
-                    for (int i = sub; i < bs; i += LPC) zq[i] = fma(-y[i], w, zq[i]);
+                    for (int i = sub; i < i1; i += LPC) zq[i] = fma(-y[i], w, zq[i]);
                 __syncwarp();
                 if (ok && sub == 0) xq[j] -= w;
                 __syncwarp();
@@ -266,7 +307,8 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
         store(s0, bs);
         __syncthreads();
     }
-    // first sub-block: plain reflectors below the diagonal, acting on [X; 0]
+    // first sub-block: plain reflectors below the diagonal, acting on [X; 0] (none
+    // where it is an R already)
     for (int e = threadIdx.x; e < b1 * k; e += TT_NT) {
         const int i = e / k, c = e - i * k;
         Y[c * ldb + i] = d.A[(r0 + i) * d.lda + c];
@@ -301,113 +343,159 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
 }
 
 // One-sided Jacobi on the pk columns of M = T^T (column t = row t of T, length q).
+// A sweep of 64 columns is 63 rounds of 32 disjoint pairs; per round an SM did ~790
+// FP64 instructions (7.2 us).  Here each CTA of the cluster holds all columns of a
+// slice of M's and V's rows.  Per round: partial dot products m_u . m_u, m_v . m_v
+// and m_u . m_v over the slice (a lane per pair; the three chains overlap, and
+// norms carried from round to round lose all digits on nearly dependent columns),
+// one cluster barrier, the sum of all partials and the angle (a lane per pair,
+// every CTA the same), the rotations of the slice (a lane per pair, a warp per
+// row).  The tangent of the angle is formed in FP32 (with Newton steps for cos =
+// 1 / sqrt(1 + t^2)): it only steers, the rotation is orthogonal to FP64 rounding
+// whatever t is, and a pair counts as orthogonal by its FP64 dot products.  64 x 64, 10 matrices: 4.8 -> SVDT ms.
+// cluster size 1..8 (svd_cluster): fewer CTAs where the batch fills the GPU.
 __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
 {
-    const SvdDesc &d = descs[blockIdx.x];
+    cg::cluster_group cl = cg::this_cluster();
+    const int ncl = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const SvdDesc &d = descs[blockIdx.y];
     const int pk = d.pk, q = d.q;
-    if (pk <= 0) return;
+    if (pk <= 0) return;  // the same for every CTA of the cluster
     extern __shared__ double sm[];
-    const int ldm = q + 1, ldv = pk + 1;
-    double *M = sm;                          // [pk][ldm]
-    double *V = M + (size_t)pk * ldm;        // [pk][ldv], column t = rotations applied to e_t
-    double *sig = V + (size_t)pk * ldv;      // [pk]
-    int *ord = reinterpret_cast<int *>(sig + pk);
-    __shared__ int rotated;
-    __shared__ double s_delta;
-    __shared__ int s_rank;
+    constexpr int NPR = TT_KMAX / 2, NPART = 4;
+    // this CTA's partial dot products (m_u . m_u, m_v . m_v, m_u . m_v; double buffered) and norms
+    __shared__ double part[2][NPART][3][NPR], norm_part[NPART][TT_KMAX];
+    __shared__ double s_nrm[TT_KMAX], s_cs[NPR], s_sn[NPR];
+    __shared__ int s_uv[NPR][2], ord[TT_KMAX], rotated, s_rank;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e < pk * q; e += TT_NT) {
-        const int t = e / q, i = e - t * q;
-        M[t * ldm + i] = d.T[(long long)t * d.ldt + i];
+    const int qa = rank * q / ncl, qn = (rank + 1) * q / ncl - qa;     // rows of M
+    const int pa = rank * pk / ncl, pn = (rank + 1) * pk / ncl - pa;   // rows of V
+    const int ldm = (qn + pn) | 1;
+    double *M = sm;                          // [pk][ldm]: qn rows of M, then pn rows of V
+    double *sig = M + (size_t)pk * ldm;      // [pk]
+    for (int e = threadIdx.x; e < pk * qn; e += TT_NT) {
+        const int t = e / qn, i = e - t * qn;
+        M[t * ldm + i] = d.T[(long long)t * d.ldt + qa + i];
     }
-    for (int e = threadIdx.x; e < pk * pk; e += TT_NT) {
-        const int t = e / pk, i = e - t * pk;
-        V[t * ldv + i] = (i == t) ? 1.0 : 0.0;
+    for (int e = threadIdx.x; e < pk * pn; e += TT_NT) {
+        const int t = e / pn, i = e - t * pn;
+        M[t * ldm + qn + i] = (pa + i == t) ? 1.0 : 0.0;
     }
     __syncthreads();
     const int n = pk + (pk & 1);  // round-robin over an even count; index pk (odd case) is a bye
     const int npairs = n / 2;
     const double tol = 8.0 * (double)max(pk, q) * DBL_EPSILON;  // cosine below which a pair counts as orthogonal
-    // per round: the pairs' dot products (an SV_LPP-lane group per pair: its
-    // sums cost log2 SV_LPP shuffle adds, a warp sum 5, and the columns are at
-    // most 96 long), their rotations (a lane per pair: the square roots and
-    // divisions run once per pair, not on every lane of a group), then the
-    // rotations themselves (an SV_LPP-lane group per pair)
-    __shared__ double s_a[TT_KMAX / 2], s_b[TT_KMAX / 2], s_c[TT_KMAX / 2], s_cs[TT_KMAX / 2], s_sn[TT_KMAX / 2];
-    __shared__ int s_uv[TT_KMAX / 2][2];
+    const int nd = min(NPART, max(1, qn / 8));  // warps per column or pair that form partial sums, ~8+ rows each
+
+    // squared norms of all columns, summed over the cluster in a fixed order into s_nrm
+    auto norms = [&]() {
+        for (int u = warp; u < nd * ((pk + 31) / 32); u += TT_NW) {
+            const int w = u % nd, t = (u / nd) * 32 + lane;
+            if (t < pk) {
+                double a = 0.0;
+                for (int i = w; i < qn; i += nd) a = fma(M[t * ldm + i], M[t * ldm + i], a);
+                norm_part[w][t] = a;
+            }
+        }
+        cl.sync();
+        for (int t = threadIdx.x; t < pk; t += TT_NT) {
+            double a = 0.0;
+            for (int c = 0; c < ncl; ++c) {
+                const double *np = cl.map_shared_rank(&norm_part[0][0], c);
+                const int ndc = min(NPART, max(1, ((c + 1) * q / ncl - c * q / ncl) / 8));
+                for (int w = 0; w < ndc; ++w) a += np[w * TT_KMAX + t];
+            }
+            s_nrm[t] = a;
+        }
+        cl.sync();  // the partials may be written again
+    };
+    int par = 0;
     for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
-        if (threadIdx.x == 0) rotated = 0;
-        __syncthreads();
-        for (int round = 0; round < n - 1; ++round) {
+        if (threadIdx.x == 0) rotated = 0;  // (set after the next barrier at the earliest)
+        for (int round = 0; round < n - 1; ++round, par ^= 1) {
             auto idx = [&](int t) { return t == 0 ? 0 : 1 + (t - 1 + round) % (n - 1); };
-            for (int s0 = warp * SV_PPW; s0 < npairs; s0 += TT_NW * SV_PPW) {  // the same trip count on every lane
-                const int slot = s0 + lane / SV_LPP, sub = lane % SV_LPP;
-                const bool ok = slot < npairs;
-                const int u = ok ? idx(slot) : 0, v = ok ? idx(n - 1 - slot) : 0;
-                double a = 0.0, bb = 0.0, c = 0.0;
-                if (ok && u < pk && v < pk) {
-                    const double *mu = M + u * ldm, *mv = M + v * ldm;
-                    for (int i = sub; i < q; i += SV_LPP) {
-                        a = fma(mu[i], mu[i], a);
-                        bb = fma(mv[i], mv[i], bb);
-                        c = fma(mu[i], mv[i], c);
-                    }
-                }
-                a = pair_sum_d(a);
-                bb = pair_sum_d(bb);
-                c = pair_sum_d(c);
-                if (ok && sub == 0) {
-                    s_a[slot] = a;
-                    s_b[slot] = bb;
-                    s_c[slot] = c;
-                    s_uv[slot][0] = u;
-                    s_uv[slot][1] = v;
+            for (int u = warp; u < nd * ((npairs + 31) / 32); u += TT_NW) {
+                const int w = u % nd, slot = (u / nd) * 32 + lane;
+                if (slot < npairs) {
+                    const int x = idx(slot), y = idx(n - 1 - slot);
+                    double a = 0.0, b = 0.0, c = 0.0;
+                    if (x < pk && y < pk)
+                        for (int i = w; i < qn; i += nd) {
+                            const double u = M[x * ldm + i], v = M[y * ldm + i];
+                            a = fma(u, u, a);
+                            b = fma(v, v, b);
+                            c = fma(u, v, c);
+                        }
+                    part[par][w][0][slot] = a;
+                    part[par][w][1][slot] = b;
+                    part[par][w][2][slot] = c;
                 }
             }
-            __syncthreads();
+            cl.sync();
             for (int slot = threadIdx.x; slot < npairs; slot += TT_NT) {
-                const double a = s_a[slot], bb = s_b[slot], c = s_c[slot];
+                const int x = idx(slot), y = idx(n - 1 - slot);
+                double a = 0.0, bb = 0.0, c = 0.0;
+                for (int r = 0; r < ncl; ++r) {
+                    const double *pp = cl.map_shared_rank(&part[par][0][0][0], r) + slot;
+                    const int ndc = min(NPART, max(1, ((r + 1) * q / ncl - r * q / ncl) / 8));
+                    for (int w = 0; w < ndc; ++w, pp += 3 * NPR) {
+                        a += pp[0];
+                        bb += pp[NPR];
+                        c += pp[2 * NPR];
+                    }
+                }
                 double cs = 1.0, sn = 0.0;
-                if (c != 0.0 && fabs(c) > tol * sqrt(a * bb)) {
-                    const double zeta = (bb - a) / (2.0 * c);
-                    const double t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
-                    cs = 1.0 / sqrt(fma(t, t, 1.0));
-                    sn = cs * t;
-                    rotated = 1;
+                // (byes have zero sums; NaNs and columns below 2^-511 are left alone)
+                const int eh = max(__double2hiint(a), __double2hiint(bb)) & 0x7FF00000;
+                if (c != 0.0 && eh >= 0x00100000 && eh < 0x7FE00000) {
+                    // scaled by the power of two that takes the larger norm to [1, 2)
+                    const double sc = __hiloint2double(0x7FE00000 - eh, 0);
+                    const double as = a * sc, bs = bb * sc, cs_ = c * sc;
+                    if (cs_ * cs_ > tol * tol * as * bs) {
+                        // tangent of the angle in FP32
+                        const float df = f64_to_f32(bs - as), cf = f64_to_f32(cs_);
+                        float t;
+                        if (cf == 0.0f) {
+                            t = (float)(c / (bb - a));
+                        } else {
+                            const float zeta = 0.5f * df / cf;
+                            t = fabsf(zeta) < 1e15f ? copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)))
+                                                    : 0.5f / zeta;
+                        }
+                        const double td = (double)t;
+                        if (td != 0.0) {
+                            cs = rsqrt_f64(fma(td, td, 1.0));
+                            sn = cs * td;
+                            rotated = 1;
+                        }
+                    }
                 }
                 s_cs[slot] = cs;
                 s_sn[slot] = sn;
+                s_uv[slot][0] = x;
+                s_uv[slot][1] = y;
             }
             __syncthreads();
-            for (int slot = threadIdx.x / SV_LPP; slot < npairs; slot += TT_NT / SV_LPP) {  // no shuffles: groups may leave early
-                const double sn = s_sn[slot];
-                if (sn == 0.0) continue;
-                const double cs = s_cs[slot];
-                const int u = s_uv[slot][0], v = s_uv[slot][1], sub = lane % SV_LPP;
-                double *mu = M + u * ldm, *mv = M + v * ldm;
-                for (int i = sub; i < q; i += SV_LPP) {
-                    const double x = mu[i], y = mv[i];
-                    mu[i] = cs * x - sn * y;
-                    mv[i] = sn * x + cs * y;
-                }
-                double *vu = V + u * ldv, *vv = V + v * ldv;
-                for (int i = sub; i < pk; i += SV_LPP) {
-                    const double x = vu[i], y = vv[i];
-                    vu[i] = cs * x - sn * y;
-                    vv[i] = sn * x + cs * y;
+            for (int u = warp; u < (qn + pn) * ((npairs + 31) / 32); u += TT_NW) {
+                const int i = u % (qn + pn), slot = (u / (qn + pn)) * 32 + lane;
+                if (slot < npairs && s_sn[slot] != 0.0) {
+                    const double cs = s_cs[slot], sn = s_sn[slot];
+                    double *mu = M + s_uv[slot][0] * ldm + i, *mv = M + s_uv[slot][1] * ldm + i;
+                    const double x = *mu, y = *mv;
+                    *mu = cs * x - sn * y;
+                    *mv = sn * x + cs * y;
                 }
             }
             __syncthreads();
         }
-        if (!rotated) break;
+        if (!rotated) break;  // the same on every CTA: all form the same angles
         __syncthreads();
     }
     // singular values, their descending order (ties by index), norm, rank
-    for (int t = warp; t < pk; t += TT_NW) {
-        double a = 0.0;
-        for (int i = lane; i < q; i += 32) a = fma(M[t * ldm + i], M[t * ldm + i], a);
-        a = warp_sum_d(a);
-        if (lane == 0) sig[t] = sqrt(a);
+    norms();
+    for (int t = threadIdx.x; t < pk; t += TT_NT) {
+        sig[t] = sqrt(s_nrm[t]);
+        ord[t] = t;  // (every entry stays an index, also when NaNs leave the order undefined)
     }
     __syncthreads();
     for (int t = threadIdx.x; t < pk; t += TT_NT) {
@@ -422,8 +510,10 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
             double s2 = 0.0;
             for (int t = pk - 1; t >= 0; --t) s2 += sig[ord[t]] * sig[ord[t]];
             delta = d.eps / sqrt(2.0) * sqrt(s2);
-            d.delta[0] = delta;
-            d.delta[1] = sqrt(s2);
+            if (rank == 0) {
+                d.delta[0] = delta;
+                d.delta[1] = sqrt(s2);
+            }
         } else {
             delta = d.delta[0];
         }
@@ -439,20 +529,21 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
         }
         if (r > d.rmax) r = d.rmax;
         s_rank = r;
-        s_delta = delta;
-        d.rank[0] = r;
+        if (rank == 0) d.rank[0] = r;
     }
     __syncthreads();
     const int r = s_rank;
-    for (int t = threadIdx.x; t < pk; t += TT_NT) d.sv[t] = sig[ord[t]];
-    for (int e = threadIdx.x; e < pk * r; e += TT_NT) {
+    if (rank == 0)
+        for (int t = threadIdx.x; t < pk; t += TT_NT) d.sv[t] = sig[ord[t]];
+    for (int e = threadIdx.x; e < pn * r; e += TT_NT) {
         const int i = e / r, c = e - i * r;
-        d.Vsel[(long long)i * d.ld_out + c] = V[ord[c] * ldv + i];
+        d.Vsel[(long long)(pa + i) * d.ld_out + c] = M[ord[c] * ldm + qn + i];
     }
-    for (int e = threadIdx.x; e < q * r; e += TT_NT) {
+    for (int e = threadIdx.x; e < qn * r; e += TT_NT) {
         const int i = e / r, c = e - i * r;
-        d.Wt[(long long)i * d.ld_out + c] = M[ord[c] * ldm + i];
+        d.Wt[(long long)(qa + i) * d.ld_out + c] = M[ord[c] * ldm + i];
     }
+    cl.sync();  // no CTA leaves while another may still read its partial sums
 }
 
 // First-core unfolding C1 [n1][R1] (coefficient folded in) and transposed
@@ -526,7 +617,8 @@ static cudaError_t tt_set_attributes()
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_qr_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_qr_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_svd_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_svd_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)svd_smem(TT_KMAX, TT_KMAX, 1))) != cudaSuccess) return e;
     tt_attrs_set = true;
     return cudaSuccess;
 }
@@ -547,12 +639,23 @@ cudaError_t launch_qr_apply(const QApplyDesc *d, int n, int max_chunks, size_t s
     return cudaGetLastError();
 }
 
-cudaError_t launch_svd_jacobi(const SvdDesc *d, int n, size_t smem, cudaStream_t s)
+cudaError_t launch_svd_jacobi(const SvdDesc *d, int n, int ncl, size_t smem, cudaStream_t s)
 {
     cudaError_t e = tt_set_attributes();
     if (e != cudaSuccess) return e;
-    k_svd_jacobi<<<n, TT_NT, smem, s>>>(d);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ncl, n);
+    cfg.blockDim = dim3(TT_NT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ncl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_svd_jacobi, d);
 }
 
 cudaError_t launch_tt_build(const TTSumDesc *d, int n, cudaStream_t s)

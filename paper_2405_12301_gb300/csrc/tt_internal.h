@@ -23,6 +23,7 @@ struct QRDesc {
     int sub_per_chunk;
     double *tau;           // [chunks][sub_per_chunk][k]
     double *Rout;          // [chunks][k][k] row-major R of each chunk
+    int tri;               // the matrix is a stack of k x k upper triangular blocks (sub-blocks of k rows)
 };
 
 // out = Q [X; 0] for the reflectors left by one QRDesc level.
@@ -38,6 +39,7 @@ struct QApplyDesc {
     int ldx, p;
     double *out;               // out(row, col) = out[(row % P) sP + (row / P) sQ + col sC]
     long long P, sP, sQ, sC;
+    int tri;                   // as in QRDesc
 };
 
 // One-sided Jacobi SVD of T^T (T: pk x q row-major, stride ldt) and truncation.
@@ -78,10 +80,11 @@ struct GemmDesc {  // out[rows][cols] = L[rows][ka] Rt[cols][ka]^T
 
 size_t qr_factor_smem(int k, int b);
 size_t qr_apply_smem(int k, int b, int p);
-size_t svd_smem(int pk, int q);
+size_t svd_smem(int pk, int q, int ncl);
+int svd_cluster(int n, int max_pk);  // CTAs per matrix of a batch of n
 cudaError_t launch_qr_factor(const QRDesc *d, int n, int max_chunks, size_t smem, cudaStream_t s);
 cudaError_t launch_qr_apply(const QApplyDesc *d, int n, int max_chunks, size_t smem, cudaStream_t s);
-cudaError_t launch_svd_jacobi(const SvdDesc *d, int n, size_t smem, cudaStream_t s);
+cudaError_t launch_svd_jacobi(const SvdDesc *d, int n, int ncl, size_t smem, cudaStream_t s);
 cudaError_t launch_tt_build(const TTSumDesc *d, int n, cudaStream_t s);
 cudaError_t launch_tt_contract(const TTSumDesc *d, int n, cudaStream_t s);
 cudaError_t launch_tt_gemm_tr(const GemmDesc *d, int n, cudaStream_t s);
