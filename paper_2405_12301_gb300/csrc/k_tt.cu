@@ -15,16 +15,17 @@
 //     chunk in reverse (eight lanes per column of X, four columns per warp,
 //     no block barrier inside a sub-block); writes the rows through a general row map so that results
 //     land directly in TT-core layout.
-//   * k_svd_jacobi: one-sided Jacobi SVD (round-robin pair ordering) of the
-//     transpose of a k x q triangular factor T: T^T V = U S gives T = V S U^T;
-//     picks the truncation rank from the singular values and writes V's kept
-//     columns and (U S)'s kept columns.  The rows of T^T and of V are spread over
-//     the CTAs of a cluster: a rotation acts on every row alone, only the dot
-//     products that choose the angles are sums over all of them.
+//   * k_svd_jacobi: SVD T = V S U^T of a k x q triangular factor by a QR with
+//     column pivoting and one-sided Jacobi (round-robin pair ordering); picks the
+//     truncation rank from the singular values and writes V's kept columns and
+//     (U S)'s kept columns.  The rows that Jacobi rotates are spread over the CTAs
+//     of a cluster: a rotation acts on every row alone, only the dot products that
+//     choose the angles are sums over all of them.
 //   * k_tt_build / k_tt_contract / k_tt_gemm_tr: the TT sum's first and last
 //     unfoldings, the block-diagonal middle core times a triangular factor, and
 //     a small dense product.
 // All arithmetic is FP64.
+#include <algorithm>
 #include <cfloat>
 
 #include <cooperative_groups.h>
@@ -110,16 +111,21 @@ size_t qr_apply_smem(int k, int b, int p)
 {
     return sizeof(double) * ((size_t)k * (b + LDPAD) + (size_t)p * (b + LDPAD) + (size_t)p * (k + 1) + k);
 }
+constexpr int SV_MAXCL = 8;  // CTAs per SVD at most
 size_t svd_smem(int pk, int q, int ncl)
 {
-    return sizeof(double) * ((size_t)pk * (((q + ncl - 1) / ncl + (pk + ncl - 1) / ncl) | 1) + pk);
+    const size_t m = (size_t)pk * ((2 * ((pk + ncl - 1) / ncl)) | 1);
+    return sizeof(double) * ((size_t)pk * (q | 1) + 2 * ncl * 3 * (TT_KMAX / 2) + (m > 8 * (size_t)(q | 1) ? m : 8 * (size_t)(q | 1)));
 }
 
-// CTAs per matrix: as many as the GPU has SMs for, at most 8 and at least ~8 rows each.
+// CTAs per matrix: as many as the GPU has SMs for, at most 8 and at least 6 rows
+// each; two where one CTA's shared memory would not do.
+constexpr int SV_ONE = 88;  // largest matrix of a single CTA
 int svd_cluster(int n, int max_pk)
 {
-    int ncl = 8;
-    while (ncl > 1 && ((long long)n * ncl > sm_count() || max_pk / ncl < 6)) ncl /= 2;
+    int ncl = SV_MAXCL;
+    const int least = max_pk > SV_ONE ? 2 : 1;
+    while (ncl > least && ((long long)n * ncl > sm_count() || max_pk / ncl < 6)) ncl /= 2;
     return ncl;
 }
 
@@ -342,18 +348,26 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
     store(r0, b1);
 }
 
-// One-sided Jacobi on the pk columns of M = T^T (column t = row t of T, length q).
-// A sweep of 64 columns is 63 rounds of 32 disjoint pairs; per round an SM did ~790
-// FP64 instructions (7.2 us).  Here each CTA of the cluster holds all columns of a
-// slice of M's and V's rows.  Per round: partial dot products m_u . m_u, m_v . m_v
-// and m_u . m_v over the slice (a lane per pair; the three chains overlap, and
-// norms carried from round to round lose all digits on nearly dependent columns),
-// one cluster barrier, the sum of all partials and the angle (a lane per pair,
-// every CTA the same), the rotations of the slice (a lane per pair, a warp per
-// row).  The tangent of the angle is formed in FP32 (with Newton steps for cos =
-// 1 / sqrt(1 + t^2)): it only steers, the rotation is orthogonal to FP64 rounding
-// whatever t is, and a pair counts as orthogonal by its FP64 dot products.  64 x 64, 10 matrices: 4.8 -> SVDT ms.
-// cluster size 1..8 (svd_cluster): fewer CTAs where the batch fills the GPU.
+// SVD of T (pk x q row-major, pk <= q): one-sided Jacobi, preconditioned by a QR with
+// column pivoting.  T^T P = Q R, Jacobi makes the columns of the lower triangular
+// R^T orthogonal, R^T J = Z, so T = P R^T Q^T = (P Z) (Q J)^T: the left vectors are
+// the columns of P Z over their norms sigma, and sigma u = Q J sigma.  On R^T Jacobi
+// takes 5 sweeps where it takes 8 to 10 on T^T itself (the nearly dependent columns
+// of a TT sum; 64 x 64).
+//   1. pivoted Householder QR of T^T, every CTA of the cluster the same;
+//   2. Jacobi: each CTA holds all columns of a slice of Z's and J's rows.  Per round
+//      of disjoint pairs: partial dot products over the slice (a lane per pair),
+//      pushed to every CTA; one cluster barrier; the sum of the partials and the
+//      angle (a lane per pair, every CTA the same); the rotations of the slice (a
+//      lane per pair, a warp per row).  The tangent of the angle is formed in FP32
+//      (with Newton steps for cos = 1 / sqrt(1 + t^2)): it only steers, the rotation
+//      is orthogonal to FP64 rounding whatever t is.  Every pair beyond 4 eps is
+//      rotated; the sweeps end when no pair's cosine was above 8 max(pk, q) eps.
+//   3. each CTA applies Q to its share of the columns of J sigma.
+// A round is a chain of latencies (FP64 68 cycles each, a cluster barrier), not
+// work: 10 matrices of 50..64, 5.1 ms on one CTA each without the QR, 3.6 ms on 8
+// CTAs with pulled partials, SVDT ms here.
+// Cluster size 1..8 (svd_cluster): fewer CTAs where the batch fills the GPU.
 __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
 {
     cg::cluster_group cl = cg::this_cluster();
@@ -362,111 +376,215 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     const int pk = d.pk, q = d.q;
     if (pk <= 0) return;  // the same for every CTA of the cluster
     extern __shared__ double sm[];
-    constexpr int NPR = TT_KMAX / 2, NPART = 4;
-    // this CTA's partial dot products (m_u . m_u, m_v . m_v, m_u . m_v; double buffered) and norms
-    __shared__ double part[2][NPART][3][NPR], norm_part[NPART][TT_KMAX];
-    __shared__ double s_nrm[TT_KMAX], s_cs[NPR], s_sn[NPR];
-    __shared__ int s_uv[NPR][2], ord[TT_KMAX], rotated, s_rank;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int qa = rank * q / ncl, qn = (rank + 1) * q / ncl - qa;     // rows of M
-    const int pa = rank * pk / ncl, pn = (rank + 1) * pk / ncl - pa;   // rows of V
-    const int ldm = (qn + pn) | 1;
-    double *M = sm;                          // [pk][ldm]: qn rows of M, then pn rows of V
-    double *sig = M + (size_t)pk * ldm;      // [pk]
-    for (int e = threadIdx.x; e < pk * qn; e += TT_NT) {
-        const int t = e / qn, i = e - t * qn;
-        M[t * ldm + i] = d.T[(long long)t * d.ldt + qa + i];
-    }
-    for (int e = threadIdx.x; e < pk * pn; e += TT_NT) {
-        const int t = e / pn, i = e - t * pn;
-        M[t * ldm + qn + i] = (pa + i == t) ? 1.0 : 0.0;
-    }
+    constexpr int NPR = TT_KMAX / 2;
+    __shared__ double sig[TT_KMAX], ts[TT_KMAX], s_cs[NPR], s_sn[NPR];
+    __shared__ float nrm[TT_KMAX];
+    __shared__ int s_uv[NPR][2], ord[TT_KMAX], perm[TT_KMAX], rotated, s_rank, s_exp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane / LPC, sub = lane % LPC;
+    const int pa = rank * pk / ncl, pn = (rank + 1) * pk / ncl - pa;   // rows of Z and of J
+    const int lda = q | 1, ldm = (2 * pn) | 1;
+    double *A = sm;                          // [pk][lda]: T^T column-major, then its reflectors and R
+    // the CTAs' partial dot products (z_u . z_u, z_v . z_v, z_u . z_v), double buffered:
+    // part + ((par * ncl + CTA) * 3 + k) * NPR
+    double *part = A + (size_t)pk * lda;
+    double *M = part + 2 * ncl * 3 * NPR;    // [pk][ldm]: pn rows of Z, then pn rows of J
+    if (threadIdx.x == 0) s_exp = 0;
     __syncthreads();
+    for (int e = threadIdx.x; e < pk * q; e += TT_NT) {
+        const int t = e / q, i = e - t * q;
+        const double x = d.T[(long long)t * d.ldt + i];
+        A[t * lda + i] = x;
+        atomicMax(&s_exp, (__double2hiint(x) >> 20) & 0x7FF);
+    }
+    for (int t = threadIdx.x; t < pk; t += TT_NT) perm[t] = t;
+    __syncthreads();
+    // FP32 value of x over the power of two of T's largest entry (0 below 2^-60 of it)
+    const int eoff = s_exp - 1023;
+    auto relative = [&](double x) {
+        const int h = __double2hiint(x), ex = ((h >> 20) & 0x7FF) - eoff;
+        const unsigned b = ((unsigned)(ex - 896) << 23) | (((unsigned)h & 0xFFFFFu) << 3) | ((unsigned)__double2loint(x) >> 29);
+        return ex < 963 ? 0.0f : __uint_as_float(b);
+    };
+
+    // ---- 1. QR with column pivoting (the pivot by FP32 norms of what is left: it only
+    // has to be near the largest)
+    for (int j = 0; j < pk; ++j) {
+        for (int c = j + warp * CPW + grp; c < pk + grp; c += TT_NW * CPW) {  // (whole warps: c - grp < pk)
+            float s = 0.0f;
+            if (c < pk)
+                for (int i = j + sub; i < q; i += LPC) {
+                    const float x = relative(A[c * lda + i]);
+                    s = fmaf(x, x, s);
+                }
+#pragma unroll
+            for (int o = LPC / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+            if (c < pk && sub == 0) nrm[c] = s;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            float best = -1.0f;
+            int bc = j;
+            for (int c = j + lane; c < pk; c += 32)
+                if (nrm[c] > best) {
+                    best = nrm[c];
+                    bc = c;
+                }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+                const int oc = __shfl_xor_sync(0xFFFFFFFFu, bc, o);
+                if (ob > best || (ob == best && oc < bc)) {
+                    best = ob;
+                    bc = oc;
+                }
+            }
+            if (bc != j)
+                for (int i = lane; i < q; i += 32) {
+                    const double x = A[j * lda + i];
+                    A[j * lda + i] = A[bc * lda + i];
+                    A[bc * lda + i] = x;
+                }
+            __syncwarp();
+            double *x = A + j * lda;
+            double s = 0.0;
+            for (int i = j + 1 + lane; i < q; i += 32) s = fma(x[i], x[i], s);
+            s = warp_sum_d(s);
+            double beta, tau, scale;
+            householder(x[j], s, beta, tau, scale);
+            for (int i = j + 1 + lane; i < q; i += 32) x[i] *= scale;
+            __syncwarp();  // every lane has read x[j]
+            if (lane == 0) {
+                x[j] = beta;
+                ts[j] = tau;
+                const int p = perm[j];
+                perm[j] = perm[bc];
+                perm[bc] = p;
+            }
+        }
+        __syncthreads();
+        const double tau = ts[j];
+        if (tau != 0.0) {
+            const double *v = A + j * lda;
+            for (int c0 = j + 1 + warp * CPW; c0 < pk; c0 += TT_NW * CPW) {
+                const int c = c0 + grp;
+                const bool ok = c < pk;
+                double *col = A + (ok ? c : 0) * lda;
+                double w = 0.0, w1 = 0.0;
+                if (ok) {
+                    int i = j + 1 + sub;
+                    for (; i + LPC < q; i += 2 * LPC) {
+                        w = fma(v[i], col[i], w);
+                        w1 = fma(v[i + LPC], col[i + LPC], w1);
+                    }
+                    if (i < q) w = fma(v[i], col[i], w);
+                }
+                w = (group_sum(w + w1) + (ok ? col[j] : 0.0)) * tau;
+                if (ok)
+                    for (int i = j + 1 + sub; i < q; i += LPC) col[i] = fma(-v[i], w, col[i]);
+                __syncwarp();
+                if (ok && sub == 0) col[j] -= w;
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- 2. Z = R^T (column t of Z is row t of R), J = identity
+    for (int e = threadIdx.x; e < pk * pn; e += TT_NT) {
+        const int t = e / pn, i = e - t * pn, c = pa + i;
+        M[t * ldm + i] = c >= t ? A[c * lda + t] : 0.0;
+        M[t * ldm + pn + i] = c == t ? 1.0 : 0.0;
+    }
+    if (threadIdx.x == 0) rotated = 0;
+    cl.sync();  // every CTA has started: partials may be pushed
     const int n = pk + (pk & 1);  // round-robin over an even count; index pk (odd case) is a bye
     const int npairs = n / 2;
-    const double tol = 8.0 * (double)max(pk, q) * DBL_EPSILON;  // cosine below which a pair counts as orthogonal
-    const int nd = min(NPART, max(1, qn / 8));  // warps per column or pair that form partial sums, ~8+ rows each
-
-    // squared norms of all columns, summed over the cluster in a fixed order into s_nrm
-    auto norms = [&]() {
-        for (int u = warp; u < nd * ((pk + 31) / 32); u += TT_NW) {
-            const int w = u % nd, t = (u / nd) * 32 + lane;
-            if (t < pk) {
-                double a = 0.0;
-                for (int i = w; i < qn; i += nd) a = fma(M[t * ldm + i], M[t * ldm + i], a);
-                norm_part[w][t] = a;
-            }
-        }
-        cl.sync();
-        for (int t = threadIdx.x; t < pk; t += TT_NT) {
-            double a = 0.0;
-            for (int c = 0; c < ncl; ++c) {
-                const double *np = cl.map_shared_rank(&norm_part[0][0], c);
-                const int ndc = min(NPART, max(1, ((c + 1) * q / ncl - c * q / ncl) / 8));
-                for (int w = 0; w < ndc; ++w) a += np[w * TT_KMAX + t];
-            }
-            s_nrm[t] = a;
-        }
-        cl.sync();  // the partials may be written again
-    };
+    const double eps_cos = 8.0 * (double)max(pk, q) * DBL_EPSILON;  // cosine below which a pair counts as orthogonal
     int par = 0;
-    for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
-        if (threadIdx.x == 0) rotated = 0;  // (set after the next barrier at the earliest)
-        for (int round = 0; round < n - 1; ++round, par ^= 1) {
-            auto idx = [&](int t) { return t == 0 ? 0 : 1 + (t - 1 + round) % (n - 1); };
-            for (int u = warp; u < nd * ((npairs + 31) / 32); u += TT_NW) {
-                const int w = u % nd, slot = (u / nd) * 32 + lane;
-                if (slot < npairs) {
-                    const int x = idx(slot), y = idx(n - 1 - slot);
-                    double a = 0.0, b = 0.0, c = 0.0;
-                    if (x < pk && y < pk)
-                        for (int i = w; i < qn; i += nd) {
-                            const double u = M[x * ldm + i], v = M[y * ldm + i];
-                            a = fma(u, u, a);
-                            b = fma(v, v, b);
-                            c = fma(u, v, c);
-                        }
-                    part[par][w][0][slot] = a;
-                    part[par][w][1][slot] = b;
-                    part[par][w][2][slot] = c;
-                }
+    // this CTA's partial sums over its rows of column pairs, into every CTA's part
+    double *dst[SV_MAXCL];
+#pragma unroll
+    for (int r = 0; r < SV_MAXCL; ++r) dst[r] = cl.map_shared_rank(part + rank * 3 * NPR, r < ncl ? r : 0);
+    auto push = [&](int slot, int x, int y) {
+        double a0 = 0.0, b0 = 0.0, c0 = 0.0, a1 = 0.0, b1 = 0.0, c1 = 0.0;
+        if (x < pk && y < pk) {
+            const double *zx = M + x * ldm, *zy = M + y * ldm;
+            int i = 0;
+            for (; i + 1 < pn; i += 2) {
+                const double u = zx[i], v = zy[i], u1 = zx[i + 1], v1 = zy[i + 1];
+                a0 = fma(u, u, a0);
+                b0 = fma(v, v, b0);
+                c0 = fma(u, v, c0);
+                a1 = fma(u1, u1, a1);
+                b1 = fma(v1, v1, b1);
+                c1 = fma(u1, v1, c1);
             }
+            if (i < pn) {
+                a0 = fma(zx[i], zx[i], a0);
+                b0 = fma(zy[i], zy[i], b0);
+                c0 = fma(zx[i], zy[i], c0);
+            }
+            a0 += a1;
+            b0 += b1;
+            c0 += c1;
+        }
+        const int o = par * ncl * 3 * NPR + slot;
+#pragma unroll
+        for (int r = 0; r < SV_MAXCL; ++r)
+            if (r < ncl) {
+                dst[r][o] = a0;
+                dst[r][o + NPR] = b0;
+                dst[r][o + 2 * NPR] = c0;
+            }
+    };
+    auto total = [&](int k, int slot) {  // over the CTAs, in a fixed order
+        const double *p = part + (par * ncl * 3 + k) * NPR + slot;
+        if (ncl == 1) return p[0];
+        double s[SV_MAXCL];
+#pragma unroll
+        for (int r = 0; r < SV_MAXCL; ++r) s[r] = r < ncl ? p[r * 3 * NPR] : 0.0;
+        const double lo = (s[0] + s[1]) + (s[2] + s[3]);
+        return ncl <= 4 ? lo : lo + ((s[4] + s[5]) + (s[6] + s[7]));
+    };
+    // a round's pair of this thread: slot t pairs the players at places t and n - 1 - t
+    // of a circle; player 0 stays, the others move one place a round
+    int px = threadIdx.x < npairs ? (int)threadIdx.x : 0, py = n - 1 - px;
+    for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
+        for (int round = 0; round < n - 1; ++round, par ^= 1) {
+            const int slot = threadIdx.x, x = px, y = py;
+            if (slot < npairs) push(slot, x, y);
             cl.sync();
-            for (int slot = threadIdx.x; slot < npairs; slot += TT_NT) {
-                const int x = idx(slot), y = idx(n - 1 - slot);
-                double a = 0.0, bb = 0.0, c = 0.0;
-                for (int r = 0; r < ncl; ++r) {
-                    const double *pp = cl.map_shared_rank(&part[par][0][0][0], r) + slot;
-                    const int ndc = min(NPART, max(1, ((r + 1) * q / ncl - r * q / ncl) / 8));
-                    for (int w = 0; w < ndc; ++w, pp += 3 * NPR) {
-                        a += pp[0];
-                        bb += pp[NPR];
-                        c += pp[2 * NPR];
-                    }
-                }
+            if (slot < npairs) {
+                const double a = total(0, slot), b = total(1, slot), c = total(2, slot);
                 double cs = 1.0, sn = 0.0;
                 // (byes have zero sums; NaNs and columns below 2^-511 are left alone)
-                const int eh = max(__double2hiint(a), __double2hiint(bb)) & 0x7FF00000;
+                const int eh = max(__double2hiint(a), __double2hiint(b)) & 0x7FF00000;
                 if (c != 0.0 && eh >= 0x00100000 && eh < 0x7FE00000) {
-                    // scaled by the power of two that takes the larger norm to [1, 2)
-                    const double sc = __hiloint2double(0x7FE00000 - eh, 0);
-                    const double as = a * sc, bs = bb * sc, cs_ = c * sc;
-                    if (cs_ * cs_ > tol * tol * as * bs) {
-                        // tangent of the angle in FP32
-                        const float df = f64_to_f32(bs - as), cf = f64_to_f32(cs_);
+                    // over the power of two of the larger norm, in FP32: the tangent of
+                    // the angle (0 below 2^-126)
+                    auto rel = [&](double v) {
+                        const int h = __double2hiint(v), ex = ((h & 0x7FF00000) - eh) >> 20;
+                        const unsigned m = ((unsigned)h & 0x800FFFFFu) | (unsigned)((ex + 127) << 20);
+                        return ex < -126 ? 0.0f
+                                         : __uint_as_float((m & 0x80000000u) | ((m & 0x0FFFFFFFu) << 3) |
+                                                           ((unsigned)__double2loint(v) >> 29));
+                    };
+                    const float cf = rel(c), len = sqrt_approx(rel(a)) * sqrt_approx(rel(b));
+                    if (fabsf(cf) > 4.0f * (float)DBL_EPSILON * len || cf == 0.0f) {
                         float t;
                         if (cf == 0.0f) {
-                            t = (float)(c / (bb - a));
+                            t = (float)(c / (b - a));
                         } else {
-                            const float zeta = 0.5f * df / cf;
-                            t = fabsf(zeta) < 1e15f ? copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.0f)))
-                                                    : 0.5f / zeta;
+                            const float zeta = 0.5f * rel(b - a) * fast_rcp(cf);
+                            t = fabsf(zeta) < 1e15f
+                                    ? copysignf(fast_rcp(fabsf(zeta) + sqrt_approx(fmaf(zeta, zeta, 1.0f))), zeta)
+                                    : 0.5f * fast_rcp(zeta);
                         }
-                        const double td = (double)t;
-                        if (td != 0.0) {
+                        if (fabsf(t) > 1e-37f) {
+                            const double td = f32_to_f64_nz(t);
                             cs = rsqrt_f64(fma(td, td, 1.0));
                             sn = cs * td;
-                            rotated = 1;
+                            // (len == 0: a norm ratio below 2^-63)
+                            if (len > 0.0f ? fabsf(cf) > (float)eps_cos * len : c * c > eps_cos * eps_cos * a * b) rotated = 1;
                         }
                     }
                 }
@@ -474,29 +592,35 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
                 s_sn[slot] = sn;
                 s_uv[slot][0] = x;
                 s_uv[slot][1] = y;
+                px = px == 0 ? 0 : px + 1 < n ? px + 1 : 1;
+                py = py == 0 ? 0 : py + 1 < n ? py + 1 : 1;
             }
             __syncthreads();
-            for (int u = warp; u < (qn + pn) * ((npairs + 31) / 32); u += TT_NW) {
-                const int i = u % (qn + pn), slot = (u / (qn + pn)) * 32 + lane;
-                if (slot < npairs && s_sn[slot] != 0.0) {
-                    const double cs = s_cs[slot], sn = s_sn[slot];
-                    double *mu = M + s_uv[slot][0] * ldm + i, *mv = M + s_uv[slot][1] * ldm + i;
-                    const double x = *mu, y = *mv;
-                    *mu = cs * x - sn * y;
-                    *mv = sn * x + cs * y;
+            for (int g = lane; g < npairs; g += 32) {
+                if (s_sn[g] == 0.0) continue;
+                const double cs = s_cs[g], sn = s_sn[g];
+                double *mu = M + s_uv[g][0] * ldm, *mv = M + s_uv[g][1] * ldm;
+                for (int i = warp; i < 2 * pn; i += TT_NW) {
+                    const double u = mu[i], v = mv[i];
+                    mu[i] = cs * u - sn * v;
+                    mv[i] = sn * u + cs * v;
                 }
             }
             __syncthreads();
         }
-        if (!rotated) break;  // the same on every CTA: all form the same angles
+        const bool more = rotated != 0;  // the same on every CTA: all form the same angles
         __syncthreads();
+        if (threadIdx.x == 0) rotated = 0;
+        if (!more) break;
     }
-    // singular values, their descending order (ties by index), norm, rank
-    norms();
-    for (int t = threadIdx.x; t < pk; t += TT_NT) {
-        sig[t] = sqrt(s_nrm[t]);
-        ord[t] = t;  // (every entry stays an index, also when NaNs leave the order undefined)
+    // ---- singular values (the norms of Z's columns), their descending order (ties by
+    // index), norm, rank
+    for (int t0 = 0; t0 < pk; t0 += NPR, par ^= 1) {  // (as pairs of a column with itself)
+        if (threadIdx.x < NPR && t0 + threadIdx.x < pk) push(threadIdx.x, t0 + threadIdx.x, t0 + threadIdx.x);
+        cl.sync();
+        if (threadIdx.x < NPR && t0 + threadIdx.x < pk) sig[t0 + threadIdx.x] = sqrt(total(0, threadIdx.x));
     }
+    for (int t = threadIdx.x; t < pk; t += TT_NT) ord[t] = t;  // every entry stays an index, also with NaNs
     __syncthreads();
     for (int t = threadIdx.x; t < pk; t += TT_NT) {
         int r = 0;
@@ -535,15 +659,80 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     const int r = s_rank;
     if (rank == 0)
         for (int t = threadIdx.x; t < pk; t += TT_NT) d.sv[t] = sig[ord[t]];
+    // left vectors: rows P of Z over sigma.  A zero column (only kept when T has fewer
+    // nonzero singular values than the rank) gets an orthonormal direction below.
     for (int e = threadIdx.x; e < pn * r; e += TT_NT) {
-        const int i = e / r, c = e - i * r;
-        d.Vsel[(long long)(pa + i) * d.ld_out + c] = M[ord[c] * ldm + qn + i];
+        const int i = e / r, c = e - i * r, t = ord[c];
+        const double s = sig[t];
+        d.Vsel[(long long)perm[pa + i] * d.ld_out + c] = s > 0.0 ? M[t * ldm + i] / s : 0.0;
+        d.Wt[(long long)(pa + i) * d.ld_out + c] = M[t * ldm + pn + i] * s;
     }
-    for (int e = threadIdx.x; e < qn * r; e += TT_NT) {
-        const int i = e / r, c = e - i * r;
-        d.Wt[(long long)(qa + i) * d.ld_out + c] = M[ord[c] * ldm + i];
+    __threadfence();
+    cl.sync();  // J sigma is complete (and no CTA reads another's shared memory any more)
+    // ---- 3. columns c = rank, rank + ncl, .. of Q [J sigma; 0], in place of J sigma
+    double *X = M;  // [..][lda] columns (M is free)
+    const int nc = (r - rank + ncl - 1) / ncl;
+    constexpr int CB = 8;
+    for (int c0 = 0; c0 < nc; c0 += CB) {
+        const int w = min(CB, nc - c0);
+        for (int e = threadIdx.x; e < w * q; e += TT_NT) {
+            const int i = e / w, c = e - i * w;
+            X[c * lda + i] = i < pk ? __ldcg(d.Wt + (long long)i * d.ld_out + rank + (c0 + c) * ncl) : 0.0;
+        }
+        __syncthreads();
+        if (warp < w) {  // a warp per column: no barrier between reflectors
+            double *x = X + warp * lda;
+            for (int j = pk - 1; j >= 0; --j) {
+                const double tau = ts[j];
+                if (tau == 0.0) continue;
+                const double *v = A + j * lda;
+                double s = 0.0;
+                for (int i = j + 1 + lane; i < q; i += 32) s = fma(v[i], x[i], s);
+                s = (warp_sum_d(s) + x[j]) * tau;
+                for (int i = j + 1 + lane; i < q; i += 32) x[i] = fma(-v[i], s, x[i]);
+                __syncwarp();
+                if (lane == 0) x[j] -= s;
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < w * q; e += TT_NT) {
+            const int i = e / w, c = e - i * w;
+            d.Wt[(long long)i * d.ld_out + rank + (c0 + c) * ncl] = X[c * lda + i];
+        }
+        __syncthreads();
     }
-    cl.sync();  // no CTA leaves while another may still read its partial sums
+    // ---- zero singular values among the kept ones: complete the left vectors to an
+    // orthonormal set (their sigma u is zero) by Gram-Schmidt on unit vectors
+    if (rank == 0 && warp == 0) {
+        int e0 = 0;
+        for (int c = 0; c < r; ++c) {
+            if (sig[ord[c]] > 0.0) continue;
+            for (; e0 < pk; ++e0) {
+                for (int pass = 0; pass < 2; ++pass) {
+                    for (int i = lane; i < pk; i += 32)
+                        if (pass == 0) X[i] = i == e0 ? 1.0 : 0.0;
+                    __syncwarp();
+                    for (int u = 0; u < c; ++u) {
+                        double s = 0.0;
+                        for (int i = lane; i < pk; i += 32) s = fma(__ldcg(d.Vsel + (long long)i * d.ld_out + u), X[i], s);
+                        s = warp_sum_d(s);
+                        for (int i = lane; i < pk; i += 32) X[i] = fma(-s, __ldcg(d.Vsel + (long long)i * d.ld_out + u), X[i]);
+                        __syncwarp();
+                    }
+                }
+                double s = 0.0;
+                for (int i = lane; i < pk; i += 32) s = fma(X[i], X[i], s);
+                s = warp_sum_d(s);
+                if (s * pk < 0.25) continue;  // some unit vector keeps at least 1 / pk of its square
+                for (int i = lane; i < pk; i += 32) d.Vsel[(long long)i * d.ld_out + c] = X[i] / sqrt(s);
+                __threadfence();
+                __syncwarp();
+                ++e0;
+                break;
+            }
+        }
+    }
 }
 
 // First-core unfolding C1 [n1][R1] (coefficient folded in) and transposed
@@ -618,7 +807,7 @@ static cudaError_t tt_set_attributes()
     if ((e = cudaFuncSetAttribute(k_qr_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_qr_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, mx)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_svd_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)svd_smem(TT_KMAX, TT_KMAX, 1))) != cudaSuccess) return e;
+                                  (int)std::max(svd_smem(SV_ONE, TT_KMAX, 1), svd_smem(TT_KMAX, TT_KMAX, 2)))) != cudaSuccess) return e;
     tt_attrs_set = true;
     return cudaSuccess;
 }
