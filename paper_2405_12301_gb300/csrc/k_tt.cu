@@ -79,6 +79,10 @@ __device__ __forceinline__ double rsqrt_f64(double s)
     return __hiloint2double(__double2hiint(y) - ((e2 / 2) << 20), __double2loint(y));
 }
 
+// The turn of a warp in taking column groups, from its distance to the warp that is
+// ahead: the warps that do not share its sub-partition first, itself last.
+__device__ __forceinline__ int turn(int dist) { return (0x54362107 >> ((dist & 7) * 4)) & 7; }
+
 // Householder vector of x = (x0, y) with ||y||^2 = sig: H = I - tau v v^T,
 // v = (1, y / (x0 - beta)), H x = (beta, 0).  sig == 0 gives tau = 0.  Every column
 // waits for this chain of dependent FP64 operations (68 cycles each), so it takes
@@ -132,7 +136,9 @@ int svd_cluster(int n, int max_pk)
 // The column loop keeps one reflector ahead: while the other warps apply reflector
 // j to their columns, one warp applies it to column j + 1 and forms reflector j + 1
 // from it, so that chain (~35 dependent FP64 operations) runs beside the updates
-// and a column takes one barrier.  64 columns of a 64-row sub-block: 195 -> QRSUB us.
+// and a column takes one barrier.  The other column groups go first to the warps of
+// the other three sub-partitions: a sub-partition issues an FP64 instruction every 64
+// cycles, whatever its warps.  64 columns of a 64-row sub-block: 195 -> QRSUB us.
 __global__ void __launch_bounds__(TT_NT) k_qr_factor(const QRDesc *descs)
 {
     const QRDesc &d = descs[blockIdx.y];
@@ -199,7 +205,7 @@ __global__ void __launch_bounds__(TT_NT) k_qr_factor(const QRDesc *descs)
                 if (j + 1 < kk) generate(j + 1);
             }
             if (tau != 0.0) {
-                for (int c0 = j + 2 + ((warp - ahead - 1) & (TT_NW - 1)) * CPW; c0 < k; c0 += TT_NW * CPW) {
+                for (int c0 = j + 2 + turn(warp - ahead) * CPW; c0 < k; c0 += TT_NW * CPW) {
                     const int c = c0 + grp;
                     const bool ok = c < k;
                     double *col = B + (ok ? c : 0) * ldb;
@@ -356,10 +362,10 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
 // of a TT sum; 64 x 64).
 //   1. pivoted Householder QR of T^T, every CTA of the cluster the same;
 //   2. Jacobi: each CTA holds all columns of a slice of Z's and J's rows.  Per round
-//      of disjoint pairs: partial dot products over the slice (a lane per pair),
-//      pushed to every CTA; one cluster barrier; the sum of the partials and the
-//      angle (a lane per pair, every CTA the same); the rotations of the slice (a
-//      lane per pair, a warp per row).  The tangent of the angle is formed in FP32
+//      of disjoint pairs: partial dot products over the slice (a lane per pair, a
+//      warp per quantity), pushed to every CTA; one cluster barrier; the sums of the
+//      partials, the angle (a lane per pair, every CTA the same); the rotations of
+//      the slice (a lane per pair, a warp per row).  The tangent of the angle is formed in FP32
 //      (with Newton steps for cos = 1 / sqrt(1 + t^2)): it only steers, the rotation
 //      is orthogonal to FP64 rounding whatever t is.  Every pair beyond 4 eps is
 //      rotated; the sweeps end when no pair's cosine was above 8 max(pk, q) eps.
@@ -377,7 +383,7 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     if (pk <= 0) return;  // the same for every CTA of the cluster
     extern __shared__ double sm[];
     constexpr int NPR = TT_KMAX / 2;
-    __shared__ double sig[TT_KMAX], ts[TT_KMAX], s_cs[NPR], s_sn[NPR];
+    __shared__ double sig[TT_KMAX], ts[TT_KMAX], s_cs[NPR], s_sn[NPR], s_tot[3][NPR];
     __shared__ float nrm[TT_KMAX];
     __shared__ int s_uv[NPR][2], ord[TT_KMAX], perm[TT_KMAX], rotated, s_rank, s_exp;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane / LPC, sub = lane % LPC;
@@ -504,37 +510,24 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     double *dst[SV_MAXCL];
 #pragma unroll
     for (int r = 0; r < SV_MAXCL; ++r) dst[r] = cl.map_shared_rank(part + rank * 3 * NPR, r < ncl ? r : 0);
-    auto push = [&](int slot, int x, int y) {
-        double a0 = 0.0, b0 = 0.0, c0 = 0.0, a1 = 0.0, b1 = 0.0, c1 = 0.0;
+    // (quantity k of a pair: z_x . z_x, z_y . z_y, z_x . z_y -- a warp each, on sub-partitions
+    // of their own: one issues an FP64 instruction every 64 cycles)
+    auto push = [&](int k, int slot, int x, int y) {
+        double s0 = 0.0, s1 = 0.0;
         if (x < pk && y < pk) {
-            const double *zx = M + x * ldm, *zy = M + y * ldm;
+            const double *zx = M + (k == 1 ? y : x) * ldm, *zy = M + (k == 0 ? x : y) * ldm;
             int i = 0;
             for (; i + 1 < pn; i += 2) {
-                const double u = zx[i], v = zy[i], u1 = zx[i + 1], v1 = zy[i + 1];
-                a0 = fma(u, u, a0);
-                b0 = fma(v, v, b0);
-                c0 = fma(u, v, c0);
-                a1 = fma(u1, u1, a1);
-                b1 = fma(v1, v1, b1);
-                c1 = fma(u1, v1, c1);
+                s0 = fma(zx[i], zy[i], s0);
+                s1 = fma(zx[i + 1], zy[i + 1], s1);
             }
-            if (i < pn) {
-                a0 = fma(zx[i], zx[i], a0);
-                b0 = fma(zy[i], zy[i], b0);
-                c0 = fma(zx[i], zy[i], c0);
-            }
-            a0 += a1;
-            b0 += b1;
-            c0 += c1;
+            if (i < pn) s0 = fma(zx[i], zy[i], s0);
+            s0 += s1;
         }
-        const int o = par * ncl * 3 * NPR + slot;
+        const int o = (par * ncl * 3 + k) * NPR + slot;
 #pragma unroll
         for (int r = 0; r < SV_MAXCL; ++r)
-            if (r < ncl) {
-                dst[r][o] = a0;
-                dst[r][o + NPR] = b0;
-                dst[r][o + 2 * NPR] = c0;
-            }
+            if (r < ncl) dst[r][o] = s0;
     };
     auto total = [&](int k, int slot) {  // over the CTAs, in a fixed order
         const double *p = part + (par * ncl * 3 + k) * NPR + slot;
@@ -545,16 +538,23 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
         const double lo = (s[0] + s[1]) + (s[2] + s[3]);
         return ncl <= 4 ? lo : lo + ((s[4] + s[5]) + (s[6] + s[7]));
     };
-    // a round's pair of this thread: slot t pairs the players at places t and n - 1 - t
-    // of a circle; player 0 stays, the others move one place a round
-    int px = threadIdx.x < npairs ? (int)threadIdx.x : 0, py = n - 1 - px;
+    // warps 0, 1, 2 (pairs 0..31) and 4, 5, 6 (pairs 32..47) form the quantities 0, 1, 2
+    const int quantity = warp & 3, qslot = lane + (warp >> 2) * 32;
+    const bool qactive = quantity < 3 && qslot < npairs;
+    // a round's pair of slot t: the players at places t and n - 1 - t of a circle; player
+    // 0 stays, the others move one place a round
+    int px = qslot < npairs ? qslot : 0, py = n - 1 - px;
     for (int sweep = 0; sweep < 60 && n > 1; ++sweep) {
         for (int round = 0; round < n - 1; ++round, par ^= 1) {
-            const int slot = threadIdx.x, x = px, y = py;
-            if (slot < npairs) push(slot, x, y);
+            const int slot = qslot, x = px, y = py;
+            if (qactive) push(quantity, slot, x, y);
             cl.sync();
-            if (slot < npairs) {
-                const double a = total(0, slot), b = total(1, slot), c = total(2, slot);
+            if (qactive) s_tot[quantity][slot] = total(quantity, slot);
+            px = px == 0 ? 0 : px + 1 < n ? px + 1 : 1;
+            py = py == 0 ? 0 : py + 1 < n ? py + 1 : 1;
+            __syncthreads();
+            if (quantity == 0 && slot < npairs) {
+                const double a = s_tot[0][slot], b = s_tot[1][slot], c = s_tot[2][slot];
                 double cs = 1.0, sn = 0.0;
                 // (byes have zero sums; NaNs and columns below 2^-511 are left alone)
                 const int eh = max(__double2hiint(a), __double2hiint(b)) & 0x7FF00000;
@@ -592,8 +592,6 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
                 s_sn[slot] = sn;
                 s_uv[slot][0] = x;
                 s_uv[slot][1] = y;
-                px = px == 0 ? 0 : px + 1 < n ? px + 1 : 1;
-                py = py == 0 ? 0 : py + 1 < n ? py + 1 : 1;
             }
             __syncthreads();
             for (int g = lane; g < npairs; g += 32) {
@@ -616,7 +614,7 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     // ---- singular values (the norms of Z's columns), their descending order (ties by
     // index), norm, rank
     for (int t0 = 0; t0 < pk; t0 += NPR, par ^= 1) {  // (as pairs of a column with itself)
-        if (threadIdx.x < NPR && t0 + threadIdx.x < pk) push(threadIdx.x, t0 + threadIdx.x, t0 + threadIdx.x);
+        if (threadIdx.x < NPR && t0 + threadIdx.x < pk) push(0, threadIdx.x, t0 + threadIdx.x, t0 + threadIdx.x);
         cl.sync();
         if (threadIdx.x < NPR && t0 + threadIdx.x < pk) sig[t0 + threadIdx.x] = sqrt(total(0, threadIdx.x));
     }
