@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(r1::NT) k_run1d(const SweepArgs a, double *U, 
     __shared__ double q[2][NF][NT];                  // the CTA's cells, double buffered
     __shared__ double sf[2 * NF][NP];                // split fluxes f(+), then f(-)
     __shared__ double sF[2 * NF][NI];                // WENO values at the interfaces
-    __shared__ unsigned list[ROUGH_CAP];
+    __shared__ unsigned list[2 * NF * NI];
     __shared__ int s_rough, s_bad;
     __shared__ unsigned long long s_max[2][K];       // wavespeed maxima of the state in the same buffer
     __shared__ double s_al[K], s_dt, s_tn;
@@ -109,12 +109,12 @@ __global__ void __launch_bounds__(r1::NT) k_run1d(const SweepArgs a, double *U, 
                     const int fs = u / nseg, j0 = (u - fs * nseg) * len, m = min(len, cnt + 1 - j0);
                     const bool minus = fs >= NF;
                     if (m > 0)
-                        weno5_slide_pair<2>(&sf[0][0], fs * NP + (minus ? j0 + m + 4 : j0), minus ? -1 : 1, P, &sF[0][0],
+                        weno5_slide_pair<2, 0>(&sf[0][0], fs * NP + (minus ? j0 + m + 4 : j0), minus ? -1 : 1, P, &sF[0][0],
                                             fs * NI + (minus ? j0 + m - 1 : j0), minus ? -1 : 1, m, rough);
                 }
             }
             __syncthreads();
-            rough_windows<2>(rough, &sf[0][0], &sF[0][0], P);
+            rough_windows<2, 0>(rough, &sf[0][0], &sF[0][0], P);
             __syncthreads();
             const bool own = tid < cnt;
             if (own) {

@@ -50,8 +50,8 @@ template <int M, int D, int DIR, bool BULK> struct Layout {
     static constexpr int NS = BULK ? 1 : 2;   // face-flux copies: FP64 keeps WENO(+) and WENO(-) apart
     static constexpr int RF = 9;              // faces per FP64 sliding run
     static constexpr size_t ref_off = align16(F_off + sizeof(T) * NS * NF * W * NI);
-    // FP32-bulk: the lines' reference states; FP64: the rough windows' list
-    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * W : sizeof(unsigned) * ROUGH_CAP);
+    // FP32-bulk: the lines' reference states; FP64: the rough windows' list (every window)
+    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * W : sizeof(unsigned) * 2 * NF * W * NI);
     static_assert(2 * NF * W * NP <= 8192 && 2 * NF * W * NI <= 8192, "offsets of a RoughList entry");
 };
 
@@ -65,7 +65,7 @@ __device__ __forceinline__ void split_flux_scalar(double u, double alpha, double
 }
 
 template <int M, int D, int DIR, bool BULK, int EPI>
-__global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
+__global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
 {
     static_assert(M == MODEL_EULER || !BULK, "the FP32-bulk form exists for the Euler equations only");
     using L = Layout<M, D, DIR, BULK>;
@@ -182,10 +182,10 @@ __global__ void __launch_bounds__(NT) k_sweep(const SweepArgs a)
             const int jp = minus ? j0 + cnt + 4 : j0, jo = minus ? j0 + cnt - 1 : j0, st_ = minus ? -pst : pst;
             const int po = fs * W * NP + (DIR == 0 ? w * NP : w) + jp * pst;
             const int oo = fs * W * NI + (DIR == 0 ? w * NI : w) + jo * pst;
-            weno5_slide_pair<W>(sfp, po, st_, P, sF, oo, st_, cnt, rough);
+            weno5_slide_pair<W, 0>(sfp, po, st_, P, sF, oo, st_, cnt, rough);
         }
         __syncthreads();
-        rough_windows<W>(rough, sfp, sF, P);
+        rough_windows<W, 0>(rough, sfp, sF, P);
     } else {
         for (int u = threadIdx.x; u < NF * W * NI; u += NT) {
             const int f = u / (W * NI);

@@ -55,9 +55,11 @@ template <int D, bool BULK> struct Layout {
     static constexpr size_t F_off = 0;                                        // Fx, Fy
     static constexpr size_t fx_off = (sizeof(T) * NS * NF * (NXI + NYI) + 15) & ~size_t(15);
     static constexpr size_t fy_off = fx_off + sizeof(T) * 2 * NF * NXP;
-    // FP32-bulk: the tile's reference state; FP64: the rough windows' list
+    // FP32-bulk: the tile's reference state; FP64: the rough windows' list (every window
+    // of a 2D tile; in 3D as many as let two CTAs share an SM)
+    static constexpr int CAP = D == 2 ? 0 : 1024, LIST = D == 2 ? 2 * NF * (NXI + TX + NYI) : CAP;
     static constexpr size_t ref_off = (fy_off + sizeof(T) * 2 * NF * NYP + 15) & ~size_t(15);
-    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) : sizeof(unsigned) * ROUGH_CAP);
+    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) : sizeof(unsigned) * LIST);
     static_assert(BULK || (2 * NF * (NXP + NYP) <= 8192 && 2 * NF * (NXI + NYI) <= 8192), "offsets of a RoughList entry");
 };
 }  // namespace xy
@@ -68,7 +70,7 @@ template <int D, bool BULK> struct Layout {
 // (stage 1, L(U)) or the stored split of U^n plus Delta_k (stages 2 and 3, the
 // stage state of k_xy2.cu).
 template <int D, bool BULK, int EPI, bool PD, int ST = 0>
-__global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
+__global__ void __launch_bounds__(xy::NT, BULK ? 5 : 2) k_xy(const SweepArgs a)
 {
     using namespace xy;
     using L = Layout<D, BULK>;
@@ -298,10 +300,10 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 1) k_xy(const SweepArgs a)
                 oo += TY * st;
                 st = -st;
             }
-            weno5_slide_pair<TX>(fx, po, st, P, Fx, oo, st, TY + 1, rough);
+            weno5_slide_pair<TX, L::CAP>(fx, po, st, P, Fx, oo, st, TY + 1, rough);
         }
         __syncthreads();
-        rough_windows<TX>(rough, fx, Fx, P);
+        rough_windows<TX, L::CAP>(rough, fx, Fx, P);
     } else {
         // WENO(+) and the mirrored WENO(-) of a face as one f32x2 pair
         auto face_x = [&](int f, int ly, int j) -> T {  // between local columns j-1 and j of row ly

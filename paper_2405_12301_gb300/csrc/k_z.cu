@@ -23,11 +23,11 @@ constexpr int NHALO = 6 * TX;               // 192 halo points
 constexpr int NF = 5;
 constexpr size_t fz_off = sizeof(double) * 2 * NF * NZI;
 constexpr size_t rough_off = fz_off + sizeof(double) * 2 * NF * NZP;
-constexpr size_t bytes = rough_off + sizeof(unsigned) * ROUGH_CAP;
+constexpr size_t bytes = rough_off + sizeof(unsigned) * 2 * NF * NZI;  // (every window)
 }  // namespace zs
 
 template <int EPI, bool PD>
-__global__ void __launch_bounds__(zs::NT) k_z(const SweepArgs a)
+__global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
 {
     using namespace zs;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -112,10 +112,10 @@ __global__ void __launch_bounds__(zs::NT) k_z(const SweepArgs a)
                 oo += TZ * TX;
                 st = -TX;
             }
-            weno5_slide_pair<TX>(fz, po, st, P, Fz, oo, st, TZ + 1, rough);
+            weno5_slide_pair<TX, 0>(fz, po, st, P, Fz, oo, st, TZ + 1, rough);
         }
         __syncthreads();
-        rough_windows<TX>(rough, fz, Fz, P);
+        rough_windows<TX, 0>(rough, fz, Fz, P);
     }
     __syncthreads();
 
