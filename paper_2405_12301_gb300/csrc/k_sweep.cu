@@ -34,8 +34,10 @@ namespace wg {
 
 constexpr int NT = 256;
 
-template <int DIR> struct Tile { static constexpr int W = 32, S = 26; };  // y, z: 32 x-lines, 26 cells
-template <> struct Tile<0> { static constexpr int W = 2, S = 122; };       // x: 2 rows, 122 cells
+// Bounds of a tile: lines, points (lines x (cells + 6 halo points)).  The launch
+// picks the tile within them for the grid (sweep_tile).
+template <int DIR> struct Tile { static constexpr int W = 32, S = 26, P = W * (S + 6); };  // y, z: 32 x-lines, 26 cells
+template <> struct Tile<0> { static constexpr int W = 28, S = 122, P = NT; };               // x: rows, 122 cells
 
 constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
@@ -43,16 +45,17 @@ template <int M> constexpr int nfields(int D) { return M == MODEL_EULER ? D + 2 
 
 template <int M, int D, int DIR, bool BULK> struct Layout {
     using T = typename std::conditional<BULK, float, double>::type;
-    static constexpr int NF = nfields<M>(D), W = Tile<DIR>::W, S = Tile<DIR>::S, NP = S + 6, NI = S + 1;
+    // (interfaces per line and component: cells + 1, fewer than points)
+    static constexpr int NF = nfields<M>(D), MP = Tile<DIR>::P, MI = DIR == 0 ? MP : Tile<DIR>::W * (Tile<DIR>::S + 1);
     static constexpr size_t fp_off = 0;
-    static constexpr size_t fm_off = fp_off + sizeof(T) * NF * W * NP;
-    static constexpr size_t F_off = fm_off + sizeof(T) * NF * W * NP;
+    static constexpr size_t fm_off = fp_off + sizeof(T) * NF * MP;
+    static constexpr size_t F_off = fm_off + sizeof(T) * NF * MP;
     static constexpr int NS = BULK ? 1 : 2;   // face-flux copies: FP64 keeps WENO(+) and WENO(-) apart
     static constexpr int RF = 9;              // faces per FP64 sliding run
-    static constexpr size_t ref_off = align16(F_off + sizeof(T) * NS * NF * W * NI);
+    static constexpr size_t ref_off = align16(F_off + sizeof(T) * NS * NF * MI);
     // FP32-bulk: the lines' reference states; FP64: the rough windows' list (every window)
-    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * W : sizeof(unsigned) * 2 * NF * W * NI);
-    static_assert(2 * NF * W * NP <= 8192 && 2 * NF * W * NI <= 8192, "offsets of a RoughList entry");
+    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * Tile<DIR>::W : sizeof(unsigned) * 2 * NF * MI);
+    static_assert(2 * NF * MP <= 8192 && 2 * NF * MI <= 8192, "offsets of a RoughList entry");
 };
 
 // Split fluxes f(+/-) = (f(u) +/- alpha u) / 2 of a scalar law (Eq. lax-friedrichs).
@@ -70,7 +73,8 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
     static_assert(M == MODEL_EULER || !BULK, "the FP32-bulk form exists for the Euler equations only");
     using L = Layout<M, D, DIR, BULK>;
     using T = typename L::T;
-    constexpr int NF = L::NF, W = L::W, S = L::S, NP = L::NP, NI = L::NI;
+    constexpr int NF = L::NF, MP = L::MP, MI = L::MI;
+    const int W = a.tile_w, S = a.tile_s, NP = S + 6, NI = S + 1;
     extern __shared__ __align__(16) unsigned char smem[];
     T *sfp = reinterpret_cast<T *>(smem + L::fp_off);
     T *sfm = reinterpret_cast<T *>(smem + L::fm_off);
@@ -158,8 +162,8 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
         }
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            sfp[f * W * NP + u] = fpv[f];
-            sfm[f * W * NP + u] = fmv[f];
+            sfp[f * MP + u] = fpv[f];
+            sfm[f * MP + u] = fmv[f];
         }
     }
     __syncthreads();
@@ -170,22 +174,24 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
     const int nfaces = n - c0 + 1 < NI ? n - c0 + 1 : NI;  // none right of the last cell's right face
     if constexpr (!BULK) {
         const PairEps P = pair_eps(eps);
-        constexpr int NSEG = (NI + L::RF - 1) / L::RF;
+        const int nseg = (nfaces + L::RF - 1) / L::RF;
         const int pst = DIR == 0 ? 1 : W;
-        for (int u = threadIdx.x; u < 2 * NF * W * NSEG; u += NT) {
-            const int w = u % W, seg_ = (u / W) % NSEG, fs = u / (W * NSEG);
+        for (int u = threadIdx.x; u < 2 * NF * W * nseg; u += NT) {
+            // neighbouring lanes: segments of a row (x), columns (y, z) -- distinct banks
+            const int q = DIR == 0 ? nseg : W, r = u / q, lo = u - r * q, hi = r % (DIR == 0 ? W : nseg);
+            const int w = DIR == 0 ? hi : lo, seg_ = DIR == 0 ? lo : hi, fs = u / (W * nseg);
             const int j0 = seg_ * L::RF, cnt = nfaces - j0 < L::RF ? nfaces - j0 : L::RF;
             long long base;
-            if (cnt <= 0 || !line(w, base)) continue;
+            if (!line(w, base)) continue;
             const bool minus = fs >= NF;
             // face j: f+ at points j..j+4, f- mirrored at j+5..j+1 (sfm follows sfp)
             const int jp = minus ? j0 + cnt + 4 : j0, jo = minus ? j0 + cnt - 1 : j0, st_ = minus ? -pst : pst;
-            const int po = fs * W * NP + (DIR == 0 ? w * NP : w) + jp * pst;
-            const int oo = fs * W * NI + (DIR == 0 ? w * NI : w) + jo * pst;
-            weno5_slide_pair<W, 0>(sfp, po, st_, P, sF, oo, st_, cnt, rough);
+            const int po = fs * MP + (DIR == 0 ? w * NP : w) + jp * pst;
+            const int oo = fs * MI + (DIR == 0 ? w * NI : w) + jo * pst;
+            weno5_slide_pair<0>(sfp, po, st_, P, sF, oo, st_, cnt, pst, rough);
         }
         __syncthreads();
-        rough_windows<W, 0>(rough, sfp, sF, P);
+        rough_windows<0>(rough, pst, sfp, sF, P);
     } else {
         for (int u = threadIdx.x; u < NF * W * NI; u += NT) {
             const int f = u / (W * NI);
@@ -194,8 +200,8 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
             if (DIR == 0) { w = r / NI; j = r - w * NI; }
             else { j = r / W; w = r - j * W; }
             if (j >= nfaces) continue;
-            const T *P = sfp + f * W * NP;
-            const T *M = sfm + f * W * NP;
+            const T *P = sfp + f * MP;
+            const T *M = sfm + f * MP;
             const int pw = DIR == 0 ? w * NP : w;
             const int ps = DIR == 0 ? 1 : W;
             // interface between local cells j-1 and j: f+ at points j..j+4, f- mirrored at j+5..j+1
@@ -203,7 +209,7 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
                                   P[pw + (j + 4) * ps], eps) +
                          weno5<T>(M[pw + (j + 5) * ps], M[pw + (j + 4) * ps], M[pw + (j + 3) * ps],
                                   M[pw + (j + 2) * ps], M[pw + (j + 1) * ps], eps);
-            sF[f * W * NI + (DIR == 0 ? w * NI + j : j * W + w)] = Fh;
+            sF[f * MI + (DIR == 0 ? w * NI + j : j * W + w)] = Fh;
         }
     }
     __syncthreads();
@@ -233,9 +239,9 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             if constexpr (BULK) {
-                rd[f] = -(sF[f * W * NI + jr] - sF[f * W * NI + jl]) * ih;
+                rd[f] = -(sF[f * MI + jr] - sF[f * MI + jl]) * ih;
             } else {
-                const T *Fp = sF + f * W * NI, *Fm = Fp + NF * W * NI;
+                const T *Fp = sF + f * MI, *Fm = Fp + NF * MI;
                 rd[f] = -((Fp[jr] + Fm[jr]) - (Fp[jl] + Fm[jl])) * ih;
             }
         }
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
                     for (int f = 0; f < NF; ++f) qf[f] = f64_to_f32(out[f]);
                     cmaxf = fmaxf(cmaxf, wavespeed_f32<D>(qf, a.gamma_f, b));
                 } else {  // (one cell per thread: its speed is formed below)
-                    static_assert(M != MODEL_EULER || W * S <= NT, "one cell per thread");
+                    static_assert(M != MODEL_EULER || MP <= NT, "one cell per thread");
 #pragma unroll
                     for (int f = 0; f < NF; ++f) qout[f] = out[f];
                     has = true;
@@ -320,14 +326,36 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
 
 static inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
+// The tile for a grid: segments of equal length (a 128-cell row is 2 x 64, not
+// 122 + 6), columns likewise, rows as many as the points allow; on small grids
+// shorter segments, so that there is a tile for every SM (a row costs 6 halo points
+// per segment, so not below 20 cells).
+template <int DIR> static void sweep_tile(SweepArgs &a)
+{
+    const int n = a.n[DIR];
+    if (DIR == 0) {
+        const long long rows = (long long)a.n[1] * a.n[2];
+        long long most = (n * rows + 4ll * sm_count() - 1) / (4ll * sm_count());
+        most = most < 20 ? 20 : most > Tile<0>::S ? Tile<0>::S : most;
+        a.tile_s = (int)cdiv(n, cdiv(n, most));
+        const int w = Tile<0>::P / (a.tile_s + 6);
+        a.tile_w = w > Tile<0>::W ? Tile<0>::W : w;
+        if (a.tile_w > a.n[1]) a.tile_w = a.n[1];
+    } else {
+        a.tile_s = (int)cdiv(n, cdiv(n, Tile<DIR>::S));
+        a.tile_w = (int)cdiv(a.n[0], cdiv(a.n[0], Tile<DIR>::W));
+    }
+}
+
 template <int M, int D, int DIR, bool BULK, int EPI>
-static cudaError_t launch_t(const SweepArgs &a, cudaStream_t s)
+static cudaError_t launch_t(SweepArgs a, cudaStream_t s)
 {
     using L = Layout<M, D, DIR, BULK>;
+    sweep_tile<DIR>(a);
     dim3 grid;
-    if (DIR == 0) grid = dim3(cdiv(a.n[0], L::S), cdiv(a.n[1], L::W), (unsigned)a.n[2]);
-    else if (DIR == 1) grid = dim3(cdiv(a.n[0], L::W), cdiv(a.n[1], L::S), (unsigned)a.n[2]);
-    else grid = dim3(cdiv(a.n[0], L::W), (unsigned)a.n[1], cdiv(a.n[2], L::S));
+    if (DIR == 0) grid = dim3(cdiv(a.n[0], a.tile_s), cdiv(a.n[1], a.tile_w), (unsigned)a.n[2]);
+    else if (DIR == 1) grid = dim3(cdiv(a.n[0], a.tile_w), cdiv(a.n[1], a.tile_s), (unsigned)a.n[2]);
+    else grid = dim3(cdiv(a.n[0], a.tile_w), (unsigned)a.n[1], cdiv(a.n[2], a.tile_s));
     k_sweep<M, D, DIR, BULK, EPI><<<grid, NT, L::bytes, s>>>(a);
     return cudaGetLastError();
 }

@@ -300,10 +300,10 @@ __global__ void __launch_bounds__(xy::NT, BULK ? 5 : 2) k_xy(const SweepArgs a)
                 oo += TY * st;
                 st = -st;
             }
-            weno5_slide_pair<TX, L::CAP>(fx, po, st, P, Fx, oo, st, TY + 1, rough);
+            weno5_slide_pair<L::CAP>(fx, po, st, P, Fx, oo, st, TY + 1, TX, rough);
         }
         __syncthreads();
-        rough_windows<TX, L::CAP>(rough, fx, Fx, P);
+        rough_windows<L::CAP>(rough, TX, fx, Fx, P);
     } else {
         // WENO(+) and the mirrored WENO(-) of a face as one f32x2 pair
         auto face_x = [&](int f, int ly, int j) -> T {  // between local columns j-1 and j of row ly

@@ -112,10 +112,10 @@ __global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
                 oo += TZ * TX;
                 st = -TX;
             }
-            weno5_slide_pair<TX, 0>(fz, po, st, P, Fz, oo, st, TZ + 1, rough);
+            weno5_slide_pair<0>(fz, po, st, P, Fz, oo, st, TZ + 1, TX, rough);
         }
         __syncthreads();
-        rough_windows<TX, 0>(rough, fz, Fz, P);
+        rough_windows<0>(rough, TX, fz, Fz, P);
     }
     __syncthreads();
 

@@ -625,8 +625,8 @@ struct RoughList {
     unsigned *list;  // shared
 };
 
-template <int S, int CAP>
-__device__ __forceinline__ void rough_windows(const RoughList &L, const double *src, double *dst, const PairEps &P)
+template <int CAP>
+__device__ __forceinline__ void rough_windows(const RoughList &L, int S, const double *src, double *dst, const PairEps &P)
 {
     const int n = CAP == 0 || *L.count < CAP ? *L.count : CAP;
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
@@ -647,9 +647,9 @@ __device__ __forceinline__ void rough_windows(const RoughList &L, const double *
 // reverse order.
 // Offsets are below 2^13 and |s| is 1 or S.  The loop stays rolled: a window is
 // ~280 instructions.
-template <int S, int CAP>
+template <int CAP>
 __device__ __forceinline__ void weno5_slide_pair(const double *src, int po, int s, const PairEps &P, double *dst, int oo,
-                                                 int os, int count, const RoughList &L)
+                                                 int os, int count, int S, const RoughList &L)
 {
     const double *p = src + po;
     double *out = dst + oo;

@@ -44,6 +44,7 @@ struct SweepArgs {
     int slot_in;         // alpha slot used for the splitting
     int slot_out;        // alpha slot the EPI_STAGE epilogue publishes to
     int check_dt;        // skip all work when ctl->dt == 0
+    int tile_w, tile_s;  // k_sweep: lines and cells per line of a tile
     int per_dir;         // LF alpha per direction (alpha_dir slots) instead of one global alpha
 };
 
