@@ -109,12 +109,12 @@ __global__ void __launch_bounds__(r1::NT) k_run1d(const SweepArgs a, double *U, 
                     const int fs = u / nseg, j0 = (u - fs * nseg) * len, m = min(len, cnt + 1 - j0);
                     const bool minus = fs >= NF;
                     if (m > 0)
-                        weno5_slide_pair<0>(&sf[0][0], fs * NP + (minus ? j0 + m + 4 : j0), minus ? -1 : 1, P, &sF[0][0],
+                        weno5_slide_pair(&sf[0][0], fs * NP + (minus ? j0 + m + 4 : j0), minus ? -1 : 1, P, &sF[0][0],
                                             fs * NI + (minus ? j0 + m - 1 : j0), minus ? -1 : 1, m, 1, rough);
                 }
             }
             __syncthreads();
-            rough_windows<0>(rough, 1, &sf[0][0], &sF[0][0], P);
+            rough_windows(rough, 1, &sf[0][0], &sF[0][0], P);
             __syncthreads();
             const bool own = tid < cnt;
             if (own) {

@@ -188,10 +188,10 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
             const int jp = minus ? j0 + cnt + 4 : j0, jo = minus ? j0 + cnt - 1 : j0, st_ = minus ? -pst : pst;
             const int po = fs * MP + (DIR == 0 ? w * NP : w) + jp * pst;
             const int oo = fs * MI + (DIR == 0 ? w * NI : w) + jo * pst;
-            weno5_slide_pair<0>(sfp, po, st_, P, sF, oo, st_, cnt, pst, rough);
+            weno5_slide_pair(sfp, po, st_, P, sF, oo, st_, cnt, pst, rough);
         }
         __syncthreads();
-        rough_windows<0>(rough, pst, sfp, sF, P);
+        rough_windows(rough, pst, sfp, sF, P);
     } else {
         for (int u = threadIdx.x; u < NF * W * NI; u += NT) {
             const int f = u / (W * NI);

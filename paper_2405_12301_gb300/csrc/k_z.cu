@@ -6,33 +6,32 @@
 
 namespace wg {
 
-// A CTA owns 32 x-cells x TZ = 8 z-cells of one y-row, one cell per thread, plus
-// the 3 + 3 halo z-planes of its 32 columns.  Phases: split fluxes of every point
-// (own and one halo point per thread), sliding WENO runs along the columns (one
-// run of 9 faces per column, component and sign), then each cell's flux
-// difference is added to the x+y part left in the accumulator by
-// k_xy<3, ..., EPI_STORE>, and the epilogue writes L(U) or applies the SSP-RK3
-// stage combination and publishes the wavespeed max.
+// A CTA owns at most 16 x-cells x MZ = 10 z-cells of one y-row, one cell per thread,
+// plus the 3 + 3 halo z-planes of its columns; the tile is fitted to the grid as in
+// k_xy64.cu.  Phases: split fluxes of every point, sliding WENO runs along the
+// columns (one per thread: column, component and sign), then each cell's flux
+// difference is added to the x+y part left in the accumulator by k_xy64<3>, and the
+// epilogue writes L(U) or applies the SSP-RK3 stage combination and publishes the
+// wavespeed max.
 namespace zs {
-constexpr int NT = 256;
-constexpr int TX = 32, TZ = 8;
-constexpr int BZ = TZ + 6;                  // column extent with halo
-constexpr int NZP = TX * BZ;                // z-flux points: 32 x 14
-constexpr int NZI = TX * (TZ + 1);          // z interfaces: 32 x 9
-constexpr int NHALO = 6 * TX;               // 192 halo points
+constexpr int MW = 16, MZ = 10;
 constexpr int NF = 5;
+constexpr int NT = 2 * NF * MW;             // a run per thread
+constexpr int NZP = MW * (MZ + 6);          // z-flux points
+constexpr int NZI = MW * (MZ + 1);          // z interfaces
 constexpr size_t fz_off = sizeof(double) * 2 * NF * NZI;
 constexpr size_t rough_off = fz_off + sizeof(double) * 2 * NF * NZP;
 constexpr size_t bytes = rough_off + sizeof(unsigned) * 2 * NF * NZI;  // (every window)
+static_assert(MW * MZ <= NT && 2 * NF * NZP <= 8192, "one cell per thread; offsets of a RoughList entry");
 }  // namespace zs
 
 template <int EPI, bool PD>
-__global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
+__global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
 {
     using namespace zs;
     extern __shared__ __align__(16) unsigned char smem[];
-    double *Fz = reinterpret_cast<double *>(smem);           // [2][NF][TZ+1][TX]
-    double *fz = reinterpret_cast<double *>(smem + fz_off);  // [2][NF][BZ][TX]
+    double *Fz = reinterpret_cast<double *>(smem);           // [2][NF][MZ+1][MW]
+    double *fz = reinterpret_cast<double *>(smem + fz_off);  // [2][NF][MZ+6][MW]
     __shared__ int s_rough;
     const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(smem + rough_off)};
     if (threadIdx.x == 0) s_rough = 0;
@@ -46,28 +45,27 @@ __global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
     const long long N = a.N, sz = a.stride[2];
     // z-tiles are the fastest grid index, so that tiles sharing halo planes run
     // close together and find those planes in L2
-    const int x0 = blockIdx.y * TX, z0 = blockIdx.x * TZ;
-    const long long yoff = (long long)blockIdx.z * a.stride[1];
-    const int tx = threadIdx.x & 31, tz = threadIdx.x >> 5;
-    const int gx = x0 + tx, gz = z0 + tz;
-    const bool own = gx < nx && gz < nz;
-    const long long cell = yoff + (long long)(gz < nz ? gz : nz - 1) * sz + (gx < nx ? gx : nx - 1);
+    const int zt = (nz + a.tile_s - 1) / a.tile_s, xt = blockIdx.x / zt;
+    const int x0 = xt * a.tile_w, z0 = (blockIdx.x - xt * zt) * a.tile_s;
+    const int W = min(a.tile_w, nx - x0), H = min(a.tile_s, nz - z0);
+    const long long yoff = (long long)blockIdx.y * a.stride[1];
+    const int tid = threadIdx.x, tz = tid / W, tx = tid - tz * W;
+    const bool own = tz < H;
+    const long long cell = yoff + (long long)(z0 + tz) * sz + (x0 + tx);
 
     double un[NF];
-    if (EPI == EPI_STAGE && a.stage > 0) {
+    if (EPI == EPI_STAGE && a.stage > 0 && own) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) un[f] = __ldg(a.Un + f * N + cell);
     }
     const double gm1 = a.gamma - 1.0;
-    const bool interior = z0 >= 3 && z0 + TZ + 3 <= nz && x0 + TX <= nx;
+    const bool interior = z0 >= 3 && z0 + H + 3 <= nz;
 
     auto load_point = [&](int lx, int lz, double *q) {
-        int cx = x0 + lx, cz = z0 + lz;
+        int cz = z0 + lz;
         bool fz_ = false;
         if (!interior) {
             int inz;
-            cx = cx < nx ? cx : nx - 1;  // columns beyond the grid only feed cells that are not written
-            cz = cz < nz + 2 ? cz : nz + 2;
             cz = ghost_map(cz, nz, a.bc[2][0], a.bc[2][1], fz_, inz);
             if (inz >= 0) {  // a ghost of an inflow side holds the given state
 #pragma unroll
@@ -75,7 +73,7 @@ __global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
                 return;
             }
         }
-        const double *src = a.U + yoff + (long long)cz * sz + cx;
+        const double *src = a.U + yoff + (long long)cz * sz + (x0 + lx);
 #pragma unroll
         for (int f = 0; f < NF; ++f) q[f] = __ldg(src + f * N);
         if (fz_) q[3] = -q[3];
@@ -83,7 +81,7 @@ __global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
     auto flux_store = [&](const double *q, int lx, int lz) {
         double fp[NF], fm[NF];
         split_flux_f64<3, 2, true>(q, alpha, gm1, fp, fm);
-        const int o = (lz + 3) * TX + lx;
+        const int o = (lz + 3) * MW + lx;
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             fz[f * NZP + o] = fp[f];
@@ -91,69 +89,58 @@ __global__ void __launch_bounds__(zs::NT, 3) k_z(const SweepArgs a)
         }
     };
 
+    // the halo's 6 W points are dealt from the last thread down
     double uk[NF], qd[NF];
-    load_point(tx, tz, uk);
-    const bool halo = threadIdx.x < NHALO;
-    const int hx = threadIdx.x & 31, hz = (threadIdx.x >> 5) < 3 ? (threadIdx.x >> 5) - 3 : TZ + (threadIdx.x >> 5) - 3;
-    if (halo) load_point(hx, hz, qd);
-    flux_store(uk, tx, tz);
-    if (halo) flux_store(qd, hx, hz);
+    if (own) load_point(tx, tz, uk);
+    const int t = NT - 1 - tid, hk = t / W, hx = t - hk * W, hz = hk < 3 ? hk - 3 : H + hk - 3;
+    if (hk < 6) load_point(hx, hz, qd);
+    if (own) flux_store(uk, tx, tz);
+    if (hk < 6) flux_store(qd, hx, hz);
     __syncthreads();
 
     {
         // the shared arrays hold 2 f(+/-): reconstruct with 4 eps (twice the WENO5 value)
         const PairEps P = pair_eps(4.0 * a.eps);
-#pragma unroll 1
-        for (int run = threadIdx.x; run < 2 * NF * TX; run += NT) {
-            const int fs = run >> 5, lx = run & 31;
-            int po = fs * NZP + lx, oo = fs * NZI + lx, st = TX;
+        const int fs = tid / W, lx = tid - fs * W;
+        if (fs < 2 * NF) {
+            int po = fs * NZP + lx, oo = fs * NZI + lx, st = MW;
             if (fs >= NF) {  // WENO(-): the same run read backwards from the far end
-                po += (TZ + 5) * TX;
-                oo += TZ * TX;
-                st = -TX;
+                po += (H + 5) * MW;
+                oo += H * MW;
+                st = -MW;
             }
-            weno5_slide_pair<0>(fz, po, st, P, Fz, oo, st, TZ + 1, TX, rough);
+            weno5_slide_pair(fz, po, st, P, Fz, oo, st, H + 1, MW, rough);
         }
         __syncthreads();
-        rough_windows<0>(rough, TX, fz, Fz, P);
+        rough_windows(rough, MW, fz, Fz, P);
     }
     __syncthreads();
 
     const double ihz = 0.5 * a.inv_h[2];  // face fluxes are twice F^
     const double *acc = reinterpret_cast<const double *>(a.acc);
     const double *FzM = Fz + NF * NZI;
-    double r[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const int o = f * NZI + tz * TX + tx;
-        const double dz = (Fz[o + TX] + FzM[o + TX]) - (Fz[o] + FzM[o]);
-        r[f] = acc[f * N + cell] + (-dz * ihz);
-    }
-    if (EPI == EPI_RHS) {
-        if (own) {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) a.Rout[f * N + cell] = r[f];
-        }
-        return;
-    }
     double out[NF];
     if (own) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            out[f] = stage_combine(a.stage, un[f], uk[f], r[f], dt);
-            a.Uout[f * N + cell] = out[f];
+            const int o = f * NZI + tz * MW + tx;
+            const double dz = (Fz[o + MW] + FzM[o + MW]) - (Fz[o] + FzM[o]);
+            const double r = acc[f * N + cell] + (-dz * ihz);
+            if (EPI == EPI_RHS) a.Rout[f * N + cell] = r;
+            else a.Uout[f * N + cell] = out[f] = stage_combine(a.stage, un[f], uk[f], r, dt);
         }
     }
-    speed_max_publish_f64<3, PD ? 4 : 1>(
-        [&](long long, double *q) {
+    if constexpr (EPI == EPI_STAGE)
+        speed_max_publish_f64<3, PD ? 4 : 1>(
+            [&](long long, double *q) {
 #pragma unroll
-            for (int f = 0; f < NF; ++f) q[f] = out[f];
-        },
-        0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
+                for (int f = 0; f < NF; ++f) q[f] = out[f];
+            },
+            0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
 }
 
 template <int EPI, bool PD>
-static cudaError_t launch_z_t(const SweepArgs &a, cudaStream_t s)
+static cudaError_t launch_z_t(SweepArgs a, cudaStream_t s)
 {
     static bool attr = false;
     if (!attr) {
@@ -161,7 +148,14 @@ static cudaError_t launch_z_t(const SweepArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    dim3 grid((unsigned)((a.n[2] + zs::TZ - 1) / zs::TZ), (unsigned)((a.n[0] + zs::TX - 1) / zs::TX), (unsigned)a.n[1]);
+    a.tile_w = fit_extent(a.n[0], zs::MW);
+    const long long gx = (a.n[0] + a.tile_w - 1) / a.tile_w;
+    const int w = a.tile_w;
+    // FP64 instructions of a tile: ~62 for a cell's flux and update, ~22 for a halo
+    // point's flux, ~8 for a window
+    a.tile_s = fit_tile(a.n[2], zs::MZ, gx * a.n[1],
+                        [&](int h) { return 62.0 * w * h + 132.0 * w + 16.0 * zs::NF * w * (h + 1); });
+    dim3 grid((unsigned)(gx * ((a.n[2] + a.tile_s - 1) / a.tile_s)), (unsigned)a.n[1]);
     k_z<EPI, PD><<<grid, zs::NT, zs::bytes, s>>>(a);
     return cudaGetLastError();
 }

@@ -1,5 +1,5 @@
 // k_z2.cu -- the z direction of the 3D FP32-bulk residual, in pair-difference
-// form, ending the stage (the x and y directions run in k_xy<3> and leave their
+// form, ending the stage (the x and y directions run in k_xy and leave their
 // part in the FP32 accumulator).
 //
 // As in k_xy2 (2D), WENO5-JS needs a stencil only through its first

@@ -275,9 +275,9 @@ static int enqueue_sweeps(weno_ctx *h, SweepArgs a, int last, cudaStream_t s)
         CK(h, launch(h, 3, s, [&] { return launch_sweep(MODEL_EULER, 1, 0, bulk(h), last, a, s); }));
     } else if (h->dim == 2) {
         if (bulk(h)) CK(h, launch(h, 4, s, [&] { return launch_xy2(last, a, s); }));
-        else CK(h, launch(h, 4, s, [&] { return launch_xy(2, false, last, a, s); }));
+        else CK(h, launch(h, 4, s, [&] { return launch_xy64(2, last, a, s); }));
     } else {
-        CK(h, launch(h, 2, s, [&] { return launch_xy(3, bulk(h), EPI_STORE, a, s); }));
+        CK(h, launch(h, 2, s, [&] { return bulk(h) ? launch_xy(a, s) : launch_xy64(3, EPI_STORE, a, s); }));
         if (bulk(h)) CK(h, launch(h, 5, s, [&] { return launch_z2(last, a, s); }));
         else CK(h, launch(h, 5, s, [&] { return launch_z(last, a, s); }));
     }

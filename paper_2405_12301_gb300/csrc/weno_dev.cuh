@@ -618,17 +618,15 @@ __device__ __forceinline__ double weno5_pair(double a, double b, double c, doubl
 // after the runs: taking weno5_rough inside a run would cost the whole warp
 // whenever one lane needs it.  An entry is the offset of the
 // window's first point, the offset of its value, and which of the strides
-// +-1, +-S its points have.  CAP: entries of the list; 0 if every window of the
-// block fits, else what does not fit is evaluated in place.
+// +-1, +-S its points have; the list holds every window of the block.
 struct RoughList {
     int *count;      // shared, zeroed before a barrier that precedes the runs
     unsigned *list;  // shared
 };
 
-template <int CAP>
 __device__ __forceinline__ void rough_windows(const RoughList &L, int S, const double *src, double *dst, const PairEps &P)
 {
-    const int n = CAP == 0 || *L.count < CAP ? *L.count : CAP;
+    const int n = *L.count;
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
         const unsigned w = L.list[e];
         const int s = (w >> 26 & 1u ? S : 1) * (w >> 27 & 1u ? -1 : 1);
@@ -647,7 +645,6 @@ __device__ __forceinline__ void rough_windows(const RoughList &L, int S, const d
 // reverse order.
 // Offsets are below 2^13 and |s| is 1 or S.  The loop stays rolled: a window is
 // ~280 instructions.
-template <int CAP>
 __device__ __forceinline__ void weno5_slide_pair(const double *src, int po, int s, const PairEps &P, double *dst, int oo,
                                                  int os, int count, int S, const RoughList &L)
 {
@@ -671,13 +668,7 @@ __device__ __forceinline__ void weno5_slide_pair(const double *src, int po, int 
         if (!rough) {
             *out = v;
         } else {
-            const int k = atomicAdd(L.count, 1);
-            if (CAP == 0 || k < CAP) {
-                L.list[k] = (unsigned)(p - 4 * s - src) | (unsigned)(out - dst) << 13 | kind;
-            } else {
-                const double b = p[-3 * s];
-                *out = weno5_diffs(b - p[-4 * s], D2, D3, D4, c, P.eps);
-            }
+            L.list[atomicAdd(L.count, 1)] = (unsigned)(p - 4 * s - src) | (unsigned)(out - dst) << 13 | kind;
         }
         out += os;
         D2 = D3;

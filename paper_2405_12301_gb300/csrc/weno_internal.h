@@ -44,7 +44,7 @@ struct SweepArgs {
     int slot_in;         // alpha slot used for the splitting
     int slot_out;        // alpha slot the EPI_STAGE epilogue publishes to
     int check_dt;        // skip all work when ctl->dt == 0
-    int tile_w, tile_s;  // k_sweep: lines and cells per line of a tile
+    int tile_w, tile_s;  // the FP64 kernels and k_sweep: extents of a tile, chosen at the launch
     int per_dir;         // LF alpha per direction (alpha_dir slots) instead of one global alpha
 };
 
@@ -55,8 +55,10 @@ cudaError_t sweep_set_attributes();
 // must be in slot 0 (k_run1d.cu).
 bool run1d_takes(long long n);
 cudaError_t launch_run1d(const SweepArgs &a, double *U, int nsteps, cudaStream_t s);
-// Fused x+y residual of a 2D grid (EPI_RHS / EPI_STAGE) or of the z-planes of a 3D grid (EPI_STORE).
-cudaError_t launch_xy(int dim, bool bulk, int epi, const SweepArgs &a, cudaStream_t s);
+// Fused FP64 x+y residual of a 2D grid (EPI_RHS / EPI_STAGE) or of the z-planes of a 3D grid (EPI_STORE).
+cudaError_t launch_xy64(int dim, int epi, const SweepArgs &a, cudaStream_t s);
+// Fused FP32-bulk x+y residual of the z-planes of a 3D grid, left in the accumulator.
+cudaError_t launch_xy(const SweepArgs &a, cudaStream_t s);
 // 2D FP32-bulk residual / stage in pair-difference form (EPI_RHS / EPI_STAGE).
 cudaError_t launch_xy2(int epi, const SweepArgs &a, cudaStream_t s);
 // z direction of a 3D FP64 grid, adding the accumulator and ending the residual (EPI_RHS / EPI_STAGE).
@@ -76,5 +78,33 @@ int sums_blocks(long long N);
 // Number of SMs of the current device (queried once per device; persistent and
 // grid-stride launches are sized from it).
 int sm_count();
+
+// Tiles of equal extent along n cells: the smallest extent that needs no more tiles
+// than `most` does (97 cells in tiles of at most 16: 7 x 14, not 6 x 16 + 1).
+inline int fit_extent(long long n, int most)
+{
+    const long long t = (n + most - 1) / most;
+    return (int)((n + t - 1) / t);
+}
+
+// The extent (2 .. most) along n cells whose fullest SM has least to do, with `others`
+// tiles across and cost(h) the work of a tile of extent h: large tiles share more of
+// their halo, but 512 tiles on 152 SMs keep a sixth of them idle.
+template <class Cost> int fit_tile(long long n, int most, long long others, Cost cost)
+{
+    int best = fit_extent(n, most);
+    double least = -1.0;
+    for (int h = most; h >= 2; --h) {
+        const int f = fit_extent(n, h);
+        const long long t = (n + f - 1) / f;
+        if (least >= 0.0 && t > 65535) break;  // (a grid dimension)
+        const double c = (double)((t * others + sm_count() - 1) / sm_count()) * cost(f);
+        if (least < 0.0 || c < least) {
+            least = c;
+            best = f;
+        }
+    }
+    return best;
+}
 
 }  // namespace wg
