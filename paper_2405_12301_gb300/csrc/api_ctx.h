@@ -30,6 +30,7 @@ struct weno_ctx {
     double *S1 = nullptr, *S2 = nullptr, *Udev = nullptr;
     void *acc = nullptr;
     double *partials = nullptr, *sums_dev = nullptr;
+    wg::Tile64 txy{}, tz{};     // tiles of the FP64 2D and 3D kernels
     double *bcs_dev = nullptr;  // weno_params.bc_state in device memory
     int nblocks_sum = 0;
     wg::Ctl *ctl = nullptr;

@@ -15,49 +15,48 @@
 //      or applies the SSP-RK3 stage combination (Eq. tt-ssprk3 without rounding)
 //      and publishes the wavespeed max of the new state.
 //
-// The FP64 pipe bounds it, so what a tile computes for nobody costs time: the tile
-// is fitted to the grid (tiles of equal size, none beyond the grid's edge; on grids
-// of a few tiles per SM the height whose fullest SM has least to do), and small
-// tiles, 4 (3D planes: 3) to an SM, even out rough and smooth ones.
+// The FP64 pipe bounds it (an SM issues one FP64 warp instruction per ~20 cycles,
+// however many lanes are active), so what a tile computes for nobody costs time.
+// The tile's extents are fitted to the grid (plan_xy64): tiles of equal size, none
+// beyond the grid's edge, whose cells, halo points and runs fill their warps and whose
+// number fills the SMs.
+#include <algorithm>
+
 #include "weno_dev.cuh"
 #include "weno_internal.h"
 
 namespace wg {
 
 namespace xy64 {
-constexpr int MW = 16, MH = 8;           // tile bounds
-constexpr int PX = MW + 6;               // row pitch of the x-flux points: 8 rows x 2 runs of a half-warp, distinct banks
-constexpr int NXP = PX * MH;             // x-flux points
-constexpr int NYP = MW * (MH + 6);       // y-flux points (row pitch MW)
-constexpr int PXI = MW + 1;
-constexpr int NXI = PXI * MH;            // x interfaces
-constexpr int NYI = MW * (MH + 1);       // y interfaces
-constexpr int RUN = MH + 1;              // most faces of a run
+constexpr int MW = 32, MH = 16, MNT = 256;  // bounds of a tile's extents and cells (one per thread)
+constexpr int RUN = 9;
 
-// 2 NF MW y runs and 2 NF MH 2 x runs: 2 per thread in 2D (256) and in 3D planes (320)
-template <int D> struct Layout {
-    static constexpr int NF = D + 2, NT = D == 2 ? 128 : 160, CTAS = D == 2 ? 4 : 3;
-    static constexpr size_t fx_off = sizeof(double) * 2 * NF * (NXI + NYI);
-    static constexpr size_t rough_off = fx_off + sizeof(double) * 2 * NF * (NXP + NYP);
-    static constexpr size_t bytes = rough_off + sizeof(unsigned) * 2 * NF * (NXI + NYI);  // (every window)
-    static_assert(2 * NF * (NXP + NYP) <= 8192 && 2 * NF * (NXI + NYI) <= 8192, "offsets of a RoughList entry");
-    static_assert(MW * MH <= NT, "one cell per thread");
+// Sizes of the shared arrays of a w x h tile, in elements per component and sign
+struct Sizes {
+    int px, nxp, nyp, pxi, nxi, nyi;
+    __host__ __device__ Sizes(int w, int h)
+        : px((w + 6) | 1), nxp(px * h), nyp(w * (h + 6)), pxi(w + 1), nxi(pxi * h), nyi(w * (h + 1))
+    {
+    }  // (odd pitch: the rows of neighbouring lanes' x-runs lie in distinct banks)
+    int points() const { return nxp + nyp; }
+    int faces() const { return nxi + nyi; }
 };
 }  // namespace xy64
 
 template <int D, int EPI, bool PD>
-__global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_xy64(const SweepArgs a)
+__global__ void __launch_bounds__(xy64::MNT, 2) k_xy64(const SweepArgs a)
 {
     using namespace xy64;
-    using L = Layout<D>;
-    constexpr int NF = L::NF, NT = L::NT;
+    constexpr int NF = D + 2;
+    const int NT = blockDim.x, TW = a.txy.w;
+    const Sizes Z(TW, a.txy.s);
     extern __shared__ __align__(16) unsigned char smem[];
-    double *Fx = reinterpret_cast<double *>(smem);              // [2][NF][MH][PXI]
-    double *Fy = Fx + 2 * NF * NXI;                             // [2][NF][MH+1][MW]
-    double *fx = reinterpret_cast<double *>(smem + L::fx_off);  // [2][NF][MH][PX]
-    double *fy = fx + 2 * NF * NXP;                             // [2][NF][MH+6][MW]
+    double *Fx = reinterpret_cast<double *>(smem);  // [2][NF][s][w+1]
+    double *Fy = Fx + 2 * NF * Z.nxi;               // [2][NF][s+1][w]
+    double *fx = Fy + 2 * NF * Z.nyi;               // [2][NF][s][px]
+    double *fy = fx + 2 * NF * Z.nxp;               // [2][NF][s+6][w]
     __shared__ int s_rough;
-    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(smem + L::rough_off)};
+    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(fy + 2 * NF * Z.nyp)};
     if (threadIdx.x == 0) s_rough = 0;
 
     const double dt = a.ctl->dt;
@@ -69,8 +68,8 @@ __global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_
 
     const int nx = a.n[0], ny = a.n[1];
     const long long N = a.N;
-    const int x0 = blockIdx.x * a.tile_w, y0 = blockIdx.y * a.tile_s;
-    const int W = min(a.tile_w, nx - x0), H = min(a.tile_s, ny - y0);
+    const int x0 = blockIdx.x * TW, y0 = blockIdx.y * a.txy.s;
+    const int W = min(TW, nx - x0), H = min(a.txy.s, ny - y0);
     const long long zoff = (long long)blockIdx.z * a.stride[2];
     const int tid = threadIdx.x, ty = tid / W, tx = tid - ty * W;
     const bool own = ty < H;
@@ -125,21 +124,21 @@ __global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_
     auto flux_x = [&](const double *q, int lx, int ly) {
         double fp[NF], fm[NF];
         split_flux_f64<D, 0, true>(q, alx, gm1, fp, fm);
-        const int o = ly * PX + lx + 3;
+        const int o = ly * Z.px + lx + 3;
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            fx[f * NXP + o] = fp[f];
-            fx[(NF + f) * NXP + o] = fm[f];
+            fx[f * Z.nxp + o] = fp[f];
+            fx[(NF + f) * Z.nxp + o] = fm[f];
         }
     };
     auto flux_y = [&](const double *q, int lx, int ly) {
         double fp[NF], fm[NF];
         split_flux_f64<D, 1, true>(q, aly, gm1, fp, fm);
-        const int o = (ly + 3) * MW + lx;
+        const int o = (ly + 3) * TW + lx;
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            fy[f * NYP + o] = fp[f];
-            fy[(NF + f) * NYP + o] = fm[f];
+            fy[f * Z.nyp + o] = fp[f];
+            fy[(NF + f) * Z.nyp + o] = fm[f];
         }
     };
 
@@ -171,12 +170,12 @@ __global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_
     }
     __syncthreads();
 
-    // ---- phase W: runs of equal length (H + 1 faces of a column; a row's W + 1 faces
-    // in segments no longer), one code path.  The shared arrays hold 2 f(+/-):
+    // ---- phase W: runs of a column's H + 1 faces and of a row's W + 1 in nseg segments,
+    // one code path.  The shared arrays hold 2 f(+/-):
     // reconstruct with 4 eps (twice the WENO5 value)
     {
         const PairEps P = pair_eps(4.0 * a.eps);
-        const int most = max(H + 1, 4), nseg = (W + most) / most, len = (W + nseg) / nseg;
+        const int nseg = a.txy.nseg, len = (W + nseg) / nseg;
         const int nry = 2 * NF * W, nrx = 2 * NF * nseg * H;
 #pragma unroll 1
         for (int run = tid; run < nry + nrx; run += NT) {
@@ -184,28 +183,29 @@ __global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_
             if (run < nry) {
                 fs = run / W;
                 const int lx = run - fs * W;
-                po = 2 * NF * NXP + fs * NYP + lx;
-                oo = 2 * NF * NXI + fs * NYI + lx;
-                st = MW;
+                po = 2 * NF * Z.nxp + fs * Z.nyp + lx;
+                oo = 2 * NF * Z.nxi + fs * Z.nyi + lx;
+                st = TW;
                 cnt = H + 1;
             } else {
                 const int u = run - nry, r = u / H, ly = u - r * H;
                 fs = r / nseg;
                 const int j0 = (r - fs * nseg) * len;
-                po = fs * NXP + ly * PX + j0;
-                oo = fs * NXI + ly * PXI + j0;
+                po = fs * Z.nxp + ly * Z.px + j0;
+                oo = fs * Z.nxi + ly * Z.pxi + j0;
                 st = 1;
                 cnt = min(len, W + 1 - j0);
+                if (cnt <= 0) continue;
             }
             if (fs >= NF) {  // WENO(-): the same run read backwards from the far end
                 po += (cnt + 4) * st;
                 oo += (cnt - 1) * st;
                 st = -st;
             }
-            weno5_slide_pair(fx, po, st, P, Fx, oo, st, cnt, MW, rough);
+            weno5_slide_pair(fx, po, st, P, Fx, oo, st, cnt, TW, rough);
         }
         __syncthreads();
-        rough_windows(rough, MW, fx, Fx, P);
+        rough_windows(rough, TW, fx, Fx, P);
     }
     __syncthreads();
 
@@ -214,12 +214,12 @@ __global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_
     double out[NF];
     if (own) {
         const double ihx = 0.5 * a.inv_h[0], ihy = 0.5 * a.inv_h[1];
-        const double *FxM = Fx + NF * NXI, *FyM = Fy + NF * NYI;
+        const double *FxM = Fx + NF * Z.nxi, *FyM = Fy + NF * Z.nyi;
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            const int ox = f * NXI + ty * PXI + tx, oy = f * NYI + ty * MW + tx;
+            const int ox = f * Z.nxi + ty * Z.pxi + tx, oy = f * Z.nyi + ty * TW + tx;
             const double dx = (Fx[ox + 1] + FxM[ox + 1]) - (Fx[ox] + FxM[ox]);
-            const double dy = (Fy[oy + MW] + FyM[oy + MW]) - (Fy[oy] + FyM[oy]);
+            const double dy = (Fy[oy + TW] + FyM[oy + TW]) - (Fy[oy] + FyM[oy]);
             const double r = -dx * ihx - dy * ihy;
             if (EPI == EPI_STORE) reinterpret_cast<double *>(a.acc)[f * N + cell] = r;
             else if (EPI == EPI_RHS) a.Rout[f * N + cell] = r;
@@ -235,27 +235,63 @@ __global__ void __launch_bounds__(xy64::Layout<D>::NT, xy64::Layout<D>::CTAS) k_
             0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
 }
 
-template <int D, int EPI, bool PD> static cudaError_t launch_xy64_t(SweepArgs a, cudaStream_t s)
+double tile64_cycles(long long tiles, const Tile64 &t, int regs, int cells, double cell, int halo, int runs, int longest)
+{
+    auto warps = [](int k) { return 4 * ((k + 127) / 128); };
+    const int k = (runs + t.nt - 1) / t.nt;
+    const double work = cell * warps(cells) + 22.0 * warps(halo) + 9.0 * k * (t.nt / 32) * (longest + 1) + 40.0;
+    const long long most = 227 * 1024, per_sm = (tiles + sm_count() - 1) / sm_count();
+    const long long res = std::min(most / (t.smem + 1024), 65536ll / (regs * t.nt));  // resident CTAs
+    if (res < 1) return -1.0;
+    const double rounds = (double)((per_sm + res - 1) / res), lone = 0.25 / (double)std::min(res, per_sm);
+    return std::max(20.0 * work * (double)per_sm, 1000.0 * (k * (longest + 1) + 4) * rounds) * (1.0 + lone);
+}
+
+// Measured at 256 x 256, 12 stages (us): 16 x 16 (the choice) 584, 32 x 7 582, 16 x 7
+// 605, 16 x 8 614, 8 x 16 619, 8 x 8 622, 16 x 4 702; at 97 x 83 x 61, L(U): 11 x 14 578,
+// 25 x 8 (the choice) 592, 25 x 7 599, 16 x 8 of 128 threads 612.  Blocks of 3 or 5 warps
+// are left out: an SM's FP64 units are its four sub-partitions', and such blocks load
+// them unevenly (8 x 8 cells, 64 / 96 / 128 threads: 622 / 737 / 659).
+Tile64 plan_xy64(int dim, const long long n[3])
 {
     using namespace xy64;
-    using L = Layout<D>;
+    const int nf = dim + 2;
+    Tile64 best{};
+    double least = -1.0;
+    for (int mw = (int)std::min(8ll, n[0]); mw <= MW; ++mw)  // (whole sectors)
+        for (int mh = 1; mh <= MH; ++mh)
+            for (int run : {std::max(4, std::min(RUN, mh + 1)), mh + 1})  // (faces of an x-run)
+                for (int nt = 128; nt <= MNT; nt += 128) {
+                    Tile64 t{mw, mh, 0, 0, nt, 0};
+                    if (fit_extent(n[0], mw) != mw || fit_extent(n[1], mh) != mh) break;
+                    const Sizes Z(mw, mh);
+                    t.nseg = (mw + run) / run;
+                    t.len = (mw + t.nseg) / t.nseg;
+                    t.smem = (unsigned)(2 * nf * (8 * Z.points() + 12 * Z.faces()));
+                    const long long gy = (n[1] + mh - 1) / mh, tiles = (n[0] + mw - 1) / mw * gy * n[2];
+                    if (mw * mh > nt || gy > 65535 || 2 * nf * std::max(Z.points(), Z.faces()) > 8192) continue;
+                    const double c = tile64_cycles(tiles, t, 112, mw * mh, dim == 2 ? 75.0 : 85.0, 6 * (mw + mh),
+                                                   2 * nf * (mw + t.nseg * mh), std::max(mh + 1, t.len));
+                    if (c >= 0.0 && (least < 0.0 || c < least)) {
+                        least = c;
+                        best = t;
+                    }
+                }
+    return best;
+}
+
+template <int D, int EPI, bool PD> static cudaError_t launch_xy64_t(const SweepArgs &a, cudaStream_t s)
+{
     static bool attr = false;
     if (!attr) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_xy64<D, EPI, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
+        cudaError_t e = cudaFuncSetAttribute(k_xy64<D, EPI, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    a.tile_w = fit_extent(a.n[0], MW);
-    const long long gx = (a.n[0] + a.tile_w - 1) / a.tile_w;
-    const int w = a.tile_w;
-    // FP64 instructions of a tile: ~75 for a cell's fluxes and update, ~22 for a halo
-    // point's flux, ~8 for a window
-    a.tile_s = fit_tile(a.n[1], MH, gx * a.n[2], [&](int h) {
-        return 75.0 * w * h + 132.0 * (w + h) + 16.0 * L::NF * (w * (h + 1) + h * (w + 1));
-    });
-    dim3 grid((unsigned)gx, (unsigned)((a.n[1] + a.tile_s - 1) / a.tile_s), (unsigned)a.n[2]);
-    k_xy64<D, EPI, PD><<<grid, L::NT, L::bytes, s>>>(a);
+    const Tile64 &t = a.txy;
+    if (t.nt == 0) return cudaErrorInvalidConfiguration;
+    dim3 grid((unsigned)((a.n[0] + t.w - 1) / t.w), (unsigned)((a.n[1] + t.s - 1) / t.s), (unsigned)a.n[2]);
+    k_xy64<D, EPI, PD><<<grid, t.nt, t.smem, s>>>(a);
     return cudaGetLastError();
 }
 

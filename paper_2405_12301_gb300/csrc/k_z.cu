@@ -1,39 +1,34 @@
 // k_z.cu -- z direction of the FP64 WENO5-JS residual for 3D grids, ending the
 // residual of a stage (the x and y directions run in k_xy.cu; FP32-bulk's z
 // direction is k_z2.cu).
+#include <algorithm>
+
 #include "weno_dev.cuh"
 #include "weno_internal.h"
 
 namespace wg {
 
-// A CTA owns at most 16 x-cells x MZ = 10 z-cells of one y-row, one cell per thread,
-// plus the 3 + 3 halo z-planes of its columns; the tile is fitted to the grid as in
-// k_xy64.cu.  Phases: split fluxes of every point, sliding WENO runs along the
-// columns (one per thread: column, component and sign), then each cell's flux
-// difference is added to the x+y part left in the accumulator by k_xy64<3>, and the
-// epilogue writes L(U) or applies the SSP-RK3 stage combination and publishes the
-// wavespeed max.
+// A CTA owns a tile of x- and z-cells of one y-row, one cell per thread, plus the
+// 3 + 3 halo z-planes of its columns; the tile is fitted to the grid as in k_xy64.cu
+// (plan_z).  Phases: split fluxes of every point, sliding WENO runs along the columns
+// (one run per column, component and sign), then each cell's flux difference is added
+// to the x+y part left in the accumulator by k_xy64<3>, and the epilogue writes L(U) or
+// applies the SSP-RK3 stage combination and publishes the wavespeed max.
 namespace zs {
-constexpr int MW = 16, MZ = 10;
+constexpr int MW = 32, MH = 24, MNT = 256;  // bounds of a tile's extents and cells
 constexpr int NF = 5;
-constexpr int NT = 2 * NF * MW;             // a run per thread
-constexpr int NZP = MW * (MZ + 6);          // z-flux points
-constexpr int NZI = MW * (MZ + 1);          // z interfaces
-constexpr size_t fz_off = sizeof(double) * 2 * NF * NZI;
-constexpr size_t rough_off = fz_off + sizeof(double) * 2 * NF * NZP;
-constexpr size_t bytes = rough_off + sizeof(unsigned) * 2 * NF * NZI;  // (every window)
-static_assert(MW * MZ <= NT && 2 * NF * NZP <= 8192, "one cell per thread; offsets of a RoughList entry");
 }  // namespace zs
 
 template <int EPI, bool PD>
-__global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
+__global__ void __launch_bounds__(zs::MNT, 2) k_z(const SweepArgs a)
 {
     using namespace zs;
     extern __shared__ __align__(16) unsigned char smem[];
-    double *Fz = reinterpret_cast<double *>(smem);           // [2][NF][MZ+1][MW]
-    double *fz = reinterpret_cast<double *>(smem + fz_off);  // [2][NF][MZ+6][MW]
+    const int NT = blockDim.x, TW = a.tz.w, NZP = TW * (a.tz.s + 6), NZI = TW * (a.tz.s + 1);
+    double *Fz = reinterpret_cast<double *>(smem);  // [2][NF][s+1][w]
+    double *fz = Fz + 2 * NF * NZI;                 // [2][NF][s+6][w]
     __shared__ int s_rough;
-    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(smem + rough_off)};
+    const RoughList rough{&s_rough, reinterpret_cast<unsigned *>(fz + 2 * NF * NZP)};
     if (threadIdx.x == 0) s_rough = 0;
 
     const double dt = a.ctl->dt;
@@ -45,9 +40,9 @@ __global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
     const long long N = a.N, sz = a.stride[2];
     // z-tiles are the fastest grid index, so that tiles sharing halo planes run
     // close together and find those planes in L2
-    const int zt = (nz + a.tile_s - 1) / a.tile_s, xt = blockIdx.x / zt;
-    const int x0 = xt * a.tile_w, z0 = (blockIdx.x - xt * zt) * a.tile_s;
-    const int W = min(a.tile_w, nx - x0), H = min(a.tile_s, nz - z0);
+    const int zt = (nz + a.tz.s - 1) / a.tz.s, xt = blockIdx.x / zt;
+    const int x0 = xt * TW, z0 = (blockIdx.x - xt * zt) * a.tz.s;
+    const int W = min(TW, nx - x0), H = min(a.tz.s, nz - z0);
     const long long yoff = (long long)blockIdx.y * a.stride[1];
     const int tid = threadIdx.x, tz = tid / W, tx = tid - tz * W;
     const bool own = tz < H;
@@ -81,7 +76,7 @@ __global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
     auto flux_store = [&](const double *q, int lx, int lz) {
         double fp[NF], fm[NF];
         split_flux_f64<3, 2, true>(q, alpha, gm1, fp, fm);
-        const int o = (lz + 3) * MW + lx;
+        const int o = (lz + 3) * TW + lx;
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             fz[f * NZP + o] = fp[f];
@@ -89,7 +84,7 @@ __global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
         }
     };
 
-    // the halo's 6 W points are dealt from the last thread down
+    // the halo's 6 W points (no more than threads) are dealt from the last thread down
     double uk[NF], qd[NF];
     if (own) load_point(tx, tz, uk);
     const int t = NT - 1 - tid, hk = t / W, hx = t - hk * W, hz = hk < 3 ? hk - 3 : H + hk - 3;
@@ -101,18 +96,19 @@ __global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
     {
         // the shared arrays hold 2 f(+/-): reconstruct with 4 eps (twice the WENO5 value)
         const PairEps P = pair_eps(4.0 * a.eps);
-        const int fs = tid / W, lx = tid - fs * W;
-        if (fs < 2 * NF) {
-            int po = fs * NZP + lx, oo = fs * NZI + lx, st = MW;
+#pragma unroll 1
+        for (int run = tid; run < 2 * NF * W; run += NT) {
+            const int fs = run / W, lx = run - fs * W;
+            int po = fs * NZP + lx, oo = fs * NZI + lx, st = TW;
             if (fs >= NF) {  // WENO(-): the same run read backwards from the far end
-                po += (H + 5) * MW;
-                oo += H * MW;
-                st = -MW;
+                po += (H + 5) * TW;
+                oo += H * TW;
+                st = -TW;
             }
-            weno5_slide_pair(fz, po, st, P, Fz, oo, st, H + 1, MW, rough);
+            weno5_slide_pair(fz, po, st, P, Fz, oo, st, H + 1, TW, rough);
         }
         __syncthreads();
-        rough_windows(rough, MW, fz, Fz, P);
+        rough_windows(rough, TW, fz, Fz, P);
     }
     __syncthreads();
 
@@ -123,8 +119,8 @@ __global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
     if (own) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
-            const int o = f * NZI + tz * MW + tx;
-            const double dz = (Fz[o + MW] + FzM[o + MW]) - (Fz[o] + FzM[o]);
+            const int o = f * NZI + tz * TW + tx;
+            const double dz = (Fz[o + TW] + FzM[o + TW]) - (Fz[o] + FzM[o]);
             const double r = acc[f * N + cell] + (-dz * ihz);
             if (EPI == EPI_RHS) a.Rout[f * N + cell] = r;
             else a.Uout[f * N + cell] = out[f] = stage_combine(a.stage, un[f], uk[f], r, dt);
@@ -139,24 +135,43 @@ __global__ void __launch_bounds__(zs::NT, 4) k_z(const SweepArgs a)
             0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
 }
 
+// Measured at 97 x 83 x 61, L(U) (us): 11 x 11 580, 9 x 11 587, 25 x 9 597, 17 x 13 604.
+Tile64 plan_z(const long long n[3])
+{
+    using namespace zs;
+    Tile64 best{};
+    double least = -1.0;
+    for (int mw = (int)std::min(8ll, n[0]); mw <= MW; ++mw)
+        for (int mh = 1; mh <= MH; ++mh)
+            for (int nt = 128; nt <= MNT; nt += 128) {
+                Tile64 t{mw, mh, 0, 0, nt, 0};
+                if (fit_extent(n[0], mw) != mw || fit_extent(n[2], mh) != mh) break;
+                const int points = mw * (mh + 6), faces = mw * (mh + 1);
+                t.smem = (unsigned)(2 * NF * (8 * points + 12 * faces));
+                if (mw * mh > nt || 6 * mw > nt || 2 * NF * points > 8192) continue;
+                const long long tiles = (n[0] + mw - 1) / mw * ((n[2] + mh - 1) / mh) * n[1];
+                const double c = tile64_cycles(tiles, t, 96, mw * mh, 62.0, 6 * mw, 2 * NF * mw, mh + 1);
+                if (c >= 0.0 && (least < 0.0 || c < least)) {
+                    least = c;
+                    best = t;
+                }
+            }
+    return best;
+}
+
 template <int EPI, bool PD>
-static cudaError_t launch_z_t(SweepArgs a, cudaStream_t s)
+static cudaError_t launch_z_t(const SweepArgs &a, cudaStream_t s)
 {
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_z<EPI, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zs::bytes);
+        cudaError_t e = cudaFuncSetAttribute(k_z<EPI, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    a.tile_w = fit_extent(a.n[0], zs::MW);
-    const long long gx = (a.n[0] + a.tile_w - 1) / a.tile_w;
-    const int w = a.tile_w;
-    // FP64 instructions of a tile: ~62 for a cell's flux and update, ~22 for a halo
-    // point's flux, ~8 for a window
-    a.tile_s = fit_tile(a.n[2], zs::MZ, gx * a.n[1],
-                        [&](int h) { return 62.0 * w * h + 132.0 * w + 16.0 * zs::NF * w * (h + 1); });
-    dim3 grid((unsigned)(gx * ((a.n[2] + a.tile_s - 1) / a.tile_s)), (unsigned)a.n[1]);
-    k_z<EPI, PD><<<grid, zs::NT, zs::bytes, s>>>(a);
+    const Tile64 &t = a.tz;
+    if (t.nt == 0) return cudaErrorInvalidConfiguration;
+    const long long gx = (a.n[0] + t.w - 1) / t.w, gz = (a.n[2] + t.s - 1) / t.s;
+    k_z<EPI, PD><<<dim3((unsigned)(gx * gz), (unsigned)a.n[1]), t.nt, t.smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -140,6 +140,10 @@ extern "C" int weno_init(weno_handle *out, const weno_grid *grid, const weno_par
             return fail(nullptr, WENO_ERR_ARG, "weno_init: scalar models need ny <= 131070 (2D)");
         }
     }
+    if (h->dim >= 2 && p.precision != WENO_FP32_BULK && p.model == WENO_MODEL_EULER) {
+        h->txy = plan_xy64(h->dim, h->n);
+        if (h->dim == 3) h->tz = plan_z(h->n);
+    }
     static bool attrs = false;
     if (!attrs) {
         cudaError_t e = sweep_set_attributes();
@@ -254,6 +258,8 @@ static SweepArgs base_args(weno_ctx *h)
     }
     a.acc = h->acc;
     a.bcs = h->bcs_dev;
+    a.txy = h->txy;
+    a.tz = h->tz;
     // a scalar law has one wavespeed |f'(u)| for every direction
     a.per_dir = h->p.alpha_mode == WENO_ALPHA_PER_DIR && h->p.model == WENO_MODEL_EULER ? 1 : 0;
     return a;

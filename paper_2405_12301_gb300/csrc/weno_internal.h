@@ -12,6 +12,13 @@ enum Epi { EPI_STORE = 0, EPI_ADD = 1, EPI_RHS = 2, EPI_STAGE = 3 };
 // Conservation law: Euler (nf = dim + 2), scalar advection or Burgers (nf = 1).
 enum Model { MODEL_EULER = 0, MODEL_ADVECT = 1, MODEL_BURGERS = 2 };
 
+// A tile of the FP64 2D and 3D kernels: w x s cells, nseg x-runs of at most len
+// faces per row (k_xy64), nt threads (0: no tile planned), its shared memory.
+struct Tile64 {
+    int w, s, nseg, len, nt;
+    unsigned smem;
+};
+
 struct SweepArgs {
     const double *U;     // stencil state U^(k) (device, FP64 SoA)
     const double *Un;    // U^n, read by the stage-2/3 combination
@@ -44,7 +51,8 @@ struct SweepArgs {
     int slot_in;         // alpha slot used for the splitting
     int slot_out;        // alpha slot the EPI_STAGE epilogue publishes to
     int check_dt;        // skip all work when ctl->dt == 0
-    int tile_w, tile_s;  // the FP64 kernels and k_sweep: extents of a tile, chosen at the launch
+    int tile_w, tile_s;  // k_sweep: lines and cells per line of a tile, chosen at the launch
+    Tile64 txy, tz;      // k_xy64, k_z: the handle's tiles
     int per_dir;         // LF alpha per direction (alpha_dir slots) instead of one global alpha
 };
 
@@ -80,31 +88,20 @@ int sums_blocks(long long N);
 int sm_count();
 
 // Tiles of equal extent along n cells: the smallest extent that needs no more tiles
-// than `most` does (97 cells in tiles of at most 16: 7 x 14, not 6 x 16 + 1).
+// than `most` does (97 cells in tiles of at most 32: 4 x 25, not 3 x 32 + 1).
 inline int fit_extent(long long n, int most)
 {
     const long long t = (n + most - 1) / most;
     return (int)((n + t - 1) / t);
 }
 
-// The extent (2 .. most) along n cells whose fullest SM has least to do, with `others`
-// tiles across and cost(h) the work of a tile of extent h: large tiles share more of
-// their halo, but 512 tiles on 152 SMs keep a sixth of them idle.
-template <class Cost> int fit_tile(long long n, int most, long long others, Cost cost)
-{
-    int best = fit_extent(n, most);
-    double least = -1.0;
-    for (int h = most; h >= 2; --h) {
-        const int f = fit_extent(n, h);
-        const long long t = (n + f - 1) / f;
-        if (least >= 0.0 && t > 65535) break;  // (a grid dimension)
-        const double c = (double)((t * others + sm_count() - 1) / sm_count()) * cost(f);
-        if (least < 0.0 || c < least) {
-            least = c;
-            best = f;
-        }
-    }
-    return best;
-}
+// Cycles of the fullest SM of a launch over Tile64 t: FP64 warp instructions at 20
+// cycles each -- `cell` for 32 cells' fluxes and update, ~22 for 32 halo points' flux,
+// ~9 for a round of windows, a phase's warps filling all four sub-partitions -- but no
+// less than the chains of windows (~1000 cycles each) that its rounds of CTAs wait for,
+// and more where few CTAs share the SM, whose phases leave it waiting.
+double tile64_cycles(long long tiles, const Tile64 &t, int regs, int cells, double cell, int halo, int runs, int longest);
+Tile64 plan_xy64(int dim, const long long n[3]);
+Tile64 plan_z(const long long n[3]);
 
 }  // namespace wg
