@@ -400,6 +400,41 @@ __device__ __forceinline__ double f32_to_f64_nz(float f)
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+// FP32 triples (about 70 bits) for what pairs do not hold.
+struct Tri {
+    float a, b, c;
+};
+// All 53 bits of |x| in [2^-79, 2^64): split_sat, then the 6 bits it drops.
+__device__ __forceinline__ Tri tr_split(double x)
+{
+    const float2 p = split_sat(x);
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), mag = h & 0x7FFFFFFFu;
+    const unsigned eb = ((mag >> 20) - 942u) << 23;  // exponent field of 2^(e - 1069): the 6 bits are worth 2^(e - 1075)
+    const float v = __uint_as_float((eb & 0x7F800000u) | ((l & 63u) << 17)) - __uint_as_float(eb & 0x7F800000u);
+    const bool ok = mag - (944u << 20) < ((1087u - 944u) << 20);
+    return Tri{p.x, p.y, ok ? __uint_as_float(__float_as_uint(v) | (h & 0x80000000u)) : 0.0f};
+}
+// x - y of two split doubles as a pair, exact to the pair's last bit (the FP64
+// difference would cost the pipe that bounds its callers ~80 issue slots, this ~35).
+__device__ __forceinline__ float2 tr_diff(Tri x, Tri y)
+{
+    const float2 h = two_sum(x.a, -y.a), l = two_sum(x.b, -y.b), m = two_sum(h.y, l.x), n = two_sum(h.x, m.x);
+    return two_sum(n.x, __fadd_rn(n.y, __fadd_rn(m.y, __fadd_rn(l.y, __fsub_rn(x.c, y.c)))));
+}
+
+// a + b + c in FP64 for a normal a (zero becomes 2^-127) and |b + c| within an ulp of
+// a: b and c are integers in units of the result's last place, so no FP64 sum.
+__device__ __forceinline__ double pr_f64(float a, float b, float c)
+{
+    const unsigned u = __float_as_uint(a);
+    const float s = __uint_as_float(0x7F000000u - (u & 0x7F800000u));  // 2^-exponent
+    int k = __float2int_rn(__fmul_rn(__fmul_rn(b, 0x1p52f), s)) + __float2int_rn(__fmul_rn(__fmul_rn(c, 0x1p52f), s));
+    k = (int)u < 0 ? -k : k;
+    if (k < 0 && (u & 0x7FFFFFu) == 0u) k += k;  // below a power of two the places are half as large
+    const long long v = ((long long)(((u & 0x7FFFFFFFu) >> 3) + 0x38000000u) << 32 | (u << 29)) + k;
+    return __hiloint2double((int)((unsigned)(v >> 32) | (u & 0x80000000u)), (int)v);
+}
+
 // 1 / x of a normal x below 2^1021: an FP32 reciprocal of the mantissa, two
 // Newton-Raphson steps r (2 - x r) (4 FP64 instructions; a division takes ~9).
 // Within an ulp: the last step's error term is exact to 2^-44.
@@ -497,8 +532,7 @@ __device__ __forceinline__ double weno5_pair_core(double D2, double D3, double c
     rough = (emh > P.thr && emh > ch - (7 << 20)) || (unsigned)(ch - 1) < (953u << 20) ||  // 0 < |c| < 2^-70
             !(mn > 0x1p-80f) || !(sum < 0x1p100f) || !(sum * sc < 0x1p66f);
     const float2 x = pr_norm(pr_add(p0, p2));
-    const double X = (fma(2.0, D3, D2) + f32_to_f64_nz(x.y)) + f32_to_f64_nz(x.x);
-    return fma(X, 1.0 / 6.0, c);
+    return fma(fma(2.0, D3, D2) + pr_f64(x.x, x.y, 0.0f), 1.0 / 6.0, c);
 }
 
 // ---- the same in FP32 triples a + b + c (about 70 bits), for windows whose X is not
@@ -506,9 +540,6 @@ __device__ __forceinline__ double weno5_pair_core(double D2, double D3, double c
 // leading parts, the last part in plain FP32 (triple-word arithmetic after Fabiano,
 // Joldes, Muller and Popescu 2019, without their final renormalisations where a
 // sum of positive terms follows).
-struct Tri {
-    float a, b, c;
-};
 __device__ __forceinline__ Tri tr_norm(Tri x)
 {
     const float2 s = two_sum(x.b, x.c), t = two_sum(x.a, s.x), u = two_sum(t.y, s.y);
@@ -541,16 +572,6 @@ __device__ __forceinline__ Tri tr_mulc(float k, Tri x)  // an FP32 factor
     const float p = __fmul_rn(k, x.a), e = __fmaf_rn(k, x.a, -p), q = __fmul_rn(k, x.b), qe = __fmaf_rn(k, x.b, -q);
     const float2 m = two_sum(e, q);
     return Tri{p, m.x, __fadd_rn(m.y, __fmaf_rn(k, x.c, qe))};
-}
-// All 53 bits of |x| in [2^-79, 2^64): split_sat, then the 6 bits it drops.
-__device__ __forceinline__ Tri tr_split(double x)
-{
-    const float2 p = split_sat(x);
-    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), mag = h & 0x7FFFFFFFu;
-    const unsigned eb = ((mag >> 20) - 942u) << 23;  // exponent field of 2^(e - 1069): the 6 bits are worth 2^(e - 1075)
-    const float v = __uint_as_float((eb & 0x7F800000u) | ((l & 63u) << 17)) - __uint_as_float(eb & 0x7F800000u);
-    const bool ok = mag - (944u << 20) < ((1087u - 944u) << 20);
-    return Tri{p.x, p.y, ok ? __uint_as_float(__float_as_uint(v) | (h & 0x80000000u)) : 0.0f};
 }
 // w / s for s normalised: three quotient words, each from the exact remainder
 __device__ __forceinline__ Tri tr_div(Tri w, Tri s, float r)
@@ -598,8 +619,7 @@ static __device__ __noinline__ double weno5_rough(double v0, double v1, double v
     const float r = fast_rcp(sw.a);
     const Tri e0 = tr_norm(tr_add(t1, tr_pow2(t0, -1.0f))), ep = tr_norm(tr_add(t2, tr_pow2(t1, -1.0f)));
     const Tri X = tr_norm(tr_add(tr_mul(tr_div(w0, sw, r), e0), tr_pow2(tr_mul(tr_div(w2, sw, r), ep), 2.0f)));
-    const double x = ((fma(2.0, D3, D2) + f32_to_f64_nz(X.c)) + f32_to_f64_nz(X.b)) + f32_to_f64_nz(X.a);
-    return fma(x, 1.0 / 6.0, v2);
+    return fma(fma(2.0, D3, D2) + pr_f64(X.a, X.b, X.c), 1.0 / 6.0, v2);
 }
 
 // One window from its five points (a rough one in place, in FP64: without a call the
@@ -654,17 +674,19 @@ __device__ __forceinline__ void weno5_slide_pair(const double *src, int po, int 
     const double v0 = *p, v1 = *(p += s);
     double c = *(p += s), d = *(p += s);
     double D2 = c - v1, D3 = d - c;
-    float2 f2 = split_sat(D2), f3 = split_sat(D3);
-    float2 u1 = split_sat(D3 - D2), u2 = split_sat(D2 - (v1 - v0));
+    Tri f2 = tr_split(D2), f3 = tr_split(D3);
+    float2 u1 = tr_diff(f3, f2), u2 = tr_diff(f2, tr_split(v1 - v0));
     float2 A1 = pair_t2(u1, P.g), A2 = pair_t2(u2, P.g), ep = pr_sub(u2, u1);
 #pragma unroll 1
     for (int m = 0; m < count; ++m) {
         const double e = *(p += s);
         const double D4 = e - d;
-        const float2 f4 = split_sat(D4), u0 = split_sat(D4 - D3);
+        const Tri f4 = tr_split(D4);
+        const float2 u0 = tr_diff(f4, f3);
         const float2 A0 = pair_t2(u0, P.g), e0 = pr_sub(u1, u0);
         bool rough;
-        const double v = weno5_pair_core(D2, D3, c, f2, f3, u0, u2, A0, A1, A2, e0, ep, P, rough);
+        const double v = weno5_pair_core(D2, D3, c, make_float2(f2.a, f2.b), make_float2(f3.a, f3.b), u0, u2, A0,
+                                         A1, A2, e0, ep, P, rough);
         if (!rough) {
             *out = v;
         } else {
