@@ -36,8 +36,10 @@ constexpr int NT = 256;
 
 // Bounds of a tile: lines, points (lines x (cells + 6 halo points)).  The launch
 // picks the tile within them for the grid (sweep_tile).
-template <int DIR> struct Tile { static constexpr int W = 32, S = 26, P = W * (S + 6); };  // y, z: 32 x-lines, 26 cells
-template <> struct Tile<0> { static constexpr int W = 28, S = 122, P = NT; };               // x: rows, 122 cells
+template <int M, int DIR> struct Tile { static constexpr int W = 32, S = 26, P = W * (S + 6); };  // y, z: 32 x-lines, 26 cells
+template <int M> struct Tile<M, 0> {  // x: rows; a scalar's runs need 1024 points to fill the warps
+    static constexpr int W = 32, S = M == MODEL_EULER ? 122 : 250, P = M == MODEL_EULER ? NT : 1024;
+};
 
 constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
@@ -46,7 +48,7 @@ template <int M> constexpr int nfields(int D) { return M == MODEL_EULER ? D + 2 
 template <int M, int D, int DIR, bool BULK> struct Layout {
     using T = typename std::conditional<BULK, float, double>::type;
     // (interfaces per line and component: cells + 1, fewer than points)
-    static constexpr int NF = nfields<M>(D), MP = Tile<DIR>::P, MI = DIR == 0 ? MP : Tile<DIR>::W * (Tile<DIR>::S + 1);
+    static constexpr int NF = nfields<M>(D), MP = Tile<M, DIR>::P, MI = DIR == 0 ? MP : Tile<M, DIR>::W * (Tile<M, DIR>::S + 1);
     static constexpr size_t fp_off = 0;
     static constexpr size_t fm_off = fp_off + sizeof(T) * NF * MP;
     static constexpr size_t F_off = fm_off + sizeof(T) * NF * MP;
@@ -54,7 +56,7 @@ template <int M, int D, int DIR, bool BULK> struct Layout {
     static constexpr int RF = 9;              // faces per FP64 sliding run
     static constexpr size_t ref_off = align16(F_off + sizeof(T) * NS * NF * MI);
     // FP32-bulk: the lines' reference states; FP64: the rough windows' list (every window)
-    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * Tile<DIR>::W : sizeof(unsigned) * 2 * NF * MI);
+    static constexpr size_t bytes = ref_off + (BULK ? sizeof(RefState<D>) * Tile<M, DIR>::W : sizeof(unsigned) * 2 * NF * MI);
     static_assert(2 * NF * MP <= 8192 && 2 * NF * MI <= 8192, "offsets of a RoughList entry");
 };
 
@@ -326,24 +328,27 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
 
 static inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) / b); }
 
-// The tile for a grid: segments of equal length (a 128-cell row is 2 x 64, not
-// 122 + 6), columns likewise, rows as many as the points allow; on small grids
-// shorter segments, so that there is a tile for every SM (a row costs 6 halo points
-// per segment, so not below 20 cells).
-template <int DIR> static void sweep_tile(SweepArgs &a)
+// The tile for a grid: segments of equal length (a 150-cell row is 2 x 75, not
+// 122 + 28), columns likewise; rows as many as the points allow while there are two
+// tiles for every SM, and on small grids shorter segments for the same reason (a row
+// costs 6 halo points per segment, so not below 20 cells).  Advection at 128^3, x:
+// 7 rows of 128 cells (210 runs, the warps full); 3 rows of 64 (48 runs) took 164 us.
+template <int M, int DIR> static void sweep_tile(SweepArgs &a)
 {
     const int n = a.n[DIR];
     if (DIR == 0) {
         const long long rows = (long long)a.n[1] * a.n[2];
         long long most = (n * rows + 4ll * sm_count() - 1) / (4ll * sm_count());
-        most = most < 20 ? 20 : most > Tile<0>::S ? Tile<0>::S : most;
+        most = most < 20 ? 20 : most > Tile<M, 0>::S ? Tile<M, 0>::S : most;
         a.tile_s = (int)cdiv(n, cdiv(n, most));
-        const int w = Tile<0>::P / (a.tile_s + 6);
-        a.tile_w = w > Tile<0>::W ? Tile<0>::W : w;
-        if (a.tile_w > a.n[1]) a.tile_w = a.n[1];
+        long long w = Tile<M, 0>::P / (a.tile_s + 6), share = rows * cdiv(n, a.tile_s) / (2ll * sm_count());
+        share = share < 2 ? 2 : share;  // (2 rows keep the grid's y extent in range)
+        w = w > Tile<M, 0>::W ? Tile<M, 0>::W : w;
+        w = w > share ? share : w;
+        a.tile_w = fit_extent(a.n[1], (int)w);
     } else {
-        a.tile_s = (int)cdiv(n, cdiv(n, Tile<DIR>::S));
-        a.tile_w = (int)cdiv(a.n[0], cdiv(a.n[0], Tile<DIR>::W));
+        a.tile_s = (int)cdiv(n, cdiv(n, Tile<M, DIR>::S));
+        a.tile_w = (int)cdiv(a.n[0], cdiv(a.n[0], Tile<M, DIR>::W));
     }
 }
 
@@ -351,7 +356,7 @@ template <int M, int D, int DIR, bool BULK, int EPI>
 static cudaError_t launch_t(SweepArgs a, cudaStream_t s)
 {
     using L = Layout<M, D, DIR, BULK>;
-    sweep_tile<DIR>(a);
+    sweep_tile<M, DIR>(a);
     dim3 grid;
     if (DIR == 0) grid = dim3(cdiv(a.n[0], a.tile_s), cdiv(a.n[1], a.tile_w), (unsigned)a.n[2]);
     else if (DIR == 1) grid = dim3(cdiv(a.n[0], a.tile_w), cdiv(a.n[1], a.tile_s), (unsigned)a.n[2]);
