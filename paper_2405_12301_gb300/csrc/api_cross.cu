@@ -66,7 +66,9 @@ static int cross_prepare(weno_ctx *h, const weno_tt_instance *inst, int32_t n_in
         c.fd = F.flux_dir;
         c.n_mode = P.ci[F.instance].n[F.mode];
         const CrossInst &ci = P.ci[F.instance];
-        c.r_mode = (F.mode == 0 ? 1 : ci.r[F.mode - 1]) * (F.mode == 2 ? 1 : ci.r[F.mode]);
+        const int rl = F.mode == 0 ? 1 : ci.r[F.mode - 1], rr = F.mode == 2 ? 1 : ci.r[F.mode];
+        c.r_mode = rl * rr;
+        c.r_row = F.flux_dir > F.mode ? rr : rl;
         c.n_left = F.n_left;
         c.n_right = F.n_right;
         c.left = F.left;

@@ -19,6 +19,7 @@ struct CrossSet {
     int inst, mode, fd;
     int n_mode;
     int r_mode;            // entries of a core row's matrix, r_{mode-1} r_mode
+    int r_row;             // entries of a contracted row
     long long n_left, n_right;
     const int *left;
     const int *right;
