@@ -252,7 +252,8 @@ __global__ void __launch_bounds__(z2::NT, 5) k_z2(const SweepArgs a)
 
     // ---- phase W: warps 0-3 run (rho, m_x) / (m_y, m_z) of column `lane`,
     // pair w & 1, sign w >> 1; warp 4 runs E of column pair lane & 15, sign
-    // lane >> 4 (a runtime stride: both signs share the warp).  Cell c's output
+    // lane >> 4 (a runtime stride, one code path: as two the warp took twice its
+    // neighbours' time and the block waited for it).  Cell c's output
     // goes to index c + 4 (WENO(+)) or c + 1 (WENO(-)); Geps = eps / 4 on
     // differences scaled by 1/4 (as in k_xy2).
     {
@@ -266,8 +267,8 @@ __global__ void __launch_bounds__(z2::NT, 5) k_z2(const SweepArgs a)
         } else if (w == 4) {
             const int sg = lane >> 4, cp = lane & 15, st = sg ? -(TX / 2) : TX / 2;
             float2 *p = reinterpret_cast<float2 *>(De + sg * NDE) + cp;
-            if (sg) weno5d_cells2<TZ + 1, false>(p + 12 * (TX / 2), st, Geps, p + TZ * (TX / 2), st);
-            else weno5d_cells2<TZ + 1, true>(p, st, Geps, p + 4 * (TX / 2), st);
+            // (a run read backwards leaves the negative: phase C subtracts it)
+            weno5d_cells2<TZ + 1, true>(p + (sg ? 12 * (TX / 2) : 0), st, Geps, p + (sg ? TZ : 4) * (TX / 2), st);
         }
     }
     __syncthreads();
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(z2::NT, 5) k_z2(const SweepArgs a)
             r[2 * pr] = rz.x;
             r[2 * pr + 1] = rz.y;
         }
-        const float se = __fadd_rn(De[c + 4 * TX], De[NDE + c + TX]);
+        const float se = __fsub_rn(De[c + 4 * TX], De[NDE + c + TX]);
         r[4] = __fmaf_rn(se, ih.x, __fmul_rn(se, ih.y));
     }
     if (own) {
