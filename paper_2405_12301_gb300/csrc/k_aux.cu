@@ -2,30 +2,77 @@
 // wavespeed max (LF alpha, Sec. 4.3), the device-side time-step control
 // (dt = lambda h / alpha with the last step shortened to land on t_end,
 // Eq. cfl-other), and the fixed-order FP64 conservation sums.
+#include <climits>
+
 #include "weno_dev.cuh"
 #include "weno_internal.h"
 
 namespace wg {
 
+// Start of a step: dt from alpha(U^n) (or the fixed dt), shortened so that the
+// time lands exactly on t_end; zero when the time is up or the step budget of
+// the current call is spent.  Clears the stage alpha slots 1..3.
+__device__ void step_begin(Ctl *c)
+{
+    double dt, tn;
+    if (next_dt(c->t, c->t_end, c->dt_req, c->cfl_h, __longlong_as_double((long long)c->alpha[0]), c->steps,
+                c->max_steps, dt, tn))
+        atomicOr(&c->status, ST_NONPHYSICAL);
+    c->dt = dt;
+    c->t_next = tn;
+    c->bdt[0] = f64_to_f32x2(dt);
+    c->bdt[1] = f64_to_f32x2(0.25 * dt);
+    c->bdt[2] = f64_to_f32x2(2.0 / 3.0 * dt);
+    for (int k = 1; k < 4; ++k) {
+        c->alpha[k] = 0ull;
+        for (int e = 0; e < 3; ++e) c->alpha_dir[k][e] = 0ull;
+    }
+}
+
+// The end of every block of an alpha kernel; the last block's takes the maxima to slot
+// 0, clears them for the next launch and does what follows -- launches of one thread
+// each (clear, set the run, begin, copy out) before.
+__device__ void alpha_done(Ctl *c, const AlphaThen &then)
+{
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&c->ticket, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    c->ticket = 0u;
+    c->alpha[0] = atomicExch(&c->alpha_new[0], 0ull);
+    for (int e = 0; e < 3; ++e) c->alpha_dir[0][e] = atomicExch(&c->alpha_new[1 + e], 0ull);
+    if (then.out) *then.out = __longlong_as_double((long long)c->alpha[0]);
+    if (then.set_run) {
+        c->t_end = then.t_end;
+        c->dt_req = then.dt_req;
+        c->cfl_h = then.cfl_h;
+        c->max_steps = (then.max_steps > LLONG_MAX - c->steps) ? LLONG_MAX : c->steps + then.max_steps;
+    }
+    if (then.begin) step_begin(c);
+}
+
 // alpha of an FP64 state (PD: and the per-direction speeds).  Bound by the FP64
 // pipe if every cell's speed is formed there (84% busy at 97 x 83 x 61); the FP32
 // estimates leave it a handful of cells per block.
 template <int D, bool PD>
-__global__ void __launch_bounds__(256) k_alpha(const double *__restrict__ U, long long N, double gamma, Ctl *ctl, int slot)
+__global__ void __launch_bounds__(256) k_alpha(const double *__restrict__ U, long long N, double gamma, Ctl *ctl,
+                                               const AlphaThen then)
 {
     speed_max_publish_f64<D, PD ? 1 + D : 1>(
         [&](long long i, double *q) {
 #pragma unroll
             for (int f = 0; f < D + 2; ++f) q[f] = __ldg(U + f * N + i);
         },
-        (long long)blockIdx.x * blockDim.x + threadIdx.x, N, (long long)gridDim.x * blockDim.x, gamma, &ctl->alpha[slot],
-        ctl->alpha_dir[slot], &ctl->status);
+        (long long)blockIdx.x * blockDim.x + threadIdx.x, N, (long long)gridDim.x * blockDim.x, gamma, &ctl->alpha_new[0],
+        &ctl->alpha_new[1], &ctl->status);
+    alpha_done(ctl, then);
 }
 
 // The same for the FP32-bulk mode: FP32 speeds, their maximum widened exactly.
 template <int D>
 __global__ void __launch_bounds__(256) k_alpha_bulk(const double *__restrict__ U, long long N, double gamma, Ctl *ctl,
-                                                    int slot, int per_dir)
+                                                    int per_dir, const AlphaThen then)
 {
     constexpr int NF = D + 2;
     float mf = 0.0f, mdf[D];
@@ -46,16 +93,17 @@ __global__ void __launch_bounds__(256) k_alpha_bulk(const double *__restrict__ U
         }
         bad |= b;
     }
-    block_max_publish_f32(mf, bad, &ctl->alpha[slot], &ctl->status);
+    block_max_publish_f32(mf, bad, &ctl->alpha_new[0], &ctl->status);
     if (per_dir) {
 #pragma unroll
-        for (int e = 0; e < D; ++e) block_max_publish_f32(mdf[e], false, &ctl->alpha_dir[slot][e], &ctl->status);
+        for (int e = 0; e < D; ++e) block_max_publish_f32(mdf[e], false, &ctl->alpha_new[1 + e], &ctl->status);
     }
+    alpha_done(ctl, then);
 }
 
 // Scalar laws: alpha = max |f'(u)| (1 for advection, |u| for Burgers).
 template <int M>
-__global__ void __launch_bounds__(256) k_alpha_scalar(const double *__restrict__ U, long long N, Ctl *ctl, int slot)
+__global__ void __launch_bounds__(256) k_alpha_scalar(const double *__restrict__ U, long long N, Ctl *ctl, const AlphaThen then)
 {
     double m = 0.0;
     bool bad = false;
@@ -64,42 +112,13 @@ __global__ void __launch_bounds__(256) k_alpha_scalar(const double *__restrict__
         bad |= !isfinite(u);
         m = fmax(m, M == MODEL_ADVECT ? 1.0 : fabs(u));
     }
-    block_max_publish(m, bad, &ctl->alpha[slot], &ctl->status);
+    block_max_publish(m, bad, &ctl->alpha_new[0], &ctl->status);
+    alpha_done(ctl, then);
 }
 
-__global__ void k_reset_slot(Ctl *ctl, int slot)
-{
-    ctl->alpha[slot] = 0ull;
-    for (int e = 0; e < 3; ++e) ctl->alpha_dir[slot][e] = 0ull;
-}
-
-__global__ void k_copy_alpha(const Ctl *ctl, int slot, double *out)
-{
-    out[0] = __longlong_as_double((long long)ctl->alpha[slot]);
-}
-
-// Start of a step: dt from alpha(U^n) (or the fixed dt), shortened so that the
-// time lands exactly on t_end; zero when the time is up or the step budget of
-// the current call is spent.  Clears the stage alpha slots 1..3.
-__global__ void k_step_begin(Ctl *c)
-{
-    double dt, tn;
-    if (next_dt(c->t, c->t_end, c->dt_req, c->cfl_h, __longlong_as_double((long long)c->alpha[0]), c->steps,
-                c->max_steps, dt, tn))
-        atomicOr(&c->status, ST_NONPHYSICAL);
-    c->dt = dt;
-    c->t_next = tn;
-    c->bdt[0] = f64_to_f32x2(dt);
-    c->bdt[1] = f64_to_f32x2(0.25 * dt);
-    c->bdt[2] = f64_to_f32x2(2.0 / 3.0 * dt);
-    for (int k = 1; k < 4; ++k) {
-        c->alpha[k] = 0ull;
-        for (int e = 0; e < 3; ++e) c->alpha_dir[k][e] = 0ull;
-    }
-}
-
-// End of a step: advance the time and carry alpha(U^{n+1}) into slot 0.
-__global__ void k_step_end(Ctl *c)
+// End of a step: advance the time and carry alpha(U^{n+1}) into slot 0; within a run
+// also the start of the next.
+__global__ void k_step_end(Ctl *c, int begin)
 {
     if (c->dt > 0.0) {
         c->t = c->t_next;
@@ -107,6 +126,7 @@ __global__ void k_step_end(Ctl *c)
         c->alpha[0] = c->alpha[3];
         for (int e = 0; e < 3; ++e) c->alpha_dir[0][e] = c->alpha_dir[3][e];
     }
+    if (begin) step_begin(c);
 }
 
 // Two-level fixed-order sums: block b reduces a fixed contiguous chunk of
@@ -180,44 +200,26 @@ int sm_count()
 }
 
 cudaError_t launch_alpha(int model, int dim, bool bulk, const double *U, long long N, double gamma, Ctl *ctl,
-                         int slot, int per_dir, cudaStream_t s)
+                         int per_dir, const AlphaThen &then, cudaStream_t s)
 {
     int blocks = (int)((N + 255) / 256);
     if (blocks > sm_count() * 8) blocks = sm_count() * 8;
     if (blocks < 1) blocks = 1;
-    if (model == MODEL_ADVECT) k_alpha_scalar<MODEL_ADVECT><<<blocks, 256, 0, s>>>(U, N, ctl, slot);
-    if (model == MODEL_BURGERS) k_alpha_scalar<MODEL_BURGERS><<<blocks, 256, 0, s>>>(U, N, ctl, slot);
+    if (model == MODEL_ADVECT) k_alpha_scalar<MODEL_ADVECT><<<blocks, 256, 0, s>>>(U, N, ctl, then);
+    if (model == MODEL_BURGERS) k_alpha_scalar<MODEL_BURGERS><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model != MODEL_EULER) return cudaGetLastError();
 #define X(D)                                                                                        \
-    if (dim == D && bulk) k_alpha_bulk<D><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, slot, per_dir);     \
-    else if (dim == D && per_dir) k_alpha<D, true><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, slot);     \
-    else if (dim == D) k_alpha<D, false><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, slot);
+    if (dim == D && bulk) k_alpha_bulk<D><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, per_dir, then);     \
+    else if (dim == D && per_dir) k_alpha<D, true><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, then);     \
+    else if (dim == D) k_alpha<D, false><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, then);
     X(1) X(2) X(3)
 #undef X
     return cudaGetLastError();
 }
 
-cudaError_t launch_reset_slot(Ctl *ctl, int slot, cudaStream_t s)
+cudaError_t launch_step_end(Ctl *ctl, bool begin, cudaStream_t s)
 {
-    k_reset_slot<<<1, 1, 0, s>>>(ctl, slot);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_copy_alpha(const Ctl *ctl, int slot, double *out, cudaStream_t s)
-{
-    k_copy_alpha<<<1, 1, 0, s>>>(ctl, slot, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_step_begin(Ctl *ctl, cudaStream_t s)
-{
-    k_step_begin<<<1, 1, 0, s>>>(ctl);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_step_end(Ctl *ctl, cudaStream_t s)
-{
-    k_step_end<<<1, 1, 0, s>>>(ctl);
+    k_step_end<<<1, 1, 0, s>>>(ctl, begin ? 1 : 0);
     return cudaGetLastError();
 }
 

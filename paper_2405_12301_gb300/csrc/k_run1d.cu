@@ -12,7 +12,7 @@
 //   256 cells, 64 steps: 2.36 ms as five kernels per step, 1.14 ms here.
 // Up to 2048 cells (256 per CTA, one cell per thread); larger grids have more
 // FP64 work than 8 SMs do in the time of the launches saved.
-// The arithmetic is that of k_sweep, k_step_begin and k_step_end, bit for bit.
+// The arithmetic is that of k_sweep and of the step control (k_aux.cu), bit for bit.
 #include <cooperative_groups.h>
 
 #include "weno_dev.cuh"

@@ -33,16 +33,6 @@ int wg::fail(weno_ctx *h, int code, const std::string &msg)
     return code;
 }
 
-
-
-__global__ static void k_set_run(Ctl *c, double t_end, double dt_req, double cfl_h, long long max_steps)
-{
-    c->t_end = t_end;
-    c->dt_req = dt_req;
-    c->cfl_h = cfl_h;
-    c->max_steps = (max_steps > LLONG_MAX - c->steps) ? LLONG_MAX : c->steps + max_steps;
-}
-
 __global__ static void k_set_time(Ctl *c, double t)
 {
     c->t = t;
@@ -290,22 +280,21 @@ static int enqueue_sweeps(weno_ctx *h, SweepArgs a, int last, cudaStream_t s)
     return WENO_OK;
 }
 
-// One SSP-RK3 step (Eq. tt-ssprk3 without rounding) on U in place; alpha(U^n)
-// must be in slot 0.  Capturable: no host synchronisation.
+// One SSP-RK3 step (Eq. tt-ssprk3 without rounding) on U in place, begun already; its
+// end begins the next if `more`.  Capturable: no host synchronisation.
 // small 1D FP64 Euler grids run whole steps inside one kernel
 static bool runs_1d(const weno_ctx *h)
 {
     return h->dim == 1 && !bulk(h) && h->p.model == WENO_MODEL_EULER && run1d_takes(h->n[0]);
 }
 
-static int enqueue_step(weno_ctx *h, double *U, cudaStream_t s)
+static int enqueue_step(weno_ctx *h, double *U, bool more, cudaStream_t s)
 {
     if (runs_1d(h)) {
         const SweepArgs a = base_args(h);
         CK(h, launch(h, 3, s, [&] { return launch_run1d(a, U, 1, s); }));
         return WENO_OK;
     }
-    CK(h, launch(h, 7, s, [&] { return launch_step_begin(h->ctl, s); }));
     double *in[3] = {U, h->S1, h->S2};
     double *outs[3] = {h->S1, h->S2, U};
     // FP32-bulk (2D and 3D) keeps the split of U^n in S1 and the FP32 increments in S2
@@ -333,18 +322,24 @@ static int enqueue_step(weno_ctx *h, double *U, cudaStream_t s)
         int r = enqueue_sweeps(h, a, EPI_STAGE, s);
         if (r) return r;
     }
-    CK(h, launch(h, 7, s, [&] { return launch_step_end(h->ctl, s); }));
+    CK(h, launch(h, 7, s, [&] { return launch_step_end(h->ctl, more, s); }));
     return WENO_OK;
 }
 
-static int enqueue_alpha0(weno_ctx *h, const double *U, cudaStream_t s)
+static int enqueue_alpha0(weno_ctx *h, const double *U, const AlphaThen &then, cudaStream_t s)
 {
-    CK(h, launch(h, 7, s, [&] { return launch_reset_slot(h->ctl, 0, s); }));
     CK(h, launch(h, 6, s, [&] {
-           return launch_alpha(h->p.model, h->dim, bulk(h), U, h->N, h->p.gamma, h->ctl, 0,
-                               h->p.alpha_mode == WENO_ALPHA_PER_DIR && h->p.model == WENO_MODEL_EULER ? 1 : 0, s);
+           return launch_alpha(h->p.model, h->dim, bulk(h), U, h->N, h->p.gamma, h->ctl,
+                               h->p.alpha_mode == WENO_ALPHA_PER_DIR && h->p.model == WENO_MODEL_EULER ? 1 : 0, then, s);
        }));
     return WENO_OK;
+}
+
+// alpha(U), the run's parameters and (unless k_run1d does) the start of its first step
+static int enqueue_start(weno_ctx *h, const double *U, double t_end, double dt, long long max_steps)
+{
+    return enqueue_alpha0(h, U, AlphaThen{nullptr, 1, runs_1d(h) ? 0 : 1, t_end, dt, h->p.cfl * min_h(h), max_steps},
+                          h->stream);
 }
 
 static int read_ctl(weno_ctx *h)
@@ -380,9 +375,7 @@ extern "C" int weno_alpha(weno_handle h, const double *U, double *alpha_dev)
     int r = need_grid(h, "weno_alpha");
     if (r) return r;
     if (!U || !alpha_dev) return fail(h, WENO_ERR_ARG, "weno_alpha: null pointer");
-    if ((r = enqueue_alpha0(h, U, h->stream))) return r;
-    CK(h, launch(h, 7, h->stream, [&] { return launch_copy_alpha(h->ctl, 0, alpha_dev, h->stream); }));
-    return WENO_OK;
+    return enqueue_alpha0(h, U, AlphaThen{alpha_dev}, h->stream);
 }
 
 extern "C" int weno_rhs(weno_handle h, const double *U, double *R, double *alpha_dev)
@@ -391,15 +384,13 @@ extern "C" int weno_rhs(weno_handle h, const double *U, double *R, double *alpha
     if (r) return r;
     if (!U || !R) return fail(h, WENO_ERR_ARG, "weno_rhs: null U or R");
     if (R == U) return fail(h, WENO_ERR_ARG, "weno_rhs: R must not alias U");
-    if ((r = enqueue_alpha0(h, U, h->stream))) return r;
+    if ((r = enqueue_alpha0(h, U, AlphaThen{alpha_dev}, h->stream))) return r;
     SweepArgs a = base_args(h);
     a.U = U;
     a.Rout = R;
     a.slot_in = 0;
     a.check_dt = 0;
-    if ((r = enqueue_sweeps(h, a, EPI_RHS, h->stream))) return r;
-    if (alpha_dev) CK(h, launch(h, 7, h->stream, [&] { return launch_copy_alpha(h->ctl, 0, alpha_dev, h->stream); }));
-    return WENO_OK;
+    return enqueue_sweeps(h, a, EPI_RHS, h->stream);
 }
 
 extern "C" int weno_set_time(weno_handle h, double t)
@@ -427,12 +418,8 @@ extern "C" int weno_ssprk3_step(weno_handle h, double *U, double t_end, double d
     if (r) return r;
     if (!U) return fail(h, WENO_ERR_ARG, "weno_ssprk3_step: null U");
     if (dt <= 0.0 && !(h->p.cfl > 0.0)) return fail(h, WENO_ERR_ARG, "weno_ssprk3_step: dt <= 0 needs cfl > 0");
-    CK(h, launch(h, 7, h->stream, [&] {
-           k_set_run<<<1, 1, 0, h->stream>>>(h->ctl, t_end, dt, h->p.cfl * min_h(h), LLONG_MAX);
-           return cudaGetLastError();
-       }));
-    if ((r = enqueue_alpha0(h, U, h->stream))) return r;
-    return enqueue_step(h, U, h->stream);
+    if ((r = enqueue_start(h, U, t_end, dt, LLONG_MAX))) return r;
+    return enqueue_step(h, U, false, h->stream);
 }
 
 static int ensure_graph(weno_ctx *h, double *U, int steps)
@@ -447,7 +434,7 @@ static int ensure_graph(weno_ctx *h, double *U, int steps)
     h->capturing = true;
     h->g_kernels = 0;
     int r = WENO_OK;
-    for (int k = 0; k < steps && r == WENO_OK; ++k) r = enqueue_step(h, U, h->capture);
+    for (int k = 0; k < steps && r == WENO_OK; ++k) r = enqueue_step(h, U, true, h->capture);
     h->capturing = false;
     cudaError_t e = cudaStreamEndCapture(h->capture, &g);
     if (r) {
@@ -471,11 +458,7 @@ extern "C" int weno_run(weno_handle h, double *U, double t_end, double dt, int64
     if (!U || max_steps < 0) return fail(h, WENO_ERR_ARG, "weno_run: null U or negative max_steps");
     if (dt <= 0.0 && !(h->p.cfl > 0.0)) return fail(h, WENO_ERR_ARG, "weno_run: dt <= 0 needs cfl > 0");
     if (steps_out) *steps_out = 0;
-    CK(h, launch(h, 7, h->stream, [&] {
-           k_set_run<<<1, 1, 0, h->stream>>>(h->ctl, t_end, dt, h->p.cfl * min_h(h), max_steps);
-           return cudaGetLastError();
-       }));
-    if ((r = enqueue_alpha0(h, U, h->stream))) return r;
+    if ((r = enqueue_start(h, U, t_end, dt, max_steps))) return r;
     if ((r = read_ctl(h))) return r;
     const long long s0 = h->ctl_host->steps;
     const int chunk = graph_steps > 0 ? graph_steps : 8;
@@ -492,7 +475,7 @@ extern "C" int weno_run(weno_handle h, double *U, double t_end, double dt, int64
             // plain launches: enqueue no step beyond max_steps
             const long long left = max_steps - (h->ctl_host->steps - s0);
             for (long long k = 0; k < chunk && k < left; ++k)
-                if ((r = enqueue_step(h, U, h->stream))) return r;
+                if ((r = enqueue_step(h, U, true, h->stream))) return r;
         }
         if ((r = read_ctl(h))) return r;
         const Ctl &c = *h->ctl_host;

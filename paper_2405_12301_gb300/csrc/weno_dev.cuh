@@ -33,8 +33,9 @@ struct Ctl {
     long long steps;       // steps taken since the last set_time
     long long max_steps;   // steps bound of the current run call
     int status;            // ST_* bits, latched
-    int pad;
+    unsigned ticket;       // blocks of k_alpha that are done (0 between launches)
     float2 bdt[3];         // b_k dt of stage k (1, 1/4, 2/3) as FP32 pairs hi + lo, set with dt
+    unsigned long long alpha_new[4];  // k_alpha's maxima, all and per direction (0 between launches)
 };
 
 // ----------------------------------------------------------------- conversions

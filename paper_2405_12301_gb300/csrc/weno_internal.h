@@ -74,12 +74,17 @@ cudaError_t launch_z(int epi, const SweepArgs &a, cudaStream_t s);
 // z direction of a 3D FP32-bulk grid in pair-difference form (EPI_RHS / EPI_STAGE).
 cudaError_t launch_z2(int epi, const SweepArgs &a, cudaStream_t s);
 
-cudaError_t launch_alpha(int model, int dim, bool bulk, const double *U, long long N, double gamma, Ctl *ctl, int slot,
-                         int per_dir, cudaStream_t s);
-cudaError_t launch_reset_slot(Ctl *ctl, int slot, cudaStream_t s);
-cudaError_t launch_step_begin(Ctl *ctl, cudaStream_t s);
-cudaError_t launch_step_end(Ctl *ctl, cudaStream_t s);
-cudaError_t launch_copy_alpha(const Ctl *ctl, int slot, double *out, cudaStream_t s);
+// What k_alpha's last block does with alpha(U) besides storing it in slot 0.
+struct AlphaThen {
+    double *out;           // not null: alpha goes there too
+    int set_run, begin;    // set t_end .. max_steps of a run; begin its first step
+    double t_end, dt_req, cfl_h;
+    long long max_steps;
+};
+cudaError_t launch_alpha(int model, int dim, bool bulk, const double *U, long long N, double gamma, Ctl *ctl,
+                         int per_dir, const AlphaThen &then, cudaStream_t s);
+// Ends a step and, if `begin`, begins the next.
+cudaError_t launch_step_end(Ctl *ctl, bool begin, cudaStream_t s);
 cudaError_t launch_sums(const double *U, int nf, long long N, double *partials, int nblocks, double *out,
                         cudaStream_t s);
 int sums_blocks(long long N);
