@@ -26,6 +26,7 @@ struct CrossSet {
     void *out;
     long long work_begin;  // first work item of this set (prefix sum)
     int jb, rows;          // fixed indices and rows of a work item (cross_plan)
+    int njb;               // blocks of jb fixed indices
     int nsl, nsr;          // shifted copies stored per left / right vector (7 or 1)
     long long lvec_off, rvec_off;  // element offsets of the set's vectors in CrossArgs::vecs
 };

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(XT, MINB) k_cross(const CrossArgs A)
         const T ih = (T)(0.5 / in.h[fd]);  // halves the doubled face fluxes
         // the item: rows i0 .. i0 + cn, fixed indices j0 .. j0 + jn
         const int jb = S.jb;
-        const long long njb = (nfix + jb - 1) / jb, w = item - S.work_begin;
+        const long long njb = S.njb, w = item - S.work_begin;
         const int i0 = (int)(w / njb) * S.rows;
         const long long j0 = (w - (w / njb) * njb) * jb;
         const int jn = nfix - j0 < jb ? (int)(nfix - j0) : jb;
@@ -738,8 +738,7 @@ void cross_default(bool fp64, int *variant, int *ctas_per_sm)
 // CTA the rows are halved.
 long long cross_items(const CrossSet &S, int rows)
 {
-    const long long nfix = S.fd > S.mode ? S.n_left : S.n_right;
-    return (nfix + S.jb - 1) / S.jb * ((S.n_mode + rows - 1) / rows);
+    return (long long)S.njb * ((S.n_mode + rows - 1) / rows);
 }
 long long cross_plan(CrossSet *sets, int n_sets, bool fp64, int variant)
 {
@@ -750,6 +749,7 @@ long long cross_plan(CrossSet *sets, int n_sets, bool fp64, int variant)
         const long long nfix = S.fd > S.mode ? S.n_left : S.n_right;
         const int most = S.fd != S.mode ? cross_jb(fp64) : fp64 || S.r_mode < 64 ? 1 : JB1;
         S.jb = (int)((nfix + (nfix + most - 1) / most - 1) / ((nfix + most - 1) / most));  // blocks of equal size
+        S.njb = (int)((nfix + S.jb - 1) / S.jb);
         if (fp64) {
             S.rows = S.fd != S.mode ? chunk / S.jb : chunk;
         } else {

@@ -1,6 +1,6 @@
 // k_maxvol.cu -- batched maxvol (the maximum-volume row selection that picks
 // the cross indices of TT-cross, Sec. 3 "TT-cross Interpolation"), FP64, five
-// launches per batch:
+// launches per batch (three for small matrices):
 //   1. the r pivot rows I of Gaussian elimination with partial pivoting on a
 //      working copy W (largest remaining |W[i][j]| of column j, ties to the
 //      smaller row); the multipliers L[i][j] overwrite column j of W, and the
@@ -31,9 +31,10 @@
 // step t, and the stash lets the owner update the winning row in place while
 // others still read it.  Slices are column-major, so a warp's row-parallel
 // accesses coalesce.
-//   16 matrices of 256..12000 x 4..32: pivot 1.10 -> MVP ms, swaps 1.82 -> MVS ms.
+//   16 matrices of 256..12000 x 4..32: pivot 1.10 -> 0.41 ms, swaps 1.82 -> 0.47 ms.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -350,6 +351,9 @@ __device__ __forceinline__ unsigned pair_low_order(float2 v)  // orders the low 
     return b & 0x80000000u ? ~b : b | 0x80000000u;
 }
 
+// F64: on FP64 values, whose rounding the result keeps: B is written back and phases 4
+// and 5 are left out.
+template <bool F64>
 __global__ void __launch_bounds__(MV_NT) k_maxvol_swap(const MaxvolDesc *descs, double delta, int max_iters, int smem_doubles)
 {
     cg::cluster_group cl = cg::this_cluster();
@@ -358,73 +362,104 @@ __global__ void __launch_bounds__(MV_NT) k_maxvol_swap(const MaxvolDesc *descs, 
     const int n = d.n, r = d.r, ncl = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     int lo, hi;
     row_slice(n, rank, ncl, lo, hi);
+    using V = typename std::conditional<F64, double, float2>::type;
     __shared__ MvStep st;
-    __shared__ float2 s_row[MV_RMAX];
+    __shared__ V s_row[MV_RMAX];
     __shared__ int I[MV_RMAX];
-    extern __shared__ float2 P[];
-    float2 *W = reinterpret_cast<float2 *>(d.W);
+    extern __shared__ double mv_smem[];
+    V *P = reinterpret_cast<V *>(mv_smem), *W = reinterpret_cast<V *>(d.W);
     const int m = hi - lo, cap = min(m, smem_doubles / r);
     for (int j = threadIdx.x; j < r; j += MV_NT) I[j] = d.idx[j];
     for (int e = threadIdx.x; e < m * r; e += MV_NT) {
         const int t = e / r, c = e - t * r;
-        const MvRow<float2> w = mv_row(P, cap, W, n, lo, t);
-        w.p[(long long)c * w.ld] = pr_norm(split_sat(d.B[(long long)lo * r + e]));
+        const MvRow<V> w = mv_row(P, cap, W, n, lo, t);
+        if constexpr (F64) w.p[(long long)c * w.ld] = d.B[(long long)lo * r + e];
+        else w.p[(long long)c * w.ld] = pr_norm(split_sat(d.B[(long long)lo * r + e]));
     }
     __syncthreads();
     // an entry's key: |hi|, then the low part's order; e = i r + c grows per thread,
     // so equal keys keep the first
-    unsigned kh = 0u, kl = 0u;
+    unsigned long long key = 0ull;
     long long be = LLONG_MAX;
-    auto consider = [&](float2 v, long long e) {
-        const unsigned h = __float_as_uint(v.x) & 0x7FFFFFFFu;
-        if (h < kh && be != LLONG_MAX) return;
-        const unsigned l = pair_low_order(v);
-        if (be == LLONG_MAX || h > kh || l > kl) {
-            kh = h;
-            kl = l;
-            be = e;
+    auto consider = [&](V v, long long e) {
+        if constexpr (F64) {
+            const unsigned long long x = absbits(v);
+            if (be == LLONG_MAX || x > key) {
+                key = x;
+                be = e;
+            }
+        } else {
+            const unsigned h = __float_as_uint(v.x) & 0x7FFFFFFFu;
+            if (h < (unsigned)(key >> 32) && be != LLONG_MAX) return;
+            const unsigned long long x = (unsigned long long)h << 32 | pair_low_order(v);
+            if (be == LLONG_MAX || x > key) {
+                key = x;
+                be = e;
+            }
         }
     };
     for (int t = threadIdx.x; t < m; t += MV_NT) {
-        const MvRow<float2> w = mv_row(P, cap, W, n, lo, t);
+        const MvRow<V> w = mv_row(P, cap, W, n, lo, t);
         for (int c = 0; c < r; ++c) consider(w.p[(long long)c * w.ld], (long long)(lo + t) * r + c);
     }
     int it = 0;
     for (; it < max_iters; ++it) {
-        const MvSlot *ws = cluster_argmax(cl, st, it & 1, ncl, (unsigned long long)kh << 32 | kl, be,
+        const MvSlot *ws = cluster_argmax(cl, st, it & 1, ncl, key, be,
                                           [&](MvSlot &s, unsigned long long, long long e) {
             if (e != LLONG_MAX) {
-                const MvRow<float2> w = mv_row(P, cap, W, n, lo, (int)(e / r - lo));
-                for (int c = threadIdx.x; c < r; c += MV_NT) reinterpret_cast<float2 *>(s.row)[c] = w.p[(long long)c * w.ld];
+                const MvRow<V> w = mv_row(P, cap, W, n, lo, (int)(e / r - lo));
+                for (int c = threadIdx.x; c < r; c += MV_NT) reinterpret_cast<V *>(s.row)[c] = w.p[(long long)c * w.ld];
             }
         });
         const long long we = st.win_e;
         const int i0 = (int)(we / r), j0 = (int)(we - (long long)i0 * r);
-        const float2 piv = reinterpret_cast<const float2 *>(ws->row)[j0];
-        if (!(fabs((double)piv.x + (double)piv.y) > 1.0 + delta)) break;  // the same decision everywhere
+        const V piv = reinterpret_cast<const V *>(ws->row)[j0];
+        double pv;
+        if constexpr (F64) pv = piv;
+        else pv = (double)piv.x + (double)piv.y;
+        if (!(fabs(pv) > 1.0 + delta)) break;  // the same decision everywhere
         if (threadIdx.x < r) {  // (row_i0 - e_j0) / piv, one residual correction of an approximate quotient
-            float2 v = reinterpret_cast<const float2 *>(ws->row)[threadIdx.x];
-            if (threadIdx.x == j0) v = pr_norm(pr_sub(v, make_float2(1.0f, 0.0f)));
-            const float q = fast_rcp(piv.x), x = __fmul_rn(v.x, q);
-            const float rem = __fadd_rn(__fmaf_rn(-x, piv.x, v.x), __fmaf_rn(-x, piv.y, v.y));
-            s_row[threadIdx.x] = make_float2(x, __fmul_rn(rem, q));
+            V v = reinterpret_cast<const V *>(ws->row)[threadIdx.x];
+            if constexpr (F64) {
+                s_row[threadIdx.x] = (threadIdx.x == j0 ? v - 1.0 : v) / piv;
+            } else {
+                if (threadIdx.x == j0) v = pr_norm(pr_sub(v, make_float2(1.0f, 0.0f)));
+                const float q = fast_rcp(piv.x), x = __fmul_rn(v.x, q);
+                const float rem = __fadd_rn(__fmaf_rn(-x, piv.x, v.x), __fmaf_rn(-x, piv.y, v.y));
+                s_row[threadIdx.x] = make_float2(x, __fmul_rn(rem, q));
+            }
         }
         if (threadIdx.x == 0) I[j0] = i0;
         __syncthreads();
         // B -= B[:, j0] (row_i0 - e_j0) / piv over the slice, with the next argmax
-        kh = kl = 0u;
+        key = 0ull;
         be = LLONG_MAX;
         for (int t = threadIdx.x; t < m; t += MV_NT) {
-            const MvRow<float2> w = mv_row(P, cap, W, n, lo, t);
-            const float2 f = w.p[(long long)j0 * w.ld];
-            float2 *wc = w.p;
+            const MvRow<V> w = mv_row(P, cap, W, n, lo, t);
+            const V f = w.p[(long long)j0 * w.ld];
+            V *wc = w.p;
             const long long e0 = (long long)(lo + t) * r;
 #pragma unroll 4
             for (int c = 0; c < r; ++c, wc += w.ld) {
-                const float2 v = pr_norm(pr_sub(*wc, pr_mul(f, s_row[c])));
+                V v;
+                if constexpr (F64) v = fma(-f, s_row[c], *wc);
+                else v = pr_norm(pr_sub(*wc, pr_mul(f, s_row[c])));
                 *wc = v;
                 consider(v, e0 + c);
             }
+        }
+    }
+    if (F64 && it > 0) {  // (the rows I exactly the unit vectors)
+        __syncthreads();
+        for (int e = threadIdx.x; e < m * r; e += MV_NT) {
+            const int t = e / r, c = e - t * r;
+            const MvRow<V> w = mv_row(P, cap, W, n, lo, t);
+            if constexpr (F64) d.B[(long long)lo * r + e] = w.p[(long long)c * w.ld];
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < r * r; e += MV_NT) {
+            const int j = e / r, c = e - j * r;
+            if (I[j] >= lo && I[j] < hi) d.B[(long long)I[j] * r + c] = c == j ? 1.0 : 0.0;
         }
     }
     cl.sync();  // no CTA leaves while another may still read its slots
@@ -561,7 +596,8 @@ static cudaError_t maxvol_attributes()
     if (done) return cudaSuccess;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_maxvol_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize, MV_SMEM)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_maxvol_swap, cudaFuncAttributeMaxDynamicSharedMemorySize, MV_SMEM)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_maxvol_swap<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MV_SMEM)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_maxvol_swap<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MV_SMEM)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(k_maxvol_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)sizeof(double) * MV_RMAX * (2 * MV_RMAX + 1))) != cudaSuccess ||
         (e = cudaFuncSetAttribute(k_maxvol_final, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -576,9 +612,11 @@ static int maxvol_cluster_size()
 {
     static int ncl = 0;
     if (ncl) return ncl;
+    if (maxvol_attributes() != cudaSuccess) return 8;
     ncl = 8;
     if (cudaFuncSetAttribute(k_maxvol_pivot, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaFuncSetAttribute(k_maxvol_swap, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaFuncSetAttribute(k_maxvol_swap<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_maxvol_swap<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(16, 1);
         cfg.blockDim = dim3(MV_NT);
@@ -590,14 +628,18 @@ static int maxvol_cluster_size()
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        int c1 = 0, c2 = 0;
+        int c1 = 0, c2 = 0, c3 = 0;
         if (cudaOccupancyMaxActiveClusters(&c1, k_maxvol_pivot, &cfg) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&c2, k_maxvol_swap, &cfg) == cudaSuccess && c1 > 0 && c2 > 0)
+            cudaOccupancyMaxActiveClusters(&c2, k_maxvol_swap<true>, &cfg) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&c3, k_maxvol_swap<false>, &cfg) == cudaSuccess && c1 > 0 && c2 > 0 && c3 > 0)
             ncl = 16;
     }
     cudaGetLastError();  // a refused query leaves no sticky state; clear the last error
     return ncl;
 }
+
+static bool maxvol_in_f64(long long max_nr) { return max_nr <= 4096ll * maxvol_cluster_size(); }
+int maxvol_launches(long long max_nr) { return maxvol_in_f64(max_nr) ? 3 : 5; }
 
 // max_nr: the largest n r of the batch.  Shared memory for a slice: what the
 // largest slice takes, and no more than lets the batch's CTAs run together.
@@ -616,7 +658,12 @@ cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_n
     if (e != cudaSuccess) return e;
     k_maxvol_b<<<dim3(64, n), 256, 0, s>>>(d);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    e = launch_cluster(k_maxvol_swap, ncl, n, smem, s, d, delta, max_iters, doubles);
+    // Small slices swap in FP64: an entry then costs a swap ~14 cycles of 32 lanes more
+    // than in pairs, but the inverse and the final product (18-23 us) fall away; at 4096
+    // entries a CTA that is ~1 us a swap.  A call on 8 matrices of up to 1233 x 9: 176 us in
+    // pairs, 147 in FP64.
+    if (maxvol_in_f64(max_nr)) return launch_cluster(k_maxvol_swap<true>, ncl, n, smem, s, d, delta, max_iters, doubles);
+    e = launch_cluster(k_maxvol_swap<false>, ncl, n, smem, s, d, delta, max_iters, doubles);
     if (e != cudaSuccess) return e;
     k_maxvol_inverse<<<n, 256, sizeof(double) * max_r * (2 * max_r + 1), s>>>(d);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -38,7 +38,7 @@ constexpr int NT = 256;
 // picks the tile within them for the grid (sweep_tile).
 template <int M, int DIR> struct Tile { static constexpr int W = 32, S = 26, P = W * (S + 6); };  // y, z: 32 x-lines, 26 cells
 template <int M> struct Tile<M, 0> {  // x: rows; a scalar's runs need 1024 points to fill the warps
-    static constexpr int W = 32, S = M == MODEL_EULER ? 122 : 250, P = M == MODEL_EULER ? NT : 1024;
+    static constexpr int W = 32, S = 250, P = M == MODEL_EULER ? NT : 1024;
 };
 
 constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
@@ -333,6 +333,7 @@ static inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b
 // tiles for every SM, and on small grids shorter segments for the same reason (a row
 // costs 6 halo points per segment, so not below 20 cells).  Advection at 128^3, x:
 // 7 rows of 128 cells (210 runs, the warps full); 3 rows of 64 (48 runs) took 164 us.
+// In 1D a tile is 250 cells, a point per thread.
 template <int M, int DIR> static void sweep_tile(SweepArgs &a)
 {
     const int n = a.n[DIR];

@@ -42,7 +42,7 @@ def check(W, mats, max_iters=200):
     return swapped
 
 
-@pytest.mark.parametrize("n,r", [(1, 1), (5, 5), (7, 3), (64, 64), (65, 64), (513, 1), (4097, 48), (3000, 64), (20000, 7),
+@pytest.mark.parametrize("n,r", [(1, 1), (5, 5), (7, 3), (64, 64), (65, 64), (513, 1), (4097, 48), (3000, 64), (20000, 7), (1365, 48), (1366, 48), (900, 18),
                                  (65536, 8)])
 def test_single_matrix(W, n, r):
     check(W, [matrix(n, r, n + r)])
