@@ -155,8 +155,9 @@ int weno_ssprk3_step(weno_handle h, double *U, double t_end, double dt);
 
 /* Up to max_steps SSP-RK3 steps (as weno_ssprk3_step) until the handle's time
  * reaches t_end.  Steps are launched as CUDA graphs of graph_steps steps
- * (graph_steps <= 0: plain launches); the graph is captured on first use for a
- * given U and reused.  alpha is carried from the last stage of one step to the
+ * (graph_steps <= 0: plain launches; the graph is captured on first use for a
+ * given U and reused; a 1D FP64 Euler grid of up to 2048 cells takes graph_steps
+ * steps in one kernel launch instead).  alpha is carried from the last stage of one step to the
  * next.  Synchronises; *steps_out (host, may be NULL) receives the number of
  * steps taken by this call. */
 int weno_run(weno_handle h, double *U, double t_end, double dt, int64_t max_steps, int32_t graph_steps,

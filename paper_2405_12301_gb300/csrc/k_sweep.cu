@@ -1,8 +1,8 @@
 // k_sweep.cu -- the fused per-direction residual kernel of the WENO5-JS scheme.
 //
 // One launch handles one direction d of one stage.  A CTA owns a tile of W
-// grid lines along d, S cells each, and runs three phases through shared
-// memory:
+// grid lines along d, S cells each (fitted to the grid, sweep_tile), and runs three
+// phases through shared memory:
 //   A. every stencil point of the tile (S + 6 per line: three ghost layers per
 //      side, Sec. 4.5) is loaded once, its ghost index mapped by the boundary
 //      rule, and its Lax-Friedrichs split flux f(+/-) (Sec. 2.2) computed once;

@@ -138,7 +138,9 @@ int svd_cluster(int n, int max_pk)
 // from it, so that chain (~35 dependent FP64 operations) runs beside the updates
 // and a column takes one barrier.  The other column groups go first to the warps of
 // the other three sub-partitions: a sub-partition issues an FP64 instruction every 64
-// cycles, whatever its warps.  64 columns of a 64-row sub-block: 195 -> QRSUB us.
+// cycles, whatever its warps.  A 64-row sub-block
+// of 64 columns takes 185 us (195 with the updates before the next reflector), a
+// triangular merge of 58 columns 158.
 __global__ void __launch_bounds__(TT_NT) k_qr_factor(const QRDesc *descs)
 {
     const QRDesc &d = descs[blockIdx.y];
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(TT_NT) k_qr_apply(const QApplyDesc *descs)
 //   3. each CTA applies Q to its share of the columns of J sigma.
 // A round is a chain of latencies (FP64 68 cycles each, a cluster barrier), not
 // work: 10 matrices of 50..64, 5.1 ms on one CTA each without the QR, 3.6 ms on 8
-// CTAs with pulled partials, SVDT ms here.
+// CTAs with pulled partials and no QR, 1.3 - 1.8 ms here.
 // Cluster size 1..8 (svd_cluster): fewer CTAs where the batch fills the GPU.
 __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
 {

@@ -9,7 +9,7 @@
 //   F^_{i+1} - F^_{i} = [f(+)_i - f(+)_{i-1}] + [f(-)_{i+1} - f(-)_i]
 //                       + [c(+)_{i+1} - c(+)_i] + [c(-)_{i+1} - c(-)_i],
 // so everything is built from the split-flux differences of neighbouring
-// points, D(a, b) = f(U_b) - f(U_a) (stored scaled for weno5d_slide2, see
+// points, D(a, b) = f(U_b) - f(U_a) (stored scaled for weno5d_cells2, see
 // pair_diff2).  Each D is formed in FP32 from the two points' FP64 states
 // alone: dU = U_b - U_a from their hi/lo splits, then the exact
 // product-difference identities with a's FP32 primitives (d(xy) = dx y_b +
@@ -44,7 +44,7 @@
 //      right (x) and upper (y) pair as one f32x2 computation (x pair in lane
 //      x, y pair in lane y), and one halo pair;
 //   W. WENO corrections of every face as sliding runs over the differences
-//      (weno5d_slide2), WENO(+) forward and the mirrored WENO(-) backward;
+//      (weno5d_cells2), WENO(+) forward and the mirrored WENO(-) backward;
 //   C. the cell's residual from its two pairs and four face corrections per
 //      direction, then L(U) or the stage update and the block's wavespeed max.
 #include "weno_dev.cuh"

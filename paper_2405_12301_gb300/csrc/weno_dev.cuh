@@ -222,62 +222,25 @@ __device__ __forceinline__ float weno5_pm(float2 a, float2 b, float2 c, float2 d
     return v.x + v.y;
 }
 
-// WENO5 correction of K consecutive windows along a line, from scaled first
+// WENO5 corrections of K consecutive windows along a line, from scaled first
 // differences (two streams as float2 pairs).  With v the values whose
 // reconstruction is wanted, D_k their first differences and t_r, s_r the
 // second differences and beta parts of the weno5 comment, the correction of a
 // window to its centre value c is
 //   sum_r omega_r v^(r) - c = (D2 + 2 D3)/6 + (w0 (t1 - t0) - 2 w2 (t1 - t2)) / (6 sum w).
-// p holds Dt = s D for a scale s, and the run returns 6 s times the correction:
+// p holds Dt = s D for a scale s; 6 s times the correction is
 //   6 s (sum_r omega_r v^(r) - c) = Ft + (w0 (tt1 - tt0) - 2 w2 (tt1 - tt2)) / sum w,
 //   Ft = Dt2 + 2 Dt3,  tt = s t,
 // with (13/3) tt_r^2 + st_r^2 = 4 s^2 beta_r (st = s s_r), so that
 // G_r = (13/3) tt_r^2 + st_r^2 + Geps with Geps = 4 s^2 eps is 4 s^2 (beta_r + eps),
 // and the weights w_r = d_r / G_r^2 up to a common factor are formed as
 // (3 g1 g2, 6 g0 g2, g0 g1) with g = G^2 (d = (3, 6, 1) / 10).  Window m takes
-// Dt1..Dt4 = p[m s] .. p[(m + 3) s] and writes to out[m os]; each window loads
-// one new difference, and its -2 (tt1 - tt2) is twice the previous window's
-// (tt1 - tt0), carried.  A mirrored window is the same run over the negated
+// Dt1..Dt4 = p[m s] .. p[(m + 3) s]; each window loads one new difference, and its
+// -2 (tt1 - tt2) is twice the previous window's (tt1 - tt0), carried.  A mirrored window is the same run over the negated
 // differences read backwards (the caller stores them negated).
-template <int K>
-__device__ __forceinline__ void weno5d_slide2(const float2 *p, int s, float Geps_, float2 *out, int os)
-{
-    const float2 k = bc2((float)(13.0 / 3.0)), Geps = bc2(Geps_);
-    float2 D1 = *p, D2 = *(p += s), D3 = *(p += s);
-    float2 t1 = sub2(D3, D2), t2 = sub2(D2, D1);
-    float2 A1 = fma2(mul2(k, t1), t1, Geps), A2 = fma2(mul2(k, t2), t2, Geps);
-    float2 h = mul2(bc2(-2.0f), sub2(t1, t2));
-#pragma unroll
-    for (int m = 0; m < K; ++m) {
-        const float2 D4 = *(p += s);
-        const float2 t0 = sub2(D4, D3);
-        const float2 A0 = fma2(mul2(k, t0), t0, Geps);
-        const float2 s0 = fma2(bc2(-3.0f), D3, D4), s1 = add2(D2, D3), s2 = fma2(bc2(-3.0f), D2, D1);
-        float2 g0 = fma2(s0, s0, A0), g1 = fma2(s1, s1, A1), g2 = fma2(s2, s2, A2);
-        g0 = mul2(g0, g0);
-        g1 = mul2(g1, g1);
-        g2 = mul2(g2, g2);
-        const float2 w0 = mul2(g1, g2), w1 = mul2(g0, g2), w2 = mul2(g0, g1);  // times 3, 6, 1
-        const float2 sw = fma2(bc2(3.0f), w0, fma2(bc2(6.0f), w1, w2));
-        const float2 e0 = sub2(t1, t0);
-        const float2 num = fma2(w0, mul2(bc2(3.0f), e0), mul2(w2, h));
-        const float2 F = fma2(bc2(2.0f), D3, D2);
-        *out = fma2(num, make_float2(fast_rcp(sw.x), fast_rcp(sw.y)), F);
-        out += os;
-        h = add2(e0, e0);
-        D1 = D2;
-        D2 = D3;
-        D3 = D4;
-        t2 = t1;
-        t1 = t0;
-        A2 = A1;
-        A1 = A0;
-    }
-}
-
-// The same run, emitting per cell instead of per face: with C_m the run's
-// output for window m, cell m - 1 (between the faces of windows m - 1 and m)
-// receives 6 D2_m + (C_m - C_{m-1}) (FWD; D2_m the window's second
+//
+// The run emits per cell: with C_m the value of window m, cell m - 1 (between the
+// faces of windows m - 1 and m) receives 6 D2_m + (C_m - C_{m-1}) (FWD; D2_m the window's second
 // difference, the cell's own pair), or -6 D2_m + (C_{m-1} - C_m) for a run read
 // backwards (!FWD), K - 1 values to out[(m - 1) os].  Those are 6 s times the
 // parts of a cell's flux difference that one run contributes (k_xy2 phase C).
@@ -328,12 +291,12 @@ __device__ __forceinline__ void weno5d_cells2(const float2 *p, int s, float Geps
 // operations form the nonlinear weights.  The value is
 //   c + [F + X] / 6,  F = D2 + 2 D3,  X = (3 g1 g2 e0 + 2 g0 g1 ep) / (3 g1 g2 + 6 g0 g2 + g0 g1),
 // with g_r = G_r^2, G_r = (13/3) t_r^2 + s_r^2 + 4 eps = 4 (beta_r + eps),
-// e0 = t1 - t0 and ep = t2 - t1 (the weno5 comment's symbols).  c, the first and
-// second differences and F stay in FP64; X is formed in unevaluated FP32 pairs
+// e0 = t1 - t0 and ep = t2 - t1 (the weno5 comment's symbols).  c, the first
+// differences and F stay in FP64; X is formed in unevaluated FP32 pairs
 // hi + lo (error-free transformations: Dekker 1971 and Knuth's two-sum; the
 // products' errors by FMA), about 47 bits, and added to F in FP64.  The second
-// differences are split after the FP64 subtraction, so X's relative error is
-// that of its own terms (~2^-46) and X is small against c wherever the data is
+// differences are formed exactly from all bits of the first (tr_diff) and then
+// rounded to pairs, so X's relative error is that of its own terms (~2^-46) and X is small against c wherever the data is
 // resolved.  Where it is not -- the two terms of X together above 2^-7 |c| --
 // where c or G leaves the range that FP32 pairs hold, the window is evaluated in
 // FP32 triples or FP64 (weno5_rough), so the error of the value stays that of FP64
@@ -344,7 +307,8 @@ __device__ __forceinline__ void weno5d_cells2(const float2 *p, int s, float Geps
 // 113-bit arithmetic, rms error in units of 2^-53 |v|, FP64 formula / this one:
 // smooth waves 0.637 / 0.637, a front 4 cells wide 0.737 / 0.744, 2 cells
 // 0.783 / 0.785, a captured shock 0.810 / 0.810, jumps 0.858 / 0.858.
-//   FP64 instructions per window of a run: 6 instead of 42.
+//   FP64 instructions per window of a run: 4 instead of 42 (L(U) at 97 x 83 x 61:
+// 2.49 -> 0.56 ms with the tiles of k_xy64.cu, scalar advection 128^3 5.0 -> 1.6).
 __device__ __forceinline__ float2 two_sum(float a, float b)
 {
     const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
@@ -587,7 +551,7 @@ __device__ __forceinline__ Tri tr_div(Tri w, Tri s, float r)
 }
 
 // The value of a rough window (its five points): differences and X in triples, c, F
-// and the final sum in FP64; the FP64 formula where G leaves the range.  9 FP64
+// and the final sum in FP64; the FP64 formula where G leaves the range.  7 FP64
 // instructions instead of 46, ~900 in FP32.  Measured as above, rms error FP64
 // formula / this one: front of 2 cells 0.780 / 0.776, captured shock 0.808 / 0.799,
 // jumps 0.855 / 0.851, random values 0.463 / 0.392.
@@ -660,8 +624,8 @@ __device__ __forceinline__ void rough_windows(const RoughList &L, int S, const d
 // `count` consecutive windows along a line: window m is the points at
 // src[po + m s], .., src[po + (m + 4) s] and its value goes to dst[oo + m os].
 // Neighbouring windows share all differences but one of each kind, so each window
-// forms one new; its value is bitwise weno5_pair of its points wherever it sits in
-// a run, so a face that two runs form gets the same value.  A negative stride walks
+// forms one new; its value depends on its five points only, bit for bit, wherever it
+// sits in a run, so a face that two runs form gets the same value.  A negative stride walks
 // a line backwards, which turns the run into the mirrored WENO(-) of the faces in
 // reverse order.
 // Offsets are below 2^13 and |s| is 1 or S.  The loop stays rolled: a window is
