@@ -238,20 +238,24 @@ __global__ void __launch_bounds__(xy64::MNT, 2) k_xy64(const SweepArgs a)
 double tile64_cycles(long long tiles, const Tile64 &t, int regs, int cells, double cell, int halo, int runs, int longest)
 {
     auto warps = [](int k) { return 4 * ((k + 127) / 128); };
-    const int k = (runs + t.nt - 1) / t.nt;
-    const double work = cell * warps(cells) + 22.0 * warps(halo) + 9.0 * k * (t.nt / 32) * (longest + 1) + 40.0;
+    const int k = (runs + t.nt - 1) / t.nt, w = t.nt / 32;
+    const double work = cell * warps(cells) + 22.0 * warps(halo) + 7.0 * k * w * (longest + 1) + 40.0;
     const long long most = 227 * 1024, per_sm = (tiles + sm_count() - 1) / sm_count();
     const long long res = std::min(most / (t.smem + 1024), 65536ll / (regs * t.nt));  // resident CTAs
     if (res < 1) return -1.0;
-    const double rounds = (double)((per_sm + res - 1) / res), lone = 0.25 / (double)std::min(res, per_sm);
-    return std::max(20.0 * work * (double)per_sm, 1000.0 * (k * (longest + 1) + 4) * rounds) * (1.0 + lone);
+    const double rounds = (double)((per_sm + res - 1) / res), ctas = (double)std::min(res, per_sm);
+    const double chain = k * (longest + 1) + 4;
+    return std::max(20.0 * work * (double)per_sm, 1000.0 * chain * rounds) * (1.0 + 0.15 / ctas + 4.0 / (ctas * w)) +
+           300.0 * chain;
 }
 
-// Measured at 256 x 256, 12 stages (us): 16 x 16 (the choice) 584, 32 x 7 582, 16 x 7
-// 605, 16 x 8 614, 8 x 16 619, 8 x 8 622, 16 x 4 702; at 97 x 83 x 61, L(U): 11 x 14 578,
-// 25 x 8 (the choice) 592, 25 x 7 599, 16 x 8 of 128 threads 612.  Blocks of 3 or 5 warps
-// are left out: an SM's FP64 units are its four sub-partitions', and such blocks load
-// them unevenly (8 x 8 cells, 64 / 96 / 128 threads: 622 / 737 / 659).
+// The estimate's choice and the best of ~30 tiles measured (us): 256 x 256, 12 stages,
+// 14 x 16 the best; 1000 x 777 (one L(U)) 16 x 16 the best; 400 x 300 16 x 16 72, 8 x 8
+// 70; 120 x 150 15 x 8 the best; 97 x 83 x 61 25 x 8 543, 11 x 14 528; 64^3 13 x 6 329,
+// 16 x 13 324; 40 x 53 x 37 10 x 11 151, 10 x 14 147 (32 x 8 of 256 threads, fixed: up to
+// 12% more).  Blocks of 3 or 5 warps are left out: an SM's FP64 units are its four
+// sub-partitions', and such blocks load them unevenly (8 x 8 cells, 64 / 96 / 128
+// threads: 622 / 737 / 659).
 Tile64 plan_xy64(int dim, const long long n[3])
 {
     using namespace xy64;

@@ -102,9 +102,9 @@ inline int fit_extent(long long n, int most)
 
 // Cycles of the fullest SM of a launch over Tile64 t: FP64 warp instructions at 20
 // cycles each -- `cell` for 32 cells' fluxes and update, ~22 for 32 halo points' flux,
-// ~9 for a round of windows, a phase's warps filling all four sub-partitions -- but no
+// ~7 for a round of windows, a phase's warps filling all four sub-partitions -- but no
 // less than the chains of windows (~1000 cycles each) that its rounds of CTAs wait for,
-// and more where few CTAs share the SM, whose phases leave it waiting.
+// more where few CTAs or warps share the SM, and part of one chain that nothing hides.
 double tile64_cycles(long long tiles, const Tile64 &t, int regs, int cells, double cell, int halo, int runs, int longest);
 Tile64 plan_xy64(int dim, const long long n[3]);
 Tile64 plan_z(const long long n[3]);
