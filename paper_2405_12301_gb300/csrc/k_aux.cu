@@ -11,12 +11,13 @@ namespace wg {
 
 // Start of a step: dt from alpha(U^n) (or the fixed dt), shortened so that the
 // time lands exactly on t_end; zero when the time is up or the step budget of
-// the current call is spent.  Clears the stage alpha slots 1..3.
-__device__ void step_begin(Ctl *c)
+// the current call is spent.  Clears the stage alpha slots 1..3.  (Values in
+// registers: one thread runs this, and every dependent load costs it ~0.4 us.)
+__device__ __forceinline__ void step_begin(Ctl *c, double t, double t_end, double dt_req, double cfl_h,
+                                           unsigned long long alpha, long long steps, long long max_steps)
 {
     double dt, tn;
-    if (next_dt(c->t, c->t_end, c->dt_req, c->cfl_h, __longlong_as_double((long long)c->alpha[0]), c->steps,
-                c->max_steps, dt, tn))
+    if (next_dt(t, t_end, dt_req, cfl_h, __longlong_as_double((long long)alpha), steps, max_steps, dt, tn))
         atomicOr(&c->status, ST_NONPHYSICAL);
     c->dt = dt;
     c->t_next = tn;
@@ -36,20 +37,28 @@ __device__ void alpha_done(Ctl *c, const AlphaThen &then)
 {
     __syncthreads();
     if (threadIdx.x != 0) return;
+    const double t = c->t;
+    const long long steps = c->steps;
     __threadfence();
     if (atomicAdd(&c->ticket, 1u) != gridDim.x - 1) return;
     __threadfence();
     c->ticket = 0u;
-    c->alpha[0] = atomicExch(&c->alpha_new[0], 0ull);
-    for (int e = 0; e < 3; ++e) c->alpha_dir[0][e] = atomicExch(&c->alpha_new[1 + e], 0ull);
-    if (then.out) *then.out = __longlong_as_double((long long)c->alpha[0]);
-    if (then.set_run) {
-        c->t_end = then.t_end;
-        c->dt_req = then.dt_req;
-        c->cfl_h = then.cfl_h;
-        c->max_steps = (then.max_steps > LLONG_MAX - c->steps) ? LLONG_MAX : c->steps + then.max_steps;
-    }
-    if (then.begin) step_begin(c);
+    unsigned long long m[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) m[e] = __ldcg(&c->alpha_new[e]);
+    c->alpha[0] = m[0];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c->alpha_new[e] = 0ull;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) c->alpha_dir[0][e] = m[1 + e];
+    if (then.out) *then.out = __longlong_as_double((long long)m[0]);
+    if (!then.set_run) return;
+    const long long max_steps = (then.max_steps > LLONG_MAX - steps) ? LLONG_MAX : steps + then.max_steps;
+    c->t_end = then.t_end;
+    c->dt_req = then.dt_req;
+    c->cfl_h = then.cfl_h;
+    c->max_steps = max_steps;
+    if (then.begin) step_begin(c, t, then.t_end, then.dt_req, then.cfl_h, m[0], steps, max_steps);
 }
 
 // alpha of an FP64 state (PD: and the per-direction speeds).  Bound by the FP64
@@ -120,13 +129,22 @@ __global__ void __launch_bounds__(256) k_alpha_scalar(const double *__restrict__
 // also the start of the next.
 __global__ void k_step_end(Ctl *c, int begin)
 {
-    if (c->dt > 0.0) {
-        c->t = c->t_next;
-        c->steps += 1;
-        c->alpha[0] = c->alpha[3];
-        for (int e = 0; e < 3; ++e) c->alpha_dir[0][e] = c->alpha_dir[3][e];
+    const double dt = c->dt, t0 = c->t, tn = c->t_next;
+    const double t_end = c->t_end, dt_req = c->dt_req, cfl_h = c->cfl_h;
+    const long long s0 = c->steps, max_steps = c->max_steps;
+    const unsigned long long a0 = c->alpha[0], a3 = c->alpha[3];
+    unsigned long long ad[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) ad[e] = c->alpha_dir[3][e];
+    const bool took = dt > 0.0;
+    if (took) {
+        c->t = tn;
+        c->steps = s0 + 1;
+        c->alpha[0] = a3;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) c->alpha_dir[0][e] = ad[e];
     }
-    if (begin) step_begin(c);
+    if (begin) step_begin(c, took ? tn : t0, t_end, dt_req, cfl_h, took ? a3 : a0, took ? s0 + 1 : s0, max_steps);
 }
 
 // Two-level fixed-order sums: block b reduces a fixed contiguous chunk of

@@ -339,7 +339,8 @@ template <int M, int DIR> static void sweep_tile(SweepArgs &a)
     const int n = a.n[DIR];
     if (DIR == 0) {
         const long long rows = (long long)a.n[1] * a.n[2];
-        long long most = (n * rows + 4ll * sm_count() - 1) / (4ll * sm_count());
+        const long long want = rows == 1 ? sm_count() : 4ll * sm_count();  // (a 1D tile is one row: a CTA per SM fills its warps best)
+        long long most = (n * rows + want - 1) / want;
         most = most < 20 ? 20 : most > Tile<M, 0>::S ? Tile<M, 0>::S : most;
         a.tile_s = (int)cdiv(n, cdiv(n, most));
         long long w = Tile<M, 0>::P / (a.tile_s + 6), share = rows * cdiv(n, a.tile_s) / (2ll * sm_count());
