@@ -85,6 +85,8 @@ def load_peaks():
 SM_COUNT = 152
 PEAK_FP32_TFLOPS = SM_COUNT * 128 * 2 * 2.070e9 / 1e12
 PEAK_FP64_TFLOPS = 1.25
+FP64_NOTE = ("all algorithmic flops against the FP64 pipe's peak: the FP64 grid kernels form the WENO weights in FP32 "
+             "pairs, so this is a speed relative to that pipe, not its use")
 
 
 def set_sm_count(n):
@@ -371,6 +373,7 @@ def roofline(w, prec_bulk, kms, kn, cells):
             "traffic": traffic, "traffic_unit": "bytes per launch (ncu dram read + write)",
             "kernel": names[k], "ms_per_launch": per_launch_ms,
             "pipe": "fp32" if prec_bulk else "fp64",
+            "note": None if prec_bulk else FP64_NOTE,
             "peak_source": "derived: %d SMs x 128 FP32 lanes x 2 flop x 2070 MHz" % SM_COUNT if prec_bulk
             else "nominal GB300 FP64 1.25 TFLOP/s"}
 
@@ -658,7 +661,7 @@ def bench_scalar(weno, I, torch, steps=4, warmup=3, N=256):
             "unit": "Mcell-stage/s", "dtype": "f64", "steps": steps, "ms_per_step": ms / steps,
             "gpu_launches": launches,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": PEAK_FP64_TFLOPS, "unit": "TFLOP/s",
-                         "frac": achieved / PEAK_FP64_TFLOPS, "traffic": None, "kernel": "sweep",
+                         "frac": achieved / PEAK_FP64_TFLOPS, "traffic": None, "kernel": "sweep", "note": FP64_NOTE,
                          "ms_per_launch": sweep_ms / max(1, kn[3]), "flops_per_cell_stage": fl,
                          "peak_source": "nominal GB300 FP64 1.25 TFLOP/s"}}
 
