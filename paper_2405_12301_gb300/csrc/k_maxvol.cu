@@ -648,7 +648,10 @@ cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_n
 {
     cudaError_t e = maxvol_attributes();
     if (e != cudaSuccess) return e;
-    const int ncl = maxvol_cluster_size();
+    // at least 64 rows to a CTA: below, the cluster barriers of a step cost more than its
+    // pass over the rows
+    int ncl = maxvol_cluster_size();
+    while (ncl > 2 && max_nr < 64ll * ncl * max_r) ncl /= 2;
     const long long per_sm = std::min(3ll, std::max(1ll, ((long long)n * ncl + sm_count() - 1) / sm_count()));
     const long long want = sizeof(double) * std::max((max_nr + ncl - 1) / ncl + max_r, 2ll * max_r * max_r);
     const long long least = sizeof(double) * 2ll * max_r * max_r;  // L[I] and its inverse
