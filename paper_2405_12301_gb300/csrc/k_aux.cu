@@ -2,6 +2,7 @@
 // wavespeed max (LF alpha, Sec. 4.3), the device-side time-step control
 // (dt = lambda h / alpha with the last step shortened to land on t_end,
 // Eq. cfl-other), and the fixed-order FP64 conservation sums.
+#include <algorithm>
 #include <climits>
 
 #include "weno_dev.cuh"
@@ -63,9 +64,11 @@ __device__ void alpha_done(Ctl *c, const AlphaThen &then)
 
 // alpha of an FP64 state (PD: and the per-direction speeds).  Bound by the FP64
 // pipe if every cell's speed is formed there (84% busy at 97 x 83 x 61); the FP32
-// estimates leave it a handful of cells per block.
+// estimates leave it a handful of cells per block, so few large blocks: at 97 x 83 x 61
+// 1216 blocks of 256 threads took 27 us, 304 of 512 take 17.
+constexpr int ALPHA_NT = 512;
 template <int D, bool PD>
-__global__ void __launch_bounds__(256) k_alpha(const double *__restrict__ U, long long N, double gamma, Ctl *ctl,
+__global__ void __launch_bounds__(ALPHA_NT, 2) k_alpha(const double *__restrict__ U, long long N, double gamma, Ctl *ctl,
                                                const AlphaThen then)
 {
     speed_max_publish_f64<D, PD ? 1 + D : 1>(
@@ -239,11 +242,12 @@ cudaError_t launch_alpha(int model, int dim, bool bulk, const double *U, long lo
     if (model == MODEL_ADVECT) k_alpha_scalar<MODEL_ADVECT><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model == MODEL_BURGERS) k_alpha_scalar<MODEL_BURGERS><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model != MODEL_EULER) return cudaGetLastError();
+    const int big = (int)std::min<long long>((N + ALPHA_NT - 1) / ALPHA_NT, 2 * sm_count());
 #define X(D)                                                                                        \
     if (dim == D && bulk)                                                                           \
         k_alpha_bulk<D><<<blocks < sm_count() * 4 ? blocks : sm_count() * 4, 256, 0, s>>>(U, N, gamma, ctl, per_dir, then); \
-    else if (dim == D && per_dir) k_alpha<D, true><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, then);     \
-    else if (dim == D) k_alpha<D, false><<<blocks, 256, 0, s>>>(U, N, gamma, ctl, then);
+    else if (dim == D && per_dir) k_alpha<D, true><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, ctl, then);   \
+    else if (dim == D) k_alpha<D, false><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, ctl, then);
     X(1) X(2) X(3)
 #undef X
     return cudaGetLastError();
