@@ -820,8 +820,9 @@ cudaError_t launch_cross(const CrossArgs &a, int variant, int ctas_per_sm, cudaS
     if (variant < 0 || variant >= kNumCrossVariants || ctas_per_sm < 1) return cudaErrorInvalidValue;
     cudaError_t ea = cross_set_attributes();
     if (ea != cudaSuccess) return ea;
-    // enough CTAs per set that all of them together fill the GPU a few times over
-    const int per_set = (int)std::min(64ll, std::max(4ll, (8ll * sm_count() + a.n_sets - 1) / a.n_sets));
+    // enough CTAs per set that the largest sets' do not outlast the rest (576 sets: with 4
+    // each the SMs stood idle half of the 138 us, with 16 it takes 107)
+    const int per_set = (int)std::min(64ll, std::max(16ll, (32ll * sm_count() + a.n_sets - 1) / a.n_sets));
     if (a.fp64) k_cross_vecs<true><<<dim3(a.n_sets, per_set), XT, 0, s>>>(a);
     else k_cross_vecs<false><<<dim3(a.n_sets, per_set), XT, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
