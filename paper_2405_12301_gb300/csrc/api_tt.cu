@@ -3,6 +3,7 @@
 // and the fixed-rank TT-cross sweep (weno_tt_cross).  Host orchestration only;
 // the kernels are in k_tt.cu, k_maxvol.cu and k_cross_drv.cu.
 #include "api_ctx.h"
+#include "qr_plan.h"
 
 using namespace wg;
 
@@ -14,94 +15,6 @@ using namespace wg;
 // the launches that follow.
 
 namespace {
-
-// A TSQR tree: level 0 factors chunks of the matrix's rows, each further level
-// groups of the R factors of the one before, until one R is left.
-struct QRPlan {
-    struct Level {
-        long long m = 0, rows = 0;  // rows of the level's matrix, rows per chunk
-        int C = 1, sub = 1;         // chunks, sub-blocks per chunk
-        double *A = nullptr, *tau = nullptr, *R = nullptr, *X = nullptr;  // (X: the stack of the chunks' top rows)
-    };
-    int k = 0, b = 32;
-    std::vector<Level> L;
-    std::vector<Level> buf;  // the buffers taken for it
-    double *T = nullptr;
-};
-constexpr int QR_MAXL = 24;  // levels at most (a matrix of 2^27 rows takes 15)
-
-// Sub-blocks of b >= k rows, at most spc per chunk, every chunk at least k rows
-// long when there are several; then g R factors per chunk: two where the batch is
-// small (the tree's depth is the time), four where it fills the GPU.
-// more: plan for that many chunks beyond what m needs (to size buffers).
-void qr_plan(QRPlan &q, long long m, int k, int spc, int g, int more = 0)
-{
-    q.k = k;
-    q.b = k <= 32 ? 32 : (k + 31) / 32 * 32;
-    q.L.clear();
-    QRPlan::Level l;
-    l.m = m;
-    const long long per = (long long)spc * q.b;
-    for (int C = (int)std::max(1LL, (m + per - 1) / per);; --C) {
-        const long long cr = (m + C - 1) / C;
-        if (C == 1 || (cr >= k && m - (long long)(C - 1) * cr >= k)) {
-            l.C = C;
-            l.rows = std::max(1LL, cr);
-            break;
-        }
-    }
-    l.sub = (int)((l.rows + q.b - 1) / q.b);
-    q.L.push_back(l);
-    q.L[0].C += more;
-    while (q.L.back().C > 1) {
-        const int C = q.L.back().C;
-        l = QRPlan::Level();
-        l.m = (long long)C * k;
-        l.C = (C + g - 1) / g;
-        l.sub = g;
-        l.rows = (long long)g * k;
-        q.L.push_back(l);
-    }
-}
-
-struct Bump {  // counts (base == nullptr) or hands out 256-byte aligned pieces
-    char *base = nullptr;
-    size_t off = 0;
-    template <class T> T *take(size_t n)
-    {
-        off = (off + 255) & ~size_t(255);
-        T *p = base ? reinterpret_cast<T *>(base + off) : nullptr;
-        off += sizeof(T) * n;
-        return p;
-    }
-};
-
-// Buffers for the QR of an m x k matrix and for applying it to p columns, also for
-// any smaller m of the same k and spc (whose plan has at most one chunk more).
-void qr_take(Bump &bp, QRPlan &q, long long m, int k, int spc, int g, int p)
-{
-    QRPlan big;
-    qr_plan(big, m, k, spc, g, 1);
-    q.buf.assign(big.L.size(), QRPlan::Level());
-    for (size_t l = 0; l < big.L.size(); ++l) {
-        const QRPlan::Level &v = big.L[l];
-        const size_t subs = l == 0 ? (size_t)(m / big.b) + 2 * (size_t)v.C + 4 : (size_t)big.L[l - 1].C + 8;
-        q.buf[l].tau = bp.take<double>(subs * k);
-        q.buf[l].R = bp.take<double>((size_t)(v.C + 1) * k * k);
-        if (l > 0) q.buf[l].X = bp.take<double>((size_t)(big.L[l - 1].C + 4) * k * p);
-    }
-}
-
-void qr_bind(QRPlan &q, double *A)
-{
-    for (size_t l = 0; l < q.L.size(); ++l) {
-        q.L[l].A = l == 0 ? A : q.buf[l - 1].R;
-        q.L[l].tau = q.buf[l].tau;
-        q.L[l].R = q.buf[l].R;
-        q.L[l].X = q.buf[l].X;
-    }
-    q.T = q.L.back().R;
-}
 
 // Sub-blocks per chunk: what spreads the batch's sub-blocks over three CTAs per SM.
 int qr_spc(long long subs) { return (int)std::min(16LL, std::max(2LL, (subs + 3LL * sm_count() - 1) / (3LL * sm_count()))); }
@@ -313,9 +226,8 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         sd[i].C1 = t.C1;
         sd[i].MA = t.MA;
         sd[i].MB = t.MB;
-        qr_bind(t.qa, t.MA);
-        qr_bind(t.qb, t.MB);
-        qr_bind(t.qc, t.MC);
+        if (!qr_bind(t.qa, t.MA) || !qr_bind(t.qb, t.MB) || !qr_bind(t.qc, t.MC))
+            return fail(h, WENO_ERR_CUDA, "weno_tt_round: a QR plan exceeds its buffers");
         sd[i].TA = t.qa.T;
     }
     // ---- phase 1: sum unfoldings; QR of the last core; middle core times TA^T; QR; first core; QR; SVD
@@ -357,7 +269,7 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         if (probs[i].cap[0] < (long long)t.n[0] * t.r1)
             return fail(h, WENO_ERR_ARG, "weno_tt_round: output core 1 capacity too small");
         qr_plan(t.qe, (long long)t.r1 * t.n[1], t.k3, pe, g);
-        qr_bind(t.qe, t.ME);
+        if (!qr_bind(t.qe, t.ME)) return fail(h, WENO_ERR_CUDA, "weno_tt_round: a QR plan exceeds its buffers");
     }
     // ---- phase 2: first output core; the middle core into the (r1 n2) x k3 unfolding; QR; SVD
     {
