@@ -30,10 +30,19 @@ struct TTPlan {
     int r1 = 0, r2 = 0;
 };
 
+// Device blocks that the launches' descriptors take in turn.  A block is written again
+// by a copy on the stream of the launches, so after the one that read it.
+struct DescRing {
+    char *base;
+    size_t block;
+    int blocks, next;
+    template <class T> T *take() { return (T *)(base + block * (next++ % blocks)); }
+};
+
 }  // namespace
 
 // Factor every plan, level by level (a plan without the level sits it out).
-static int tt_factor(weno_ctx *h, std::vector<QRPlan *> &ps, char *dev)
+static int tt_factor(weno_ctx *h, std::vector<QRPlan *> &ps, DescRing &ring)
 {
     const int n = (int)ps.size();
     size_t levels = 0;
@@ -52,7 +61,7 @@ static int tt_factor(weno_ctx *h, std::vector<QRPlan *> &ps, char *dev)
             maxC = std::max(maxC, v.C);
             smem = std::max(smem, qr_factor_smem(q.k, q.b));
         }
-        QRDesc *dd = (QRDesc *)(dev + sizeof(QRDesc) * n * l);
+        QRDesc *dd = ring.take<QRDesc>();
         CK(h, cudaMemcpyAsync(dd, ds.data(), sizeof(QRDesc) * n, cudaMemcpyHostToDevice, h->stream));
         CK(h, launch(h, 0, h->stream, [&] { return launch_qr_factor(dd, n, maxC, smem, h->stream); }));
     }
@@ -69,7 +78,7 @@ struct ApplyReq {  // Q [X; 0] of one plan into an output row map
 
 // From the top of each plan's tree down: a level's result is the stack of the top
 // rows of the level below.
-static int tt_apply(weno_ctx *h, std::vector<ApplyReq> &rs, char *dev)
+static int tt_apply(weno_ctx *h, std::vector<ApplyReq> &rs, DescRing &ring)
 {
     const int n = (int)rs.size();
     size_t levels = 0;
@@ -92,7 +101,7 @@ static int tt_apply(weno_ctx *h, std::vector<ApplyReq> &rs, char *dev)
             maxC = std::max(maxC, v.C);
             smem = std::max(smem, qr_apply_smem(q.k, q.b, r.p));
         }
-        QApplyDesc *dd = (QApplyDesc *)(dev + sizeof(QApplyDesc) * n * l);
+        QApplyDesc *dd = ring.take<QApplyDesc>();
         CK(h, cudaMemcpyAsync(dd, ds.data(), sizeof(QApplyDesc) * n, cudaMemcpyHostToDevice, h->stream));
         CK(h, launch(h, 0, h->stream, [&] { return launch_qr_apply(dd, n, maxC, smem, h->stream); }));
     }
@@ -172,9 +181,9 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
         qr_plan(t.qb, t.mB, t.R1, pb, g);
         qr_plan(t.qc, t.n[0], t.k2, pc, g);
     }
-    // scratch: descriptors (a QR or apply step takes one block per level), ranks, then
-    // per problem matrices and QR data
-    const int NDESC = 8 * QR_MAXL + 8;
+    // scratch: descriptors (the sums' block, which two launches read, and a ring for the
+    // others), ranks, then per problem matrices and QR data
+    const int NDESC = 24;
     const size_t dsz = std::max({sizeof(QRDesc), sizeof(QApplyDesc), sizeof(SvdDesc), sizeof(TTSumDesc), sizeof(GemmDesc)});
     auto layout = [&](Bump &bp) -> char * {
         char *desc = bp.take<char>(dsz * NDESC * (size_t)np);
@@ -214,12 +223,7 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
     bp.base = (char *)h->tbuf;
     char *desc = layout(bp);
     int *ranks = (int *)((char *)h->tbuf + rank_off);
-    int slot = 0;
-    auto next_desc = [&](int blocks = 1) {
-        char *p = desc + dsz * (size_t)np * slot;
-        slot += blocks;
-        return p;
-    };
+    DescRing ring{desc + dsz * (size_t)np, dsz * (size_t)np, NDESC - 1, 0};
 
     for (int i = 0; i < np; ++i) {
         TTPlan &t = pl[i];
@@ -232,32 +236,32 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
     }
     // ---- phase 1: sum unfoldings; QR of the last core; middle core times TA^T; QR; first core; QR; SVD
     {
-        TTSumDesc *d = (TTSumDesc *)next_desc();
+        TTSumDesc *d = (TTSumDesc *)desc;
         CK(h, cudaMemcpyAsync(d, sd.data(), sizeof(TTSumDesc) * np, cudaMemcpyHostToDevice, h->stream));
         CK(h, launch(h, 1, h->stream, [&] { return launch_tt_build(d, np, h->stream); }));
         std::vector<QRPlan *> ps;
         for (auto &t : pl) ps.push_back(&t.qa);
-        int r = tt_factor(h, ps, next_desc(QR_MAXL));
+        int r = tt_factor(h, ps, ring);
         if (r) return r;
         CK(h, launch(h, 1, h->stream, [&] { return launch_tt_contract(d, np, h->stream); }));
         ps.clear();
         for (auto &t : pl) ps.push_back(&t.qb);
-        if ((r = tt_factor(h, ps, next_desc(QR_MAXL)))) return r;
+        if ((r = tt_factor(h, ps, ring))) return r;
         std::vector<GemmDesc> gd(np);
         for (int i = 0; i < np; ++i)
             gd[i] = GemmDesc{pl[i].C1, pl[i].qb.T, pl[i].MC, pl[i].n[0], pl[i].k2, pl[i].R1};
-        GemmDesc *gdev = (GemmDesc *)next_desc();
+        GemmDesc *gdev = ring.take<GemmDesc>();
         CK(h, cudaMemcpyAsync(gdev, gd.data(), sizeof(GemmDesc) * np, cudaMemcpyHostToDevice, h->stream));
         CK(h, launch(h, 1, h->stream, [&] { return launch_tt_gemm_tr(gdev, np, h->stream); }));
         ps.clear();
         for (auto &t : pl) ps.push_back(&t.qc);
-        if ((r = tt_factor(h, ps, next_desc(QR_MAXL)))) return r;
+        if ((r = tt_factor(h, ps, ring))) return r;
         std::vector<SvdDesc> sv(np);
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
             sv[i] = SvdDesc{t.qc.T, t.k2, t.kc, t.k2, eps_tt, 1, t.delta, ranks + 2 * i, t.kc, t.svC, t.VC, t.WC, t.kc};
         }
-        if ((r = tt_svd(h, sv, (SvdDesc *)next_desc()))) return r;
+        if ((r = tt_svd(h, sv, ring.take<SvdDesc>()))) return r;
     }
     std::vector<int> rk(2 * np);
     CK(h, cudaMemcpyAsync(rk.data(), ranks, sizeof(int) * 2 * np, cudaMemcpyDeviceToHost, h->stream));
@@ -278,23 +282,23 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
             TTPlan &t = pl[i];
             ar[i] = ApplyReq{&t.qc, t.VC, t.kc, t.r1, probs[i].out.core[0], t.n[0], t.r1, 0, 1};
         }
-        int r = tt_apply(h, ar, next_desc(QR_MAXL));
+        int r = tt_apply(h, ar, ring);
         if (r) return r;
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
             ar[i] = ApplyReq{&t.qb, t.WC, t.kc, t.r1, t.ME, t.mB, 1, 0, t.mB};
         }
-        if ((r = tt_apply(h, ar, next_desc(QR_MAXL)))) return r;
+        if ((r = tt_apply(h, ar, ring))) return r;
         std::vector<QRPlan *> ps;
         for (auto &t : pl) ps.push_back(&t.qe);
-        if ((r = tt_factor(h, ps, next_desc(QR_MAXL)))) return r;
+        if ((r = tt_factor(h, ps, ring))) return r;
         std::vector<SvdDesc> sv(np);
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
             const int pk = (int)std::min<long long>((long long)t.r1 * t.n[1], t.k3);
             sv[i] = SvdDesc{t.qe.T, t.k3, pk, t.k3, eps_tt, 0, t.delta, ranks + 2 * i + 1, pk, t.svE, t.VE, t.WE, t.ke};
         }
-        if ((r = tt_svd(h, sv, (SvdDesc *)next_desc()))) return r;
+        if ((r = tt_svd(h, sv, ring.take<SvdDesc>()))) return r;
     }
     std::vector<double> norms(2 * np);
     CK(h, cudaMemcpyAsync(rk.data(), ranks, sizeof(int) * 2 * np, cudaMemcpyDeviceToHost, h->stream));
@@ -316,13 +320,13 @@ extern "C" int weno_tt_round(weno_handle h, weno_tt_round_problem *probs, int32_
             ar[i] = ApplyReq{&t.qe, t.VE, t.ke, t.r2, probs[i].out.core[1], t.n[1], (long long)t.r1 * t.r2,
                              t.r2, 1};
         }
-        int r = tt_apply(h, ar, next_desc(QR_MAXL));
+        int r = tt_apply(h, ar, ring);
         if (r) return r;
         for (int i = 0; i < np; ++i) {
             TTPlan &t = pl[i];
             ar[i] = ApplyReq{&t.qa, t.WE, t.ke, t.r2, probs[i].out.core[2], t.n[2], t.r2, 0, 1};
         }
-        if ((r = tt_apply(h, ar, next_desc(QR_MAXL)))) return r;
+        if ((r = tt_apply(h, ar, ring))) return r;
     }
     for (int i = 0; i < np; ++i) {
         weno_tt3 &o = probs[i].out;
