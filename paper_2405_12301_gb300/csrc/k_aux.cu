@@ -68,15 +68,15 @@ __device__ void alpha_done(Ctl *c, const AlphaThen &then)
 // 1216 blocks of 256 threads took 27 us, 304 of 512 take 17.
 constexpr int ALPHA_NT = 512;
 template <int D, bool PD>
-__global__ void __launch_bounds__(ALPHA_NT, 2) k_alpha(const double *__restrict__ U, long long N, double gamma, Ctl *ctl,
-                                               const AlphaThen then)
+__global__ void __launch_bounds__(ALPHA_NT, 2) k_alpha(const double *__restrict__ U, long long N, double gamma, float gg,
+                                                       Ctl *ctl, const AlphaThen then)
 {
     speed_max_publish_f64<D, PD ? 1 + D : 1>(
         [&](long long i, double *q) {
 #pragma unroll
             for (int f = 0; f < D + 2; ++f) q[f] = __ldg(U + f * N + i);
         },
-        (long long)blockIdx.x * blockDim.x + threadIdx.x, N, (long long)gridDim.x * blockDim.x, gamma, &ctl->alpha_new[0],
+        (long long)blockIdx.x * blockDim.x + threadIdx.x, N, (long long)gridDim.x * blockDim.x, gamma, gg, &ctl->alpha_new[0],
         &ctl->alpha_new[1], &ctl->status);
     alpha_done(ctl, then);
 }
@@ -242,12 +242,13 @@ cudaError_t launch_alpha(int model, int dim, bool bulk, const double *U, long lo
     if (model == MODEL_ADVECT) k_alpha_scalar<MODEL_ADVECT><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model == MODEL_BURGERS) k_alpha_scalar<MODEL_BURGERS><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model != MODEL_EULER) return cudaGetLastError();
+    const float gg = (float)(gamma * (gamma - 1.0));
     const int big = (int)std::min<long long>((N + ALPHA_NT - 1) / ALPHA_NT, 2 * sm_count());
 #define X(D)                                                                                        \
     if (dim == D && bulk)                                                                           \
         k_alpha_bulk<D><<<blocks < sm_count() * 4 ? blocks : sm_count() * 4, 256, 0, s>>>(U, N, gamma, ctl, per_dir, then); \
-    else if (dim == D && per_dir) k_alpha<D, true><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, ctl, then);   \
-    else if (dim == D) k_alpha<D, false><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, ctl, then);
+    else if (dim == D && per_dir) k_alpha<D, true><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, gg, ctl, then);   \
+    else if (dim == D) k_alpha<D, false><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, gg, ctl, then);
     X(1) X(2) X(3)
 #undef X
     return cudaGetLastError();

@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(r1::NT) k_run1d(const SweepArgs a, double *U, 
 #pragma unroll
                     for (int f = 0; f < NF; ++f) s[f] = uk[f];
                 },
-                0, own ? 1 : 0, 1, a.gamma, s_max[buf], &s_bad);
+                0, own ? 1 : 0, 1, a.gamma, a.gg_f, s_max[buf], &s_bad);
             __syncthreads();
             if (tid == 0 && s_bad) atomicOr(&a.ctl->status, ST_NONPHYSICAL);
             cl.sync();

@@ -313,10 +313,10 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
             for (int f = 0; f < NF; ++f) q[f] = qout[f];
         };
         if (K == 2)
-            speed_max_publish_f64<D, 2>(load, 0, has ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out],
+            speed_max_publish_f64<D, 2>(load, 0, has ? 1 : 0, 1, a.gamma, a.gg_f, &a.ctl->alpha[a.slot_out],
                                         a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
         else
-            speed_max_publish_f64<D, 1>(load, 0, has ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out],
+            speed_max_publish_f64<D, 1>(load, 0, has ? 1 : 0, 1, a.gamma, a.gg_f, &a.ctl->alpha[a.slot_out],
                                         a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
     } else if (EPI == EPI_STAGE) {
         if (BULK) cmax = (double)cmaxf;

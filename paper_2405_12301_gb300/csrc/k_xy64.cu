@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(xy64::MNT, 2) k_xy64(const SweepArgs a)
 #pragma unroll
                 for (int f = 0; f < NF; ++f) q[f] = out[f];
             },
-            0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
+            0, own ? 1 : 0, 1, a.gamma, a.gg_f, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
 }
 
 double tile64_cycles(long long tiles, const Tile64 &t, int regs, int cells, double cell, int halo, int runs, int longest)

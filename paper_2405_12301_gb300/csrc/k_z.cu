@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(zs::MNT, 2) k_z(const SweepArgs a)
 #pragma unroll
                 for (int f = 0; f < NF; ++f) q[f] = out[f];
             },
-            0, own ? 1 : 0, 1, a.gamma, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
+            0, own ? 1 : 0, 1, a.gamma, a.gg_f, &a.ctl->alpha[a.slot_out], a.ctl->alpha_dir[a.slot_out], &a.ctl->status);
 }
 
 // Measured at 97 x 83 x 61, L(U) (us): 11 x 11 580, 9 x 11 587, 25 x 9 597, 17 x 13 604.

@@ -924,12 +924,13 @@ __device__ __forceinline__ float wavespeed_f32(const float *q, float gamma, bool
 }
 
 // FP32 estimates of the speeds of an FP64 state: est[0] = |u| + a and, for K > 1,
-// est[1 + e] = |u_e| + a.  Returns whether the state is certainly physical and the
+// est[1 + e] = |u_e| + a; gg = gamma (gamma - 1), formed from the FP64 gamma (an FP32
+// one less 1 has few bits left near 1).  Returns whether the state is certainly physical and the
 // estimates are within 2^-16 of the FP64 values: the conserved fields of ordinary
 // size and the internal energy at least 2^-5 of the total and kinetic energies
 // (its FP32 rounding is 2^-21 of those).
 template <int D, int K>
-__device__ __forceinline__ bool speed_estimate(const double *q, float gamma, float *est)
+__device__ __forceinline__ bool speed_estimate(const double *q, float gg, float *est)
 {
     float f[D + 2];
 #pragma unroll
@@ -942,7 +943,7 @@ __device__ __forceinline__ bool speed_estimate(const double *q, float gamma, flo
         u2 = fmaf(ue, ue, u2);
     }
     const float ke = 0.5f * f[0] * u2, ie = f[D + 1] - ke;
-    const float a = sqrt_approx(gamma * (gamma - 1.0f) * ie * ir);
+    const float a = sqrt_approx(gg * ie * ir);
     est[0] = sqrt_approx(u2) + a;
     if (K > 1) {
 #pragma unroll
@@ -965,7 +966,7 @@ __device__ __forceinline__ bool speed_estimate(const double *q, float gamma, flo
 // block must call it.
 template <int D, int K, class Load>
 __device__ __forceinline__ void speed_max_block_f64(Load load, long long begin, long long end, long long step,
-                                                    double gamma, unsigned long long *s_max, int *s_bad)
+                                                    double gamma, float gg, unsigned long long *s_max, int *s_bad)
 {
     __shared__ unsigned s_est[K];
     if (threadIdx.x < K) {
@@ -973,7 +974,6 @@ __device__ __forceinline__ void speed_max_block_f64(Load load, long long begin, 
         s_max[threadIdx.x] = 0ull;
     }
     if (threadIdx.x == 0) *s_bad = 0;
-    const float gf = (float)gamma;
     float mine[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) mine[k] = 0.0f;
@@ -982,7 +982,7 @@ __device__ __forceinline__ void speed_max_block_f64(Load load, long long begin, 
         double q[D + 2];
         float est[K];
         load(i, q);
-        if (speed_estimate<D, K>(q, gf, est)) {
+        if (speed_estimate<D, K>(q, gg, est)) {
 #pragma unroll
             for (int k = 0; k < K; ++k) mine[k] = fmaxf(mine[k], est[k]);
         } else {
@@ -1012,7 +1012,7 @@ __device__ __forceinline__ void speed_max_block_f64(Load load, long long begin, 
                 double q[D + 2], v[K];
                 float est[K];
                 load(i, q);
-                bool go = !speed_estimate<D, K>(q, gf, est), bad;
+                bool go = !speed_estimate<D, K>(q, gg, est), bad;
 #pragma unroll
                 for (int k = 0; k < K; ++k) go = go || est[k] >= thr[k];
                 if (!go) continue;
@@ -1039,12 +1039,12 @@ __device__ __forceinline__ void speed_max_block_f64(Load load, long long begin, 
 // also slot_dir[e].
 template <int D, int K, class Load>
 __device__ __forceinline__ void speed_max_publish_f64(Load load, long long begin, long long end, long long step,
-                                                      double gamma, unsigned long long *slot0,
+                                                      double gamma, float gg, unsigned long long *slot0,
                                                       unsigned long long *slot_dir, int *status)
 {
     __shared__ unsigned long long s_max[K];
     __shared__ int s_bad;
-    speed_max_block_f64<D, K>(load, begin, end, step, gamma, s_max, &s_bad);
+    speed_max_block_f64<D, K>(load, begin, end, step, gamma, gg, s_max, &s_bad);
     __syncthreads();
     if (threadIdx.x < K && s_max[threadIdx.x])
         atomicMax(threadIdx.x == 0 ? slot0 : slot_dir + (threadIdx.x - 1), s_max[threadIdx.x]);

@@ -45,6 +45,7 @@ struct SweepArgs {
     double gamma;
     double eps;
     float gamma_f, gm1_f, eps_f;  // the same constants in FP32, rounded on the host
+    float gg_f;          // gamma (gamma - 1) in FP32
     float inv_h_f[3];
     float2 ih23[3];      // -(2/3) / h_d as FP32 pairs hi + lo (the 2D FP32-bulk residual factor)
     int stage;           // 0, 1, 2
