@@ -927,8 +927,10 @@ __device__ __forceinline__ float wavespeed_f32(const float *q, float gamma, bool
 // est[1 + e] = |u_e| + a; gg = gamma (gamma - 1), formed from the FP64 gamma (an FP32
 // one less 1 has few bits left near 1).  Returns whether the state is certainly physical and the
 // estimates are within 2^-16 of the FP64 values: the conserved fields of ordinary
-// size and the internal energy at least 2^-5 of the total and kinetic energies
-// (its FP32 rounding is 2^-21 of those).
+// size, the internal energy at least 2^-5 of the total and kinetic energies (its FP32
+// rounding is 2^-21 of those), density and sound speed above 1e-12 (so that what FP32
+// flushes to zero on the way -- momenta below 2^-103, squares below 2^-126 -- is below
+// 2^-16 of the sound speed).
 template <int D, int K>
 __device__ __forceinline__ bool speed_estimate(const double *q, float gg, float *est)
 {
@@ -953,7 +955,7 @@ __device__ __forceinline__ bool speed_estimate(const double *q, float gg, float 
     bool in = true;
 #pragma unroll
     for (int k = 0; k < D + 2; ++k) in = in && (__double2hiint(q[k]) & 0x7FFFFFFF) < (1123 << 20);  // |q| < 2^100
-    return in && f[0] > 1e-30f && ie > 0.03125f * (fabsf(f[D + 1]) + ke) && est[0] < 1e30f;
+    return in && f[0] > 1e-12f && a > 1e-12f && ie > 0.03125f * (fabsf(f[D + 1]) + ke) && est[0] < 1e30f;
 }
 
 // max over the block of the FP64 speeds of its threads' states (K = 1: |u| + a

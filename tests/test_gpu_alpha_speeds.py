@@ -1,6 +1,7 @@
 """alpha where the FP32 estimates that pick the cells whose FP64 speeds are formed could mislead: gases with gamma near 1,
-where gamma - 1 has few bits in FP32 once 1 has been taken from an FP32 gamma.  Fast cold cells and slow hot cells of
-nearly the same speed compete for the maximum; alpha is the oracle's, bit for bit, of the state given and (through dt) of
+where gamma - 1 has few bits in FP32 once 1 has been taken from an FP32 gamma, and states whose speeds are so small that
+their squares leave the FP32 range.  Fast cold cells and slow hot cells of nearly the same speed compete for the
+maximum; alpha is the oracle's, bit for bit, of the state given and (through dt) of
 the one a step leaves."""
 import numpy as np
 import pytest
@@ -84,3 +85,15 @@ def test_alpha_of_the_state_a_step_leaves(W, n, gamma, mode):
         s.run(U, 1e30, max_steps=2, graph_steps=2)
         assert s.time()[0] == t1 + cfl * h / O.alpha(cfg, V.cpu().numpy())[0]
         s.close()
+
+
+@pytest.mark.parametrize("rho,speed", [(1e10, 1e-20), (1e6, 1e-19), (1.0, 1e-15), (1e-14, 1e-13), (1e-20, 1.0), (1e20, 1e12)])
+@pytest.mark.parametrize("n", SHAPES)
+def test_speeds_far_from_one(W, n, rho, speed):
+    rng = np.random.default_rng(3 + len(n))
+    cfg = O.Cfg(dim=len(n), n=n)
+    s = solver(W, n, 1.4)
+    for _ in range(12):
+        U = state(rng, n, 1.4, rho, speed)
+        assert alpha_of(s, U) == O.alpha(cfg, U)[0]
+    s.close()
