@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(ALPHA_NT, 2) k_alpha(const double *__restrict_
 // by memory: a thread loads four cells before it uses the first (one cell at a time
 // took 45 us at 2048 x 2048, 3 TB/s; now 28).
 template <int D>
-__global__ void __launch_bounds__(256, 4) k_alpha_bulk(const double *__restrict__ U, long long N, double gamma, Ctl *ctl,
-                                                       int per_dir, const AlphaThen then)
+__global__ void __launch_bounds__(256, 4) k_alpha_bulk(const double *__restrict__ U, long long N, float gamma, float gm1,
+                                                       Ctl *ctl, int per_dir, const AlphaThen then)
 {
     constexpr int NF = D + 2, UN = 4;
     float mf = 0.0f, mdf[D];
@@ -108,10 +108,10 @@ __global__ void __launch_bounds__(256, 4) k_alpha_bulk(const double *__restrict_
 #pragma unroll
             for (int f = 0; f < NF; ++f) qf[f] = f64_to_f32(u[k][f]);
             bool b;
-            mf = fmaxf(mf, wavespeed_f32<D>(qf, (float)gamma, b));
+            mf = fmaxf(mf, wavespeed_f32<D>(qf, gamma, gm1, b));
             if (per_dir) {
                 float sd[D];
-                dirspeeds_f32<D>(qf, (float)gamma, sd);
+                dirspeeds_f32<D>(qf, gamma, gm1, sd);
 #pragma unroll
                 for (int e = 0; e < D; ++e) mdf[e] = fmaxf(mdf[e], b ? 0.0f : sd[e]);
             }
@@ -242,11 +242,11 @@ cudaError_t launch_alpha(int model, int dim, bool bulk, const double *U, long lo
     if (model == MODEL_ADVECT) k_alpha_scalar<MODEL_ADVECT><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model == MODEL_BURGERS) k_alpha_scalar<MODEL_BURGERS><<<blocks, 256, 0, s>>>(U, N, ctl, then);
     if (model != MODEL_EULER) return cudaGetLastError();
-    const float gg = (float)(gamma * (gamma - 1.0));
+    const float gm1 = speed_gm1(gamma), gg = (float)(gamma * (gamma - 1.0));
     const int big = (int)std::min<long long>((N + ALPHA_NT - 1) / ALPHA_NT, 2 * sm_count());
 #define X(D)                                                                                        \
     if (dim == D && bulk)                                                                           \
-        k_alpha_bulk<D><<<blocks < sm_count() * 4 ? blocks : sm_count() * 4, 256, 0, s>>>(U, N, gamma, ctl, per_dir, then); \
+        k_alpha_bulk<D><<<blocks < sm_count() * 4 ? blocks : sm_count() * 4, 256, 0, s>>>(U, N, (float)gamma, gm1, ctl, per_dir, then); \
     else if (dim == D && per_dir) k_alpha<D, true><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, gg, ctl, then);   \
     else if (dim == D) k_alpha<D, false><<<big, ALPHA_NT, 0, s>>>(U, N, gamma, gg, ctl, then);
     X(1) X(2) X(3)

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
                     float qf[NF];
 #pragma unroll
                     for (int f = 0; f < NF; ++f) qf[f] = f64_to_f32(out[f]);
-                    cmaxf = fmaxf(cmaxf, wavespeed_f32<D>(qf, a.gamma_f, b));
+                    cmaxf = fmaxf(cmaxf, wavespeed_f32<D>(qf, a.gamma_f, a.gms_f, b));
                 } else {  // (one cell per thread: its speed is formed below)
                     static_assert(M != MODEL_EULER || MP <= NT, "one cell per thread");
 #pragma unroll

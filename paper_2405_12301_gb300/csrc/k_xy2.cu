@@ -455,8 +455,8 @@ __global__ void __launch_bounds__(xy2::NT, 5) k_xy2(const SweepArgs a)
         }
         const float q[NF] = {qq[0].x, qq[0].y, qq[1].x, qq[1].y};
         if (ST < 2) reinterpret_cast<float4 *>(a.dout)[cell] = cat4(dn[0], dn[1]);
-        s = wavespeed_f32<2>(q, a.gamma_f, bad);
-        if (PD && !bad) dirspeeds_f32<2>(q, a.gamma_f, sd);
+        s = wavespeed_f32<2>(q, a.gamma_f, a.gms_f, bad);
+        if (PD && !bad) dirspeeds_f32<2>(q, a.gamma_f, a.gms_f, sd);
     }
     const float v[3] = {s, sd[0], sd[1]};
     block_max_publish_f32_1b<PD ? 3 : 1>(v, bad, s_max, &s_bad, &a.ctl->alpha[a.slot_out],

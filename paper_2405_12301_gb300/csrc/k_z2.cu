@@ -335,8 +335,8 @@ __global__ void __launch_bounds__(z2::NT, 5) k_z2(const SweepArgs a)
             reinterpret_cast<float4 *>(a.dout)[(unsigned)cell] = make_float4(dn[0], dn[1], dn[2], dn[3]);
             a.dout1[(unsigned)cell] = dn[4];
         }
-        s = wavespeed_f32<3>(qn, a.gamma_f, bad);
-        if (PD && !bad) dirspeeds_f32<3>(qn, a.gamma_f, sd);
+        s = wavespeed_f32<3>(qn, a.gamma_f, a.gms_f, bad);
+        if (PD && !bad) dirspeeds_f32<3>(qn, a.gamma_f, a.gms_f, sd);
     }
     const float v[4] = {s, sd[0], sd[1], sd[2]};
     block_max_publish_f32_1b<PD ? 4 : 1>(v, bad, s_max, &s_bad, &a.ctl->alpha[a.slot_out],

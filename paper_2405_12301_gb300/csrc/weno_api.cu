@@ -239,6 +239,7 @@ static SweepArgs base_args(weno_ctx *h)
     a.eps = h->p.eps_weno;
     a.gamma_f = (float)h->p.gamma;
     a.gm1_f = (float)(h->p.gamma - 1.0);
+    a.gms_f = speed_gm1(h->p.gamma);
     a.gg_f = (float)(h->p.gamma * (h->p.gamma - 1.0));
     a.eps_f = (float)h->p.eps_weno;
     for (int d = 0; d < 3; ++d) {

@@ -880,8 +880,9 @@ __device__ __forceinline__ void dirspeeds_f64(const double *q, double gamma, dou
     for (int e = 0; e < D; ++e) sd[e] = __dadd_rn(fabs(__ddiv_rn(q[1 + e], rho)), a);
 }
 
+// (gm1: speed_gm1)
 template <int D>
-__device__ __forceinline__ void dirspeeds_f32(const float *q, float gamma, float *sd)
+__device__ __forceinline__ void dirspeeds_f32(const float *q, float gamma, float gm1, float *sd)
 {
     const float rho = q[0];
     const float ir = 1.0f / rho;
@@ -891,7 +892,7 @@ __device__ __forceinline__ void dirspeeds_f32(const float *q, float gamma, float
         const float ue = q[1 + e] * ir;
         u2 += ue * ue;
     }
-    const float p = (gamma - 1.0f) * (q[D + 1] - 0.5f * rho * u2);
+    const float p = gm1 * (q[D + 1] - 0.5f * rho * u2);
     const float a = sqrtf(gamma * p * ir);
 #pragma unroll
     for (int e = 0; e < D; ++e) sd[e] = fabsf(q[1 + e] * ir) + a;
@@ -908,7 +909,7 @@ __device__ __forceinline__ float sqrt_approx(float x)
 }
 
 template <int D>
-__device__ __forceinline__ float wavespeed_f32(const float *q, float gamma, bool &bad)
+__device__ __forceinline__ float wavespeed_f32(const float *q, float gamma, float gm1, bool &bad)
 {
     const float rho = q[0];
     const float ir = fast_rcp(rho);
@@ -918,7 +919,7 @@ __device__ __forceinline__ float wavespeed_f32(const float *q, float gamma, bool
         const float ue = q[1 + e] * ir;
         u2 += ue * ue;
     }
-    const float p = (gamma - 1.0f) * (q[D + 1] - 0.5f * rho * u2);
+    const float p = gm1 * (q[D + 1] - 0.5f * rho * u2);
     bad = !(rho > 0.0f) || !(p > 0.0f) || !isfinite(u2) || !isfinite(q[D + 1]);
     return bad ? 0.0f : sqrt_approx(u2) + sqrt_approx(gamma * p * ir);
 }

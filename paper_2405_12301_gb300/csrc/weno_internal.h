@@ -46,6 +46,7 @@ struct SweepArgs {
     double eps;
     float gamma_f, gm1_f, eps_f;  // the same constants in FP32, rounded on the host
     float gg_f;          // gamma (gamma - 1) in FP32
+    float gms_f;         // gamma - 1 of the FP32 wavespeeds (speed_gm1)
     float inv_h_f[3];
     float2 ih23[3];      // -(2/3) / h_d as FP32 pairs hi + lo (the 2D FP32-bulk residual factor)
     int stage;           // 0, 1, 2
@@ -56,6 +57,11 @@ struct SweepArgs {
     Tile64 txy, tz;      // k_xy64, k_z: the handle's tiles
     int per_dir;         // LF alpha per direction (alpha_dir slots) instead of one global alpha
 };
+
+// gamma - 1 of the FP32 wavespeeds: the FP32 gamma less 1, good to 2^-21 from 1.25 up
+// (alpha and dt keep their bits there), and the rounded FP64 difference below, where the
+// FP32 one loses its bits (none left at 1 + 1e-8).
+inline float speed_gm1(double gamma) { return gamma < 1.25 ? (float)(gamma - 1.0) : (float)gamma - 1.0f; }
 
 // Launches the sweep of direction dir for a dim-dimensional grid.
 cudaError_t launch_sweep(int model, int dim, int dir, bool bulk, int epi, const SweepArgs &a, cudaStream_t s);

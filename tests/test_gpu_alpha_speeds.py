@@ -1,8 +1,8 @@
 """alpha where the FP32 estimates that pick the cells whose FP64 speeds are formed could mislead: gases with gamma near 1,
 where gamma - 1 has few bits in FP32 once 1 has been taken from an FP32 gamma, and states whose speeds are so small that
 their squares leave the FP32 range.  Fast cold cells and slow hot cells of nearly the same speed compete for the
-maximum; alpha is the oracle's, bit for bit, of the state given and (through dt) of
-the one a step leaves."""
+maximum; alpha is the oracle's, bit for bit, of the state given and (through dt) of the one a step leaves.  FP32-bulk:
+within 2^-18 (its speeds are sums of FP32 roundings of a few ulp)."""
 import numpy as np
 import pytest
 
@@ -62,6 +62,29 @@ def test_gamma_near_one(W, n, gamma):
     for _ in range(24):
         U = state(rng, n, gamma)
         assert alpha_of(s, U) == O.alpha(cfg, U)[0]
+    s.close()
+
+
+@pytest.mark.parametrize("gamma", [1.4, 1.01, 1.001, 1.0001, 1.00001, 1 + 1e-8])
+@pytest.mark.parametrize("n", SHAPES)
+def test_gamma_near_one_fp32_bulk(W, n, gamma):
+    rng = np.random.default_rng(len(n))
+    cfg = O.Cfg(dim=len(n), n=n, gamma=gamma)
+    h, cfl = 1.0 / max(n), 1e-9
+    s = solver(W, n, gamma, precision=W.FP32_BULK, cfl=cfl)
+    for _ in range(24):
+        U = state(rng, n, gamma)
+        want = O.alpha(cfg, U)[0]
+        assert abs(alpha_of(s, U) - want) <= 2.0 ** -18 * want
+    if gamma < 1.001:  # (the jumps of E, ~1 / (gamma - 1), to the eighth power leave the FP32 range of the weights)
+        return s.close()
+    t, Ud = [], [torch.from_numpy(U).cuda() for _ in range(2)]
+    for k in range(2):  # and of the state a step leaves, through the second step's dt
+        s.set_time(0.0)
+        s.run(Ud[k], 1e30, max_steps=k + 1, graph_steps=k + 1)
+        t.append(s.time()[0])
+    want = O.alpha(cfg, Ud[0].cpu().numpy())[0]
+    assert abs(cfl * h / (t[1] - t[0]) - want) <= 2.0 ** -18 * want
     s.close()
 
 
