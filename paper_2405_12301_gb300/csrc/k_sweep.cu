@@ -40,6 +40,10 @@ template <int M, int DIR> struct Tile { static constexpr int W = 32, S = 26, P =
 template <int M> struct Tile<M, 0> {  // x: rows; a scalar's runs need 1024 points to fill the warps
     static constexpr int W = 32, S = 250, P = M == MODEL_EULER ? NT : 1024;
 };
+// FP32-bulk: a row's points lie within 124 cells of its reference, the middle cell (the
+// rounding errors of L(U) grow with that distance: 250 cells with the reference in the
+// first have twice the error of 243 cells at 200000 cells).
+constexpr int BULK_S = 243;
 
 constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
@@ -116,13 +120,13 @@ __global__ void __launch_bounds__(NT, 4) k_sweep(const SweepArgs a)
     const double gm1 = a.gamma - 1.0;
     const T eps = BULK ? (T)a.eps_f : (T)a.eps;
 
-    // ---- phase 0 (FP32-bulk): reference state of every line
+    // ---- phase 0 (FP32-bulk): reference state of every line, its middle cell's
     if constexpr (BULK) {
         for (int w = threadIdx.x; w < W; w += NT) {
             long long base;
             const bool ok = line(w, base);
             double q[NF];
-            const int cr = c0 < n ? c0 : n - 1;
+            const int cr = c0 + S / 2 < n ? c0 + S / 2 : n - 1;
 #pragma unroll
             for (int f = 0; f < NF; ++f)
                 q[f] = ok ? a.U[f * N + base + (long long)cr * st] : (f == 0 || f == NF - 1 ? 1.0 : 0.0);
@@ -333,15 +337,16 @@ static inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b
 // tiles for every SM, and on small grids shorter segments for the same reason (a row
 // costs 6 halo points per segment, so not below 20 cells).  Advection at 128^3, x:
 // 7 rows of 128 cells (210 runs, the warps full); 3 rows of 64 (48 runs) took 164 us.
-// In 1D a tile is 250 cells, a point per thread.
-template <int M, int DIR> static void sweep_tile(SweepArgs &a)
+// In 1D a tile is 250 cells (FP32-bulk: 243), a point per thread.
+template <int M, int DIR, bool BULK> static void sweep_tile(SweepArgs &a)
 {
     const int n = a.n[DIR];
     if (DIR == 0) {
         const long long rows = (long long)a.n[1] * a.n[2];
         const long long want = rows == 1 ? sm_count() : 4ll * sm_count();  // (a 1D tile is one row: a CTA per SM fills its warps best)
         long long most = (n * rows + want - 1) / want;
-        most = most < 20 ? 20 : most > Tile<M, 0>::S ? Tile<M, 0>::S : most;
+        constexpr int longest = BULK ? BULK_S : Tile<M, 0>::S;
+        most = most < 20 ? 20 : most > longest ? longest : most;
         a.tile_s = (int)cdiv(n, cdiv(n, most));
         long long w = Tile<M, 0>::P / (a.tile_s + 6), share = rows * cdiv(n, a.tile_s) / (2ll * sm_count());
         share = share < 2 ? 2 : share;  // (2 rows keep the grid's y extent in range)
@@ -358,7 +363,7 @@ template <int M, int D, int DIR, bool BULK, int EPI>
 static cudaError_t launch_t(SweepArgs a, cudaStream_t s)
 {
     using L = Layout<M, D, DIR, BULK>;
-    sweep_tile<M, DIR>(a);
+    sweep_tile<M, DIR, BULK>(a);
     dim3 grid;
     if (DIR == 0) grid = dim3(cdiv(a.n[0], a.tile_s), cdiv(a.n[1], a.tile_w), (unsigned)a.n[2]);
     else if (DIR == 1) grid = dim3(cdiv(a.n[0], a.tile_w), cdiv(a.n[1], a.tile_s), (unsigned)a.n[2]);
