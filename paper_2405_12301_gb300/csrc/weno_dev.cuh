@@ -417,14 +417,14 @@ __device__ __forceinline__ double rcp_f64(double x)
 // The smoothness parameter as the pair formula takes it.
 struct PairEps {
     double eps;
-    float2 g;  // 4 eps as a pair
+    float2 g;  // 4 eps as a pair; infinite (every window is rough) from eps = 2^60 on, where pairs end
     int thr;   // high word of a double near 2^-30 sqrt(4 eps)
 };
 __device__ __forceinline__ PairEps pair_eps(double eps)
 {
     PairEps P;
     P.eps = eps;
-    P.g = split_sat(4.0 * eps);
+    P.g = __double2hiint(eps) < (1083 << 20) ? split_sat(4.0 * eps) : make_float2(__int_as_float(0x7F800000), 0.0f);
     P.thr = ((__double2hiint(eps) - 0x3FF00000) >> 1) + 0x3FF00000 - (29 << 20);
     return P;
 }
@@ -569,7 +569,8 @@ static __device__ __noinline__ double weno5_rough(double v0, double v1, double v
     const float mn = fminf(G0.a, fminf(G1.a, G2.a)), sum = G0.a + G1.a + G2.a;
     const float sc = __uint_as_float(0x75000000u - (__float_as_uint(mn) & 0x7F800000u));
     const float big = fmaxf(fmaxf(fabsf(d1.a), fabsf(d2.a)), fmaxf(fabsf(d3.a), fabsf(d4.a)));
-    if (!(mn > 0x1p-80f) || !(sum < 0x1p100f) || !(sum * sc < 0x1p66f) || !(big > 0x1p-60f))
+    if (!(mn > 0x1p-80f) || !(sum < 0x1p100f) || !(sum * sc < 0x1p66f) || !(big > 0x1p-60f) ||
+        __double2hiint(eps) >= (1083 << 20))  // eps of 2^60 and more
         return weno5_diffs(D1, D2, D3, D4, v2, eps);
     auto scaled = [&](Tri G) {
         const float x = __fmul_rn(G.a, sc);
