@@ -1,6 +1,6 @@
 """The FP64 WENO5 value at the edges of the FP32 pairs' range: a smoothness parameter beyond what an FP32 number's square
-holds.  The reference and the tolerance are those of test_gpu_weno_pairs.py, without its allowance for terms below
-2^-30 sqrt(4 eps)."""
+holds, and fields far below sqrt(eps), where the weights are the linear ones.  The reference and the tolerance are those
+of test_gpu_weno_pairs.py, without its allowance for terms below 2^-30 sqrt(4 eps)."""
 import numpy as np
 import pytest
 
@@ -32,3 +32,11 @@ def check(W, u, eps):
 def test_large_eps(W, kind, eps, over):
     n = 300
     check(W, P.field(kind, n, np.random.default_rng(n)) * over * np.sqrt(eps), eps)
+
+
+@pytest.mark.parametrize("kind", ["wave", "zero mean", "front", "shock", "jumps", "noise", "wide range"])
+@pytest.mark.parametrize("eps", [1e-6, 1.0, 1e6, 1e-30])
+@pytest.mark.parametrize("below", [2.0 ** -25, 2.0 ** -28, 2.0 ** -29, 2.0 ** -30, 2.0 ** -31, 2.0 ** -32, 2.0 ** -34, 2.0 ** -50])
+def test_fields_below_sqrt_eps(W, kind, eps, below):
+    n = 301
+    check(W, P.field(kind, n, np.random.default_rng(n)) * below * np.sqrt(eps), eps)
