@@ -375,7 +375,7 @@ extern "C" int weno_maxvol(weno_handle h, const weno_maxvol_problem *probs, int3
     MaxvolDesc *dd = (MaxvolDesc *)(base + off_desc);
     CK(h, cudaMemcpyAsync(dd, ds.data(), sizeof(MaxvolDesc) * n_probs, cudaMemcpyHostToDevice, h->stream));
     CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, n_probs, max_r, max_nr, delta, max_iters, h->stream); },
-                 maxvol_launches(max_nr)));
+                 maxvol_launches(max_nr, delta)));
     std::vector<int> st(2 * n_probs);
     CK(h, cudaMemcpyAsync(st.data(), ints, sizeof(int) * 2 * n_probs, cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
@@ -530,7 +530,7 @@ extern "C" int weno_tt_cross(weno_handle h, const weno_tt_instance *inst, int32_
         maxvol_order(md.data(), np);
         MaxvolDesc *dd = (MaxvolDesc *)slot(3);
         CK(h, cudaMemcpyAsync(dd, md.data(), sizeof(MaxvolDesc) * np, cudaMemcpyHostToDevice, h->stream));
-        CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, np, mr, mnr, delta, 200, h->stream); }, maxvol_launches(mnr)));
+        CK(h, launch(h, 1, h->stream, [&] { return launch_maxvol(dd, np, mr, mnr, delta, 200, h->stream); }, maxvol_launches(mnr, delta)));
         ++mv_call;
         return WENO_OK;
     };

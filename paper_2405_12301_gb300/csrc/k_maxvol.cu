@@ -638,8 +638,13 @@ static int maxvol_cluster_size()
     return ncl;
 }
 
-static bool maxvol_in_f64(long long max_nr) { return max_nr <= 4096ll * maxvol_cluster_size(); }
-int maxvol_launches(long long max_nr) { return maxvol_in_f64(max_nr) ? 3 : 5; }
+// FP64 swaps: for small matrices (launch_maxvol), and where delta is within 2^10 of the
+// pairs' 2^-46 -- an entry of a selected row, 1 but for its rounding, would pass for a swap.
+static bool maxvol_in_f64(long long max_nr, double delta)
+{
+    return delta < 0x1p-36 || max_nr <= 4096ll * maxvol_cluster_size();
+}
+int maxvol_launches(long long max_nr, double delta) { return maxvol_in_f64(max_nr, delta) ? 3 : 5; }
 
 // max_nr: the largest n r of the batch.  Shared memory for a slice: what the
 // largest slice takes, and no more than lets the batch's CTAs run together.
@@ -665,7 +670,7 @@ cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_n
     // than in pairs, but the inverse and the final product (18-23 us) fall away; at 4096
     // entries a CTA that is ~1 us a swap.  A call on 8 matrices of up to 1233 x 9: 176 us in
     // pairs, 147 in FP64.
-    if (maxvol_in_f64(max_nr)) return launch_cluster(k_maxvol_swap<true>, ncl, n, smem, s, d, delta, max_iters, doubles);
+    if (maxvol_in_f64(max_nr, delta)) return launch_cluster(k_maxvol_swap<true>, ncl, n, smem, s, d, delta, max_iters, doubles);
     e = launch_cluster(k_maxvol_swap<false>, ncl, n, smem, s, d, delta, max_iters, doubles);
     if (e != cudaSuccess) return e;
     k_maxvol_inverse<<<n, 256, sizeof(double) * max_r * (2 * max_r + 1), s>>>(d);

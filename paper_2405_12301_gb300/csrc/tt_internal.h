@@ -103,7 +103,7 @@ struct MaxvolDesc {
     int *swaps;
     int n, r;
 };
-int maxvol_launches(long long max_nr);  // kernels of one launch_maxvol
+int maxvol_launches(long long max_nr, double delta);  // kernels of one launch_maxvol
 // Orders a batch largest first (n r^2), so the biggest matrices start first.
 void maxvol_order(MaxvolDesc *d, int n);
 cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_nr, double delta, int max_iters,
