@@ -406,8 +406,16 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     }
     for (int t = threadIdx.x; t < pk; t += TT_NT) perm[t] = t;
     __syncthreads();
+    // T over a power of four near its largest entry, so that the squares that Jacobi
+    // works on stay normal whatever T's scale is (a T of norm 1e-146 left its small
+    // columns, of norms below 2^-511, unrotated; exact, so no bit of the result moves
+    // where nothing underflowed); the singular values are scaled back at the end
+    const int e4 = max(-1000, min(1000, (s_exp - 1023) & ~1));
+    const double down = __hiloint2double((1023 - e4) << 20, 0), up = __hiloint2double((1023 + e4) << 20, 0);
+    for (int e = threadIdx.x; e < pk * q; e += TT_NT) A[(e / q) * lda + e % q] *= down;
+    __syncthreads();
     // FP32 value of x over the power of two of T's largest entry (0 below 2^-60 of it)
-    const int eoff = s_exp - 1023;
+    const int eoff = s_exp - 1023 - e4;
     auto relative = [&](double x) {
         const int h = __double2hiint(x), ex = ((h >> 20) & 0x7FF) - eoff;
         const unsigned b = ((unsigned)(ex - 896) << 23) | (((unsigned)h & 0xFFFFFu) << 3) | ((unsigned)__double2loint(x) >> 29);
@@ -635,11 +643,11 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
             for (int t = pk - 1; t >= 0; --t) s2 += sig[ord[t]] * sig[ord[t]];
             delta = d.eps / sqrt(2.0) * sqrt(s2);
             if (rank == 0) {
-                d.delta[0] = delta;
-                d.delta[1] = sqrt(s2);
+                d.delta[0] = delta * up;
+                d.delta[1] = sqrt(s2) * up;
             }
         } else {
-            delta = d.delta[0];
+            delta = d.delta[0] * down;
         }
         // smallest r >= 1 whose discarded singular values have a 2-norm <= delta
         int r = pk;
@@ -658,14 +666,14 @@ __global__ void __launch_bounds__(TT_NT) k_svd_jacobi(const SvdDesc *descs)
     __syncthreads();
     const int r = s_rank;
     if (rank == 0)
-        for (int t = threadIdx.x; t < pk; t += TT_NT) d.sv[t] = sig[ord[t]];
+        for (int t = threadIdx.x; t < pk; t += TT_NT) d.sv[t] = sig[ord[t]] * up;
     // left vectors: rows P of Z over sigma.  A zero column (only kept when T has fewer
     // nonzero singular values than the rank) gets an orthonormal direction below.
     for (int e = threadIdx.x; e < pn * r; e += TT_NT) {
         const int i = e / r, c = e - i * r, t = ord[c];
         const double s = sig[t];
         d.Vsel[(long long)perm[pa + i] * d.ld_out + c] = s > 0.0 ? M[t * ldm + i] / s : 0.0;
-        d.Wt[(long long)(pa + i) * d.ld_out + c] = M[t * ldm + pn + i] * s;
+        d.Wt[(long long)(pa + i) * d.ld_out + c] = M[t * ldm + pn + i] * (s * up);
     }
     __threadfence();
     cl.sync();  // J sigma is complete (and no CTA reads another's shared memory any more)
