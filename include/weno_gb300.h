@@ -405,7 +405,8 @@ typedef struct {
  * flags); the selection and the cores are FP64.  inst, probs: HOST arrays;
  * synchronises once at the end.  Uses the handle's gamma and eps_weno.
  * Errors: WENO_ERR_ARG for bad ranks, null pointers or a fiber matrix of rank
- * below the cross rank; those of weno_cross_eval. */
+ * below the cross rank; WENO_ERR_UNSUPPORTED when a fiber matrix has more than
+ * 65536 rows (n1, r1 n2, 5 n3 or n2 r2); those of weno_cross_eval. */
 int weno_tt_cross(weno_handle h, const weno_tt_instance *inst, int32_t n_inst, int32_t flux_dir,
                   weno_tt_cross_problem *probs, int32_t sweeps, double delta, int32_t flags);
 

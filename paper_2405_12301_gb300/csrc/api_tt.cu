@@ -428,6 +428,8 @@ extern "C" int weno_tt_cross(weno_handle h, const weno_tt_instance *inst, int32_
         if (x.r1 < 1 || x.r1 > MV_RMAX || x.r1 > n1 || x.r1 > 5 * n2 * n3 || x.r2 < 1 || x.r2 > MV_RMAX ||
             x.r2 > (long long)x.r1 * n2 || x.r2 > 5 * n3 || x.r1 > n2 * x.r2)
             return fail(h, WENO_ERR_ARG, "weno_tt_cross: need 1 <= r1 <= min(n1, n2 r2, 64), 1 <= r2 <= min(r1 n2, 5 n3, 64)");
+        if (std::max({n1, x.r1 * n2, 5 * n3, n2 * x.r2}) > MV_NMAX)
+            return fail(h, WENO_ERR_UNSUPPORTED, "weno_tt_cross: n1, r1 n2, 5 n3 and n2 r2 may be 65536 at most");
         if (!P.J1 || !P.J2 || !P.I1 || !P.I2 || !P.core[0] || !P.core[1] || !P.core[2])
             return fail(h, WENO_ERR_ARG, "weno_tt_cross: null index set or core");
         max_r = std::max({max_r, x.r1, x.r2});
