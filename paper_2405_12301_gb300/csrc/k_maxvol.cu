@@ -16,10 +16,13 @@
 // A is ill-conditioned: |L| <= 1 under partial pivoting, and the scale of
 // A's columns stays in U.  The swaps only choose rows: their rank-one updates
 // would hold the FP64 pipe for n r instructions each (12000 x 32: 15 us a swap
-// on 8 SMs), while a choice that the pairs' 2^-46 could change is a tie for FP64
-// rounding as well; the final B is one FP64 product of the accurate B of step 2
-// with the inverse of a well-conditioned matrix, without the swaps' accumulated
-// rounding.  Phases 1 and 3 are sequences of (argmax, rank-one
+// on 8 SMs).  Entries closer than the pairs' 2^-46 may be taken in another order than
+// FP64 swaps would; equal rows stay equal bit for bit, so ties go to the first entry, and
+// a delta too small for pairs takes FP64 swaps.  The final B is one FP64 product of the
+// accurate B of step 2 with the inverse of its rows I, without the swaps' accumulated
+// rounding: the inverse's entries are those of the final B (1 + delta at most once the
+// swaps have ended), so its error is that of a sum of r products of B's entries, bounded
+// by the elimination's growth as B's own error is.  Phases 1 and 3 are sequences of (argmax, rank-one
 // update) steps.  Each matrix gets a thread-block cluster whose CTAs own
 // contiguous slices of its rows, held in shared memory as far as they fit (a slice
 // in L2 costs a round trip per step and column batch) and in W beyond.  Per step
@@ -47,6 +50,7 @@ namespace wg {
 namespace cg = cooperative_groups;
 
 constexpr int MV_NT = 512, MV_NW = MV_NT / 32;
+constexpr int MV_ROWS = 64;  // rows that a CTA of a cluster gets at least (launch_maxvol)
 // A pivot |w| <= MV_RANK_TOL r max_i |A[i][j]| counts as zero: the residual
 // of a column that lies in the span of the earlier ones is a few rounding
 // errors of the column's own scale (a full-rank matrix reaches it only with a
@@ -189,7 +193,10 @@ __global__ void __launch_bounds__(MV_NT) k_maxvol_pivot(const MaxvolDesc *descs,
     row_slice(n, rank, ncl, lo, hi);
     __shared__ MvStep st;
     __shared__ int I[MV_RMAX];
-    __shared__ unsigned chosen[MV_NMAX / 8 / 32];  // rows of this slice already picked (slices have <= n/8 + 1 rows)
+    // rows of this slice already picked: a slice has MV_NMAX / 8 rows at most on 8 CTAs or
+    // more, and fewer than 2 MV_ROWS r on a cluster that launch_maxvol halved below 8
+    static_assert(2 * MV_ROWS * MV_RMAX <= MV_NMAX / 8, "chosen holds a slice's rows");
+    __shared__ unsigned chosen[MV_NMAX / 8 / 32];
     __shared__ int s_fail;
     __shared__ unsigned long long cbits[MV_RMAX];  // this CTA's column maxima of |A| (bit patterns)
     __shared__ double ctol[MV_RMAX];
@@ -653,10 +660,10 @@ cudaError_t launch_maxvol(const MaxvolDesc *d, int n, int max_r, long long max_n
 {
     cudaError_t e = maxvol_attributes();
     if (e != cudaSuccess) return e;
-    // at least 64 rows to a CTA: below, the cluster barriers of a step cost more than its
+    // at least MV_ROWS rows to a CTA: below, the cluster barriers of a step cost more than its
     // pass over the rows
     int ncl = maxvol_cluster_size();
-    while (ncl > 2 && max_nr < 64ll * ncl * max_r) ncl /= 2;
+    while (ncl > 2 && max_nr < (long long)MV_ROWS * ncl * max_r) ncl /= 2;
     const long long per_sm = std::min(3ll, std::max(1ll, ((long long)n * ncl + sm_count() - 1) / sm_count()));
     const long long want = sizeof(double) * std::max((max_nr + ncl - 1) / ncl + max_r, 2ll * max_r * max_r);
     const long long least = sizeof(double) * 2ll * max_r * max_r;  // L[I] and its inverse

@@ -15,7 +15,8 @@
 //      SSP-RK3 stage combination (Eq. tt-ssprk3 without rounding) and
 //      publishes the wavespeed max of the new state for the next stage's alpha.
 //
-// FP64 mode computes everything in FP64.  FP32-bulk mode computes phases A-C
+// FP64 mode computes everything in FP64 but the WENO weights (FP32 pairs and triples at
+// FP64's accuracy, weno5_slide_pair).  FP32-bulk mode computes phases A-C
 // in FP32 on differences from a per-line reference state (exact to FP32
 // relative precision of the differences), and only the final state update
 // U^(k+1) = U^(k) + D is an FP64 add.
@@ -380,7 +381,7 @@ static cudaError_t attr_t()
                                 (int)L::bytes);
 }
 
-// Euler: 1D grids only (2D and 3D grids run in the fused k_xy and k_z kernels).
+// Euler: 1D grids only (2D and 3D grids run in the fused k_xy* and k_z* kernels).
 // Scalar laws (FP64): every direction; the first stores, the middle one of 3D
 // adds, the last runs the residual or stage epilogue.
 #define WG_SWEEP_TABLE(X)                                                                       \

@@ -24,7 +24,8 @@
 //   * k_tt_build / k_tt_contract / k_tt_gemm_tr: the TT sum's first and last
 //     unfoldings, the block-diagonal middle core times a triangular factor, and
 //     a small dense product.
-// All arithmetic is FP64.
+// All sums, factors and vectors are FP64.  FP32 only steers: the pivot norms and the
+// tangents of the Jacobi angles (k_svd_jacobi), and the seeds of Newton iterations.
 #include <algorithm>
 #include <cfloat>
 

@@ -1,5 +1,5 @@
 // k_z.cu -- z direction of the FP64 WENO5-JS residual for 3D grids, ending the
-// residual of a stage (the x and y directions run in k_xy.cu; FP32-bulk's z
+// residual of a stage (the x and y directions run in k_xy64.cu; FP32-bulk's z
 // direction is k_z2.cu).
 #include <algorithm>
 

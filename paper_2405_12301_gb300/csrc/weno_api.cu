@@ -282,14 +282,15 @@ static int enqueue_sweeps(weno_ctx *h, SweepArgs a, int last, cudaStream_t s)
     return WENO_OK;
 }
 
-// One SSP-RK3 step (Eq. tt-ssprk3 without rounding) on U in place, begun already; its
-// end begins the next if `more`.  Capturable: no host synchronisation.
-// small 1D FP64 Euler grids run whole steps inside one kernel
+// Small 1D FP64 Euler grids run whole steps inside one kernel.
 static bool runs_1d(const weno_ctx *h)
 {
     return h->dim == 1 && !bulk(h) && h->p.model == WENO_MODEL_EULER && run1d_takes(h->n[0]);
 }
 
+// One SSP-RK3 step (Eq. tt-ssprk3 without rounding) on U in place, begun already; its
+// end begins the next if `more`.  (k_run1d begins and ends its steps itself: nothing is
+// begun for it, and `more` says nothing.)  Capturable: no host synchronisation.
 static int enqueue_step(weno_ctx *h, double *U, bool more, cudaStream_t s)
 {
     if (runs_1d(h)) {

@@ -401,7 +401,8 @@ __device__ __forceinline__ double pr_f64(float a, float b, float c)
 
 // 1 / x of a normal x below 2^1021: an FP32 reciprocal of the mantissa, two
 // Newton-Raphson steps r (2 - x r) (4 FP64 instructions; a division takes ~9).
-// Within an ulp: the last step's error term is exact to 2^-44.
+// The last step forms r (1 + e), e ~ 2^-46, in one rounding and drops e^2, so the
+// result is the correctly rounded one but within 2^-38 of a tie (20 million random x: all).
 __device__ __forceinline__ double rcp_f64(double x)
 {
     const unsigned h = (unsigned)__double2hiint(x);

@@ -23,3 +23,9 @@ def test_small_delta(W, n, r, delta):
     assert delta == 0.0 or swaps == so
     B = B.cpu().numpy()
     assert np.abs(B).max() <= 1 + max(delta, 1e-13)
+
+
+@pytest.mark.parametrize("n", [32767, 16383, 16384])
+def test_longest_slices(W, n):
+    """A rank-1 matrix beside one of rank 64: slices of up to 8192 rows, all that a CTA's row mask holds."""
+    M.check(W, [M.matrix(n, 1, 2), M.matrix(64, 64, 3)])
